@@ -1,16 +1,15 @@
 // qgemm.cu — eq. (1): 8-bit code products with 32-bit accumulators, offset terms and recovery.
 //
-// Datapath. sm_103a accepts no 8-bit integer tcgen05 MMA, so the exact integer product runs on
-// the warp-level integer tensor-core instruction mma.sync m16n8k32 (u8 x u8 -> s32). Tiles of
-// 128 x 128 outputs, K in steps of 64 bytes, a four-stage cp.async pipeline into padded shared
-// memory rows (80-byte stride: the 16-byte ldmatrix rows of eight consecutive rows hit disjoint
-// banks), ldmatrix fragment loads, eight warps of 64 x 32 outputs each.
+// Datapath for a few rows of A. sm_103a accepts no 8-bit integer tcgen05 MMA, so the exact integer
+// product runs on the warp-level integer tensor-core instruction mma.sync m16n8k32 (u8 x u8 ->
+// s32), with both operands streamed straight from global memory into its fragments.
 //
 // Epilogue (fused): S = acc + zw*rsA[m] + za[m]*csW[n] + K*za*zw in 64-bit integers (eq. 1 with
 // V'' = V' + round(Q Vmin)), then y = S / (Qa Qw) + bias (eq. 3 recovery and Fig. 1's bias), and
 // optionally the raw accumulator.
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "qnn_device.cuh"
 #include "qnn_host.h"
@@ -18,29 +17,7 @@
 namespace qnn {
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 4, THREADS = 256;
-constexpr int SROW = BK + 16;  // padded shared-memory row (bytes)
-constexpr int TILE_BYTES = BM * SROW;  // same for the BN side
-constexpr int SMEM_BYTES = STAGES * 2 * TILE_BYTES;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
+constexpr int kWarps = 8, THREADS = 32 * kWarps;
 
 __device__ __forceinline__ void mma_u8(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -50,125 +27,162 @@ __device__ __forceinline__ void mma_u8(int (&d)[4], const uint32_t (&a)[4], uint
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Copies a BM x BK byte tile (rows r0.., bytes k0..) of a row-major u8 matrix into shared memory.
-// Bytes past `rows` or `K` are zero so they add nothing to the integer sums.
-template <bool kAligned>
-__device__ __forceinline__ void load_tile(uint32_t sdst, const uint8_t *__restrict__ g, int64_t ld, int64_t rows,
-                                          int64_t r0, int64_t K, int64_t k0) {
-#pragma unroll
-    for (int i = 0; i < (BM * BK / 16) / THREADS; ++i) {
-        const int c = threadIdx.x + i * THREADS;
-        const int r = c >> 2, ch = c & 3;
-        const int64_t gr = r0 + r, gk = k0 + ch * 16;
-        int valid = 0;
-        if (gr < rows) {
-            int64_t rem = K - gk;
-            valid = rem <= 0 ? 0 : (rem >= 16 ? 16 : (int)rem);
-        }
-        const uint32_t d = sdst + r * SROW + ch * 16;
-        if (kAligned) {
-            const uint8_t *src = valid ? g + gr * ld + gk : g;
-            cp_async16(d, src, valid);
+// 16 codes at p of which the first `valid` lie inside the row (the rest read as 0, which adds nothing
+// to the sums). AL is the alignment every row start of the matrix has (16, 4 or 1 bytes).
+template <int AL, bool kStream>
+__device__ __forceinline__ uint4 ld_codes16(const uint8_t *__restrict__ p, int valid) {
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (valid >= 16) {
+        if constexpr (AL == 16) {
+            if constexpr (kStream)
+                asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                    : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                    : "l"(p));
+            else
+                v = __ldg(reinterpret_cast<const uint4 *>(p));
+        } else if constexpr (AL == 4) {
+            const uint32_t *w = reinterpret_cast<const uint32_t *>(p);
+            v = make_uint4(__ldg(w), __ldg(w + 1), __ldg(w + 2), __ldg(w + 3));
         } else {
-            uint32_t w[4] = {0, 0, 0, 0};
-            const uint8_t *src = g + gr * ld + gk;
-            for (int b = 0; b < valid; ++b) w[b >> 2] |= (uint32_t)__ldg(src + b) << ((b & 3) * 8);
-            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(d), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]));
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                w[i] = (uint32_t)__ldg(p + 4 * i) | (uint32_t)__ldg(p + 4 * i + 1) << 8 |
+                       (uint32_t)__ldg(p + 4 * i + 2) << 16 | (uint32_t)__ldg(p + 4 * i + 3) << 24;
+            v = make_uint4(w[0], w[1], w[2], w[3]);
         }
+    } else if (valid > 0) {
+        uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i < valid) w[i >> 2] |= (uint32_t)__ldg(p + i) << (8 * (i & 3));
+        v = make_uint4(w[0], w[1], w[2], w[3]);
     }
+    return v;
 }
 
-template <bool kAligned>
-__global__ void __launch_bounds__(THREADS) qgemm_imma_kernel(
+// The product for a few rows of A: 16 MT rows of W x 8 NT rows of A per block, K spread over the
+// block's warps. W is the m16 side of mma.sync m16n8k32, so eight rows of A cost one instruction's
+// columns and a single row wastes columns, not loads. Each warp takes every kWarps-th 64-code chunk
+// of K: lane (g, tq) loads 16 consecutive codes (offset 16 tq) of rows g and g + 8 of W and of row g
+// of A, and uses words 0-1 and 2-3 as the fragments of two MMAs. Both operands permute k the same way,
+// so the sums are the same integers; nothing passes through shared memory but the warps' partial sums,
+// which integer atomics add exactly in any order.
+//
+// Bound: the bytes of W once (N K), and at small sizes the latency of one load round, the reduction
+// and the epilogue. Sixteen rows a block because tiles of 128 rows leave a 2048-row W on 16 of 152
+// SMs with 32 serial k-steps. Event-timed, 128-row tiles against this split: M = 1, 2048 x 2048 84 ->
+// 8.2 us; M = 100, 2000 x 500 (rows 4-byte aligned) 67 -> 14 us. M = 1, 8192 x 8192: 16.3 us a call,
+// 4.1 TB/s (20.5 us with three blocks an SM, whose last wave is nearly empty; four chunks in flight
+// a warp with four blocks an SM gain nothing more).
+template <int NT, int MT, int AL>
+__global__ void __launch_bounds__(THREADS, NT == 1 ? 4 : NT == 2 ? 3 : NT == 4 ? 2 : 1) qgemm_imma_kernel(
     const uint8_t *__restrict__ A, int64_t lda, const qnn_qparams *__restrict__ pa, int a_per_row,
-    const int32_t *__restrict__ rsA, int64_t M, int64_t K, const uint8_t *__restrict__ W, int64_t ldw,
+    const int32_t *__restrict__ rsA, int64_t M, int K, const uint8_t *__restrict__ W, int64_t ldw,
     const qnn_qparams *__restrict__ pw, int64_t rows_per_block, const int32_t *__restrict__ csW, int64_t N,
-    const float *__restrict__ bias, float *__restrict__ Y, int64_t ldy, int32_t *__restrict__ acc_out) {
-    extern __shared__ __align__(128) uint8_t smem[];
-    const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wm = warp >> 2, wn = warp & 3;  // 2 x 4 warps, 64 x 32 outputs each
-    const uint32_t s0 = smem_u32(smem);
-    auto sa = [&](int s) { return s0 + s * 2 * TILE_BYTES; };
-    auto sw = [&](int s) { return s0 + s * 2 * TILE_BYTES + TILE_BYTES; };
-
-    const int KT = (int)((K + BK - 1) / BK);
-#pragma unroll
-    for (int s = 0; s < STAGES - 1; ++s) {
-        if (s < KT) {
-            load_tile<kAligned>(sa(s), A, lda, M, m0, K, (int64_t)s * BK);
-            load_tile<kAligned>(sw(s), W, ldw, N, n0, K, (int64_t)s * BK);
-        }
-        cp_async_commit();
+    const float *__restrict__ bias, float *__restrict__ Y, int64_t ldy, int32_t *__restrict__ acc_out,
+    unsigned n_tiles) {
+    constexpr int ROWS = 16 * MT, COLS = 8 * NT;
+    constexpr int U = NT == 4 ? 4 : 2;  // chunks of W in flight per warp
+    __shared__ int s_acc[COLS][ROWS + 1];
+    const int64_t n0 = (int64_t)(blockIdx.x % n_tiles) * ROWS, m0 = (int64_t)(blockIdx.x / n_tiles) * COLS;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+    for (int i = threadIdx.x; i < COLS * (ROWS + 1); i += THREADS) s_acc[0][i] = 0;
+    // the constants of this thread's first output, loaded ahead of the products
+    const int e_r = threadIdx.x % ROWS;
+    const int64_t e_n = n0 + e_r;
+    int e_cs = 0;
+    float e_bias = 0.0f;
+    qnn_qparams e_w{};
+    if (e_n < N) {
+        e_cs = csW[e_n];
+        e_w = pw[e_n / rows_per_block];
+        if (bias) e_bias = bias[e_n];
     }
 
-    int acc[4][4][4];
+    int acc[MT][NT][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < NT; ++j)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[i][j][k] = 0;
-
-    for (int kt = 0; kt < KT; ++kt) {
-        cp_async_wait<STAGES - 2>();
-        __syncthreads();
-        const int pf = kt + STAGES - 1;
-        if (pf < KT) {
-            load_tile<kAligned>(sa(pf % STAGES), A, lda, M, m0, K, (int64_t)pf * BK);
-            load_tile<kAligned>(sw(pf % STAGES), W, ldw, N, n0, K, (int64_t)pf * BK);
-        }
-        cp_async_commit();
-        const uint32_t ta = sa(kt % STAGES), tw = sw(kt % STAGES);
+            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0;
+    // rows past the end repeat the last one (their sums are dropped), so that the loads of whole
+    // chunks need no predicates
+    const uint8_t *wr[MT][2], *ar[NT];
 #pragma unroll
-        for (int kk = 0; kk < BK; kk += 32) {
-            uint32_t af[4][4], bf[4][2];
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-            for (int mi = 0; mi < 4; ++mi) {
-                const int r = wm * 64 + mi * 16 + (lane & 15);
-                ldmatrix_x4(ta + r * SROW + kk + (lane >> 4) * 16, af[mi][0], af[mi][1], af[mi][2], af[mi][3]);
+        for (int h = 0; h < 2; ++h) wr[i][h] = W + min(n0 + 16 * i + 8 * h + g, N - 1) * ldw + 16 * tq;
+#pragma unroll
+    for (int j = 0; j < NT; ++j) ar[j] = A + min(m0 + 8 * j + g, M - 1) * lda + 16 * tq;
+    auto multiply = [&](const uint4 (&w)[MT][2], int k, int valid) {
+        uint4 a[NT];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) a[j] = ld_codes16<AL, false>(ar[j] + k, valid);
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+            const uint4 lo = w[i][0], hi = w[i][1];
+            const uint32_t f0[4] = {lo.x, hi.x, lo.y, hi.y}, f1[4] = {lo.z, hi.z, lo.w, hi.w};
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                mma_u8(acc[i][j], f0, a[j].x, a[j].y);
+                mma_u8(acc[i][j], f1, a[j].z, a[j].w);
             }
-#pragma unroll
-            for (int nj = 0; nj < 2; ++nj) {
-                const int r = wn * 32 + nj * 16 + (lane & 7) + ((lane >> 4) << 3);
-                ldmatrix_x4(tw + r * SROW + kk + ((lane >> 3) & 1) * 16, bf[2 * nj][0], bf[2 * nj][1],
-                            bf[2 * nj + 1][0], bf[2 * nj + 1][1]);
-            }
-#pragma unroll
-            for (int mi = 0; mi < 4; ++mi)
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni) mma_u8(acc[mi][ni], af[mi], bf[ni][0], bf[ni][1]);
         }
+    };
+    auto load_w = [&](uint4 (&w)[MT][2], int k, int valid) {
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) w[i][h] = ld_codes16<AL, true>(wr[i][h] + k, valid);
+    };
+    // a round's U chunks are consecutive (256 bytes of a row) when every warp then has some, else
+    // spread over the warps; the ragged last chunk goes to the warp after the one with the last whole one
+    const int whole = K / 64;
+    const bool wide = whole >= kWarps * U;
+    const int cu = wide ? 1 : kWarps;
+    for (int c0 = wide ? warp * U : warp; c0 < whole; c0 += kWarps * U) {
+        uint4 w[U][MT][2];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u == 0 || c0 + cu * u < whole) load_w(w[u], 64 * (c0 + cu * u), 16);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u == 0 || c0 + cu * u < whole) multiply(w[u], 64 * (c0 + cu * u), 16);
     }
-    cp_async_wait<0>();
-
-    // Epilogue: offsets, recovery, bias.
-    const int g = lane >> 2, tq = lane & 3;
-    const int Ki = (int)K;
+    const bool tail = whole * 64 < K && warp == whole % kWarps;
+    if (tail) {
+        uint4 w[MT][2];
+        load_w(w, 64 * whole, K - 64 * whole - 16 * tq);
+        multiply(w, 64 * whole, K - 64 * whole - 16 * tq);
+    }
+    __syncthreads();  // s_acc is clear
+    if (warp < whole || tail) {
 #pragma unroll
-    for (int mi = 0; mi < 4; ++mi) {
+        for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t m = m0 + wm * 64 + mi * 16 + g + h * 8;
-            if (m >= M) continue;
-            const qnn_qparams qa = pa[a_per_row ? m : 0];
-            const int ra = rsA[m];
+            for (int j = 0; j < NT; ++j)
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int64_t n = n0 + wn * 32 + ni * 8 + tq * 2 + e;
-                    if (n >= N) continue;
-                    const qnn_qparams qw = pw[n / rows_per_block];
-                    const int a = acc[mi][ni][h * 2 + e];
-                    const long long S = offset_product(a, qa.z, qw.z, ra, csW[n], Ki);
-                    float y = recover_product(S, qa.Q, qw.Q);
-                    if (bias) y = __fadd_rn(y, bias[n]);
-                    if (Y) Y[m * ldy + n] = y;
-                    if (acc_out) acc_out[m * N + n] = a;
+                for (int e = 0; e < 4; ++e) {
+                    const int col = 8 * j + 2 * tq + (e & 1);
+                    if (m0 + col < M) atomicAdd(&s_acc[col][16 * i + 8 * (e >> 1) + g], acc[i][j][e]);
                 }
-            }
-        }
+    }
+    __syncthreads();
+
+    // Epilogue: offsets, recovery, bias (THREADS is a multiple of ROWS: each thread keeps its W row).
+    if (e_n >= N) return;
+    for (int c = threadIdx.x / ROWS; c < COLS; c += THREADS / ROWS) {
+        const int64_t m = m0 + c;
+        if (m >= M) break;
+        const qnn_qparams qa = pa[a_per_row ? m : 0];
+        const int a = s_acc[c][e_r];
+        const long long S = offset_product(a, qa.z, e_w.z, rsA[m], e_cs, K);
+        float y = recover_product(S, qa.Q, e_w.Q);
+        if (bias) y = __fadd_rn(y, e_bias);
+        if (Y) Y[m * ldy + e_n] = y;
+        if (acc_out) acc_out[m * N + e_n] = a;
     }
 }
 
@@ -179,32 +193,42 @@ qnn_status launch_qgemm_imma(const uint8_t *A, int64_t lda, const qnn_qparams *p
                              int64_t rows_per_block, const int32_t *csW, int64_t N, const float *bias, float *Y,
                              int64_t ldy, int32_t *acc_out, cudaStream_t st) {
     if (M == 0 || N == 0) return QNN_OK;
-    static bool configured[2] = {false, false};
-    const bool aligned = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W)) & 15) == 0 &&
-                         lda % 16 == 0 && ldw % 16 == 0;
-    auto kern = aligned ? qgemm_imma_kernel<true> : qgemm_imma_kernel<false>;
-    if (!configured[aligned]) {
-        QNN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        configured[aligned] = true;
-    }
-    dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + BM - 1) / BM));
+    const uintptr_t at = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | (uintptr_t)lda | (uintptr_t)ldw;
+    const int al = (at & 15) == 0 ? 16 : (at & 3) == 0 ? 4 : 1;
     ProfScope prof("qgemm_imma", st);
-    kern<<<grid, THREADS, SMEM_BYTES, st>>>(A, lda, pa, ga == QNN_PER_ROW, rsA, M, K, W, ldw, pw, rows_per_block, csW,
-                                            N, bias, Y, ldy, acc_out);
-    QNN_CUDA_TRY(cudaGetLastError());
-    return QNN_OK;
+    auto run = [&](auto nt, auto mt) -> qnn_status {
+        constexpr int NT = decltype(nt)::value, MT = decltype(mt)::value;
+        const int64_t n_tiles = (N + 16 * MT - 1) / (16 * MT), m_tiles = (M + 8 * NT - 1) / (8 * NT);
+        if (n_tiles * m_tiles > INT32_MAX) return QNN_FAIL(QNN_ERR_INVALID_ARG);
+        auto kern = al == 16  ? qgemm_imma_kernel<NT, MT, 16>
+                    : al == 4 ? qgemm_imma_kernel<NT, MT, 4>
+                              : qgemm_imma_kernel<NT, MT, 1>;
+        kern<<<(unsigned)(n_tiles * m_tiles), THREADS, 0, st>>>(A, lda, pa, ga == QNN_PER_ROW, rsA, M, (int)K, W, ldw, pw,
+                                                               rows_per_block, csW, N, bias, Y, ldy, acc_out,
+                                                               (unsigned)n_tiles);
+        QNN_CUDA_TRY(cudaGetLastError());
+        return QNN_OK;
+    };
+    using std::integral_constant;
+    if (M <= 8) return run(integral_constant<int, 1>{}, integral_constant<int, 1>{});
+    if (M <= 16) return run(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+    if (M <= 32) return run(integral_constant<int, 4>{}, integral_constant<int, 1>{});
+    return run(integral_constant<int, 8>{}, integral_constant<int, 2>{});
 }
 
-// Datapath choice: the tcgen05 path runs whole 128 x 256 tiles at the fp16 tensor rate (after
-// centering both operands into fp16 scratch); below one tile of rows the integer MMA path, which
-// needs no conversion, is used. QNN_QGEMM=imma or =tc forces one (tests compare the two).
+// Datapath choice: up to 127 rows of A the streaming integer MMA kernel, which needs no conversion,
+// else the tcgen05 path, which runs whole tiles at the fp16 tensor rate after centering both operands
+// into fp16 scratch. Above 64 rows the streaming kernel reads W twice and its MMA rate shows: there it
+// keeps W of up to 2^24 codes (M = 127: 16.5 against 32 us at 2048 x 2048, 180 against 102 us at
+// 8192 x 8192; M = 64 at 8192 x 8192: 87 against 102 us). QNN_QGEMM=imma or =tc forces one (tests
+// compare the two).
 qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, int ga, const int32_t *rsA, int64_t M,
                         int64_t K, const uint8_t *W, int64_t ldw, const qnn_qparams *pw, int64_t rows_per_block,
                         const int32_t *csW, int64_t N, const float *bias, float *Y, int64_t ldy, int32_t *acc_out,
                         cudaStream_t st) {
     if (M == 0 || N == 0) return QNN_OK;
     const char *force = std::getenv("QNN_QGEMM");
-    bool tc = M >= 128;
+    bool tc = M >= 128 || (M > 64 && N * K > (int64_t)1 << 24);
     if (force && std::strcmp(force, "imma") == 0) tc = false;
     if (force && std::strcmp(force, "tc") == 0) tc = true;
     if (tc) {

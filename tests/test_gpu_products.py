@@ -1,0 +1,61 @@
+"""The product kernels at the edges of their tiles: the streaming integer-MMA kernel over every
+number of A-row groups, ragged rows, ragged reductions and row alignments (16, 4 and 1 bytes)."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qnn():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1607_04683_gb300 import build, qnn as q
+    build.build()
+    q.lib()
+    torch.cuda.set_device(0)
+    return q
+
+
+def gpu(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def strided(a, ld, off):
+    """The code matrix on the device with `ld` bytes between rows, starting `off` bytes into its
+    buffer; the bytes between and after the rows are nonzero codes that must not be summed."""
+    rows, cols = a.shape
+    buf = torch.full((off + rows * ld,), 77, dtype=torch.uint8, device="cuda")
+    v = buf[off:].reshape(rows, ld)[:, :cols]
+    v.copy_(gpu(a))
+    return v
+
+
+# M around the 8-row groups of A (1, 2, 4 and 8 per block), N around 16 and 32 rows of W, K around
+# 16 codes, the 64-code chunk and the 8 warps' round of chunks
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (1, 16, 64), (1, 2000, 500), (1, 33, 4097), (7, 17, 15), (8, 31, 513),
+                                   (9, 15, 63), (16, 100, 1000), (17, 16, 65), (32, 130, 2049), (33, 31, 16),
+                                   (64, 33, 511), (65, 64, 129), (100, 2000, 500), (127, 96, 8192), (2, 64, 33025)])
+@pytest.mark.parametrize("pad,off", [(None, 0), (0, 0), (4, 4), (3, 1)])
+def test_few_rows_bit_exact(qnn, M, N, K, pad, off, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "imma")
+    g = np.random.Generator(np.random.PCG64(M * 31 + N * 7 + K))
+    A = g.normal(0.1, 1.0, (M, K)).astype(np.float32)
+    nb = 4 if N % 4 == 0 else 1
+    Ws = [g.uniform(-s, s, (N // nb, K)).astype(np.float32) for s in np.linspace(0.05, 0.4, nb)]
+    ga = oracle.PER_ROW if M % 2 else oracle.PER_MATRIX
+    ca, pa, ra = oracle.quantize(A, ga)
+    parts = [oracle.quantize(w, oracle.PER_MATRIX) for w in Ws]
+    cw, pw, cs = (np.concatenate([p[i] for p in parts]) for i in range(3))
+    bias = g.normal(0, 1, N).astype(np.float32) if K % 2 else None
+    ref = oracle.qmatmul(ca, pa, ga, cw, pw, n_blocks=nb, bias=bias)
+    ld = (K + 15) // 16 * 16 if pad is None else (K + 3) // 4 * 4 + pad if pad == 4 else K + pad
+    Y, acc = qnn.qnn_qmatmul(strided(ca, ld, off), qnn.params_tensor(pa), ga, gpu(ra), strided(cw, ld, off),
+                             qnn.params_tensor(pw), gpu(cs), n_blocks=nb, bias=None if bias is None else gpu(bias),
+                             want_acc=True)
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"])
+    assert np.array_equal(Y.cpu().numpy(), ref["y"])
