@@ -59,3 +59,24 @@ def test_few_rows_bit_exact(qnn, M, N, K, pad, off, monkeypatch):
     assert qnn.device_status() == qnn.QNN_OK
     assert np.array_equal(acc.cpu().numpy(), ref["acc"])
     assert np.array_equal(Y.cpu().numpy(), ref["y"])
+
+
+# The float output layer on each of its tiles (32, 64 and 128 rows and classes, chosen by the number of
+# tiles), with ragged rows and classes and K not a multiple of 4 or of 16, against the oracle's fp64
+# sums within the fp32 dot-product bound (parity.float_logit_bound).
+@pytest.mark.parametrize("B,T,H,C", [(5, 3, 50, 33), (7, 5, 64, 300), (70, 9, 50, 1999), (64, 10, 36, 2000),
+                                     (65, 20, 49, 2001), (100, 17, 64, 1300)])
+def test_float_output_layer_tiles(qnn, B, T, H, C):
+    import parity
+    from paper_1607_04683_gb300 import inputs
+    wl = inputs.LstmWorkload("float", seed=3, num_layers=1, input_dim=12, hidden=H, proj=0, num_classes=C, batch=B,
+                             frames=T, w_range=0.3, forget_bias=1.0, output_mode=2, out_w_range=0.5)
+    params, x = wl.make()
+    model = qnn.LstmModel(qnn.lstm_desc(1, 12, H, 0, C, qnn.OUT_FLOAT), gpu(params))
+    lg = torch.full((B, T, C), float("nan"), device="cuda")
+    y = model.forward(gpu(x), logits=lg)
+    assert qnn.device_status() == qnn.QNN_OK
+    ref = oracle.lstm_forward(oracle.desc(1, 12, H, 0, C, oracle.OUT_FLOAT), params, x, want_h_all=True,
+                              want_logits=True)
+    parity.check_logits(lg.cpu().numpy(), ref["logits"], 2, ref["h_all"][0], wl.out_weights(params))
+    parity.check_posteriors(y.cpu().numpy(), ref["y"])
