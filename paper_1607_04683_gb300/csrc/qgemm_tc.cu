@@ -270,10 +270,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     const uint32_t pxfull0 = su32(bars + 2 * STAGES + 4), pxempty0 = su32(bars + 2 * STAGES + 6);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr bool LX = EPI == kEpiLstmX;
-    const int KB = args.KB + (LX ? args.KB_x : 0);  // k-blocks of the K loop (kEpiLstmX: x's, then h's)
-    const int kpc = LX ? 64 : KCHUNK / TBK;        // k-blocks per chunk (16; kEpiLstmX: the whole loop, each
-                                                   // accumulator summing at most 1024)
-    const int nchunks = (KB + kpc - 1) / kpc;
+    const int nchunks = (args.KB + KCHUNK / TBK - 1) / (KCHUNK / TBK);  // K chunks of a tile (kEpiLinear)
     const int tiles_n = (int)((args.N + BN - 1) / BN);
     const int64_t tiles_m = (args.M + TBM - 1) / TBM;
     const int64_t tiles = tiles_m * tiles_n;
@@ -296,18 +293,11 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         n0 += (j & 1) * (BN / 2);
         return true;
     };
-    // the A and W tiles of k-block kb (kEpiLstmX: x_t and Wx for kb < KB_x, then h_{t-1} and Wh)
-    auto load_a = [&](uint32_t dst, uint32_t bar, int kb, int m0) {
-        if (LX && kb < args.KB_x)
-            tma_load_2d(dst, &mapAX, bar, kb * TBK, m0);
-        else
-            tma_load_2d(dst, &mapA, bar, (kb - (LX ? args.KB_x : 0)) * TBK, m0);
-    };
-    auto load_w = [&](uint32_t dst, uint32_t bar, int kb, int n0) {
-        if (LX && kb < args.KB_x)
-            tma_load_2d(dst, &mapWX, bar, kb * TBK, n0);
-        else
-            tma_load_2d(dst, &mapW, bar, (kb - (LX ? args.KB_x : 0)) * TBK, n0);
+    // The k-blocks of an item in two segments: kEpiLstmX's x_t and Wx (segment 0), then A and W (segment 1;
+    // an item's own K range for split-K). A stage holds k-blocks of one segment.
+    auto segment = [&](int seg, int64_t item, int &kb, int &end) {
+        kb = seg == 0 || LX ? 0 : (int)(item % splits) * args.kbs;
+        end = seg == 0 ? args.KB_x : LX ? args.KB : min(args.KB, kb + args.kbs);
     };
     __shared__ int s_abort;
 
@@ -353,31 +343,19 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         if (args.w_static && blockIdx.x < items) {
             int64_t m0, n0;
             item_origin(blockIdx.x / splits, m0, n0);
-            const int kb0 = (int)(blockIdx.x % splits) * args.kbs, kb1 = min(KB, kb0 + args.kbs);
-            if constexpr (TL::KPS == 1) {
-                w_early = min(STAGES, kb1 - kb0);
-                for (int j = 0; j < w_early; ++j) {
-                    const uint32_t sb = su32(smem + j * TL::STAGE_BYTES) + A_BYTES;
-                    mb_expect(full0 + 8 * j, TL::STAGE_BYTES);
-                    load_w(sb, full0 + 8 * j, kb0 + j, (int)n0);
-                    if (LX && full_early == j && kb0 + j < args.KB_x) {
-                        load_a(sb - A_BYTES, full0 + 8 * j, kb0 + j, (int)m0);
-                        ++full_early;
+#pragma unroll
+            for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
+                int kb, end;
+                segment(seg, blockIdx.x, kb, end);
+                for (; kb < end && w_early < STAGES; kb += TL::KPS, ++w_early) {
+                    const int nv = min(TL::KPS, end - kb);
+                    const uint32_t sa = su32(smem + w_early * TL::STAGE_BYTES), bar = full0 + 8 * w_early;
+                    mb_expect(bar, (uint32_t)(nv * TL::SUB_BYTES));
+                    for (int v = 0; v < nv; ++v) {
+                        tma_load_2d(sa + TL::KPS * A_BYTES + v * TL::B_BYTES, seg == 0 ? &mapWX : &mapW, bar, (kb + v) * TBK, (int)n0);
+                        if (seg == 0) tma_load_2d(sa + v * A_BYTES, &mapAX, bar, (kb + v) * TBK, (int)m0);
                     }
-                }
-            } else {
-                w_early = min(STAGES, (kb1 - kb0 + TL::KPS - 1) / TL::KPS);
-                for (int j = 0; j < w_early; ++j) {
-                    const int kbj = kb0 + j * TL::KPS, nv = min(TL::KPS, kb1 - kbj);
-                    const uint32_t sb = su32(smem + j * TL::STAGE_BYTES) + TL::KPS * A_BYTES;
-                    mb_expect(full0 + 8 * j, (uint32_t)(nv * TL::SUB_BYTES));
-                    for (int v = 0; v < nv; ++v)
-                        load_w(sb + v * TL::B_BYTES, full0 + 8 * j, kbj + v, (int)n0);
-                    if (LX && full_early == j && kbj + nv <= args.KB_x) {
-                        for (int v = 0; v < nv; ++v)
-                            load_a(sb - TL::KPS * A_BYTES + v * A_BYTES, full0 + 8 * j, kbj + v, (int)m0);
-                        ++full_early;
-                    }
+                    if (seg == 0) ++full_early;
                 }
             }
         }
@@ -394,176 +372,114 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     // epilogue overlaps the next tile's MMAs.
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        if constexpr (TL::KPS == 1) {
-            if (lane == 0) {
-                int64_t g = 0;  // k-blocks issued by this block
-                for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                    int64_t m0, n0;
-                    item_origin(item / splits, m0, n0);
-                    const int kb0 = (int)(item % splits) * args.kbs, kb1 = min(KB, kb0 + args.kbs);
-                    for (int kb = kb0; kb < kb1; ++kb, ++g) {
-                        const int s = (int)(g % STAGES);
-                        if (g >= STAGES && !mb_wait(empty0 + 8 * s, (unsigned)((g / STAGES) - 1) & 1, args.status)) {
+        // One thread issues every copy and every instruction of its loop is on the critical path of the
+        // operand stream (a few cycles each, one after the other), so the ring position advances
+        // incrementally in 32-bit registers.
+        if (lane == 0) {
+            const uint32_t ring0 = su32(smem);
+            uint32_t dst = ring0, bar = full0;
+            unsigned free_parity = 1;
+            int issued = 0;
+            for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                int64_t m0l, n0l;
+                item_origin(item / splits, m0l, n0l);
+                const int m0 = (int)m0l, n0 = (int)n0l;
+#pragma unroll
+                for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
+                    const CUtensorMap *const ma = seg == 0 ? &mapAX : &mapA, *const mw = seg == 0 ? &mapWX : &mapW;
+                    int kb, end;
+                    segment(seg, item, kb, end);
+                    for (; kb < end; kb += TL::KPS) {
+                        // (not on a slot's first use: an early stage may already be freed again)
+                        if (issued >= STAGES && !mb_wait(bar + 8 * STAGES, free_parity, args.status)) {
                             s_abort = 1;
                             break;
                         }
-                        const uint32_t sa = su32(smem + s * TL::STAGE_BYTES), sb = sa + A_BYTES;
-                        if (g < full_early) continue;  // issued whole before the wait
-                        if (g < w_early) {  // W already on its way (expect set with it)
-                            load_a(sa, full0 + 8 * s, kb, (int)m0);
-                            continue;
-                        }
-                        mb_expect(full0 + 8 * s, TL::STAGE_BYTES);
-                        load_a(sa, full0 + 8 * s, kb, (int)m0);
-                        load_w(sb, full0 + 8 * s, kb, (int)n0);
-                    }
-                }
-            }
-        } else {
-            if (lane == 0) {
-                // One thread issues every copy; its loop is on the critical path of the operand stream,
-                // so the ring position (slot, phase, shared-memory address) advances incrementally in
-                // 32-bit registers instead of being derived from a 64-bit counter every stage.
-                const uint32_t ring0 = su32(smem);
-                int slot = 0, issued = 0;  // ring slot; stages issued (saturating at STAGES)
-                unsigned phase = 0;        // parity of the slot's current use
-                uint32_t st_addr = ring0, bar_full = full0, bar_empty = empty0;
-                for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                    int64_t m0l, n0l;
-                    item_origin(item / splits, m0l, n0l);
-                    const int m0 = (int)m0l, n0 = (int)n0l;
-                    const int kb0 = (int)(item % splits) * args.kbs, kb1 = min(KB, kb0 + args.kbs);
-                    for (int kb = kb0; kb < kb1; kb += TL::KPS) {
-                        if (issued >= STAGES && !mb_wait(bar_empty, phase ^ 1u, args.status)) {
-                            s_abort = 1;
-                            break;
-                        }
-                        const int nv = min(TL::KPS, kb1 - kb);  // k-blocks in this stage (the last may be short)
-                        const uint32_t sb = st_addr + TL::KPS * A_BYTES;
-                        const bool w_sent = issued < w_early;   // W already on its way (expect set with it)
-                        if (issued >= full_early) {             // (else issued whole before the wait)
-                            if (!w_sent) mb_expect(bar_full, (uint32_t)(nv * TL::SUB_BYTES));
+                        const int nv = min(TL::KPS, end - kb);   // k-blocks in this stage (the last may be short)
+                        const bool w_sent = issued < w_early;    // W already on its way (expect set with it)
+                        if (issued >= full_early) {              // (else issued whole before the wait)
+                            if (!w_sent) mb_expect(bar, (uint32_t)(nv * TL::SUB_BYTES));
 #pragma unroll
                             for (int v = 0; v < TL::KPS; ++v) {
                                 if (v >= nv) break;
-                                load_a(st_addr + v * A_BYTES, bar_full, kb + v, m0);
-                                if (!w_sent) load_w(sb + v * TL::B_BYTES, bar_full, kb + v, n0);
+                                tma_load_2d(dst + v * A_BYTES, ma, bar, (kb + v) * TBK, m0);
+                                if (!w_sent)
+                                    tma_load_2d(dst + TL::KPS * A_BYTES + v * TL::B_BYTES, mw, bar, (kb + v) * TBK, n0);
                             }
                         }
-                        if (issued < STAGES) ++issued;
-                        if (++slot == STAGES) {
-                            slot = 0;
-                            phase ^= 1u;
-                            st_addr = ring0, bar_full = full0, bar_empty = empty0;
-                        } else {
-                            st_addr += TL::STAGE_BYTES, bar_full += 8, bar_empty += 8;
-                        }
+                        ++issued;
+                        dst += TL::STAGE_BYTES, bar += 8;
+                        if (bar == full0 + 8 * STAGES) dst = ring0, bar = full0, free_parity ^= 1u;
                     }
+                    if (s_abort) break;
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if constexpr (TL::KPS == 1) {
-            if (lane == 0) {
-                int64_t g = 0, gc = 0;  // k-blocks and chunks consumed by this block
-                for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                    const int kb0 = (int)(item % splits) * args.kbs, kb1 = min(KB, kb0 + args.kbs);
-                    const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
-                    for (int kb = kb0; kb < kb1; ++kb, ++g) {
-                        const int s = (int)(g % STAGES);
-                        const int kc = (kb - kb0) % kpc;
-                        const int buf = (int)(gc & 1);
-                        if (kc == 0 && gc >= 2 &&
-                            !mb_wait(drained0 + 8 * buf, (unsigned)((gc / 2) - 1) & 1, args.status)) {  // buffer free
-                            s_abort = 1;
-                            break;
-                        }
-                        if (!mb_wait(full0 + 8 * s, (unsigned)(g / STAGES) & 1, args.status)) {
-                            s_abort = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t sa = su32(smem + s * TL::STAGE_BYTES), sb = sa + A_BYTES;
-                        // kEpiLstmX: x's k-blocks into the buffer's first accumulator, h's into the second
-                        const bool hpart = LX && kb >= args.KB_x;
-                        const uint32_t tmem_d = tmem_base + (uint32_t)(buf * TL::ACC_COLS + (hpart ? BN : 0));
-                        const bool fresh = kc == 0 || (LX && kb == args.KB_x);
+        // Its loop is what a k-block costs when it is longer than the MMAs themselves: four MMAs issue in
+        // about 230 cycles (a floor for N <= 128; 521 at N = 256), a commit takes about 250, and everything
+        // else here adds to that. So the descriptors are 32-bit additions to a running low word (the high
+        // word is constant) and the accumulate flag a constant after the first MMA. Probe of the loop
+        // alone, cycles per 64-wide k-block: 761 with descriptors built per MMA and a 64-bit ring counter;
+        // 535 so (N = 128, one k-block a stage), 381 with two k-blocks a stage, 544 at N = 256.
+        if (lane == 0) {
+            const uint32_t desc0 = smem_desc_lo(su32(smem));
+            uint32_t da = desc0, bar = full0;
+            unsigned parity = 0;
+            unsigned gc = 0;  // chunks accumulated by this block
+            for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
 #pragma unroll
-                        for (int k = 0; k < TBK / 16; ++k) {
-                            // advance 16 fp16 = 32 bytes along K inside the swizzled 128-byte rows
-                            mma_f16(tmem_d, smem_desc(sa + 32 * k), smem_desc(sb + 32 * k), idesc,
-                                    (fresh && k == 0) ? 0u : 1u);
+                for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
+                    int kb, end;
+                    segment(seg, item, kb, end);
+                    int kc = 0;  // position in the K chunk (chunks hold whole stages)
+                    uint32_t tmem_d = 0;
+                    for (; kb < end; kb += TL::KPS) {
+                        const bool fresh = kc == 0;
+                        if (fresh) {
+                            // kEpiLstmX: x's k-blocks into the buffer's first accumulator, h's into the second
+                            tmem_d = tmem_base + (gc & 1) * TL::ACC_COLS + (LX && seg == 1 ? BN : 0);
+                            if ((!LX || seg == 0) && gc >= 2 &&
+                                !mb_wait(drained0 + 8 * (gc & 1), ((gc >> 1) - 1) & 1, args.status)) {  // buffer free
+                                s_abort = 1;
+                                break;
+                            }
                         }
-                        mma_commit(empty0 + 8 * s);  // frees the stage when these MMAs have read it
-                        if (kc == kpc - 1 || kb == kb1 - 1) {
-                            mma_commit(chunk0 + 8 * buf);
-                            ++gc;
-                        }
-                    }
-                    if (s_abort) break;
-                }
-            }
-        } else {
-            if (lane == 0) {
-                // The same incremental ring position as the producer's; the shared-memory descriptors of
-                // a stage are its base descriptor plus the byte offset / 16 in the address field (the
-                // address stays below 2^18, so the 14-bit field never carries).
-                const uint32_t ring0 = su32(smem);
-                int slot = 0;
-                unsigned phase = 0;
-                uint32_t st_addr = ring0, bar_full = full0, bar_empty = empty0;
-                int64_t gc = 0;  // chunks accumulated by this block
-                for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                    const int kb0 = (int)(item % splits) * args.kbs, kb1 = min(KB, kb0 + args.kbs);
-                    const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
-                    int kc = 0;  // position of the stage in its K chunk (chunks hold whole stages)
-                    for (int kb = kb0; kb < kb1; kb += TL::KPS) {
-                        const int nv = min(TL::KPS, kb1 - kb);
-                        const int buf = (int)(gc & 1);
-                        if (kc == 0 && gc >= 2 &&
-                            !mb_wait(drained0 + 8 * buf, (unsigned)((gc / 2) - 1) & 1, args.status)) {  // buffer free
-                            s_abort = 1;
-                            break;
-                        }
-                        if (!mb_wait(bar_full, phase, args.status)) {
+                        if (!mb_wait(bar, parity, args.status)) {
                             s_abort = 1;
                             break;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint64_t da = smem_desc(st_addr), db = smem_desc(st_addr + TL::KPS * A_BYTES);
+                        const uint32_t db = da + ((TL::KPS * A_BYTES) >> 4);
 #pragma unroll
                         for (int v = 0; v < TL::KPS; ++v) {
-                            if (v >= nv) break;
-                            // kEpiLstmX: x's k-blocks into the buffer's first accumulator, h's into the second
-                            const bool hpart = LX && kb + v >= args.KB_x;
-                            const uint32_t tmem_d = tmem_base + (uint32_t)(buf * TL::ACC_COLS + (hpart ? BN : 0));
-                            const bool fresh = (kc == 0 && v == 0) || (LX && kb + v == args.KB_x);
+                            if (v > 0 && kb + v >= end) break;
 #pragma unroll
                             for (int k = 0; k < TBK / 16; ++k) {
                                 // advance 16 fp16 = 32 bytes along K inside the swizzled 128-byte rows
-                                mma_f16(tmem_d, da + (uint64_t)((v * A_BYTES + 32 * k) >> 4),
-                                        db + (uint64_t)((v * TL::B_BYTES + 32 * k) >> 4), idesc,
-                                        (fresh && k == 0) ? 0u : 1u);
+                                const uint32_t x = da + ((v * A_BYTES + 32 * k) >> 4), w = db + ((v * TL::B_BYTES + 32 * k) >> 4);
+                                if (v == 0 && k == 0)
+                                    mma_f16_lo(tmem_d, x, w, idesc, fresh ? 0u : 1u);
+                                else
+                                    mma_f16_lo(tmem_d, x, w, idesc, 1u);
                             }
                         }
-                        mma_commit(bar_empty);  // frees the stage when these MMAs have read it
-                        kc += nv;
-                        if (kc >= kpc || kb + nv >= kb1) {
-                            mma_commit(chunk0 + 8 * buf);
+                        mma_commit(bar + 8 * STAGES);  // frees the stage when these MMAs have read it
+                        kc += TL::KPS;
+                        const bool last = kb + TL::KPS >= end;
+                        if (LX ? (seg == 1 && last) : (kc == KCHUNK / TBK || last)) {
+                            mma_commit(chunk0 + 8 * (gc & 1));
                             ++gc;
                             kc = 0;
                         }
-                        if (++slot == STAGES) {
-                            slot = 0;
-                            phase ^= 1u;
-                            st_addr = ring0, bar_full = full0, bar_empty = empty0;
-                        } else {
-                            st_addr += TL::STAGE_BYTES, bar_full += 8, bar_empty += 8;
-                        }
+                        da += TL::STAGE_BYTES >> 4, bar += 8;
+                        if (bar == full0 + 8 * STAGES) da = desc0, bar = full0, parity ^= 1u;
                     }
                     if (s_abort) break;
                 }
+                if (s_abort) break;
             }
         }
     } else if constexpr (EPI == kEpiLinear) {

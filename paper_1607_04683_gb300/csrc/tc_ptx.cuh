@@ -30,16 +30,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
 }
 
 // Shared-memory matrix descriptor of a K-major tile with 128-byte swizzle: rows of 128 bytes,
-// 8-row groups 1024 bytes apart (stride byte offset), tcgen05 descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFF) >> 4);        // start address
-    d |= (uint64_t)1 << 16;                          // leading byte offset (unused with this swizzle)
-    d |= (uint64_t)(1024 >> 4) << 32;                // stride byte offset
-    d |= (uint64_t)1 << 46;                          // version
-    d |= (uint64_t)2 << 61;                          // 128-byte swizzle
-    return d;
-}
+// 8-row groups 1024 bytes apart (stride byte offset), tcgen05 descriptor version 1. The low word holds
+// the start address / 16 (the leading byte offset is unused with this swizzle); byte offsets / 16 may be
+// added to it, since shared-memory addresses stay below 2^18 and the 14-bit field never carries.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) { return ((addr & 0x3FFFF) >> 4) | (1u << 16); }
+constexpr uint32_t kSmemDescHi = (1024u >> 4)   // stride byte offset
+                                 | (1u << 14)   // version
+                                 | (2u << 29);  // 128-byte swizzle
 
 // Instruction descriptor of tcgen05.mma kind::f16: fp32 accumulator, fp16 A and B, both K-major,
 // M rows x N columns.
@@ -47,13 +44,14 @@ __host__ __device__ constexpr uint32_t mma_idesc_f16(int M, int N) {
     return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D (tensor memory) += A (shared) x B (shared)^T, or = when accumulate is 0; idesc from mma_idesc_f16.
-__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
+// D (tensor memory) += A (shared) x B (shared)^T, or = when accumulate is 0; idesc from mma_idesc_f16,
+// operands by the low words of their descriptors.
+__device__ __forceinline__ void mma_f16_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                           uint32_t accumulate) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}" ::"r"(tmem_d),
+        "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kSmemDescHi)
         : "memory");
 }
 // Arrives on `bar` once every MMA issued so far by this thread has completed.
