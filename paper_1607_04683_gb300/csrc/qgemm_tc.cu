@@ -561,6 +561,42 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 if (nb >= args.N) continue;
                 const bool full = vec && nb + 32 <= args.N;
                 float *yr = args.Y ? args.Y + m * args.ldy + nb : nullptr;
+                int *const ar = args.acc_out ? args.acc_out + m * args.N + nb : nullptr;
+                // The usual block: 32 columns of one weight unit, whole rows, sums S of eq. (1) that fit 32 bits
+                // (K max|a' + za| max|w' + zw| < 2^31: wrapping 32-bit arithmetic gives them exactly) and a
+                // divisor far from the ends of the fp32 range (div_by_recip: the IEEE quotient). The block's
+                // outputs then cost a few instructions each; with a 64-bit sum and an IEEE divide apiece the
+                // tile's epilogue outlasts the two K chunks the accumulators can run ahead.
+                if (full && (!ar || (reinterpret_cast<uintptr_t>(ar) & 15) == 0) && cu[c0].unit == cu[c0 + 31].unit) {
+                    const int zw = cc[c0].zw;
+                    const float den = __fmul_rn(Qa, cc[c0].Qw);
+                    if ((long long)K * max(abs(za), abs(za + 255)) * (long long)max(abs(zw), abs(zw + 255)) < (1LL << 31) &&
+                        den >= 0x1p-60f && den <= 0x1p60f) {
+                        const float rden = __frcp_rn(den);
+                        const uint32_t rt = (uint32_t)(128 + zw) * (uint32_t)ra + (uint32_t)K * ((uint32_t)za * (uint32_t)zw - 16384u);
+                        const uint32_t za128 = (uint32_t)(128 + za);
+#pragma unroll
+                        for (int v4 = 0; v4 < 8; ++v4) {
+                            float y[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int i = 4 * v4 + e;
+                                const int S = (int)((uint32_t)run[j][i] + rt + za128 * (uint32_t)cc[c0 + i].cs);
+                                y[e] = div_by_recip(__int2float_rn(S), den, rden);
+                                if (args.bias) y[e] = __fadd_rn(y[e], cc[c0 + i].bias);
+                            }
+                            *reinterpret_cast<float4 *>(yr + 4 * v4) = make_float4(y[0], y[1], y[2], y[3]);
+                            if (ar) {  // raw code products
+                                const int base = 128 * ra - 16384 * K;
+                                int o[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) o[e] = run[j][4 * v4 + e] + base + 128 * cc[c0 + 4 * v4 + e].cs;
+                                *reinterpret_cast<int4 *>(ar + 4 * v4) = make_int4(o[0], o[1], o[2], o[3]);
+                            }
+                        }
+                        continue;
+                    }
+                }
 #pragma unroll
                 for (int v4 = 0; v4 < 8; ++v4) {
                     float y[4];
