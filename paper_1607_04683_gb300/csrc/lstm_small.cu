@@ -386,8 +386,8 @@ __global__ void __launch_bounds__(kSThreads, 1) lstm_small_kernel(const __grid_c
                 mn = fminf(mn, S.hbuf[1][warp][k]);
                 mx = fmaxf(mx, S.hbuf[1][warp][k]);
             }
-            mn = warp_min(mn);
-            mx = warp_max(mx);
+            mn = warp_min_quick(mn);
+            mx = warp_max_quick(mx);
             for (int i = lane; i < kHParts; i += 32) S.hmm[1][warp][i] = make_float2(mn, mx);
         }
         // Wx rows of this block, local row 4c + g <- global row g H + j0 + c
@@ -464,8 +464,8 @@ __global__ void __launch_bounds__(kSThreads, 1) lstm_small_kernel(const __grid_c
                         }
                     }
                 }
-                mn = warp_min(mn);
-                mx = warp_max(mx);
+                mn = warp_min_quick(mn);
+                mx = warp_max_quick(mx);
                 bad = __any_sync(0xffffffffu, bad);
                 if (bad) {
                     if (lane == 0) record_status(a.status, QNN_ERR_NONFINITE);
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kSThreads, 1) lstm_small_kernel(const __grid_c
 #pragma unroll
             for (int b = 0; b < kMaxB; ++b) {
                 if (b >= B) break;
-                const float m = warp_max(mine ? lg[b] : -FLT_MAX);
+                const float m = warp_max_quick(mine ? lg[b] : -FLT_MAX);
                 if (lane == 0) S.red_m[warp][b] = m;
             }
             named_bar(1, kPT);
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(kSThreads, 1) lstm_small_kernel(const __grid_c
                         }
                         if (i < a.nout) M = fmaxf(M, __uint_as_float((unsigned)mv));
                     }
-                    M = warp_max(M);
+                    M = warp_max_quick(M);
                     float part = 0.0f;
 #pragma unroll 1
                     for (int q = 0; q < rounds; ++q) {
@@ -659,8 +659,8 @@ __global__ void __launch_bounds__(kSThreads, 1) lstm_small_kernel(const __grid_c
                             mx = fmaxf(mx, mm.y);
                         }
                     }
-                    mn = warp_min(mn);
-                    mx = warp_max(mx);
+                    mn = warp_min_quick(mn);
+                    mx = warp_max_quick(mx);
                     const qnn_qparams p = params_from_range(mn, mx);
                     code_row(S.hbuf[pb][b], R, p, S.codes_h[b], tid);
                     if (tid == 0) S.meta_h[par][b] = RowMeta{p.z, p.Q, 0, 0};

@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(256) proj_finish_kernel(const FinishArgs a) {
                d >= 0x1p-60f && d <= 0x1p60f;
     }
     if (fast) {
-        const float rcp = __frcp_rn(d);
+        const float rcp = rcp_rn(d);
         const uint32_t rt = (uint32_t)(128 + qw0.z) * (uint32_t)ra + (uint32_t)a.K * (uint32_t)(za * qw0.z - 16384);
         const int4 c0 = *reinterpret_cast<const int4 *>(a.wp_sum + k0), c1 = *reinterpret_cast<const int4 *>(a.wp_sum + k0 + 4);
         const int cs[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};

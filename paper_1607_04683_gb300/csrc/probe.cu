@@ -112,32 +112,43 @@ __global__ void s64_to_f32_kernel(const int64_t *__restrict__ in, float *__restr
 
 __device__ __forceinline__ bool bits_differ(float a, float b) { return __float_as_uint(a) != __float_as_uint(b); }
 
-// Pairs (in[2i], in[2i+1]) through the paired-instruction functions and the scalar ones: counts
-// the pairs where any of E, sigma, tanh, the cell update and the reciprocal-based quotient differ.
+// Pairs (in[2i], in[2i+1]) through the functions the gate kernels use and through the same operations
+// with IEEE divides: counts the pairs where any of sigma, tanh, the cell update, the reciprocal and the
+// reciprocal-based quotient differ.
 __global__ void pair_functions_kernel(const float *__restrict__ in, int64_t npairs, unsigned long long *mismatches) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npairs; i += (int64_t)gridDim.x * blockDim.x) {
         const float2 x = make_float2(in[2 * i], in[2 * i + 1]);
         bool bad = false;
-        const float2 e = pexp2(x), sg = psigmoid2(x), th = ptanh2(x);
-        bad |= bits_differ(e.x, pexp(x.x)) || bits_differ(e.y, pexp(x.y));
-        bad |= bits_differ(sg.x, psigmoid(x.x)) || bits_differ(sg.y, psigmoid(x.y));
-        bad |= bits_differ(th.x, ptanh(x.x)) || bits_differ(th.y, ptanh(x.y));
-        // a cell with gates built from both values, and its scalar twins
+        auto sigma = [](float v) { return __fdiv_rn(1.0f, __fadd_rn(1.0f, pexp(-v))); };
+        auto tangent = [](float v) { return __fsub_rn(1.0f, __fdiv_rn(2.0f, __fadd_rn(pexp(__fmul_rn(2.0f, v)), 1.0f))); };
+        bad |= bits_differ(gate_activation(x.x, false), sigma(x.x)) || bits_differ(gate_activation(x.y, true), tangent(x.y));
+        bad |= bits_differ(psigmoid(x.y), sigma(x.y)) || bits_differ(ptanh(x.x), tangent(x.x));
+        // a cell with gates built from both values
+        auto cell = [&](float pi, float pf, float pg, float po, float &c) {
+            c = __fadd_rn(__fmul_rn(sigma(pf), c), __fmul_rn(sigma(pi), tangent(pg)));
+            return __fmul_rn(sigma(po), tangent(c));
+        };
         const float qx = __fmul_rn(0.25f, x.x), qy = __fmul_rn(0.5f, x.y);
-        float c0 = __fmul_rn(x.x, 0.37f), c1 = __fmul_rn(x.y, -0.51f);
+        float c0 = __fmul_rn(x.x, 0.37f), c1 = __fmul_rn(x.y, -0.51f), c2 = c0, m2;
         float2 c = make_float2(c0, c1);
         const float2 m = lstm_cell2(x, make_float2(x.y, x.x), make_float2(-x.x, qy), make_float2(qx, x.y), c);
-        float m0, m1;
-        lstm_cell(x.x, x.y, -x.x, qx, c0, m0);
-        lstm_cell(x.y, x.x, qy, x.y, c1, m1);
+        lstm_cell(x.x, x.y, -x.x, qx, c2, m2);
+        const float m0 = cell(x.x, x.y, -x.x, qx, c0), m1 = cell(x.y, x.x, qy, x.y, c1);
         bad |= bits_differ(m.x, m0) || bits_differ(m.y, m1) || bits_differ(c.x, c0) || bits_differ(c.y, c1);
+        bad |= bits_differ(m2, m0) || bits_differ(c2, c0);
+        // reciprocals of the values within the short form's range, and a quotient of each
+        for (const float v : {fabsf(x.x), fabsf(x.y)})
+            if (v >= 0x1p-100f && v < 0x1p126f) {
+                bad |= bits_differ(rcp_rn(v), __frcp_rn(v));
+                bad |= bits_differ(div_rn(kScale, v), __fdiv_rn(kScale, v));
+            }
         // the recovery's quotient: integer numerators (converted from int, as the kernel's exact sums
         // are, so never -0) over a divisor from its correctly rounded reciprocal
         const float d = __fadd_rn(__fmul_rn(fabsf(x.x), 977.0f), 0.75f);
         const float2 v = make_float2(__int2float_rn(__float2int_rn(__fmul_rn(x.y, 1.0e6f))),
                                      __int2float_rn(__float2int_rn(__fmul_rn(x.x, 3.0e5f))));
         const float2 q = div_by_recip2(v, d, __frcp_rn(d));
-        bad |= bits_differ(q.x, __fdiv_rn(v.x, d)) || bits_differ(q.y, __fdiv_rn(v.y, d));
+        if (d <= 0x1p60f) bad |= bits_differ(q.x, __fdiv_rn(v.x, d)) || bits_differ(q.y, __fdiv_rn(v.y, d));
         if (bad) atomicAdd(mismatches, 1ull);
     }
 }

@@ -572,7 +572,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                     const float den = __fmul_rn(Qa, cc[c0].Qw);
                     if ((long long)K * max(abs(za), abs(za + 255)) * (long long)max(abs(zw), abs(zw + 255)) < (1LL << 31) &&
                         den >= 0x1p-60f && den <= 0x1p60f) {
-                        const float rden = __frcp_rn(den);
+                        const float rden = rcp_rn(den);
                         const uint32_t rt = (uint32_t)(128 + zw) * (uint32_t)ra + (uint32_t)K * ((uint32_t)za * (uint32_t)zw - 16384u);
                         const uint32_t za128 = (uint32_t)(128 + za);
 #pragma unroll
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 if (one_unit && full && !args.acc_out) {  // the usual block: no per-element branches
                     if (den >= 0x1p-60f && den <= 0x1p60f &&
                         llabs(rt) + (long long)abs(za128) * 255 * K < (1LL << 24)) {
-                        const float rden = __frcp_rn(den);
+                        const float rden = rcp_rn(den);
                         if (args.bias)
                             row_block_f32<true>(r, cc + c0, (float)rt, (float)za128, den, rden, yr);
                         else
@@ -891,7 +891,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                     const long long rtx = (long long)(128 + qw.z) * rsx + (long long)args.K_x * ((long long)zx * qw.z - 16384);
                     const long long rth = (long long)(128 + qh.z) * rs + (long long)K * ((long long)za * qh.z - 16384);
                     // (rt_x, rt_h exact when the bound below holds)
-                    rq[32 * g] = make_float4(__frcp_rn(dx), __frcp_rn(dh), (float)rtx, (float)rth);
+                    rq[32 * g] = make_float4(rcp_rn(dx), rcp_rn(dh), (float)rtx, (float)rth);
                     rd[32 * g] = make_float2(dx, dh);
                     f &= (long long)args.K_x * ax * (long long)max(abs(qw.z), abs(qw.z + 255)) < (1LL << 31) &&
                          (long long)K * ah * (long long)max(abs(qh.z), abs(qh.z + 255)) < (1LL << 31) &&
