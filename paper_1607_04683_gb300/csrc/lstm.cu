@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__res
 }  // namespace
 
 // The largest tile whose tiles give every SM at least one block, else the smallest.
-static qnn_status launch_float_linear(const float *X, int64_t M, int64_t K, const float *Wt, int64_t C, const float *bias,
+qnn_status launch_float_linear(const float *X, int64_t M, int64_t K, const float *Wt, int64_t C, const float *bias,
                                float *Y, cudaStream_t st) {
     ProfScope prof("float_linear", st);
     auto tiles = [&](int64_t b) { return ((M + b - 1) / b) * ((C + b - 1) / b); };
@@ -771,6 +771,8 @@ extern "C" void qnn_lstm_model_destroy(qnn_lstm_model *m) {
     cudaFree(m->ws);
     cudaFree(m->sws);
     cudaFree(m->tcw);
+    cudaFree(m->pw);
+    cudaFree(m->pws);
     cudaFree(m->fws);
     for (cudaStream_t w : m->wave_st) cudaStreamDestroy(w);
     for (cudaEvent_t e : m->wave_ev) cudaEventDestroy(e);
@@ -1033,6 +1035,12 @@ qnn_status forward_impl(qnn_lstm_model *m, const float *x, int64_t B, int64_t T,
         QNN_TRY(small_path_forward(m, x, B, T, y, logits, h_state, c_state, h_all, st, &used));
         if (used) return QNN_OK;
         if (choice == PathChoice::kSmall) return QNN_ERR_INVALID_ARG;
+    }
+    if (choice == PathChoice::kPersist || (choice == PathChoice::kAuto && persist_preferred(m, B, y_map != nullptr))) {
+        bool used = false;
+        QNN_TRY(persist_path_forward(m, x, B, T, y, logits, h_state, c_state, h_all, st, &used));
+        if (used) return QNN_OK;
+        if (choice == PathChoice::kPersist) return QNN_ERR_INVALID_ARG;
     }
     // recurrence: tensor cores for large batches, else the persistent integer-MMA kernel
     const bool use_tc = tc_recurrence_supported(m) && (!ha_dev || (reinterpret_cast<uintptr_t>(h_all) & 15) == 0) &&

@@ -45,6 +45,11 @@ struct TcFusedInput {
     int32_t *rs = nullptr;
 };
 
+struct PersistWeights {  // one layer's weights in the persistent stack kernel's layout (lstm_persist.cu)
+    __half *wx16 = nullptr, *wh16 = nullptr;  // gate rows by cell pair, [4 round_up(H, 2)][kx], [..][kh]
+    float2 *pairc = nullptr;                  // column constants by cell pair
+};
+
 }  // namespace qnn
 
 struct qnn_lstm_model {
@@ -81,6 +86,13 @@ struct qnn_lstm_model {
     // the 8-bit output layer's Wo as centered fp16 [C][round_up(R, 64)] (in tcw)
     __half *wo16 = nullptr;
     std::vector<qnn::TcLayer> tc_layers;
+    // the persistent tensor-core stack's weights (made on first use), the 8-bit output layer's with them,
+    // and its workspace
+    void *pw = nullptr;
+    __half *pw_wo16 = nullptr;
+    std::vector<qnn::PersistWeights> pw_layers;
+    void *pws = nullptr;
+    size_t pws_bytes = 0;
     // host mirror of the unit parameters (filled at creation)
     std::vector<qnn_qparams> host_params;
 };
@@ -114,10 +126,28 @@ struct SmallStreamArgs {
 qnn_status small_stream_plan(const qnn_lstm_model *m, int64_t B, int *writer_blocks, int *nout);
 qnn_status small_stream_launch(const qnn_lstm_model *m, const SmallStreamArgs &s, cudaStream_t st);
 
+// Runs qnn_lstm_forward on the persistent tensor-core stack (lstm_persist.cu) if the model and batch
+// qualify (no projection, one unit per gate matrix, at most 256 sequences, a stack whose blocks fit the
+// SMs); *used tells whether it ran. Arguments as for qnn_lstm_forward_logits (logits nullable).
+qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, int64_t T, float *y, float *logits,
+                                float *h_state, float *c_state, float *h_all, cudaStream_t st, bool *used);
+// Whether that path is the better one where it qualifies (see there).
+bool persist_preferred(const qnn_lstm_model *m, int64_t B, bool host_posteriors);
+
+// Rows of fp32 values -> centered fp16 codes [rows][kp], units and code sums (the tensor-core
+// recurrences' row quantizer, lstm_tc.cu); with tm_T > 0 source row b tm_T + t goes to row t tm_B + b.
+qnn_status quantize_rows_f16(const float *src, int64_t ld, int64_t rows, int64_t len, int64_t kp, __half *dst,
+                             qnn_qparams *prm, int32_t *rsum, int *status, cudaStream_t st, int64_t tm_T, int64_t tm_B);
+
+// The float output layer: Y [M][C] = X [M][K] Wt^T + bias in fp32 (lstm.cu).
+qnn_status launch_float_linear(const float *X, int64_t M, int64_t K, const float *Wt, int64_t C, const float *bias,
+                               float *Y, cudaStream_t st);
+
 // Which forward path to take, from the QNN_LSTM_PATH environment variable: "layerwise" (the
-// persistent integer-MMA recurrence), "tc" (the tensor-core recurrence), "small" or unset/"auto"
-// (small when it qualifies, else tc for batches of at least kTcMinBatch, else layerwise).
-enum class PathChoice { kAuto, kLayerwise, kTc, kSmall };
+// persistent integer-MMA recurrence), "tc" (the tensor-core recurrence), "persist" (the persistent
+// tensor-core stack), "small" or unset/"auto" (small when it qualifies, else persist when it does, else
+// tc for batches of at least kTcMinBatch, else layerwise).
+enum class PathChoice { kAuto, kLayerwise, kTc, kSmall, kPersist };
 PathChoice path_choice();
 constexpr int64_t kTcMinBatch = 64;
 

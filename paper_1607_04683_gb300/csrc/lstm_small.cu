@@ -976,6 +976,7 @@ PathChoice path_choice() {
     if (std::strcmp(v, "layerwise") == 0) return PathChoice::kLayerwise;
     if (std::strcmp(v, "small") == 0) return PathChoice::kSmall;
     if (std::strcmp(v, "tc") == 0) return PathChoice::kTc;
+    if (std::strcmp(v, "persist") == 0) return PathChoice::kPersist;
     return PathChoice::kAuto;
 }
 

@@ -448,6 +448,11 @@ bool pdl_enabled() {
 
 }  // namespace
 
+qnn_status quantize_rows_f16(const float *src, int64_t ld, int64_t rows, int64_t len, int64_t kp, __half *dst,
+                             qnn_qparams *prm, int32_t *rsum, int *status, cudaStream_t st, int64_t tm_T, int64_t tm_B) {
+    return launch_quantize_rows_f16(src, ld, rows, len, kp, dst, prm, rsum, status, false, st, tm_T, tm_B);
+}
+
 bool tc_recurrence_supported(const qnn_lstm_model *m) {
     return m->H % 4 == 0 && (m->H / m->S) % 4 == 0 && round_up(m->R, 64) <= 1024;
 }

@@ -1285,6 +1285,23 @@ qnn_status dispatch_lstm(const TcOperands &op, const TcArgs &a, cudaStream_t st)
 
 }  // namespace
 
+qnn_status tc_map_f16(CUtensorMap *map, const __half *base, int64_t rows, int64_t ld, int box_rows) {
+    return make_map(map, base, rows, ld, box_rows);
+}
+
+qnn_status tc_map_kblocks(CUtensorMap *map, const __half *base, int64_t rows, int64_t ld, int box_rows, int box_kb) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
+    QNN_TRY(get_encode(&enc));
+    cuuint64_t dims[3] = {(cuuint64_t)TBK, (cuuint64_t)rows, (cuuint64_t)(ld / TBK)};
+    cuuint64_t strides[2] = {(cuuint64_t)(ld * 2), (cuuint64_t)(TBK * 2)};
+    cuuint32_t box[3] = {(cuuint32_t)TBK, (cuuint32_t)box_rows, (cuuint32_t)box_kb};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half *>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? QNN_OK : QNN_FAIL(QNN_ERR_CUDA);
+}
+
 int tc_choose_bn(int64_t M, int64_t N, const int *cands, int n) {
     if (const char *e = std::getenv("QNN_TC_BN")) {
         const int v = std::atoi(e);

@@ -30,6 +30,11 @@ struct TcOperands {
     int max_blocks = 0;
 };
 qnn_status tc_operands(TcOperands *op, const __half *A16, int64_t M, const __half *W16, int64_t N, int64_t kp, int bn);
+// Tensor map of centered fp16 codes [rows][ld] (ld a multiple of 64) in boxes of 64 x box_rows, 128-byte swizzle.
+qnn_status tc_map_f16(CUtensorMap *map, const __half *base, int64_t rows, int64_t ld, int box_rows);
+// The same matrix as [ld / 64 k-blocks][rows][64], in boxes of box_kb k-blocks x box_rows x 64: one load
+// brings box_kb consecutive k-blocks of the rows, each a swizzled tile of its own.
+qnn_status tc_map_kblocks(CUtensorMap *map, const __half *base, int64_t rows, int64_t ld, int box_rows, int box_kb);
 // Default tile width of a linear product (QNN_TC_BN overrides).
 int tc_pick_bn(int64_t M, int64_t N, int64_t kp);
 // Of the candidate tile widths (widest first), the widest whose share of busy SMs over the last
