@@ -756,17 +756,18 @@ qnn_status prepare(qnn_lstm_model *m) {
 
 }  // namespace
 
-// Where the launch-per-step recurrences are better although the stack qualifies. Stacks gain from layers
-// running side by side in one launch (40 frames, this against the best other path, us: 5 x 500 B = 16 472
-// : 2257, B = 256 1017 : 1211; 2 x 128 B = 256 374 : 635). A single layer is one chain either way, and two
-// row tiles or long reductions share one block's operand stream there, while the tensor-core recurrence
-// spreads a step over every SM: 1 x 500 B = 100 359 : 392 but B = 150 564 : 415; 1 x 1024 B = 64 450 : 462
-// but B = 100 524 : 482; with a few rows 1 x 1024 B = 1 383 : 369 (layerwise), B = 5 383 : 391. Posteriors in
-// pinned host memory cross the link during the wavefront's recurrence but only after this one: 5 x 500
-// B = 256 end to end 14.8 : 14.6 ms.
+// Where the launch-per-step recurrences keep a stack that qualifies. Stacks gain from layers running side
+// by side in one launch (40 frames, this against the best other path, us: 5 x 500 B = 16 472 : 2257,
+// B = 256 1017 : 1211; 2 x 128 B = 256 374 : 635). A single layer is one chain either way, and two row
+// tiles or long reductions share one block's operand stream there, while the tensor-core recurrence
+// spreads a step over every SM: it keeps single layers from its smallest batch on (1 x 500 B = 64 314 : 375,
+// B = 150 564 : 415; 1 x 1024 B = 64 450 : 462, B = 100 524 : 482). With a few rows of a wide layer the
+// layerwise kernel is as good (1 x 1024 B = 1 383 : 369, B = 5 383 : 391). Posteriors in pinned host memory
+// cross the link during the wavefront's recurrence but only after this one: 5 x 500 B = 256 end to end
+// 14.8 : 14.6 ms.
 bool persist_preferred(const qnn_lstm_model *m, int64_t B, bool host_posteriors) {
     const bool tc = tc_recurrence_supported(m) && B >= kTcMinBatch;
-    if (m->L == 1) return m->H > 512 ? (B > 4 && (B <= 64 || !tc)) : (B <= kTile || !tc);
+    if (m->L == 1) return !tc && (m->H <= 512 || B > 4);
     return !(host_posteriors && B > kTile && tc && tc_stack_supported(m));
 }
 
