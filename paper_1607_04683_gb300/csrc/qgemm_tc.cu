@@ -101,9 +101,12 @@ struct Tile {
     // memory across the block's tiles: per warp [4 gates][32 lanes] float4 (1/dx, 1/dh, rt_x, rt_h),
     // then [4 gates][32 lanes] float2 (dx, dh)
     static constexpr int RC_BYTES = EPI == kEpiLstmX ? EPI_WARPS * 24 * 32 * 4 : 0;
+    // kEpiRow: each epilogue warp's staging, 32 rows x BN / 4 fp32 columns, for its TMA stores
+    static constexpr int ROW_COLS = BN / 4, STG_BYTES = EPI == kEpiRow ? 32 * ROW_COLS * 4 : 0;
     static constexpr int EPI_BYTES = IS_LSTM              ? 2 * LSTM_BUF + RC_BYTES
                                      : EPI == kEpiPartial ? 0
-                                                          : 2 * BN * (int)(sizeof(ColConst) + sizeof(ColUnit));
+                                                          : 2 * BN * (int)(sizeof(ColConst) + sizeof(ColUnit)) +
+                                                                EPI_WARPS * STG_BYTES;
     static constexpr int SMEM_CAP = 227 * 1024 - 1024 - 256;  // dynamic shared memory left for stages + EPI_BYTES
     static constexpr int FIT_STAGES = (SMEM_CAP - EPI_BYTES) / STAGE_BYTES;
     static constexpr int WANT_STAGES = BASE_STAGES / KPS < 2 ? 2 : BASE_STAGES / KPS;
@@ -154,6 +157,7 @@ struct TcArgs {
     const int32_t *csW_x;
     const float *bias_x;
     int K_x, KB_x;
+    int y_map;  // kEpiRow: mapPX is a map of Y for TMA stores
     // LSTM epilogues: tiles from full_tiles on (the last, partial wave of the persistent grid) run as
     // two half-width items each, so that the blocks of that wave finish together (0: none)
     int64_t full_tiles;
@@ -201,17 +205,17 @@ __device__ __forceinline__ void tile_origin(int64_t tile, int64_t tiles_m, int t
     n0 = (local / rows) * bn;
 }
 
-// Recovered outputs of one 16-column block of one row that lies in one weight unit, in fp32: the
+// Recovered outputs of one block of COLS columns of one row that lies in one weight unit, in fp32: the
 // tensor-core sum P is an exact integer and, when |rt| + |za + 128| 255 K < 2^24, so is the offset
 // term rt + (za + 128) cs, formed by one fused multiply-add without rounding; the one rounded add
 // P + (offset term) then equals the rounded integer sum S of eq. (1), and S / (Qa Qw) comes from the
 // divisor's correctly rounded reciprocal (div_by_recip2: the IEEE quotient while the divisor lies
 // within 2^-60 .. 2^60). Two columns at a time with paired fp32 instructions; four 16-byte stores.
-template <bool BIAS>
-__device__ __forceinline__ void row_block_f32(const uint32_t (&r)[16], const ColConst *cc, float rtf, float za128f,
-                                              float den, float rden, float *yr) {
+template <bool BIAS, int COLS, typename Put>
+__device__ __forceinline__ void row_block_f32(const uint32_t (&r)[COLS], const ColConst *cc, float rtf, float za128f,
+                                              float den, float rden, Put put) {
 #pragma unroll
-    for (int v4 = 0; v4 < 4; ++v4) {
+    for (int v4 = 0; v4 < COLS / 4; ++v4) {
         float y[4];
 #pragma unroll
         for (int e2 = 0; e2 < 4; e2 += 2) {
@@ -222,27 +226,26 @@ __device__ __forceinline__ void row_block_f32(const uint32_t (&r)[16], const Col
             if (BIAS) q = fadd2_rn(q, make_float2(cc[i].bias, cc[i + 1].bias));
             y[e2] = q.x, y[e2 + 1] = q.y;
         }
-        *reinterpret_cast<float4 *>(yr + 4 * v4) = make_float4(y[0], y[1], y[2], y[3]);
+        put(v4, make_float4(y[0], y[1], y[2], y[3]));
     }
 }
 
 // The same block with the integer sum formed in 64 bits and an IEEE divide (rows outside the
 // bounds above).
-template <bool BIAS>
-__device__ __forceinline__ void row_block_fast(const uint32_t (&r)[16], const ColConst *cc, long long rt, int za128,
-                                               float den, float *yr) {
+template <bool BIAS, int COLS, typename Put>
+__device__ __forceinline__ void row_block_fast(const uint32_t (&r)[COLS], const ColConst *cc, long long rt, int za128,
+                                               float den, Put put) {
 #pragma unroll
-    for (int v4 = 0; v4 < 4; ++v4) {
+    for (int v4 = 0; v4 < COLS / 4; ++v4) {
         float y[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const int i = 4 * v4 + e;
             const long long S = (long long)f32_integer_to_s32(__uint_as_float(r[i])) + rt + (long long)za128 * cc[i].cs;
-            const float x = s64_to_f32_rn(S);
-            y[e] = __fdiv_rn(x, den);
+            y[e] = fdiv_any(s64_to_f32_rn(S), den);
             if (BIAS) y[e] = __fadd_rn(y[e], cc[i].bias);
         }
-        *reinterpret_cast<float4 *>(yr + 4 * v4) = make_float4(y[0], y[1], y[2], y[3]);
+        put(v4, make_float4(y[0], y[1], y[2], y[3]));
     }
 }
 
@@ -621,11 +624,12 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         }
     } else if constexpr (EPI == kEpiRow) {
         // ---------------- epilogue (warps 2..17): recovered product, one row per lane ----------------
-        // Each lane owns one output row; the four warps of a lane quarter take its 16-column blocks
-        // in turn: eq. (1)'s offsets and eq. (3)'s recovery per element, stored as 16-byte vectors
-        // (ragged edges element by element). The column constants of the tile are staged in shared
-        // memory (double-buffered by tile parity; one named barrier of the epilogue warps per tile).
-        ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES);
+        // Each lane owns one output row; the four warps of a lane quarter take a quarter of its columns
+        // each: eq. (1)'s offsets and eq. (3)'s recovery per element. The column constants of the tile are
+        // staged in shared memory (double-buffered by tile parity; one named barrier of the epilogue warps
+        // per tile).
+        uint8_t *const stg = smem + STAGES * TL::STAGE_BYTES + (warp - 2) * TL::STG_BYTES;
+        ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES + TL::EPI_WARPS * TL::STG_BYTES);
         ColUnit *sunit = reinterpret_cast<ColUnit *>(scol + 2 * BN);
         const int q = warp & 3;
         const int part = (warp - 2) >> 2;
@@ -676,14 +680,51 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 if (failed) *reinterpret_cast<volatile int *>(&s_abort) = 1;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            // The usual tile: every warp takes a quarter of the columns of its 32 rows; when they lie in one
+            // weight unit (and no raw products are wanted) the outputs go through the warp's staging buffer,
+            // swizzled so that neither side conflicts, and out as one TMA store of whole row segments. (Stored
+            // from registers, one 16-byte piece of 32 different rows an instruction, they take most of the
+            // epilogue's time: 128000 x 2000 x 500 535 us, so 389; 102400 x 8192 x 512 1884 us, so 1343.)
+            constexpr int RC = TL::ROW_COLS;
+            const int cq = part * RC;
+            const bool staged = args.y_map && !args.acc_out && cu[cq].unit >= 0 && cu[cq].unit == cu[cq + RC - 1].unit;
+            if (staged && !failed) {
+                uint32_t r[RC];
+                if constexpr (RC == 32)
+                    tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + cq), r);
+                else
+                    tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + cq), r);
+                if (lane == 0) bulk_wait_read();  // the buffer's previous store has read it
+                __syncwarp();
+                const int zw = cc[cq].zw;
+                const long long rt = (long long)(128 + zw) * ra + (long long)K * ((long long)za * zw - 16384);
+                const float den = __fmul_rn(Qa, cc[cq].Qw);
+                uint8_t *const row = stg + lane * RC * 4;
+                const int sw = RC == 32 ? lane & 7 : (lane >> 1) & 3;  // 128- or 64-byte swizzle
+                auto put = [&](int i, float4 v) { *reinterpret_cast<float4 *>(row + ((i ^ sw) << 4)) = v; };
+                if (den >= 0x1p-60f && den <= 0x1p60f && llabs(rt) + (long long)abs(za128) * 255 * K < (1LL << 24)) {
+                    const float rden = rcp_rn(den);
+                    if (args.bias)
+                        row_block_f32<true>(r, cc + cq, (float)rt, (float)za128, den, rden, put);
+                    else
+                        row_block_f32<false>(r, cc + cq, (float)rt, (float)za128, den, rden, put);
+                } else if (args.bias) {
+                    row_block_fast<true>(r, cc + cq, rt, za128, den, put);
+                } else {
+                    row_block_fast<false>(r, cc + cq, rt, za128, den, put);
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) tma_store_2d(&mapPX, su32(stg), (int)n0 + cq, (int)m0 + 32 * q);
+            }
 #pragma unroll 1
-            for (int j = part; j < BN / 16 && !failed; j += TL::EPI_WARPS / 4) {
+            for (int j = part * (RC / 16); j < (part + 1) * (RC / 16) && !failed && !staged; ++j) {
                 const int c0 = 16 * j;
                 uint32_t r[16];
                 tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + c0), r);
                 const int64_t nb = n0 + c0;
                 if (!mv || nb >= args.N) continue;
-                // one weight unit across the 16 columns (the usual case): row terms hoisted
+                // row terms hoisted when one weight unit covers the 16 columns
                 const bool one_unit = cu[c0].unit == cu[c0 + 15].unit;  // -1 past N: ragged blocks take the general way
                 long long rt = 0;
                 float den = 0.0f;
@@ -694,21 +735,6 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 }
                 float *yr = args.Y ? args.Y + m * args.ldy + nb : nullptr;
                 const bool full = vec && nb + 16 <= args.N;
-                if (one_unit && full && !args.acc_out) {  // the usual block: no per-element branches
-                    if (den >= 0x1p-60f && den <= 0x1p60f &&
-                        llabs(rt) + (long long)abs(za128) * 255 * K < (1LL << 24)) {
-                        const float rden = rcp_rn(den);
-                        if (args.bias)
-                            row_block_f32<true>(r, cc + c0, (float)rt, (float)za128, den, rden, yr);
-                        else
-                            row_block_f32<false>(r, cc + c0, (float)rt, (float)za128, den, rden, yr);
-                    } else if (args.bias) {
-                        row_block_fast<true>(r, cc + c0, rt, za128, den, yr);
-                    } else {
-                        row_block_fast<false>(r, cc + c0, rt, za128, den, yr);
-                    }
-                    continue;
-                }
 #pragma unroll
                 for (int v4 = 0; v4 < 4; ++v4) {
                     float y[4];
@@ -727,7 +753,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                                 (long long)K * ((long long)za * v.zw - 16384);
                             dn = __fmul_rn(Qa, v.Qw);
                         }
-                        y[e] = __fdiv_rn(s64_to_f32_rn(S), dn);
+                        y[e] = fdiv_any(s64_to_f32_rn(S), dn);
                         if (args.bias) y[e] = __fadd_rn(y[e], v.bias);
                         if (args.acc_out && nb + i < args.N)
                             args.acc_out[m * args.N + nb + i] = P + 128 * (ra + v.cs) - 16384 * K;  // raw code product
@@ -746,6 +772,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             if (lane == 0) mb_arrive(drained0 + 8 * buf);
             ++gc;
         }
+        if (lane == 0) bulk_wait();  // (the staging buffers are read until then)
     } else if constexpr (EPI == kEpiPartial) {
         // ---------------- epilogue (warps 2..17): split-K partial sums ----------------
         // The item's K range is at most one accumulation chunk, so its fp32 accumulator holds the
@@ -1156,9 +1183,10 @@ qnn_status get_encode(PFN_cuTensorMapEncodeTiled_v12000 *out) {
 }
 
 // 2-D fp32 tensor: rows of `cols` values, `ld` values apart (ld a multiple of 4, base 16-byte
-// aligned), boxes of box_cols x box_rows, no swizzle (rows of the box land box_cols * 4 bytes apart).
+// aligned), boxes of box_cols x box_rows; swizzle 0 (rows of the box land box_cols * 4 bytes apart), or
+// 64 or 128 bytes, then box_cols * 4.
 qnn_status make_map_f32(CUtensorMap *map, const float *base, int64_t rows, int64_t cols, int64_t ld, int box_cols,
-                        int box_rows) {
+                        int box_rows, int swizzle = 0) {
     if ((reinterpret_cast<uintptr_t>(base) & 15) || ld % 4 || box_cols % 4) return QNN_ERR_INVALID_ARG;
     PFN_cuTensorMapEncodeTiled_v12000 enc = nullptr;
     QNN_TRY(get_encode(&enc));
@@ -1167,7 +1195,10 @@ qnn_status make_map_f32(CUtensorMap *map, const float *base, int64_t rows, int64
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     swizzle == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                     : swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                     : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? QNN_OK : QNN_FAIL(QNN_ERR_CUDA);
 }
@@ -1254,9 +1285,15 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
 
 qnn_status dispatch_linear(const TcOperands &op, const TcArgs &a, cudaStream_t st) {
     if (op.row_epilogue) {
+        // Y by TMA where its rows are 16-byte aligned (else from registers)
+        CUtensorMap map_y;
+        TcArgs r = a;
+        r.y_map = a.Y && a.ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0 && a.M <= INT32_MAX && a.N <= INT32_MAX;
+        if (r.y_map) QNN_TRY(make_map_f32(&map_y, a.Y, a.M, a.N, a.ldy, op.bn / 4, 32, op.bn == 128 ? 128 : 64));
+        const CUtensorMap *my = r.y_map ? &map_y : nullptr;
         switch (op.bn) {
-            case 64: return launch_tc<64, kEpiRow>(op, a, "qgemm_tc", st);
-            case 128: return launch_tc<128, kEpiRow>(op, a, "qgemm_tc", st);
+            case 64: return launch_tc<64, kEpiRow>(op, r, "qgemm_tc", st, my);
+            case 128: return launch_tc<128, kEpiRow>(op, r, "qgemm_tc", st, my);
             default: return QNN_ERR_INVALID_ARG;
         }
     }

@@ -80,3 +80,31 @@ def test_float_output_layer_tiles(qnn, B, T, H, C):
                               want_logits=True)
     parity.check_logits(lg.cpu().numpy(), ref["logits"], 2, ref["h_all"][0], wl.out_weights(params))
     parity.check_posteriors(y.cpu().numpy(), ref["y"])
+
+
+# The tensor-core product's outputs without raw sums: K <= 1024 stores them by TMA from staging buffers
+# (whole units, ragged rows and columns, rows further apart than N, unaligned rows from registers), longer K
+# whole blocks of 32 columns in 32-bit sums; offsets beyond the fp32 and the 32-bit forms take the others.
+@pytest.mark.parametrize("bn", ["64", "128", "256"])
+@pytest.mark.parametrize("M,N,K,pad", [(1, 8, 1, 0), (33, 64, 64, 0), (128, 256, 64, 4), (130, 260, 100, 0), (257, 2000, 500, 8),
+                                       (200, 136, 1000, 1), (384, 512, 1024, 0), (129, 260, 1025, 0), (257, 320, 3000, 4)])
+@pytest.mark.parametrize("shift", [0.0, 20.0, 3000.0])
+def test_tensor_core_outputs(qnn, M, N, K, pad, bn, shift, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "tc")
+    monkeypatch.setenv("QNN_TC_BN", bn)
+    g = np.random.Generator(np.random.PCG64(M + N + K))
+    A = (g.normal(0.1, 1.0, (M, K)) + shift).astype(np.float32)
+    nb = 4 if N % 4 == 0 else 1
+    Ws = [g.uniform(-s, s, (N // nb, K)).astype(np.float32) for s in np.linspace(0.05, 0.4, nb)]
+    ga = oracle.PER_ROW if M % 2 else oracle.PER_MATRIX
+    ca, pa, ra = oracle.quantize(A, ga)
+    parts = [oracle.quantize(w, oracle.PER_MATRIX) for w in Ws]
+    cw, pw, cs = (np.concatenate([p[i] for p in parts]) for i in range(3))
+    bias = g.normal(0, 1, N).astype(np.float32) if K % 2 == 0 else None
+    ref = oracle.qmatmul(ca, pa, ga, cw, pw, n_blocks=nb, bias=bias)
+    out = torch.full((M + 1, N + pad), 7.0, device="cuda")
+    qnn.qnn_qmatmul(gpu(ca), qnn.params_tensor(pa), ga, gpu(ra), gpu(cw), qnn.params_tensor(pw), gpu(cs), n_blocks=nb,
+                    bias=None if bias is None else gpu(bias), out=out[:M, :N])
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(out[:M, :N].cpu().numpy(), ref["y"])
+    assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
