@@ -97,13 +97,14 @@ struct Tile {
     static constexpr int COL_BYTES = 12 * (BN / 4) * 4;
     static constexpr int LSTM_TX = EPI == kEpiLstmX ? PX_BOX + COL_BYTES : 5 * PX_BOX;  // bytes of one fill
     static constexpr int LSTM_BUF = (LSTM_TX + 1023) / 1024 * 1024;  // [4 px boxes +] the c box [+ constants]
-    // kEpiLstmX: per epilogue thread, its row's per-gate constants of eq. (1)/(3), kept in shared
-    // memory across the block's tiles: per warp [4 gates][32 lanes] float4 (1/dx, 1/dh, rt_x, rt_h),
-    // then [4 gates][32 lanes] float2 (dx, dh)
-    static constexpr int RC_BYTES = EPI == kEpiLstmX ? EPI_WARPS * 24 * 32 * 4 : 0;
+    // kEpiLstmX: the tile's cell outputs, staged for their TMA stores (as the new cell state is in the c
+    // box), and by row quarter its rows' per-gate constants of eq. (1)/(3), kept across the block's tiles:
+    // [4 gates][32 rows] float4 (1/dx, 1/dh, rt_x, rt_h), then [4 gates][32 rows] float2 (dx, dh)
+    static constexpr int OUT_BYTES = EPI == kEpiLstmX ? PX_BOX : 0;
+    static constexpr int RC_BYTES = EPI == kEpiLstmX ? 4 * 24 * 32 * 4 : 0;
     // kEpiRow: each epilogue warp's staging, 32 rows x BN / 4 fp32 columns, for its TMA stores
     static constexpr int ROW_COLS = BN / 4, STG_BYTES = EPI == kEpiRow ? 32 * ROW_COLS * 4 : 0;
-    static constexpr int EPI_BYTES = IS_LSTM              ? 2 * LSTM_BUF + RC_BYTES
+    static constexpr int EPI_BYTES = IS_LSTM              ? 2 * LSTM_BUF + OUT_BYTES + RC_BYTES
                                      : EPI == kEpiPartial ? 0
                                                           : 2 * BN * (int)(sizeof(ColConst) + sizeof(ColUnit)) +
                                                                 EPI_WARPS * STG_BYTES;
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     qgemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapW,
                     const __grid_constant__ CUtensorMap mapPX, const __grid_constant__ CUtensorMap mapC,
                     const __grid_constant__ CUtensorMap mapAX, const __grid_constant__ CUtensorMap mapWX,
+                    const __grid_constant__ CUtensorMap mapH,
                     const TcArgs args) {
     using TL = Tile<BN, EPI>;
     constexpr int STAGES = TL::STAGES;
@@ -314,7 +316,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             mb_init(chunk0 + 8 * i, 1);      // MMA -> epilogue: chunk accumulated in buffer i
             mb_init(drained0 + 8 * i, TL::EPI_WARPS);  // epilogue -> MMA: buffer i read out by every epilogue warp
             mb_init(pxfull0 + 8 * i, 1);
-            mb_init(pxempty0 + 8 * i, TL::EPI_WARPS);
+            mb_init(pxempty0 + 8 * i, LX ? 4 : TL::EPI_WARPS);  // by epilogue warp, or row quarter (LX)
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -830,9 +832,10 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         const int K = args.K;
         const TcLstmOut &E = args.lstm;
         const int H = E.H;
-        // px and c of a tile come into shared memory by TMA, two tiles ahead: buffer i % 2 holds
-        // the block's i-th tile; one thread (warp 2, lane 0) refills a buffer once every epilogue
-        // warp has released it, so the loads overlap the arithmetic of the tile in between
+        // px and c of a tile come into shared memory by TMA, ahead of it: buffer i % 2 holds the block's
+        // i-th tile; one thread (warp 2, lane 0) refills a buffer once it is released, at the end of a
+        // tile for the tile two on (kEpiLstm), or halfway through the next one (kEpiLstmX, whose new
+        // cell state leaves from the buffer)
         constexpr int CW = BN / 4;  // cells per tile
         constexpr int C_OFF = LX ? 0 : 4 * TL::PX_BOX;  // the c box within a buffer (after the px boxes)
         float *const pxs0 = reinterpret_cast<float *>(smem + STAGES * TL::STAGE_BYTES);
@@ -851,30 +854,46 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                       // then maps the [12][H] constant table)
                 tma_load_2d(dst + TL::PX_BOX, &mapPX, bar, (int)(n1 / 4), 0);
             }
-            tma_load_2d(dst + C_OFF, &mapC, bar, (int)(n1 / 4), (int)m1);
+            if constexpr (LX) {  // swizzled, a row quarter each
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    tma_load_2d(dst + i * (TL::PX_BOX / 4), &mapC, bar, (int)(n1 / 4), (int)m1 + 32 * i);
+            } else {
+                tma_load_2d(dst + C_OFF, &mapC, bar, (int)(n1 / 4), (int)m1);
+            }
         };
         if (issuer) {
             if (blockIdx.x < work) issue_px(blockIdx.x, 0);
             if (blockIdx.x + gridDim.x < work) issue_px(blockIdx.x + gridDim.x, 1);
         }
-        // kEpiLstmX with one weight unit per gate matrix: the correctly rounded reciprocals of the
-        // per-row, per-gate divisors Qa Qw of eq. (3) are computed once for the block's row tile and
-        // kept (in this thread's shared-memory slots) while it stays on that tile; the other row
-        // terms are cheap to re-form
+        // kEpiLstmX with one weight unit per gate matrix: the rows' divisors Qa Qw of eq. (3), their
+        // correctly rounded reciprocals and the constant parts of the sums are formed once while the block
+        // stays on a row tile, a gate by each of the quarter's warps
+        static_assert(!LX || TL::EPI_WARPS == 16, "a gate per warp");
         int64_t cm0 = -1;
         bool fastrow = false;
-        float *const rcw = pxs0 + 2 * (TL::LSTM_BUF / 4) + (warp - 2) * 24 * 32;  // this warp's constants
-        float4 *const rq = reinterpret_cast<float4 *>(rcw) + lane;                 // rq[32 g]
-        float2 *const rd = reinterpret_cast<float2 *>(rcw + 16 * 32) + lane;       // rd[32 g]
+        uint8_t *const hst = reinterpret_cast<uint8_t *>(pxs0) + 2 * TL::LSTM_BUF;  // staged outputs
+        float *const rcw = reinterpret_cast<float *>(hst + TL::OUT_BYTES) + q * 24 * 32;
+        float4 *const rq = reinterpret_cast<float4 *>(rcw) + lane;            // rq[32 g]
+        float2 *const rd = reinterpret_cast<float2 *>(rcw + 16 * 32) + lane;  // rd[32 g]
+        auto quarter_bar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + q), "n"(8 * TL::EPI_WARPS) : "memory"); };
+        // 16-byte chunk i of the row's cells in a swizzled box (128-, 64- or 32-byte rows and swizzle)
+        const int sw = BN == 128 ? lane & 7 : BN == 64 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+        auto cells_at = [&](uint8_t *box, int cell) {
+            return reinterpret_cast<float *>(box + (32 * q + lane) * CW * 4 + (((cell >> 2) ^ sw) << 4) + (cell & 3) * 4);
+        };
         int64_t gc = 0;
         bool ok = true;
         // row b's units and code sums: za, Qa, rs of h_{t-1}; zx, Qx, rsx of x_t (kEpiLstmX)
         int64_t lm0 = -1;
         int za = 0, rs = 0, zx = 0, rsx = 0;
         float Qa = 1.0f, Qx = 1.0f;
-        for (int64_t tile = blockIdx.x; tile < work && ok; tile += gridDim.x) {
+        // kEpiLstmX: every warp runs every tile (the quarter's barriers count on it); after a wait gave up
+        // the remaining tiles are skipped without waiting
+        for (int64_t tile = blockIdx.x; tile < work && (LX || ok); tile += gridDim.x) {
             int64_t m0, n0;
-            const int slices = item_origin(tile, m0, n0) ? SLICES / 2 : SLICES;  // half-width items: half the slices
+            const bool half = item_origin(tile, m0, n0);
+            const int slices = half ? SLICES / 2 : SLICES;  // half-width items: half the slices
             const int pbuf = (int)(gc & 1);  // this tile's px/c buffer (gc counts the block's tiles)
             const float *pxb = pxs0 + pbuf * (TL::LSTM_BUF / 4);
             const int rl = 32 * q + lane;    // row within the tile
@@ -899,42 +918,54 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             const int za128 = 128 + za;
             const float za128f = (float)za128;
             const float zx128f = (float)(128 + zx);
+            if constexpr (LX) {
+                // the previous tile's stores have read their boxes: its c buffer may be refilled, and once
+                // the quarter has met, the staged outputs overwritten
+                if (eh == 0 && lane == 0 && gc > 0) {
+                    bulk_wait_read();
+                    mb_arrive(pxempty0 + 8 * (pbuf ^ 1));
+                }
+                quarter_bar();
+            }
             if (LX && E.ups == 1 && m0 != cm0) {
                 // The fast path forms S = P + rt_g + (128 + z_row) cs of eq. (1) in fp32: the tensor-core
                 // sum P is an exact integer, and when |rt_g| + |128 + z_row| 255 K < 2^24 the offset term
                 // rt_g + (128 + z_row) cs is an exact integer too (cs <= 255 K) and one fused multiply-add
                 // forms it without rounding, so the single rounded addition P + (offset term) equals the
-                // correctly rounded S (S itself stays below 2^31 when K max|a' + za| max|w' + zw| < 2^31).
+                // correctly rounded S.
                 // The quotient S / (Qa Qw) is the correctly rounded q + (S - q d) r with r = RN(1/d),
                 // q = RN(S r) (Markstein's final step), which needs d and r far from the ends of the fp32
                 // range. Rows outside these bounds take the general path below.
                 cm0 = m0;
-                const long long ax = max(abs(zx), abs(zx + 255)), ah = max(abs(za), abs(za + 255));
-                bool f = bv;
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
+                {
+                    const int g = eh;
                     const qnn_qparams qw = args.pw_x[g], qh = args.pw[g];
                     const float dx = __fmul_rn(Qx, qw.Q), dh = __fmul_rn(Qa, qh.Q);
                     const long long rtx = (long long)(128 + qw.z) * rsx + (long long)args.K_x * ((long long)zx * qw.z - 16384);
                     const long long rth = (long long)(128 + qh.z) * rs + (long long)K * ((long long)za * qh.z - 16384);
-                    // (rt_x, rt_h exact when the bound below holds)
+                    const bool f = llabs(rtx) + (long long)abs(128 + zx) * 255 * args.K_x < (1LL << 24) &&
+                                   llabs(rth) + (long long)abs(za128) * 255 * K < (1LL << 24) && dx >= 0x1p-60f &&
+                                   dx <= 0x1p60f && dh >= 0x1p-60f && dh <= 0x1p60f;
+                    // (rt_x, rt_h exact when the bound holds; dx = 0 where a bound does not)
                     rq[32 * g] = make_float4(rcp_rn(dx), rcp_rn(dh), (float)rtx, (float)rth);
-                    rd[32 * g] = make_float2(dx, dh);
-                    f &= (long long)args.K_x * ax * (long long)max(abs(qw.z), abs(qw.z + 255)) < (1LL << 31) &&
-                         (long long)K * ah * (long long)max(abs(qh.z), abs(qh.z + 255)) < (1LL << 31) &&
-                         llabs(rtx) + (long long)abs(128 + zx) * 255 * args.K_x < (1LL << 24) &&
-                         llabs(rth) + (long long)abs(za128) * 255 * K < (1LL << 24) &&
-                         dx >= 0x1p-60f && dx <= 0x1p60f && dh >= 0x1p-60f && dh <= 0x1p60f;
+                    rd[32 * g] = make_float2(f ? dx : 0.0f, dh);
                 }
+                quarter_bar();
+                const bool f = bv && rd[0].x != 0.0f && rd[32].x != 0.0f && rd[64].x != 0.0f && rd[96].x != 0.0f;
                 fastrow = f;
             }
             const int buf = (int)(gc & 1);
-            ok = __all_sync(0xffffffffu, mb_wait(chunk0 + 8 * buf, (unsigned)(gc / 2) & 1, args.status) &&
-                                             mb_wait(pxfull0 + 8 * pbuf, (unsigned)(gc / 2) & 1, args.status));
-            if (!ok) break;
+            if (LX && ok && *reinterpret_cast<volatile int *>(&s_abort)) ok = false;
+            if (ok)
+                ok = __all_sync(0xffffffffu, mb_wait(chunk0 + 8 * buf, (unsigned)(gc / 2) & 1, args.status) &&
+                                                 mb_wait(pxfull0 + 8 * pbuf, (unsigned)(gc / 2) & 1, args.status));
+            if (!ok) {
+                if (!LX) break;
+                *reinterpret_cast<volatile int *>(&s_abort) = 1;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
-            for (int s = eh; s < slices; s += TL::EPI_WARPS / 4) {
+            for (int s = eh; s < slices && ok; s += TL::EPI_WARPS / 4) {
                 const int gi = s / SPG, part = s % SPG;
                 const int j0 = (int)(n0 / 4) + gi * 8 + part * CPS;  // H is a multiple of 4: all CPS valid or none
                 if constexpr (LX) {
@@ -954,7 +985,8 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                     const int unit = j0 / E.cpu;
                     // the slice's cell state in, and its new state and outputs out, as one vector each
                     float cst[CPS], mst[CPS];
-                    if (valid) ld_vec(pxb + C_OFF / 4 + rl * CW + jt, cst);
+                    uint8_t *const cbox = reinterpret_cast<uint8_t *>(pxs0) + pbuf * TL::LSTM_BUF;
+                    if (valid) ld_vec(cells_at(cbox, jt), cst);
 #pragma unroll
                     for (int c2 = 0; c2 < CPS; c2 += 2) {
                         uint32_t rx[4][2], rh[4][2];
@@ -1031,10 +1063,16 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                         cst[c2] = cv.x, cst[c2 + 1] = cv.y;
                         mst[c2] = mv.x, mst[c2 + 1] = mv.y;
                     }
-                    if (valid) {
+                    if (valid && !half) {  // whole tiles leave by TMA below
+                        st_vec(cells_at(cbox, jt), cst);
+                        st_vec(cells_at(hst, jt), mst);
+                    } else if (valid) {
                         st_vec(E.c + b * (int64_t)H + j0, cst);
                         st_vec(E.h + b * E.h_ld + j0, mst);
                     }
+                    if (s == eh && issuer && gc > 0 && tile + (int64_t)gridDim.x < work &&
+                        mb_wait(pxempty0 + 8 * (pbuf ^ 1), (unsigned)((gc - 1) / 2) & 1, args.status))
+                        issue_px(tile + (int64_t)gridDim.x, pbuf ^ 1);
                     continue;
                 }
                 uint32_t r[4][CPS];
@@ -1095,14 +1133,27 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             __syncwarp();
             if (lane == 0) {
                 mb_arrive(drained0 + 8 * buf);
-                mb_arrive(pxempty0 + 8 * pbuf);
+                if (!LX) mb_arrive(pxempty0 + 8 * pbuf);
+            }
+            if constexpr (LX) {
+                // the quarter's new cell state and outputs, 32 rows each, as whole row segments (stored from
+                // registers, 16 bytes of 32 rows an instruction, they and the unswizzled reads of c took a
+                // quarter of the shared-memory and L1 cycles that bound a tile)
+                fence_async_smem();
+                quarter_bar();
+                if (ok && !half && eh == 0 && lane == 0) {
+                    tma_store_2d(&mapC, su32(pxs0) + (uint32_t)(pbuf * TL::LSTM_BUF + q * (TL::PX_BOX / 4)), (int)(n0 / 4),
+                                 (int)m0 + 32 * q);
+                    tma_store_2d(&mapH, su32(hst) + (uint32_t)(q * (TL::PX_BOX / 4)), (int)(n0 / 4), (int)m0 + 32 * q);
+                }
             }
             // refill the buffer with the tile two ahead once every epilogue warp has released it
-            if (issuer && tile + 2 * (int64_t)gridDim.x < work &&
+            if (!LX && issuer && tile + 2 * (int64_t)gridDim.x < work &&
                 mb_wait(pxempty0 + 8 * pbuf, (unsigned)(gc / 2) & 1, args.status))
                 issue_px(tile + 2 * (int64_t)gridDim.x, pbuf);
             ++gc;
         }
+        if (LX && lane == 0) bulk_wait();
         if (!ok) s_abort = 1;  // copies may still be in flight: the block waits for them before leaving
     }
     __syncwarp();
@@ -1184,7 +1235,7 @@ qnn_status get_encode(PFN_cuTensorMapEncodeTiled_v12000 *out) {
 
 // 2-D fp32 tensor: rows of `cols` values, `ld` values apart (ld a multiple of 4, base 16-byte
 // aligned), boxes of box_cols x box_rows; swizzle 0 (rows of the box land box_cols * 4 bytes apart), or
-// 64 or 128 bytes, then box_cols * 4.
+// 32, 64 or 128 bytes, then box_cols * 4.
 qnn_status make_map_f32(CUtensorMap *map, const float *base, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                         int box_rows, int swizzle = 0) {
     if ((reinterpret_cast<uintptr_t>(base) & 15) || ld % 4 || box_cols % 4) return QNN_ERR_INVALID_ARG;
@@ -1198,6 +1249,7 @@ qnn_status make_map_f32(CUtensorMap *map, const float *base, int64_t rows, int64
                      CU_TENSOR_MAP_INTERLEAVE_NONE,
                      swizzle == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                      : swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                     : swizzle == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
                                      : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? QNN_OK : QNN_FAIL(QNN_ERR_CUDA);
@@ -1230,7 +1282,8 @@ namespace {
 template <int BN, int EPI>
 qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cudaStream_t st,
                      const CUtensorMap *map_px = nullptr, const CUtensorMap *map_c = nullptr,
-                     const CUtensorMap *map_ax = nullptr, const CUtensorMap *map_wx = nullptr) {
+                     const CUtensorMap *map_ax = nullptr, const CUtensorMap *map_wx = nullptr,
+                     const CUtensorMap *map_h = nullptr) {
     using TL = Tile<BN, EPI>;
     static int configured = -1;
     int dev = 0;
@@ -1277,9 +1330,9 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = op.pdl ? 1 : 0;
-    // the px, c, x and Wx maps are read by the LSTM kernels only (the others get A's map, unused)
+    // the px, c, x, Wx and output maps are read by the LSTM kernels only (the others get A's map, unused)
     QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, qgemm_tc_kernel<BN, EPI>, op.a, op.w, map_px ? *map_px : op.a,
-                                    map_c ? *map_c : op.a, map_ax ? *map_ax : op.a, map_wx ? *map_wx : op.w, args));
+                                    map_c ? *map_c : op.a, map_ax ? *map_ax : op.a, map_wx ? *map_wx : op.w, map_h ? *map_h : op.a, args));
     return QNN_OK;
 }
 
@@ -1424,16 +1477,16 @@ qnn_status tc_lstm_gates_x(const TcOperands &op, const qnn_qparams *pa, const in
              1, kbh + kbx, nullptr, 0, 1};
     a.pa_x = in.pa, a.x_stride = in.stride, a.rsA_x = in.rs, a.pw_x = in.pw4, a.csW_x = in.cs, a.bias_x = in.bias;
     a.K_x = in.K_x, a.KB_x = kbx;
-    CUtensorMap map_c, map_ax, map_wx, map_col;
-    QNN_TRY(make_map_f32(&map_c, out.c, op.M, out.H, out.H, op.bn / 4, TBM));
+    CUtensorMap map_c, map_h, map_ax, map_wx, map_col;
+    QNN_TRY(make_map_f32(&map_c, out.c, op.M, out.H, out.H, op.bn / 4, 32, op.bn));
+    QNN_TRY(make_map_f32(&map_h, out.h, op.M, out.H, out.h_ld, op.bn / 4, 32, op.bn));
     QNN_TRY(make_map_f32(&map_col, reinterpret_cast<const float *>(in.colc), 12, out.H, out.H, op.bn / 4, 12));
     QNN_TRY(make_map(&map_ax, in.x16, op.M, in.kx, TBM, in.x_pitch));
     QNN_TRY(make_map(&map_wx, in.wx16, op.N, in.kx, op.bn));
     switch (op.bn) {
-        case 32: return launch_tc<32, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx);
-        case 64: return launch_tc<64, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx);
-        case 96: return launch_tc<96, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx);
-        case 128: return launch_tc<128, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx);
+        case 32: return launch_tc<32, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx, &map_h);
+        case 64: return launch_tc<64, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx, &map_h);
+        case 128: return launch_tc<128, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx, &map_h);
         default: return QNN_ERR_INVALID_ARG;
     }
 }
