@@ -4,8 +4,13 @@
 // flagged) and a code pass (eq. 2 with the unit's Q and z, four codes per 32-bit store, row code
 // sums). Per-row units (one frame of one sequence) take one warp per row; rows of up to 1024
 // values stay in the warp's registers between the passes (read once), longer ones are re-read
-// from L1/L2. A per-matrix unit first reduces block partials into a small scratch array;
-// the last block to finish folds them into the unit's parameters, then a second launch writes codes.
+// from L1/L2. A per-matrix unit first reduces block partials into a small scratch array; the last
+// block to finish folds them into the unit's parameters, then a second launch writes codes.
+//
+// Bound: HBM (5 bytes a value for rows, 9 for a matrix beyond L2). Per matrix 8192 x 8192: 117 us with one
+// 16-byte load in flight a lane and both passes from HBM; 101 us with eight in flight and the code pass
+// starting where the range pass ended, in rows that L2 still holds.
+#include <algorithm>
 #include <cfloat>
 #include <cstdlib>
 
@@ -18,39 +23,44 @@ namespace {
 
 constexpr int kRowWarps = 8;  // warps (rows) per block in the per-row kernels
 
+constexpr int kFlight = 8;    // 16-byte loads in flight per lane in the passes over long rows
+
+// Running range of values and whether one was not finite: v * 0 is NaN then, and so is the sum.
+struct Range {
+    float mn = FLT_MAX, mx = -FLT_MAX, bad = 0.0f;
+    __device__ __forceinline__ void add(float v) {
+        mn = fminf(mn, v);
+        mx = fmaxf(mx, v);
+        bad = __fmaf_rn(v, 0.0f, bad);
+    }
+    __device__ __forceinline__ void add(const float4 &v) { add(v.x), add(v.y), add(v.z), add(v.w); }
+    __device__ __forceinline__ bool finite() const { return bad == 0.0f; }
+};
+
 // Range of one row held by one warp; returns false if a value is not finite.
 template <bool kVec>
 __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int cols, float &mn, float &mx) {
     const int lane = threadIdx.x & 31;
-    mn = FLT_MAX;
-    mx = -FLT_MAX;
-    bool bad = false;
+    Range r;
+    int done = 0;
     if (kVec) {
         const float4 *x4 = reinterpret_cast<const float4 *>(xr);
         const int n4 = cols >> 2;
-        for (int i = lane; i < n4; i += 32) {
-            float4 v = __ldg(x4 + i);
-            bad |= !isfinite(v.x) | !isfinite(v.y) | !isfinite(v.z) | !isfinite(v.w);
-            mn = fminf(fminf(mn, v.x), fminf(v.y, fminf(v.z, v.w)));
-            mx = fmaxf(fmaxf(mx, v.x), fmaxf(v.y, fmaxf(v.z, v.w)));
+        for (int i = lane; i < n4; i += 32 * kFlight) {
+            float4 v[kFlight];
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u)
+                if (i + 32 * u < n4) v[u] = __ldg(x4 + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u)
+                if (i + 32 * u < n4) r.add(v[u]);
         }
-        for (int i = (n4 << 2) + lane; i < cols; i += 32) {
-            float v = __ldg(xr + i);
-            bad |= !isfinite(v);
-            mn = fminf(mn, v);
-            mx = fmaxf(mx, v);
-        }
-    } else {
-        for (int i = lane; i < cols; i += 32) {
-            float v = __ldg(xr + i);
-            bad |= !isfinite(v);
-            mn = fminf(mn, v);
-            mx = fmaxf(mx, v);
-        }
+        done = n4 << 2;
     }
-    mn = warp_min(mn);
-    mx = warp_max(mx);
-    return !__any_sync(0xffffffffu, bad);
+    for (int i = done + lane; i < cols; i += 32) r.add(__ldg(xr + i));
+    mn = warp_min(r.mn);
+    mx = warp_max(r.mx);
+    return __all_sync(0xffffffffu, r.finite());
 }
 
 // Codes of one row (eq. 2) and their sum, one warp.
@@ -63,12 +73,19 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
         const float4 *x4 = reinterpret_cast<const float4 *>(xr);
         uint32_t *c4 = reinterpret_cast<uint32_t *>(cr);
         const int n4 = cols >> 2;
-        for (int i = lane; i < n4; i += 32) {
-            float4 v = __ldg(x4 + i);
-            uint32_t a = quant_code(v.x, Q, z), b = quant_code(v.y, Q, z), c = quant_code(v.z, Q, z),
-                     d = quant_code(v.w, Q, z);
-            s += (int)(a + b + c + d);
-            c4[i] = a | (b << 8) | (c << 16) | (d << 24);
+        for (int i = lane; i < n4; i += 32 * kFlight) {
+            float4 v[kFlight];
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u)
+                if (i + 32 * u < n4) v[u] = __ldg(x4 + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < kFlight; ++u) {
+                if (i + 32 * u >= n4) break;
+                const uint32_t a = quant_code(v[u].x, Q, z), b = quant_code(v[u].y, Q, z), c = quant_code(v[u].z, Q, z),
+                               d = quant_code(v[u].w, Q, z);
+                s += (int)(a + b + c + d);
+                c4[i + 32 * u] = a | (b << 8) | (c << 16) | (d << 24);
+            }
         }
         for (int i = (n4 << 2) + lane; i < cols; i += 32) {
             uint32_t a = quant_code(__ldg(xr + i), Q, z);
@@ -109,20 +126,13 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
 }
 
 // Per-row units of at most 1024 values (16-byte aligned input rows): the warp holds its row in
-// registers, NV float4 per lane, all loads issued before any is used, so the row is read once and
-// the code pass needs no second read.
+// registers, NV float4 per lane, so the row is read once and the code pass needs no second read. A warp
+// takes every gridDim kRowWarps-th row, and rows of at most 512 values are loaded while the row before is
+// reduced and coded: the loads of one row alone leave memory idle through its reductions (128000 x 500:
+// 71.9 us, 4.5 TB/s, with a row a warp; 59.4 us, 5.4 TB/s, so).
 template <int NV>
-__global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_reg_kernel(const float *__restrict__ x, int64_t rows,
-                                                                          int cols, int64_t ldx,
-                                                                          uint8_t *__restrict__ codes, int64_t ldc,
-                                                                          qnn_qparams *__restrict__ params,
-                                                                          int32_t *__restrict__ sums, int *status,
-                                                                          bool pack) {
-    const int64_t row = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
-    if (row >= rows) return;
+__device__ __forceinline__ void load_row(float4 (&v)[NV], const float *__restrict__ xr, int cols) {
     const int lane = threadIdx.x & 31;
-    const float *xr = x + row * ldx;
-    float4 v[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
         const int k = 4 * (lane + 32 * i);
@@ -135,57 +145,88 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_reg_kernel(const
             v[i].w = k + 3 < cols ? __ldg(xr + k + 3) : 0.0f;
         }
     }
-    float mn = FLT_MAX, mx = -FLT_MAX;
-    bool bad = false;
+}
+
+// Blocks per SM the registers leave room for.
+constexpr int rows_reg_blocks(int NV) { return NV <= 1 ? 7 : NV <= 2 ? 5 : NV <= 4 ? 4 : 3; }
+
+template <int NV>
+__global__ void __launch_bounds__(kRowWarps * 32, rows_reg_blocks(NV))
+    quantize_rows_reg_kernel(const float *__restrict__ x, int64_t rows, int cols, int64_t ldx, uint8_t *__restrict__ codes,
+                             int64_t ldc, qnn_qparams *__restrict__ params, int32_t *__restrict__ sums, int *status,
+                             bool pack) {
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * kRowWarps;
+    int64_t row = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+    if (row >= rows) return;
+    float4 v[NV];
+    load_row<NV>(v, x + row * ldx, cols);
+    while (true) {
+        constexpr bool kAhead = NV <= 4;
+        float4 w[kAhead ? NV : 1];
+        const int64_t next = row + step;
+        if constexpr (kAhead)
+            if (next < rows) load_row<NV>(w, x + next * ldx, cols);
+        Range r;
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int k = 4 * (lane + 32 * i);
-        const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        for (int i = 0; i < NV; ++i) {
+            const int k = 4 * (lane + 32 * i);
+            if (k + 4 <= cols) {
+                r.add(v[i]);
+            } else {
+                const float e[3] = {v[i].x, v[i].y, v[i].z};
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (k + j < cols) {
-                bad |= !isfinite(e[j]);
-                mn = fminf(mn, e[j]);
-                mx = fmaxf(mx, e[j]);
+                for (int j = 0; j < 3; ++j)
+                    if (k + j < cols) r.add(e[j]);
             }
-    }
-    mn = warp_min(mn);
-    mx = warp_max(mx);
-    if (__any_sync(0xffffffffu, bad)) {
-        if (lane == 0) record_status(status, QNN_ERR_NONFINITE);
-        mn = 0.0f;
-        mx = 0.0f;
-    }
-    const qnn_qparams p = params_from_range(mn, mx);
-    uint8_t *cr = codes + row * ldc;
-    int s = 0;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int k = 4 * (lane + 32 * i);
-        if (k >= cols) continue;
-        const uint32_t a = quant_code(v[i].x, p.Q, p.z), b = quant_code(v[i].y, p.Q, p.z),
-                       c = quant_code(v[i].z, p.Q, p.z), d = quant_code(v[i].w, p.Q, p.z);
-        if (pack && k + 4 <= cols) {  // 4-byte aligned code rows: one store for four codes
-            s += (int)(a + b + c + d);
-            *reinterpret_cast<uint32_t *>(cr + k) = a | (b << 8) | (c << 16) | (d << 24);
-        } else {
-            const uint32_t q4[4] = {a, b, c, d};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (k + j < cols) {
-                    s += (int)q4[j];
-                    cr[k + j] = (uint8_t)q4[j];
-                }
         }
-    }
-    s = warp_sum(s);
-    if (lane == 0) {
-        params[row] = p;
-        if (sums) sums[row] = s;
+        float mn = warp_min(r.mn), mx = warp_max(r.mx);
+        if (!__all_sync(0xffffffffu, r.finite())) {
+            if (lane == 0) record_status(status, QNN_ERR_NONFINITE);
+            mn = 0.0f;
+            mx = 0.0f;
+        }
+        const qnn_qparams p = params_from_range(mn, mx);
+        uint8_t *cr = codes + row * ldc;
+        int s = 0;
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int k = 4 * (lane + 32 * i);
+            if (k >= cols) continue;
+            const uint32_t a = quant_code(v[i].x, p.Q, p.z), b = quant_code(v[i].y, p.Q, p.z),
+                           c = quant_code(v[i].z, p.Q, p.z), d = quant_code(v[i].w, p.Q, p.z);
+            if (pack && k + 4 <= cols) {  // 4-byte aligned code rows: one store for four codes
+                s += (int)(a + b + c + d);
+                *reinterpret_cast<uint32_t *>(cr + k) = a | (b << 8) | (c << 16) | (d << 24);
+            } else {
+                const uint32_t q4[4] = {a, b, c, d};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (k + j < cols) {
+                        s += (int)q4[j];
+                        cr[k + j] = (uint8_t)q4[j];
+                    }
+            }
+        }
+        s = warp_sum(s);
+        if (lane == 0) {
+            params[row] = p;
+            if (sums) sums[row] = s;
+        }
+        if (next >= rows) return;
+        row = next;
+        if constexpr (kAhead) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) v[i] = w[i];
+        } else {
+            load_row<NV>(v, x + row * ldx, cols);
+        }
     }
 }
 
-// Per-matrix pass 1: block partial ranges; the last block folds them into params[0].
+// Per-matrix pass 1: block partial ranges; the last block folds them into params[0]. The warps take segments
+// of kSegment values of the rows in turn (whole rows leave a last, nearly empty round).
+constexpr int kSegment = 2048;
 template <bool kVec>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const float *__restrict__ x, int64_t rows,
                                                                      int cols, int64_t ldx, float *__restrict__ partials,
@@ -198,9 +239,14 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     float mn = FLT_MAX, mx = -FLT_MAX;
-    for (int64_t row = (int64_t)blockIdx.x * kRowWarps + warp; row < rows; row += (int64_t)gridDim.x * kRowWarps) {
+    grid_dependents_launch();
+    const int segs = (cols - 1) / kSegment + 1;
+    const int64_t items = rows * segs;
+    for (int64_t i = (int64_t)blockIdx.x * kRowWarps + warp; i < items; i += (int64_t)gridDim.x * kRowWarps) {
+        const int64_t row = i / segs;
+        const int k0 = (int)(i - row * segs) * kSegment;
         float a, b;
-        if (!warp_row_range<kVec>(x + row * ldx, cols, a, b)) {
+        if (!warp_row_range<kVec>(x + row * ldx + k0, min(kSegment, cols - k0), a, b)) {
             if (lane == 0) s_bad = 1;
         } else {
             mn = fminf(mn, a);
@@ -247,16 +293,43 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     }
 }
 
-// Per-matrix pass 2: codes and row sums with the single unit's parameters.
+// Per-matrix pass 2: codes and row sums with the single unit's parameters. Rows of at least kLongRow values
+// take a block each (contiguous parts of the row by warp), shorter ones a warp. Last rows first: the range
+// pass read them last, so about an L2 of them is still there.
+constexpr int kLongRow = 2048;
+template <bool kVec>
+__global__ void __launch_bounds__(kRowWarps * 32) matrix_long_rows_kernel(const float *__restrict__ x, int cols, int64_t ldx,
+                                                                         uint8_t *__restrict__ codes, int64_t ldc,
+                                                                         const qnn_qparams *__restrict__ params,
+                                                                         int32_t *__restrict__ sums) {
+    __shared__ int s_sum[kRowWarps];
+    const int64_t row = gridDim.x - 1 - blockIdx.x;
+    const int warp = threadIdx.x >> 5, part = ((cols + kRowWarps - 1) / kRowWarps + 3) & ~3, k0 = warp * part;
+    grid_dependency_wait();
+    const float Q = __ldcg(&params[0].Q);
+    const int z = __ldcg(&params[0].z);
+    const int s = k0 < cols ? warp_row_codes<kVec>(x + row * ldx + k0, min(part, cols - k0), Q, z, codes + row * ldc + k0) : 0;
+    if (!sums) return;
+    if ((threadIdx.x & 31) == 0) s_sum[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+#pragma unroll
+        for (int w = 0; w < kRowWarps; ++w) t += s_sum[w];
+        sums[row] = t;
+    }
+}
+
 template <bool kVec>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_codes_kernel(const float *__restrict__ x, int64_t rows,
                                                                      int cols, int64_t ldx, uint8_t *__restrict__ codes,
                                                                      int64_t ldc, const qnn_qparams *__restrict__ params,
                                                                      int32_t *__restrict__ sums) {
-    const int64_t row = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+    const int64_t row = (int64_t)(gridDim.x - 1 - blockIdx.x) * kRowWarps + (threadIdx.x >> 5);
+    grid_dependency_wait();
     if (row >= rows) return;
-    const float Q = params[0].Q;
-    const int z = params[0].z;
+    const float Q = __ldcg(&params[0].Q);
+    const int z = __ldcg(&params[0].z);
     int s = warp_row_codes<kVec>(x + row * ldx, cols, Q, z, codes + row * ldc);
     if ((threadIdx.x & 31) == 0 && sums) sums[row] = s;
 }
@@ -280,6 +353,7 @@ qnn_status launch_quantize_rows(const float *x, int64_t rows, int64_t cols, int6
     if (x_ok && nv <= 8) {
         const bool pack = ((reinterpret_cast<uintptr_t>(codes) & 3) == 0) && (ldc % 4 == 0);
         const int r = nv <= 1 ? 1 : nv <= 2 ? 2 : nv <= 4 ? 4 : 8;
+        grid.x = std::min<unsigned>(grid.x, (unsigned)(sm_count() * rows_reg_blocks(r)));  // one wave
         switch (r) {
             case 1: quantize_rows_reg_kernel<1><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
             case 2: quantize_rows_reg_kernel<2><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
@@ -299,8 +373,9 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
                                   int max_blocks, cudaStream_t st) {
     int *status = nullptr;
     QNN_TRY(status_word(&status));
-    int64_t want = (rows + kRowWarps - 1) / kRowWarps;
-    unsigned nb = (unsigned)(want < max_blocks ? want : max_blocks);
+    const int64_t want = (rows + kRowWarps - 1) / kRowWarps;
+    const int64_t range = (rows * ((cols - 1) / kSegment + 1) + kRowWarps - 1) / kRowWarps;
+    const unsigned nb = (unsigned)(range < max_blocks ? range : max_blocks);
     const bool v = vec_ok(x, ldx, codes, ldc);
     {
     ProfScope prof("quantize_matrix_range", st);
@@ -311,12 +386,23 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     QNN_CUDA_TRY(cudaGetLastError());
     }
     ProfScope prof("quantize_matrix_codes", st);
-    dim3 grid((unsigned)want);
-    if (v)
-        matrix_codes_kernel<true><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums);
+    // programmatic dependent launch: the blocks are set up while the range pass ends (they wait for it)
+    cudaLaunchConfig_t cfg = {};
+    const bool long_rows = cols >= kLongRow && rows <= INT32_MAX;
+    cfg.gridDim = dim3((unsigned)(long_rows ? rows : want));
+    cfg.blockDim = dim3(kRowWarps * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (long_rows)
+        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, v ? matrix_long_rows_kernel<true> : matrix_long_rows_kernel<false>, x, (int)cols, ldx,
+                                        codes, ldc, (const qnn_qparams *)params, sums));
     else
-        matrix_codes_kernel<false><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums);
-    QNN_CUDA_TRY(cudaGetLastError());
+        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, v ? matrix_codes_kernel<true> : matrix_codes_kernel<false>, x, rows, (int)cols,
+                                        ldx, codes, ldc, (const qnn_qparams *)params, sums));
     return QNN_OK;
 }
 

@@ -1,0 +1,69 @@
+"""The quantizer kernels at the edges of their splits, against the oracle: rows around the register
+kernel's widths and its rows per wave, matrices around the range pass's segments and the code pass's
+long rows, unaligned and strided inputs, rows after others in one warp."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qnn():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1607_04683_gb300 import build, qnn as q
+    build.build()
+    q.lib()
+    torch.cuda.set_device(0)
+    return q
+
+
+def check(qnn, x, ld, off, granularity):
+    rows, cols = x.shape
+    buf = torch.full((off + rows * ld,), float("nan"), device="cuda")
+    v = buf[off:].reshape(rows, ld)[:, :cols]
+    v.copy_(torch.from_numpy(x))
+    codes, params, sums = qnn.qnn_quantize(v, granularity)
+    assert qnn.device_status() == qnn.QNN_OK
+    c, p, s = oracle.quantize(x, granularity)
+    assert np.array_equal(codes.cpu().numpy(), c)
+    assert np.array_equal(qnn.params_view(params).view(np.int32), p.view(np.int32))
+    assert np.array_equal(sums.cpu().numpy(), s)
+
+
+def values(rows, cols, seed):
+    g = np.random.Generator(np.random.PCG64(seed))
+    x = g.normal(0, 1, (rows, cols)) * np.exp2(g.integers(-20, 20, (rows, 1))) + g.choice([0.0, 0.0, 30.0, -1e3], (rows, 1))
+    return x.astype(np.float32)
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 1), (7, 127), (9, 128), (5, 129), (3000, 256), (2500, 260), (20000, 500), (9000, 512),
+                                       (9001, 516), (5000, 1000), (17, 1024), (33, 1028), (4, 4100)])
+@pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
+def test_rows(qnn, rows, cols, pad, off):
+    check(qnn, values(rows, cols, rows + cols), cols + pad, off, oracle.PER_ROW)
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 1), (3, 2047), (8, 2048), (9, 2049), (700, 2052), (130, 4099), (5, 16384), (3000, 40),
+                                       (1, 100001), (513, 2500)])
+@pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
+def test_matrix(qnn, rows, cols, pad, off):
+    g = np.random.Generator(np.random.PCG64(rows * 7 + cols))
+    check(qnn, (g.normal(0, 0.05, (rows, cols)) + g.choice([0.0, 5.0])).astype(np.float32), cols + pad, off, oracle.PER_MATRIX)
+
+
+@pytest.mark.parametrize("granularity", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(12, 300), (6, 3000)])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_non_finite_values_are_reported(qnn, rows, cols, value, granularity):
+    x = values(rows, cols, 3)
+    for at in ((0, 0), (rows - 1, cols - 1), (rows // 2, cols // 2)):
+        bad = x.copy()
+        bad[at] = value
+        qnn.qnn_quantize(torch.from_numpy(bad).cuda(), granularity)
+        assert qnn.device_status() == qnn.QNN_ERR_NONFINITE
+    qnn.qnn_quantize(torch.from_numpy(x).cuda(), granularity)
+    assert qnn.device_status() == qnn.QNN_OK
