@@ -216,22 +216,35 @@ qnn_status launch_qgemm_imma(const uint8_t *A, int64_t lda, const qnn_qparams *p
     return run(integral_constant<int, 8>{}, integral_constant<int, 2>{});
 }
 
-// Datapath choice: up to 127 rows of A the streaming integer MMA kernel, which needs no conversion,
-// else the tcgen05 path, which runs whole tiles at the fp16 tensor rate after centering both operands
-// into fp16 scratch. Above 64 rows the streaming kernel reads W twice and its MMA rate shows: there it
-// keeps W of up to 2^24 codes (M = 127: 16.5 against 32 us at 2048 x 2048, 180 against 102 us at
-// 8192 x 8192; M = 64 at 8192 x 8192: 87 against 102 us). QNN_QGEMM=imma or =tc forces one (tests
-// compare the two).
+// Datapath choice, between three kernels that differ in what they do to the operands first:
+//   - the streaming integer MMA kernel, nothing at all: up to 32 rows of A (8192 x 8192: 42 us at M = 32 against
+//     72 for the codes kernel), and up to 127 while its blocks (64 rows of A, 32 of W) are one wave (M = 127, 2048 x
+//     2048: 16.5 against 18.3; 4096 x 4096: 49.8 against 30.0);
+//   - the codes kernel, converting on the way into shared memory: while its tiles of 128 x 128 are one wave
+//     (M = 256, 8192 x 8192: 83 against 97 us; 1100 x 2000 x 500: 16.6 against 22.6; 128 x 2048 x 2048: 18.3 against
+//     28.8; at two waves M = 512, 8192 x 8192: 161 against 117; 1536 x 2000 x 500: 31.4 against 26.7);
+//   - the fp16 tensor-core product after a pass that centers both operands into scratch: the rest.
+// QNN_QGEMM=imma, =codes or =tc forces one (tests compare them).
 qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, int ga, const int32_t *rsA, int64_t M,
                         int64_t K, const uint8_t *W, int64_t ldw, const qnn_qparams *pw, int64_t rows_per_block,
                         const int32_t *csW, int64_t N, const float *bias, float *Y, int64_t ldy, int32_t *acc_out,
                         cudaStream_t st) {
     if (M == 0 || N == 0) return QNN_OK;
     const char *force = std::getenv("QNN_QGEMM");
-    bool tc = M >= 128 || (M > 64 && N * K > (int64_t)1 << 24);
-    if (force && std::strcmp(force, "imma") == 0) tc = false;
-    if (force && std::strcmp(force, "tc") == 0) tc = true;
-    if (tc) {
+    enum { kImma, kCodes, kTc } path = kTc;
+    const int64_t sms = sm_count();
+    if (M <= 32 || (M < 128 && (M + 63) / 64 * ((N + 31) / 32) <= sms))
+        path = kImma;
+    else if ((M + 127) / 128 * ((N + 127) / 128) <= sms)
+        path = kCodes;
+    if (force && std::strcmp(force, "imma") == 0) path = kImma;
+    if (force && std::strcmp(force, "codes") == 0) path = kCodes;
+    if (force && std::strcmp(force, "tc") == 0) path = kTc;
+    // the codes kernel loads aligned 16-byte units, and each operand has to hold one
+    if (path == kCodes && ((M - 1) * lda + K < 31 || (N - 1) * ldw + K < 31)) path = kTc;
+    if (path == kCodes)
+        return launch_qgemm_codes(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out, st);
+    if (path == kTc) {
         void *ws = nullptr;
         QNN_TRY(scratch(kScratchTc, tc_scratch_bytes(M, N, K), &ws));
         return launch_qgemm_tc(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out, ws,

@@ -1172,16 +1172,6 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     }
 }
 
-// Two codes (bytes lo and hi of w selected by sel) as two centered fp16 values c - 128: the byte
-// placed under the exponent pattern 0x64 is the fp16 value 1024 + c (exact), and 1024 + 128 is
-// then subtracted (exact: integers below 2048).
-__device__ __forceinline__ uint32_t center2(uint32_t w, uint32_t sel) {
-    const uint32_t bits = __byte_perm(w, 0x64646464u, sel);
-    const __half2 v = __hsub2(*reinterpret_cast<const __half2 *>(&bits), __halves2half2(__ushort_as_half(0x6480),
-                                                                                      __ushort_as_half(0x6480)));
-    return *reinterpret_cast<const uint32_t *>(&v);
-}
-
 // u8 codes -> centered fp16 (c - 128), rows padded with zeros to ldo (a multiple of 64). A thread
 // converts 16 codes: one 16-byte load and two 16-byte stores when the row is 16-byte aligned and
 // the 16 codes lie inside K, element by element otherwise (ragged tail, padding, unaligned rows).

@@ -90,6 +90,10 @@ qnn_status launch_qgemm_tc(const uint8_t *A, int64_t lda, const qnn_qparams *pa,
                            const int32_t *csW, int64_t N, const float *bias, float *Y, int64_t ldy, int32_t *acc_out,
                            void *scratch, cudaStream_t st);
 size_t tc_scratch_bytes(int64_t M, int64_t N, int64_t K);
+qnn_status launch_qgemm_codes(const uint8_t *A, int64_t lda, const qnn_qparams *pa, int ga, const int32_t *rsA, int64_t M,
+                              int64_t K, const uint8_t *W, int64_t ldw, const qnn_qparams *pw, int64_t rows_per_block,
+                              const int32_t *csW, int64_t N, const float *bias, float *Y, int64_t ldy, int32_t *acc_out,
+                              cudaStream_t st);
 // Softmax of rows of logits into y. With tm_B > 0 the rows are time-major, frames tm_t0 .. of tm_B
 // sequences (row i: frame tm_t0 + i / tm_B of sequence i % tm_B), and each goes to its row of the
 // sequence-major y [tm_B][tm_T][C].

@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <cuda.h>
+#include <cuda_fp16.h>
 
 namespace qnn {
 
@@ -113,6 +114,16 @@ __device__ __forceinline__ void tmem_ld_nowait(uint32_t taddr, uint32_t (&r)[4])
 }
 __device__ __forceinline__ void tmem_ld_nowait(uint32_t taddr, uint32_t (&r)[2]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+
+// Two codes (bytes lo and hi of w selected by sel) as two centered fp16 values c - 128: the byte
+// placed under the exponent pattern 0x64 is the fp16 value 1024 + c (exact), and 1024 + 128 is
+// then subtracted (exact: integers below 2048).
+__device__ __forceinline__ uint32_t center2(uint32_t w, uint32_t sel) {
+    const uint32_t bits = __byte_perm(w, 0x64646464u, sel);
+    const __half2 v = __hsub2(*reinterpret_cast<const __half2 *>(&bits), __halves2half2(__ushort_as_half(0x6480),
+                                                                                      __ushort_as_half(0x6480)));
+    return *reinterpret_cast<const uint32_t *>(&v);
 }
 
 }  // namespace qnn

@@ -1,5 +1,6 @@
 """The product kernels at the edges of their tiles: the streaming integer-MMA kernel over every
-number of A-row groups, ragged rows, ragged reductions and row alignments (16, 4 and 1 bytes)."""
+number of A-row groups, ragged rows, ragged reductions and row alignments (16, 4 and 1 bytes), the
+tensor-core product's outputs, and the product from the codes at its own edges."""
 import numpy as np
 import pytest
 
@@ -108,3 +109,48 @@ def test_tensor_core_outputs(qnn, M, N, K, pad, bn, shift, monkeypatch):
     assert qnn.device_status() == qnn.QNN_OK
     assert np.array_equal(out[:M, :N].cpu().numpy(), ref["y"])
     assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
+
+
+# The product from the codes: rows of A around its 64 and 128 columns, rows of W around 128, K around 16
+# codes, the ring's four stages and three k-blocks of loads ahead, chunks of 1024 (drained late, a last chunk
+# of one to three k-blocks), every row shift, raw sums, sums of 32 and of 64 bits.
+@pytest.mark.parametrize("M,N,K", [(1, 1, 40), (5, 6, 7), (63, 127, 15), (64, 128, 16), (65, 129, 17), (100, 260, 63), (129, 2000, 64),
+                                   (130, 500, 65), (200, 9000, 127), (128, 20000, 193), (128, 130, 256), (129, 136, 321),
+                                   (300, 300, 1000), (128, 64, 1024), (130, 132, 1025), (96, 128, 1088), (70, 200, 1153),
+                                   (128, 14600, 1217), (128, 129, 2048), (128, 128, 2113), (66, 65, 3300), (64, 33, 33025)])
+@pytest.mark.parametrize("pad,off,shift", [(None, 0, 0.0), (0, 0, 20.0), (4, 4, 3000.0), (3, 1, 0.0), (6, 15, 0.0)])
+def test_codes_bit_exact(qnn, M, N, K, pad, off, shift, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "codes")
+    g = np.random.Generator(np.random.PCG64(M * 31 + N * 7 + K))
+    A = (g.normal(0.1, 1.0, (M, K)) + shift).astype(np.float32)
+    nb = 4 if N % 4 == 0 else 1
+    Ws = [g.uniform(-s, s, (N // nb, K)).astype(np.float32) for s in np.linspace(0.05, 0.4, nb)]
+    ga = oracle.PER_ROW if M % 2 else oracle.PER_MATRIX
+    ca, pa, ra = oracle.quantize(A, ga)
+    parts = [oracle.quantize(w, oracle.PER_MATRIX) for w in Ws]
+    cw, pw, cs = (np.concatenate([p[i] for p in parts]) for i in range(3))
+    bias = g.normal(0, 1, N).astype(np.float32) if K % 2 else None
+    ref = oracle.qmatmul(ca, pa, ga, cw, pw, n_blocks=nb, bias=bias)
+    ld = (K + 15) // 16 * 16 if pad is None else (K + 3) // 4 * 4 + pad if pad == 4 else K + pad
+    out = torch.full((M + 1, N + 3), 7.0, device="cuda")
+    _, acc = qnn.qnn_qmatmul(strided(ca, ld, off), qnn.params_tensor(pa), ga, gpu(ra), strided(cw, ld, off),
+                             qnn.params_tensor(pw), gpu(cs), n_blocks=nb, bias=None if bias is None else gpu(bias),
+                             want_acc=True, out=out[:M, :N])
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"])
+    assert np.array_equal(out[:M, :N].cpu().numpy(), ref["y"])
+    assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
+
+
+# Operands too small to hold one aligned unit take another path than the one the sizes ask for.
+@pytest.mark.parametrize("M,N,K", [(130, 1, 1), (200, 2, 15), (129, 1, 30), (128, 1, 31)])
+@pytest.mark.parametrize("off", [0, 1, 15])
+def test_few_codes(qnn, M, N, K, off):
+    g = np.random.Generator(np.random.PCG64(M + K))
+    ca, pa, ra = oracle.quantize(g.normal(0.1, 1.0, (M, K)).astype(np.float32), oracle.PER_ROW)
+    cw, pw, cs = oracle.quantize(g.normal(0.0, 1.0, (N, K)).astype(np.float32), oracle.PER_MATRIX)
+    ref = oracle.qmatmul(ca, pa, oracle.PER_ROW, cw, pw)
+    Y, acc = qnn.qnn_qmatmul(strided(ca, K, off), qnn.params_tensor(pa), oracle.PER_ROW, gpu(ra), strided(cw, K, off),
+                             qnn.params_tensor(pw), gpu(cs), want_acc=True)
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"]) and np.array_equal(Y.cpu().numpy(), ref["y"])
