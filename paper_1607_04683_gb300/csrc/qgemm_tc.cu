@@ -102,8 +102,9 @@ struct Tile {
     // [4 gates][32 rows] float4 (1/dx, 1/dh, rt_x, rt_h), then [4 gates][32 rows] float2 (dx, dh)
     static constexpr int OUT_BYTES = EPI == kEpiLstmX ? PX_BOX : 0;
     static constexpr int RC_BYTES = EPI == kEpiLstmX ? 4 * 24 * 32 * 4 : 0;
-    // kEpiRow: each epilogue warp's staging, 32 rows x BN / 4 fp32 columns, for its TMA stores
-    static constexpr int ROW_COLS = BN / 4, STG_BYTES = EPI == kEpiRow ? 32 * ROW_COLS * 4 : 0;
+    // kEpiRow, kEpiLinear: each epilogue warp's staging of outputs, 32 rows x ROW_COLS fp32 columns
+    static constexpr int ROW_COLS = EPI == kEpiRow ? BN / 4 : 16;
+    static constexpr int STG_BYTES = EPI == kEpiRow || EPI == kEpiLinear ? 32 * ROW_COLS * 4 : 0;
     static constexpr int EPI_BYTES = IS_LSTM              ? 2 * LSTM_BUF + OUT_BYTES + RC_BYTES
                                      : EPI == kEpiPartial ? 0
                                                           : 2 * BN * (int)(sizeof(ColConst) + sizeof(ColUnit)) +
@@ -158,7 +159,7 @@ struct TcArgs {
     const int32_t *csW_x;
     const float *bias_x;
     int K_x, KB_x;
-    int y_map;  // kEpiRow: mapPX is a map of Y for TMA stores
+    int y_map;  // kEpiRow, kEpiLinear: mapPX is a map of Y for TMA stores
     // LSTM epilogues: tiles from full_tiles on (the last, partial wave of the persistent grid) run as
     // two half-width items each, so that the blocks of that wave finish together (0: none)
     int64_t full_tiles;
@@ -248,6 +249,31 @@ __device__ __forceinline__ void row_block_fast(const uint32_t (&r)[COLS], const 
         }
         put(v4, make_float4(y[0], y[1], y[2], y[3]));
     }
+}
+
+// A warp's staged outputs (32 rows x COLS columns, 16-byte pieces of a row swizzled: 128 bytes, or 64) to Y
+// at column n of rows m .. m + 31: by TMA where Y has a map, else whole row segments by plain stores (rows of
+// any alignment; a lane storing its own row would touch 32 rows an instruction).
+template <int COLS>
+__device__ __forceinline__ void store_staged(const uint8_t *stg, const CUtensorMap *map, bool by_map, float *Y, int64_t ldy,
+                                             int64_t m, int64_t n, int64_t M) {
+    const int lane = threadIdx.x & 31;
+    if (by_map) {
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) tma_store_2d(map, su32(stg), (int)n, (int)m);
+        return;
+    }
+    __syncwarp();
+    constexpr int RPI = 32 / COLS;  // rows an instruction
+    const int c = lane % COLS, r0 = lane / COLS, rows = (int)min((int64_t)32, M - m);
+    float *y = Y + (m + r0) * ldy + n + c;
+#pragma unroll 8
+    for (int i = 0; i < 32; i += RPI) {
+        const int r = i + r0, sw = COLS == 32 ? r & 7 : (r >> 1) & 3;
+        if (r < rows) y[i * ldy] = *reinterpret_cast<const float *>(stg + r * COLS * 4 + (((c >> 2) ^ sw) << 4) + (c & 3) * 4);
+    }
+    __syncwarp();
 }
 
 // Persistent tile loop. Warp 0: TMA producer; warp 1: tensor-memory owner and MMA issuer; warps
@@ -495,7 +521,8 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         // registers (ragged or unaligned outputs element by element). Column constants are staged
         // in shared memory per tile (double-buffered; one named barrier of the epilogue warps).
         constexpr int NJ = BN / 64;             // 32-column blocks per warp
-        ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES);
+        uint8_t *const stg = smem + STAGES * TL::STAGE_BYTES + (warp - 2) * TL::STG_BYTES;
+        ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES + TL::EPI_WARPS * TL::STG_BYTES);
         ColUnit *sunit = reinterpret_cast<ColUnit *>(scol + 2 * BN);
         const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
         const int half = (warp - 2) >> 2;       // column half: [0, BN/2) or [BN/2, BN)
@@ -555,9 +582,10 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 if (lane == 0) mb_arrive(drained0 + 8 * buf);
             }
             const int64_t m = m0 + 32 * q + lane;
-            if (failed || m >= args.M) continue;
-            const qnn_qparams qa = args.pa[args.a_per_row ? m : 0];
-            const int za = qa.z, ra = args.rsA[m];
+            if (failed || m0 + 32 * q >= args.M) continue;
+            const bool mv = m < args.M;
+            const qnn_qparams qa = args.pa[args.a_per_row && mv ? m : 0];
+            const int za = qa.z, ra = mv ? args.rsA[m] : 0;
             const float Qa = qa.Q;
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {
@@ -566,42 +594,64 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 if (nb >= args.N) continue;
                 const bool full = vec && nb + 32 <= args.N;
                 float *yr = args.Y ? args.Y + m * args.ldy + nb : nullptr;
-                int *const ar = args.acc_out ? args.acc_out + m * args.N + nb : nullptr;
-                // The usual block: 32 columns of one weight unit, whole rows, sums S of eq. (1) that fit 32 bits
+                // The usual block: 32 columns of one weight unit, sums S of eq. (1) that fit 32 bits
                 // (K max|a' + za| max|w' + zw| < 2^31: wrapping 32-bit arithmetic gives them exactly) and a
                 // divisor far from the ends of the fp32 range (div_by_recip: the IEEE quotient). The block's
-                // outputs then cost a few instructions each; with a 64-bit sum and an IEEE divide apiece the
-                // tile's epilogue outlasts the two K chunks the accumulators can run ahead.
-                if (full && (!ar || (reinterpret_cast<uintptr_t>(ar) & 15) == 0) && cu[c0].unit == cu[c0 + 31].unit) {
+                // outputs then cost a few instructions each (with a 64-bit sum and an IEEE divide apiece the
+                // tile's epilogue outlasts the two K chunks the accumulators can run ahead), and leave through the
+                // warp's staging, 16 columns at a time (stored from registers, a lane its own row: 16384 x 8192 x 8192
+                // 1593 us, so 1527; 9374 x 3033 x 2052, whose rows no 16-byte store fits, 308 us, so 185).
+                if (args.Y && cu[c0].unit >= 0 && cu[c0].unit == cu[c0 + 31].unit) {
                     const int zw = cc[c0].zw;
                     const float den = __fmul_rn(Qa, cc[c0].Qw);
-                    if ((long long)K * max(abs(za), abs(za + 255)) * (long long)max(abs(zw), abs(zw + 255)) < (1LL << 31) &&
-                        den >= 0x1p-60f && den <= 0x1p60f) {
+                    const bool fits = (long long)K * max(abs(za), abs(za + 255)) * (long long)max(abs(zw), abs(zw + 255)) < (1LL << 31) &&
+                                      den >= 0x1p-60f && den <= 0x1p60f;
+                    if (__all_sync(0xffffffffu, fits || !mv)) {
                         const float rden = rcp_rn(den);
                         const uint32_t rt = (uint32_t)(128 + zw) * (uint32_t)ra + (uint32_t)K * ((uint32_t)za * (uint32_t)zw - 16384u);
                         const uint32_t za128 = (uint32_t)(128 + za);
+                        uint8_t *const row = stg + lane * 64;
 #pragma unroll
-                        for (int v4 = 0; v4 < 8; ++v4) {
-                            float y[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int i = 4 * v4 + e;
-                                const int S = (int)((uint32_t)run[j][i] + rt + za128 * (uint32_t)cc[c0 + i].cs);
-                                y[e] = div_by_recip(__int2float_rn(S), den, rden);
-                                if (args.bias) y[e] = __fadd_rn(y[e], cc[c0 + i].bias);
+                        for (int g = 0; g < 2; ++g) {
+                            if (args.y_map) {
+                                if (lane == 0) bulk_wait_read();  // the buffer's previous store has read it
+                                __syncwarp();
                             }
-                            *reinterpret_cast<float4 *>(yr + 4 * v4) = make_float4(y[0], y[1], y[2], y[3]);
-                            if (ar) {  // raw code products
-                                const int base = 128 * ra - 16384 * K;
+#pragma unroll
+                            for (int v4 = 0; v4 < 4; ++v4) {
+                                float y[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const int i = 16 * g + 4 * v4 + e;
+                                    const int S = (int)((uint32_t)run[j][i] + rt + za128 * (uint32_t)cc[c0 + i].cs);
+                                    y[e] = div_by_recip(__int2float_rn(S), den, rden);
+                                    if (args.bias) y[e] = __fadd_rn(y[e], cc[c0 + i].bias);
+                                }
+                                *reinterpret_cast<float4 *>(row + ((v4 ^ ((lane >> 1) & 3)) << 4)) = make_float4(y[0], y[1], y[2], y[3]);
+                            }
+                            store_staged<16>(stg, &mapPX, args.y_map, args.Y, args.ldy, m0 + 32 * q, nb + 16 * g, args.M);
+                        }
+                        if (args.acc_out && mv) {  // raw code products
+                            int *const ar = args.acc_out + m * args.N + nb;
+                            const int base = 128 * ra - 16384 * K;
+                            const bool ar16 = (reinterpret_cast<uintptr_t>(ar) & 15) == 0;
+#pragma unroll
+                            for (int v4 = 0; v4 < 8; ++v4) {
                                 int o[4];
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) o[e] = run[j][4 * v4 + e] + base + 128 * cc[c0 + 4 * v4 + e].cs;
-                                *reinterpret_cast<int4 *>(ar + 4 * v4) = make_int4(o[0], o[1], o[2], o[3]);
+                                if (ar16) {
+                                    *reinterpret_cast<int4 *>(ar + 4 * v4) = make_int4(o[0], o[1], o[2], o[3]);
+                                } else {
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) ar[4 * v4 + e] = o[e];
+                                }
                             }
                         }
                         continue;
                     }
                 }
+                if (!mv) continue;
 #pragma unroll
                 for (int v4 = 0; v4 < 8; ++v4) {
                     float y[4];
@@ -624,6 +674,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 }
             }
         }
+        if (lane == 0) bulk_wait();  // (the staging buffers are read until then)
     } else if constexpr (EPI == kEpiRow) {
         // ---------------- epilogue (warps 2..17): recovered product, one row per lane ----------------
         // Each lane owns one output row; the four warps of a lane quarter take a quarter of its columns
@@ -684,20 +735,23 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // The usual tile: every warp takes a quarter of the columns of its 32 rows; when they lie in one
             // weight unit (and no raw products are wanted) the outputs go through the warp's staging buffer,
-            // swizzled so that neither side conflicts, and out as one TMA store of whole row segments. (Stored
+            // swizzled so that neither side conflicts, and out as whole row segments, one TMA store where Y has a
+            // map and a row an instruction where it does not (8000 x 2001 x 500: 99 us, so 77). (Stored
             // from registers, one 16-byte piece of 32 different rows an instruction, they take most of the
             // epilogue's time: 128000 x 2000 x 500 535 us, so 389; 102400 x 8192 x 512 1884 us, so 1343.)
             constexpr int RC = TL::ROW_COLS;
             const int cq = part * RC;
-            const bool staged = args.y_map && !args.acc_out && cu[cq].unit >= 0 && cu[cq].unit == cu[cq + RC - 1].unit;
+            const bool staged = args.Y && !args.acc_out && cu[cq].unit >= 0 && cu[cq].unit == cu[cq + RC - 1].unit;
             if (staged && !failed) {
                 uint32_t r[RC];
                 if constexpr (RC == 32)
                     tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + cq), r);
                 else
                     tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + cq), r);
-                if (lane == 0) bulk_wait_read();  // the buffer's previous store has read it
-                __syncwarp();
+                if (args.y_map) {
+                    if (lane == 0) bulk_wait_read();  // the buffer's previous store has read it
+                    __syncwarp();
+                }
                 const int zw = cc[cq].zw;
                 const long long rt = (long long)(128 + zw) * ra + (long long)K * ((long long)za * zw - 16384);
                 const float den = __fmul_rn(Qa, cc[cq].Qw);
@@ -715,9 +769,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 } else {
                     row_block_fast<false>(r, cc + cq, rt, za128, den, put);
                 }
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) tma_store_2d(&mapPX, su32(stg), (int)n0 + cq, (int)m0 + 32 * q);
+                store_staged<RC>(stg, &mapPX, args.y_map, args.Y, args.ldy, m0 + 32 * q, n0 + cq, args.M);
             }
 #pragma unroll 1
             for (int j = part * (RC / 16); j < (part + 1) * (RC / 16) && !failed && !staged; ++j) {
@@ -1327,13 +1379,14 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
 }
 
 qnn_status dispatch_linear(const TcOperands &op, const TcArgs &a, cudaStream_t st) {
+    // Y by TMA where its rows are 16-byte aligned (else by plain stores)
+    CUtensorMap map_y;
+    TcArgs r = a;
+    r.y_map = a.Y && a.ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0 && a.M <= INT32_MAX && a.N <= INT32_MAX;
+    const int box = op.row_epilogue ? op.bn / 4 : 16;
+    if (r.y_map) QNN_TRY(make_map_f32(&map_y, a.Y, a.M, a.N, a.ldy, box, 32, box == 32 ? 128 : 64));
+    const CUtensorMap *my = r.y_map ? &map_y : nullptr;
     if (op.row_epilogue) {
-        // Y by TMA where its rows are 16-byte aligned (else from registers)
-        CUtensorMap map_y;
-        TcArgs r = a;
-        r.y_map = a.Y && a.ldy % 4 == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0 && a.M <= INT32_MAX && a.N <= INT32_MAX;
-        if (r.y_map) QNN_TRY(make_map_f32(&map_y, a.Y, a.M, a.N, a.ldy, op.bn / 4, 32, op.bn == 128 ? 128 : 64));
-        const CUtensorMap *my = r.y_map ? &map_y : nullptr;
         switch (op.bn) {
             case 64: return launch_tc<64, kEpiRow>(op, r, "qgemm_tc", st, my);
             case 128: return launch_tc<128, kEpiRow>(op, r, "qgemm_tc", st, my);
@@ -1341,9 +1394,9 @@ qnn_status dispatch_linear(const TcOperands &op, const TcArgs &a, cudaStream_t s
         }
     }
     switch (op.bn) {
-        case 64: return launch_tc<64, kEpiLinear>(op, a, "qgemm_tc", st);
-        case 128: return launch_tc<128, kEpiLinear>(op, a, "qgemm_tc", st);
-        case 256: return launch_tc<256, kEpiLinear>(op, a, "qgemm_tc", st);
+        case 64: return launch_tc<64, kEpiLinear>(op, r, "qgemm_tc", st, my);
+        case 128: return launch_tc<128, kEpiLinear>(op, r, "qgemm_tc", st, my);
+        case 256: return launch_tc<256, kEpiLinear>(op, r, "qgemm_tc", st, my);
         default: return QNN_ERR_INVALID_ARG;
     }
 }
