@@ -22,9 +22,12 @@
 // Bound: the chain of one frame (operand stream of h_{t-1}, gate arithmetic, two exchanges). A step
 // as launches of a quantizer and a gate kernel per layer takes two launches' latency and streams the
 // weights again; the grid barriers of lstm_recurrent_kernel keep one layer at a time on the GPU. 5 x 500
-// cells, 2000 classes, 100 frames, this kernel alone (whole pass before): B = 16 878 us (5.5 ms), B = 64
-// 1057 us (2.3 ms), B = 128 1231 us (2.6 ms), B = 256 1908 us (3.0 ms). A frame at B = 32 is about 15,000
-// cycles: h's operand stream and products 4,700, gates 5,000, range exchange 2,200, codes and release 2,700.
+// cells, 2000 classes, 100 frames, this kernel alone (whole pass before): B = 16 717 us (5.5 ms), B = 64
+// 1030 us (2.3 ms), B = 128 1231 us (2.6 ms), B = 256 1908 us (3.0 ms). A frame at B = 32 took about 15,000
+// cycles while one row quarter's warps, all on one scheduler, did all its cells: h's operand stream and
+// products 4,700, gates 5,000, range exchange 2,200, codes and release 2,700. With the cells spread over the
+// four schedulers (SP = 4) B = 16 went from 869 to 717 us; two quarters' over all four (SP = 2), 5 x 300, 40
+// frames, B = 48, from 376 to 350 us, 5 x 512 551 to 529, 1 x 128 231 to 224.
 //
 // Every wait is bounded in time: one that gives up records QNN_ERR_TIMEOUT and raises the abort
 // flag, after which all waits return at once and the launch runs to its end with meaningless outputs.
@@ -33,6 +36,7 @@
 #include <cfloat>
 #include <climits>
 #include <cstdlib>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -244,20 +248,31 @@ __device__ __noinline__ PairPre pair_pre_general(const PairSums s, float Qx, int
     return pre;
 }
 
-template <int NC, int MT>
+// SP: with one (SP = 4) or two (SP = 2) row quarters in use, the warps of the other quarters, which cannot read
+// those rows' tensor memory and would leave their schedulers idle, take SP - 1 of SP cell pairs: the warp that
+// can hands it their sums through shared memory.
+template <int NC, int MT, int SP>
 struct Cfg {
-    static constexpr int CB = 4 * NC, N = 16 * NC;      // cells and gate columns of a block
-    static constexpr int SL = MT == 1 ? 4 : 2;          // cell slices of a tile: a warp each per row quarter
-    static constexpr int PAIRS = MT == 1 ? NC / 2 : NC;  // cell pairs of a thread
-    static constexpr bool ODD = MT == 1 && (NC & 1);     // and one more cell
+    static_assert(SP == 1 || MT == 1, "two row tiles use every quarter");
+    static constexpr int CB = 4 * NC, N = 16 * NC;           // cells and gate columns of a block
+    static constexpr int SL = (MT == 1 ? 4 : 2) * SP;        // cell slices of a tile: a warp each per row quarter
+    static constexpr int PAIRS = SP > 1 ? (2 * NC + SL - 1) / SL : MT == 1 ? NC / 2 : NC;  // cell pairs of a thread
+    static constexpr bool ODD = SP == 1 && MT == 1 && (NC & 1);  // and one more cell
+    static constexpr int GIVEN = SP > 1 ? 2 * NC - (2 * NC + SP - 1) / SP : 0;  // pairs handed over per row quarter
     static constexpr int TMEM_COLS = 3 * MT * N <= 128 ? 128 : (3 * MT * N <= 256 ? 256 : 512);
     static constexpr int KB_BYTES = N * 128;             // a k-block of weights
-    static constexpr int MISC = 8 * (2 * kMaxSlots + 8) + 16 + 4 * kTile * 4 + (MT == 1 ? 2 * NC * 64 : 0);
 };
 
-template <int NC, int MT>
+// Shared memory beside the ring and the weights: barriers, ranges, (MT = 1) the pairs' code sums, and the sums
+// handed over, [quarter][pair][16 words][32 rows].
+constexpr int misc_bytes(int NC, int MT, int SP) {
+    return 8 * (2 * kMaxSlots + 8) + 16 + 4 * kTile * 4 + (MT == 1 ? 2 * NC * 64 : 0) +
+           (SP > 1 ? (2 * NC - (2 * NC + SP - 1) / SP) * (4 / SP) * 64 * 32 : 0);
+}
+
+template <int NC, int MT, int SP>
 __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_constant__ PersistArgs a) {
-    using C = Cfg<NC, MT>;
+    using C = Cfg<NC, MT, SP>;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int l = blockIdx.x / a.G, blk = blockIdx.x % a.G;
@@ -284,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
         mb_init(wfull, 1);
         for (int i = 0; i < MT; ++i) {
             mb_init(acc0 + 8 * i, 1);
-            mb_init(drained0 + 8 * i, C::SL * quarters(i));
+            mb_init(drained0 + 8 * i, C::SL / SP * quarters(i));  // the warps that read the accumulators
             mb_init(ready0 + 8 * i, 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -401,7 +416,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
         }
     } else {
         // ---------------- epilogue ----------------
-        const int tile = MT == 2 ? warp >> 3 : 0, q = warp & 3, e = (warp >> 2) & (C::SL - 1);
+        // row quarter q, slice e; `own`: this warp may read the quarter's tensor-memory lanes
+        const int tile = MT == 2 ? warp >> 3 : 0, q = warp & (4 / SP - 1), rep = (warp & 3) / (4 / SP);
+        const int e = SP > 1 ? (warp >> 2) * SP + rep : (warp >> 2) & (C::SL - 1);
+        const bool own = SP == 1 || rep == 0;
         const int rows = tile_rows(tile);
         if (32 * q < rows) {
             constexpr int GT = 32 * C::SL;  // threads of a row quarter
@@ -418,7 +436,15 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
             // cells of this thread: pairs e PAIRS .. of the block, and for odd NC one of pair 2 NC - 2 ..
             const int pair0 = e * C::PAIRS, pair_odd = 4 * C::PAIRS + (e >> 1), odd = e & 1;
             float c[2 * C::PAIRS + 1], h[2 * C::PAIRS + 1];
-            auto cell_of = [&](int k) { return j_blk + (k < 2 * C::PAIRS ? 2 * pair0 + k : 2 * pair_odd + odd); };
+            // (SP > 1: pairs e, e + SL of the block; cells of no pair lie past every row)
+            auto pair_of = [&](int k) { return SP > 1 ? e + C::SL * k : pair0 + k; };
+            auto cell_of = [&](int k) {
+                if (SP > 1) return pair_of(k / 2) < 2 * NC ? j_blk + 2 * pair_of(k / 2) + (k & 1) : 1 << 30;
+                return j_blk + (k < 2 * C::PAIRS ? 2 * pair0 + k : 2 * pair_odd + odd);
+            };
+            // sums of a pair handed over: 16-byte words v = 0 .. 3 of each row
+            float4 *const xch = reinterpret_cast<float4 *>(s_min + 4 * kTile) + (MT == 1 ? 8 * NC : 0);
+            auto given = [&](int p, int v) { return xch + ((q * C::GIVEN + p - p / SP - 1) * 4 + v) * 32 + lane; };
             constexpr int CELLS = 2 * C::PAIRS + (C::ODD ? 1 : 0);
 #pragma unroll
             for (int k = 0; k < CELLS; ++k) {
@@ -449,8 +475,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
 #pragma unroll
                     for (int g = 0; g < 4; ++g) X.r[g] = Hh.r[g] = 0.0f;
                 }
-                wait_bar(a, acc0 + 8 * tile, (unsigned)t & 1);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (own) {
+                    wait_bar(a, acc0 + 8 * tile, (unsigned)t & 1);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
                 // ---- gates and cells ----
                 const uint32_t tx = acc_x(t, tile) + lane_base, th = acc_h(tile) + lane_base;
                 int kmin = INT_MAX, kmax = INT_MIN;
@@ -460,11 +488,43 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
                         kmin = min(kmin, k), kmax = max(kmax, k);
                     }
                 };
+                if constexpr (SP > 1) {
+                    const int hand = 5 + 4 * q + (warp >> 2);  // barrier of a reading warp and those it hands sums to
+                    if (own) {
+#pragma unroll
+                        for (int i = 0; i < C::PAIRS * (SP - 1); ++i) {
+                            const int p = pair_of(i / (SP - 1)) + 1 + i % (SP - 1);
+                            if (p >= 2 * NC) continue;
+                            uint32_t x[8], y[8];
+                            tmem_ld8_nowait(tx + 8 * p, x);
+                            tmem_ld8_nowait(th + 8 * p, y);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int v = 0; v < 2; ++v) {
+                                *reinterpret_cast<uint4 *>(given(p, v)) = make_uint4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+                                *reinterpret_cast<uint4 *>(given(p, 2 + v)) = make_uint4(y[4 * v], y[4 * v + 1], y[4 * v + 2], y[4 * v + 3]);
+                            }
+                        }
+                        asm volatile("bar.arrive %0, %1;" ::"r"(hand), "n"(32 * SP) : "memory");
+                    } else {
+                        bar_sync(hand, 32 * SP);
+                    }
+                }
                 auto pre_of = [&](int p) {  // pre-activations of a pair of the block's cells
                     PairSums P;
-                    tmem_ld8_nowait(tx + 8 * p, P.x);
-                    tmem_ld8_nowait(th + 8 * p, P.h);
-                    tmem_wait_ld();
+                    if (own) {
+                        tmem_ld8_nowait(tx + 8 * p, P.x);
+                        tmem_ld8_nowait(th + 8 * p, P.h);
+                        tmem_wait_ld();
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < 2; ++v) {
+                            const uint4 x = *reinterpret_cast<const uint4 *>(given(p, v)),
+                                        y = *reinterpret_cast<const uint4 *>(given(p, 2 + v));
+                            P.x[4 * v] = x.x, P.x[4 * v + 1] = x.y, P.x[4 * v + 2] = x.z, P.x[4 * v + 3] = x.w;
+                            P.h[4 * v] = y.x, P.h[4 * v + 1] = y.y, P.h[4 * v + 2] = y.z, P.h[4 * v + 3] = y.w;
+                        }
+                    }
                     const float2 *cc = ly.pairc + min(blk * 2 * NC + p, last_pair) * kPairConsts;
                     PairPre pre;
                     if (fast)
@@ -475,7 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
                 };
 #pragma unroll
                 for (int p = 0; p < C::PAIRS; ++p) {
-                    const PairPre pre = pre_of(pair0 + p);
+                    if (SP > 1 && pair_of(p) >= 2 * NC) continue;  // (uniform in the warp)
+                    const PairPre pre = pre_of(pair_of(p));
                     float2 cv = make_float2(c[2 * p], c[2 * p + 1]);
                     const float2 m = lstm_cell2(pre.g[0], pre.g[1], pre.g[2], pre.g[3], cv);
                     c[2 * p] = cv.x, c[2 * p + 1] = cv.y;
@@ -492,7 +553,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mb_arrive(drained0 + 8 * tile);
+                if (own && lane == 0) mb_arrive(drained0 + 8 * tile);
                 // ---- the row's range over the layer's blocks ----
                 atomicMin(my_min, kmin);
                 atomicMax(my_max, kmax);
@@ -649,12 +710,10 @@ __global__ void pair_constants_kernel(const float *__restrict__ bias, const int3
 }
 
 struct Plan {
-    int NC = 0, MT = 1, G = 0;
+    int NC = 0, MT = 1, SP = 1, G = 0;
     int rows_box = 0, kps = 0, slots = 0, slot_bytes = 0;
     size_t smem = 0;
 };
-
-int misc_bytes(int NC, int MT) { return Cfg<2, 2>::MISC + (MT == 1 ? 128 * NC : 0); }
 
 // The smallest cell count per block for which the stack's blocks fit the SMs one each and the widest
 // layer's weights leave room for the operand ring.
@@ -667,32 +726,34 @@ bool make_plan(const qnn_lstm_model *m, int64_t B, Plan *p) {
     if (kx > 1024) return false;
     p->MT = B > kTile ? 2 : 1;
     p->rows_box = (int)std::min<int64_t>(kTile, round_up(B, 8));
-    p->kps = std::max(1, std::min(8, kSlotBytes / (p->rows_box * 128)));
-    p->slot_bytes = p->kps * p->rows_box * 128;
+    p->SP = B <= 32 ? 4 : B <= 64 ? 2 : 1;
     for (int NC : {2, 4, 5, 6}) {
         const int64_t G = (m->H + 4 * NC - 1) / (4 * NC);
         if (G * m->L > sm_count()) continue;
         const int64_t weights = (kx + kh) / 64 * NC * 2048;
         // (by the widest slots, so that a model's layout does not depend on the batch)
-        const int64_t left = kSmemMax - weights - misc_bytes(NC, p->MT);
-        if (kSmemMax - weights - std::max(misc_bytes(NC, 1), misc_bytes(NC, 2)) < 2 * kSlotBytes) continue;
+        const int64_t left = kSmemMax - weights - misc_bytes(NC, p->MT, p->SP);
+        if (kSmemMax - weights - std::max(misc_bytes(NC, 1, 1), misc_bytes(NC, 2, 1)) < 2 * kSlotBytes) continue;
+        // (handed-over sums take up to 24 KB: where two whole slots don't fit beside them, two halves do)
+        p->kps = std::max(1, std::min(8, (left >= 2 * kSlotBytes ? kSlotBytes : kSlotBytes / 2) / (p->rows_box * 128)));
+        p->slot_bytes = p->kps * p->rows_box * 128;
         const int64_t slots = std::min<int64_t>(kMaxSlots, left / p->slot_bytes);
         p->NC = NC, p->G = (int)G, p->slots = (int)slots;
         // an operand box of fewer than 128 rows is multiplied as 128: its last slot's reads stay inside
-        const int64_t used = slots * p->slot_bytes + weights + misc_bytes(NC, p->MT);
+        const int64_t used = slots * p->slot_bytes + weights + misc_bytes(NC, p->MT, p->SP);
         p->smem = (size_t)std::min<int64_t>(kSmemMax, std::max(used, slots * p->slot_bytes + kTile * 128));
         return (int64_t)p->smem >= slots * p->slot_bytes + kTile * 128;
     }
     return false;
 }
 
-template <int NC, int MT>
+template <int NC, int MT, int SP>
 qnn_status launch(const PersistArgs &a, const Plan &p, int64_t L, cudaStream_t st) {
     static std::atomic<int> configured{-1};
     int dev = 0;
     QNN_CUDA_TRY(cudaGetDevice(&dev));
     if (configured.load() != dev) {
-        QNN_CUDA_TRY(cudaFuncSetAttribute(lstm_persist_kernel<NC, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+        QNN_CUDA_TRY(cudaFuncSetAttribute(lstm_persist_kernel<NC, MT, SP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
         configured.store(dev);
     }
     cudaLaunchConfig_t cfg = {};
@@ -705,7 +766,7 @@ qnn_status launch(const PersistArgs &a, const Plan &p, int64_t L, cudaStream_t s
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, lstm_persist_kernel<NC, MT>, a);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, lstm_persist_kernel<NC, MT, SP>, a);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         cudaGetLastError();
         return QNN_ERR_NO_COOP;
@@ -879,16 +940,16 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
     }
     {
         ProfScope prof("lstm_persist", st);
-        switch (10 * p.NC + p.MT) {
-            case 21: QNN_TRY((launch<2, 1>(a, p, L, st))); break;
-            case 22: QNN_TRY((launch<2, 2>(a, p, L, st))); break;
-            case 41: QNN_TRY((launch<4, 1>(a, p, L, st))); break;
-            case 42: QNN_TRY((launch<4, 2>(a, p, L, st))); break;
-            case 51: QNN_TRY((launch<5, 1>(a, p, L, st))); break;
-            case 52: QNN_TRY((launch<5, 2>(a, p, L, st))); break;
-            case 61: QNN_TRY((launch<6, 1>(a, p, L, st))); break;
-            default: QNN_TRY((launch<6, 2>(a, p, L, st))); break;
-        }
+        auto run = [&](auto nc) -> qnn_status {
+            constexpr int NC = decltype(nc)::value;
+            if (p.MT == 2) return launch<NC, 2, 1>(a, p, L, st);
+            return p.SP == 4 ? launch<NC, 1, 4>(a, p, L, st) : p.SP == 2 ? launch<NC, 1, 2>(a, p, L, st) : launch<NC, 1, 1>(a, p, L, st);
+        };
+        using std::integral_constant;
+        QNN_TRY(p.NC == 2   ? run(integral_constant<int, 2>{})
+                : p.NC == 4 ? run(integral_constant<int, 4>{})
+                : p.NC == 5 ? run(integral_constant<int, 5>{})
+                            : run(integral_constant<int, 6>{}));
     }
     float *const lg = C > 0 ? at(o_lg) : nullptr;
     float *const yd = y_dev ? y : y_map ? y_map : at(o_y);
