@@ -22,7 +22,7 @@
 // Bound: the chain of one frame (operand stream of h_{t-1}, gate arithmetic, two exchanges). A step
 // as launches of a quantizer and a gate kernel per layer takes two launches' latency and streams the
 // weights again; the grid barriers of lstm_recurrent_kernel keep one layer at a time on the GPU. 5 x 500
-// cells, 2000 classes, 100 frames, this kernel alone (whole pass before): B = 16 717 us (5.5 ms), B = 64
+// cells, 2000 classes, 100 frames, this kernel alone (whole pass before): B = 16 592 us (5.5 ms), B = 64
 // 1030 us (2.3 ms), B = 128 1231 us (2.6 ms), B = 256 1908 us (3.0 ms). A frame at B = 32 took about 15,000
 // cycles while one row quarter's warps, all on one scheduler, did all its cells: h's operand stream and
 // products 4,700, gates 5,000, range exchange 2,200, codes and release 2,700. With the cells spread over the
@@ -50,7 +50,12 @@ namespace {
 
 constexpr int kMaxL = 8;               // layers of a launch (tensor maps are kernel arguments)
 constexpr int kEpiWarps = 16;
-constexpr int kThreads = 32 * (kEpiWarps + 2);
+constexpr int kThreads = 32 * (kEpiWarps + 4);  // (two warps only complete the last warpgroup)
+// Registers a thread: 96 at launch (640 threads), of which the producer's warpgroup leaves its share to the
+// four epilogue ones (4 x 112 + 32 = 5 x 96). With 96 their rows' constants and cells spill, and a reload
+// misses the little L1 that the weights leave: 5 x 500 cells, B = 16 and 64, 100 frames 714 and 1435 us, B = 256,
+// 500 frames 9.59 ms; so 630, 1352 us and 8.37 ms.
+constexpr int kRegsEpi = 112, kRegsIssue = 32;
 constexpr int kMaxSlots = 4;           // operand ring slots
 constexpr int kSlotBytes = 32 * 1024;  // at most (two k-blocks of 128 rows)
 constexpr int kTile = 128;             // rows (sequences) of a tile
@@ -326,96 +331,100 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
     auto acc_x = [&](int t, int i) { return tmem + (uint32_t)(((t & 1) * MT + i) * C::N); };
     auto acc_h = [&](int i) { return tmem + (uint32_t)((2 * MT + i) * C::N); };
 
-    if (warp == kEpiWarps) {
-        // ---------------- producer ----------------
-        if (lane == 0) {
-            const uint32_t w0 = su32(wts);
-            mb_expect(wfull, (uint32_t)(kbw * C::KB_BYTES));
-            for (int kb = 0; kb < ly.kbx; ++kb) tma_load_2d(w0 + kb * C::KB_BYTES, &a.mwx[l], wfull, 64 * kb, blk * C::N);
-            for (int kb = 0; kb < a.kbh; ++kb)
-                tma_load_2d(w0 + (ly.kbx + kb) * C::KB_BYTES, &a.mwh[l], wfull, 64 * kb, blk * C::N);
-            // (one thread: its loop is on the critical path, so the ring advances by additions)
-            const uint32_t ring = su32(smem), ring_end = ring + a.slots * a.slot_bytes, slot_bytes = a.slot_bytes;
-            const int kps = a.kps;
-            uint32_t dst = ring, bar = full0;
-            unsigned parity = 1;  // a fresh slot's empty barrier passes with parity 1
-            auto stream = [&](const CUtensorMap *map, int kbs, int row) {
-                for (int kb = 0; kb < kbs; kb += kps) {
-                    wait_bar(a, bar + 8 * kMaxSlots, parity);
-                    mb_expect(bar, slot_bytes);
-                    tma_load_3d(dst, map, bar, 0, row, kb);  // k-blocks past the matrix read as zero
-                    dst += slot_bytes, bar += 8;
-                    if (dst == ring_end) dst = ring, bar = full0, parity ^= 1u;
-                }
-            };
-            for (int t = 0; t < T; ++t) {
-#pragma unroll
-                for (int i = 0; i < MT; ++i) {
-                    if (l > 0) {
-                        wait_counter(a, a.ctr + 2 * (l - 1) + i, (unsigned)(quarters(i) * a.G * (t + 1)));
-                        asm volatile("fence.proxy.async.global;" ::: "memory");
+    if (warp >= kEpiWarps) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
+        if (warp == kEpiWarps) {
+            // ---------------- producer ----------------
+            if (lane == 0) {
+                const uint32_t w0 = su32(wts);
+                mb_expect(wfull, (uint32_t)(kbw * C::KB_BYTES));
+                for (int kb = 0; kb < ly.kbx; ++kb) tma_load_2d(w0 + kb * C::KB_BYTES, &a.mwx[l], wfull, 64 * kb, blk * C::N);
+                for (int kb = 0; kb < a.kbh; ++kb)
+                    tma_load_2d(w0 + (ly.kbx + kb) * C::KB_BYTES, &a.mwh[l], wfull, 64 * kb, blk * C::N);
+                // (one thread: its loop is on the critical path, so the ring advances by additions)
+                const uint32_t ring = su32(smem), ring_end = ring + a.slots * a.slot_bytes, slot_bytes = a.slot_bytes;
+                const int kps = a.kps;
+                uint32_t dst = ring, bar = full0;
+                unsigned parity = 1;  // a fresh slot's empty barrier passes with parity 1
+                auto stream = [&](const CUtensorMap *map, int kbs, int row) {
+                    for (int kb = 0; kb < kbs; kb += kps) {
+                        wait_bar(a, bar + 8 * kMaxSlots, parity);
+                        mb_expect(bar, slot_bytes);
+                        tma_load_3d(dst, map, bar, 0, row, kb);  // k-blocks past the matrix read as zero
+                        dst += slot_bytes, bar += 8;
+                        if (dst == ring_end) dst = ring, bar = full0, parity ^= 1u;
                     }
-                    stream(&a.mx[l], ly.kbx, t * B + kTile * i);
-                }
+                };
+                for (int t = 0; t < T; ++t) {
 #pragma unroll
-                for (int i = 0; i < MT; ++i) {
-                    if (t > 0) wait_counter(a, a.ctr + 2 * l + i, (unsigned)(quarters(i) * a.G * t));
-                    mb_arrive(ready0 + 8 * i);  // x_t and h_{t-1}: their units and code sums may be read
-                    asm volatile("fence.proxy.async.global;" ::: "memory");
-                    if (t > 0)
-                        stream(&a.mh[l], a.kbh, (t - 1) * B + kTile * i);
-                    else
-                        stream(&a.mh0, a.kbh, l * B + kTile * i);
+                    for (int i = 0; i < MT; ++i) {
+                        if (l > 0) {
+                            wait_counter(a, a.ctr + 2 * (l - 1) + i, (unsigned)(quarters(i) * a.G * (t + 1)));
+                            asm volatile("fence.proxy.async.global;" ::: "memory");
+                        }
+                        stream(&a.mx[l], ly.kbx, t * B + kTile * i);
+                    }
+#pragma unroll
+                    for (int i = 0; i < MT; ++i) {
+                        if (t > 0) wait_counter(a, a.ctr + 2 * l + i, (unsigned)(quarters(i) * a.G * t));
+                        mb_arrive(ready0 + 8 * i);  // x_t and h_{t-1}: their units and code sums may be read
+                        asm volatile("fence.proxy.async.global;" ::: "memory");
+                        if (t > 0)
+                            stream(&a.mh[l], a.kbh, (t - 1) * B + kTile * i);
+                        else
+                            stream(&a.mh0, a.kbh, l * B + kTile * i);
+                    }
                 }
             }
-        }
-    } else if (warp == kEpiWarps + 1) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            constexpr uint32_t idesc = mma_idesc_f16(kTile, C::N);
-            const uint32_t da0 = smem_desc_lo(su32(smem)), sub = (uint32_t)a.rows_box * 128 / 16, slot16 = a.slot_bytes / 16;
-            const uint32_t bar_end = full0 + 8 * a.slots;
-            const int kps = a.kps;
-            uint32_t da = da0, bar = full0;
-            unsigned parity = 0;
-            wait_bar(a, wfull, 0);
-            // d = the k-blocks of one operand against the weights at w; `done` (0: none) completes with them
-            auto multiply = [&](uint32_t d, uint32_t w, int kbs, uint32_t done) {
-                uint32_t accumulate = 0;
-                for (int kb = 0; kb < kbs; kb += kps) {
-                    wait_bar(a, bar, parity);
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const int nv = min(kps, kbs - kb);
-                    uint32_t x = da;
+        } else if (warp == kEpiWarps + 1) {
+            // ---------------- MMA issuer ----------------
+            if (lane == 0) {
+                constexpr uint32_t idesc = mma_idesc_f16(kTile, C::N);
+                const uint32_t da0 = smem_desc_lo(su32(smem)), sub = (uint32_t)a.rows_box * 128 / 16, slot16 = a.slot_bytes / 16;
+                const uint32_t bar_end = full0 + 8 * a.slots;
+                const int kps = a.kps;
+                uint32_t da = da0, bar = full0;
+                unsigned parity = 0;
+                wait_bar(a, wfull, 0);
+                // d = the k-blocks of one operand against the weights at w; `done` (0: none) completes with them
+                auto multiply = [&](uint32_t d, uint32_t w, int kbs, uint32_t done) {
+                    uint32_t accumulate = 0;
+                    for (int kb = 0; kb < kbs; kb += kps) {
+                        wait_bar(a, bar, parity);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const int nv = min(kps, kbs - kb);
+                        uint32_t x = da;
 #pragma unroll 2
-                    for (int v = 0; v < nv; ++v) {
-                        mma_f16_lo(d, x, w, idesc, accumulate);
-                        accumulate = 1;
+                        for (int v = 0; v < nv; ++v) {
+                            mma_f16_lo(d, x, w, idesc, accumulate);
+                            accumulate = 1;
 #pragma unroll
-                        for (int k = 1; k < 4; ++k) mma_f16_lo(d, x + 2 * k, w + 2 * k, idesc, 1u);  // 16 fp16 = 32 bytes
-                        x += sub, w += C::KB_BYTES / 16;
+                            for (int k = 1; k < 4; ++k) mma_f16_lo(d, x + 2 * k, w + 2 * k, idesc, 1u);  // 16 fp16 = 32 bytes
+                            x += sub, w += C::KB_BYTES / 16;
+                        }
+                        if (done && kb + kps >= kbs) mma_commit(done);  // (before the slot's: a commit takes 250 cycles)
+                        mma_commit(bar + 8 * kMaxSlots);
+                        da += slot16, bar += 8;
+                        if (bar == bar_end) da = da0, bar = full0, parity ^= 1u;
                     }
-                    if (done && kb + kps >= kbs) mma_commit(done);  // (before the slot's: a commit takes 250 cycles)
-                    mma_commit(bar + 8 * kMaxSlots);
-                    da += slot16, bar += 8;
-                    if (bar == bar_end) da = da0, bar = full0, parity ^= 1u;
-                }
-            };
-            const uint32_t wx = smem_desc_lo(su32(wts)), wh = wx + ly.kbx * (C::KB_BYTES / 16);
-            for (int t = 0; t < T; ++t) {
+                };
+                const uint32_t wx = smem_desc_lo(su32(wts)), wh = wx + ly.kbx * (C::KB_BYTES / 16);
+                for (int t = 0; t < T; ++t) {
 #pragma unroll
-                for (int i = 0; i < MT; ++i) multiply(acc_x(t, i), wx, ly.kbx, 0);
+                    for (int i = 0; i < MT; ++i) multiply(acc_x(t, i), wx, ly.kbx, 0);
 #pragma unroll
-                for (int i = 0; i < MT; ++i) {
-                    // both accumulators of frame t - 1 read out (and, one frame back, x's of this parity)
-                    if (t > 0) wait_bar(a, drained0 + 8 * i, (unsigned)(t - 1) & 1);
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    multiply(acc_h(i), wh, a.kbh, acc0 + 8 * i);
+                    for (int i = 0; i < MT; ++i) {
+                        // both accumulators of frame t - 1 read out (and, one frame back, x's of this parity)
+                        if (t > 0) wait_bar(a, drained0 + 8 * i, (unsigned)(t - 1) & 1);
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        multiply(acc_h(i), wh, a.kbh, acc0 + 8 * i);
+                    }
                 }
             }
         }
     } else {
         // ---------------- epilogue ----------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
         // row quarter q, slice e; `own`: this warp may read the quarter's tensor-memory lanes
         const int tile = MT == 2 ? warp >> 3 : 0, q = warp & (4 / SP - 1), rep = (warp & 3) / (4 / SP);
         const int e = SP > 1 ? (warp >> 2) * SP + rep : (warp >> 2) & (C::SL - 1);
@@ -435,7 +444,8 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
             const int j_blk = blk * C::CB;
             // cells of this thread: pairs e PAIRS .. of the block, and for odd NC one of pair 2 NC - 2 ..
             const int pair0 = e * C::PAIRS, pair_odd = 4 * C::PAIRS + (e >> 1), odd = e & 1;
-            float c[2 * C::PAIRS + 1], h[2 * C::PAIRS + 1];
+            constexpr int CELLS = 2 * C::PAIRS + (C::ODD ? 1 : 0);
+            float c[CELLS];
             // (SP > 1: pairs e, e + SL of the block; cells of no pair lie past every row)
             auto pair_of = [&](int k) { return SP > 1 ? e + C::SL * k : pair0 + k; };
             auto cell_of = [&](int k) {
@@ -445,7 +455,6 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
             // sums of a pair handed over: 16-byte words v = 0 .. 3 of each row
             float4 *const xch = reinterpret_cast<float4 *>(s_min + 4 * kTile) + (MT == 1 ? 8 * NC : 0);
             auto given = [&](int p, int v) { return xch + ((q * C::GIVEN + p - p / SP - 1) * 4 + v) * 32 + lane; };
-            constexpr int CELLS = 2 * C::PAIRS + (C::ODD ? 1 : 0);
 #pragma unroll
             for (int k = 0; k < CELLS; ++k) {
                 const int j = cell_of(k);
@@ -458,6 +467,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_
                 Qh = p.Q, zh = p.z;
             }
             for (int t = 0; t < T; ++t) {
+                float h[CELLS];
                 // ---- units and code sums of the row's x_t and h_{t-1} ----
                 float Qx = 1.0f;
                 int zx = 0, rsx = 0, rsh = 0;
