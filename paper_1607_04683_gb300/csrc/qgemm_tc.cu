@@ -20,6 +20,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1224,35 +1225,83 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     }
 }
 
-// u8 codes -> centered fp16 (c - 128), rows padded with zeros to ldo (a multiple of 64). A thread
-// converts 16 codes: one 16-byte load and two 16-byte stores when the row is 16-byte aligned and
-// the 16 codes lie inside K, element by element otherwise (ragged tail, padding, unaligned rows).
-__global__ void center_fp16_kernel(const uint8_t *__restrict__ in, int64_t rows, int K, int64_t ldi,
-                                   __half *__restrict__ out, int ldo) {
-    const int per_row = ldo / 16;
-    const int64_t total = rows * (int64_t)per_row;
-    const bool vec = (reinterpret_cast<uintptr_t>(in) & 15) == 0 && ldi % 16 == 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / per_row;
-        const int k0 = (int)(i - r * per_row) * 16;
-        uint4 o[2];
-        if (vec && k0 + 16 <= K) {
-            const uint4 w = *reinterpret_cast<const uint4 *>(in + r * ldi + k0);
-            o[0] = make_uint4(center2(w.x, 0x4140u), center2(w.x, 0x4342u), center2(w.y, 0x4140u), center2(w.y, 0x4342u));
-            o[1] = make_uint4(center2(w.z, 0x4140u), center2(w.z, 0x4342u), center2(w.w, 0x4140u), center2(w.w, 0x4342u));
-        } else {
-            __align__(16) __half v[16];
+// u8 codes -> centered fp16 (c - 128) of two matrices of K columns (N may be 0), rows padded with zeros to ldo
+// (a multiple of 64), the second matrix's rows after the first's in `out`. A thread converts 8 codes at a
+// time (its warp then stores 512 consecutive bytes), kCenterFlight times in flight. With SHIFT the rows have
+// any alignment: a thread loads the aligned 8-byte unit its codes begin in and the one after (its neighbour's
+// first), and shifts. Codes that a row's or a matrix's end cuts go byte by byte.
+//
+// Bound: HBM (3 bytes a code). 16 codes a thread, stored as 16-byte halves of 32 bytes, one load in flight and a
+// launch a matrix: 16384 + 8192 rows of 8192 122 us, 4.9 TB/s; so 109 us, 5.5 TB/s. Rows without an alignment byte by
+// byte: 9374 + 3033 rows of 2052 28 us; so 23 us.
+struct CenterArgs {
+    const uint8_t *in[2];
+    int64_t ld[2], rows[2];
+    int K;
+    int per_row;    // groups of 8 codes a row
+    int64_t total;  // groups of both
+    __half *out;
+};
+constexpr int kCenterFlight = 4;
+
+template <bool SHIFT>
+__global__ void __launch_bounds__(256) center_fp16_kernel(const CenterArgs a) {
+    grid_dependents_launch();
+    const int64_t step = (int64_t)gridDim.x * 256;
+    const bool small = a.total <= INT_MAX;
+    for (int64_t i0 = (int64_t)blockIdx.x * 256 + threadIdx.x; i0 < a.total; i0 += step * kCenterFlight) {
+        uint2 u[kCenterFlight], v[SHIFT ? kCenterFlight : 1];
+        int sh[kCenterFlight];  // where the codes begin in u; -1: to be taken byte by byte
 #pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int k = k0 + e;
-                v[e] = k < K ? __int2half_rn((int)in[r * ldi + k] - 128) : __int2half_rn(0);
+        for (int j = 0; j < kCenterFlight; ++j) {
+            const int64_t i = i0 + j * step;
+            sh[j] = -1;
+            if (i >= a.total) continue;
+            int64_t row = small ? (int64_t)((unsigned)i / (unsigned)a.per_row) : i / a.per_row;
+            const int k0 = (int)(i - row * a.per_row) * 8;
+            const bool m = row >= a.rows[0];
+            const uint8_t *const base = m ? a.in[1] : a.in[0];
+            const int64_t ld = m ? a.ld[1] : a.ld[0];
+            if (m) row -= a.rows[0];
+            if (k0 + 8 > a.K) continue;
+            const uint8_t *const c = base + row * ld + k0;
+            if constexpr (SHIFT) {
+                const int s = (int)(reinterpret_cast<uintptr_t>(c) & 7);
+                if (c - s < base || c - s + 16 > base + ((m ? a.rows[1] : a.rows[0]) - 1) * ld + a.K) continue;
+                u[j] = __ldg(reinterpret_cast<const uint2 *>(c - s));
+                v[j] = __ldg(reinterpret_cast<const uint2 *>(c - s) + 1);
+                sh[j] = s;
+            } else {
+                u[j] = __ldg(reinterpret_cast<const uint2 *>(c));
+                sh[j] = 0;
             }
-            o[0] = reinterpret_cast<const uint4 *>(v)[0];
-            o[1] = reinterpret_cast<const uint4 *>(v)[1];
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(out + r * ldo + k0);
-        dst[0] = o[0];
-        dst[1] = o[1];
+#pragma unroll
+        for (int j = 0; j < kCenterFlight; ++j) {
+            const int64_t i = i0 + j * step;
+            if (i >= a.total) break;
+            uint32_t w[2] = {u[j].x, u[j].y};
+            if (sh[j] < 0) {
+                int64_t row = i / a.per_row;
+                const int k0 = (int)(i - row * a.per_row) * 8;
+                const bool m = row >= a.rows[0];
+                const uint8_t *const c = m ? a.in[1] + (row - a.rows[0]) * a.ld[1] + k0 : a.in[0] + row * a.ld[0] + k0;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    w[e] = 0;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)  // (128, a centered zero, past the row)
+                        w[e] |= (k0 + 4 * e + b < a.K ? (uint32_t)__ldg(c + 4 * e + b) : 128u) << (8 * b);
+                }
+            } else if constexpr (SHIFT) {
+                const bool word = sh[j] & 4;
+                const uint32_t e0 = word ? w[1] : w[0], e1 = word ? v[j].x : w[1], e2 = word ? v[j].y : v[j].x;
+                w[0] = __funnelshift_r(e0, e1, 8 * (sh[j] & 3));
+                w[1] = __funnelshift_r(e1, e2, 8 * (sh[j] & 3));
+            }
+            reinterpret_cast<uint4 *>(a.out)[i] =
+                make_uint4(center2(w[0], 0x4140u), center2(w[0], 0x4342u), center2(w[1], 0x4140u), center2(w[1], 0x4342u));
+        }
     }
 }
 
@@ -1558,14 +1607,24 @@ qnn_status tc_partial(const TcOperands &op, int splits, int32_t *part, int64_t l
                        : launch_tc<128, kEpiPartial>(op, a, "qgemm_tc_partial", st);
 }
 
+static qnn_status launch_center_pair(const uint8_t *A, int64_t lda, int64_t M, const uint8_t *W, int64_t ldw, int64_t N,
+                                     int64_t K, __half *out, int64_t ldo, cudaStream_t st) {
+    CenterArgs a{{A, W}, {lda, ldw}, {M, N}, (int)K, (int)(ldo / 8), (M + N) * (ldo / 8), out};
+    const uintptr_t at = reinterpret_cast<uintptr_t>(A) | (uintptr_t)lda | (N ? reinterpret_cast<uintptr_t>(W) | (uintptr_t)ldw : 0);
+    const int64_t blocks = (a.total + 256 * kCenterFlight - 1) / (256 * kCenterFlight);
+    const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)sm_count() * 8);
+    if ((at & 7) == 0)
+        center_fp16_kernel<false><<<grid, 256, 0, st>>>(a);
+    else
+        center_fp16_kernel<true><<<grid, 256, 0, st>>>(a);
+    QNN_CUDA_TRY(cudaGetLastError());
+    return QNN_OK;
+}
+
 qnn_status launch_center_fp16(const uint8_t *in, int64_t rows, int64_t K, int64_t ldi, __half *out, int64_t ldo,
                               cudaStream_t st) {
     if (rows == 0) return QNN_OK;
-    const int64_t tot = rows * (ldo / 16);
-    center_fp16_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, (int64_t)sm_count() * 16), 256, 0, st>>>(
-        in, rows, (int)K, ldi, out, (int)ldo);
-    QNN_CUDA_TRY(cudaGetLastError());
-    return QNN_OK;
+    return launch_center_pair(in, ldi, rows, nullptr, 0, 0, K, out, ldo, st);
 }
 
 // Centers A and W into fp16 scratch and runs the tensor-core product (K <= QNN_K_MAX).
@@ -1579,11 +1638,13 @@ qnn_status launch_qgemm_tc(const uint8_t *A, int64_t lda, const qnn_qparams *pa,
     __half *W16 = A16 + M * kp;
     {
         ProfScope prof("center_fp16", st);
-        QNN_TRY(launch_center_fp16(A, M, K, lda, A16, kp, st));
-        QNN_TRY(launch_center_fp16(W, N, K, ldw, W16, kp, st));
+        QNN_TRY(launch_center_pair(A, lda, M, W, ldw, N, K, A16, kp, st));
     }
     TcOperands op;
     QNN_TRY(tc_operands(&op, A16, M, W16, N, kp, tc_pick_bn(M, N, kp)));
+    // its block setup overlaps a short centering pass (a long one loses more: 16384 x 8192 x 8192 1521 us so, 1511
+    // without; 4096 x 2048 x 512 34.9 against 36.5)
+    op.pdl = (M + N) * kp <= (int64_t)1 << 26;
     return tc_linear(op, pa, ga == QNN_PER_ROW, rsA, K, pw, rows_per_block, csW, bias, Y, ldy, acc_out, st);
 }
 

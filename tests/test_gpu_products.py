@@ -155,3 +155,20 @@ def test_few_codes(qnn, M, N, K, off):
                              qnn.params_tensor(pw), gpu(cs), want_acc=True)
     assert qnn.device_status() == qnn.QNN_OK
     assert np.array_equal(acc.cpu().numpy(), ref["acc"]) and np.array_equal(Y.cpu().numpy(), ref["y"])
+
+
+# Centering both operands, rows of any alignment: around 8 codes, whole and ragged rows, the first and last
+# codes of a matrix, more than one round of a thread's groups.
+@pytest.mark.parametrize("M,N,K", [(130, 70, 1), (130, 70, 7), (129, 65, 8), (131, 64, 9), (200, 3, 23), (150, 150, 65), (140, 90, 1030),
+                                   (9000, 2000, 517)])
+@pytest.mark.parametrize("pad,off", [(0, 0), (0, 1), (3, 7), (8, 8)])
+def test_centered_operands(qnn, M, N, K, pad, off, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "tc")
+    g = np.random.Generator(np.random.PCG64(M + N + K))
+    ca, pa, ra = oracle.quantize(g.normal(0.1, 1.0, (M, K)).astype(np.float32), oracle.PER_ROW)
+    cw, pw, cs = oracle.quantize(g.normal(0.0, 1.0, (N, K)).astype(np.float32), oracle.PER_MATRIX)
+    ref = oracle.qmatmul(ca, pa, oracle.PER_ROW, cw, pw)
+    _, acc = qnn.qnn_qmatmul(strided(ca, K + pad, off), qnn.params_tensor(pa), oracle.PER_ROW, gpu(ra), strided(cw, K + pad, off),
+                             qnn.params_tensor(pw), gpu(cs), want_acc=True)
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"])
