@@ -11,9 +11,10 @@
 // memory buffer (two, alternating) and is drained into int32 registers as soon as it completes.
 //
 // Tile: 128 rows of A x 256 rows of W per block, K in steps of 64 fp16 (128-byte rows, TMA with
-// 128-byte swizzle into a 4-stage shared-memory ring). Warp 0 issues TMA, warp 1 issues the MMAs
+// 128-byte swizzle into a 4-stage shared-memory ring). By role, warp 0 issues TMA, warp 1 the MMAs
 // (tcgen05.mma.cta_group::1.kind::f16, M 128 N 256 K 16) and owns the tensor memory, warps 2-9 are
-// the epilogue (each tensor-memory lane quarter is read by two warps, one per column half).
+// the epilogue (each tensor-memory lane quarter is read by two warps, one per column half); the epilogue's
+// warps come first in the block (SPLIT below).
 // Every wait is bounded in time; a wait that gives up records QNN_ERR_TIMEOUT and the block skips
 // ahead, waits (bounded) for its own copies in flight, frees its tensor memory and returns.
 #include <cuda.h>
@@ -63,7 +64,7 @@ struct ColUnit {  // and the weight unit of each column (-1 past N)
 // register cap, the epilogue's shared staging, and the MMA instruction descriptor (fp32
 // accumulator, fp16 A and B, both K-major, M = 128, N = BN). A block that allocates tensor memory
 // has its SM to itself, so the ALU-bound row and LSTM epilogues run sixteen warps (four per
-// tensor-memory lane quarter); eighteen warps fit the register file at 96 registers a thread.
+// tensor-memory lane quarter); eighteen to twenty warps fit the register file at 96 registers a thread.
 template <int BN, int EPI>
 struct Tile {
     static_assert(EPI == kEpiLinear || BN <= 128, "row and LSTM epilogues take tiles of at most 128 columns");
@@ -74,7 +75,12 @@ struct Tile {
     static constexpr int EPI_WARPS = EPI == kEpiLinear ? 8 : (LSTM96 ? 24 : 16);
     // LSTM: cells per epilogue slice (a 32-column tile has 8 cells: 2-cell slices keep 4 warps busy)
     static constexpr int CPS = BN == 32 ? 2 : 4;
-    static constexpr int THREADS = 32 * (2 + EPI_WARPS);
+    // SPLIT: the epilogue warps come first and the two issuing ones after them, in a warpgroup of their own that
+    // leaves most of its registers to the epilogue's. (At the registers an even share leaves a thread the
+    // epilogues spill, and their reloads go through the same port as the operands: 16384 x 8192 x 8192 1521 us,
+    // so 1421; 9374 x 3032 x 2052 142 and 128; LSTMP 5 x 2048p512, B = 1024, 100 frames 20.35 and 19.88 ms.)
+    static constexpr bool SPLIT = EPI == kEpiLinear || EPI == kEpiRow || (IS_LSTM && !LSTM96);
+    static constexpr int THREADS = 32 * ((SPLIT ? 4 : 2) + EPI_WARPS);
     static constexpr int B_BYTES = BN * TBK * 2;
     // a pipeline stage carries KPS consecutive k-blocks (A sub-tiles first, then the W sub-tiles):
     // the operand stream advances by stages at a pace that hardly depends on their size, so short
@@ -122,6 +128,9 @@ struct Tile {
     // warps sit on the four SM sub-partitions by index: 18 warps put 5 on one (5 x 32 x 96 <= 16384),
     // 26 warps put 7 on one (7 x 32 x 72 <= 16384)
     static constexpr int MAX_REGS = EPI == kEpiLinear ? 168 : (LSTM96 ? 72 : 96);
+    // SPLIT: per warpgroup, EPI_WARPS / 4 REGS_EPI + REGS_ISSUE <= (EPI_WARPS / 4 + 1) MAX_REGS
+    static constexpr int REGS_ISSUE = 32, REGS_EPI = EPI_WARPS == 8 ? 232 : 112;
+    static_assert(!SPLIT || EPI_WARPS / 4 * REGS_EPI + REGS_ISSUE <= (EPI_WARPS / 4 + 1) * MAX_REGS, "registers of the block");
     static constexpr uint32_t IDESC = mma_idesc_f16(TBM, BN);
     static constexpr uint32_t IDESC_HALF = mma_idesc_f16(TBM, BN / 2 >= 16 ? BN / 2 : 16);  // half-width items
     static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + EPI_BYTES + 256;
@@ -198,14 +207,11 @@ __device__ __forceinline__ void st_vec(float *p, const float (&v)[2]) {
 // Tile order: groups of kGroupM row tiles, columns outer within a group, so that the tiles one
 // wave of blocks works on span a compact block of A and W (both stay in L2 across the wave).
 constexpr int kGroupM = 16;
-__device__ __forceinline__ void tile_origin(int64_t tile, int64_t tiles_m, int tiles_n, int bn, int64_t &m0,
-                                            int64_t &n0) {
-    const int64_t per_group = (int64_t)kGroupM * tiles_n;
-    const int64_t first = (tile / per_group) * kGroupM;
-    const int64_t rows = tiles_m - first < kGroupM ? tiles_m - first : kGroupM;
-    const int64_t local = tile % per_group;
-    m0 = (first + local % rows) * TBM;
-    n0 = (local / rows) * bn;
+__device__ __forceinline__ void tile_origin(int tile, int tiles_m, int tiles_n, int bn, int64_t &m0, int64_t &n0) {
+    const int per_group = kGroupM * tiles_n, group = tile / per_group, first = group * kGroupM;
+    const int rows = min(tiles_m - first, kGroupM), local = tile - group * per_group, col = local / rows;
+    m0 = (int64_t)(first + local - col * rows) * TBM;
+    n0 = (int64_t)col * bn;
 }
 
 // Recovered outputs of one block of COLS columns of one row that lies in one weight unit, in fp32: the
@@ -300,35 +306,36 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                    drained0 = su32(bars + 2 * STAGES + 2);
     // LSTM only: px/c buffer i loaded (pxfull0 + 8 i) and released by every epilogue warp (pxempty0 + 8 i)
     const uint32_t pxfull0 = su32(bars + 2 * STAGES + 4), pxempty0 = su32(bars + 2 * STAGES + 6);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // roles by `warp`: 0 producer, 1 MMA issuer, 2 .. EPI_WARPS + 1 epilogue (tensor-memory lane quarter hw & 3)
+    const int hw = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = !TL::SPLIT || hw >= TL::EPI_WARPS + 2 ? hw : hw < TL::EPI_WARPS ? hw + 2 : hw - TL::EPI_WARPS;
     constexpr bool LX = EPI == kEpiLstmX;
     const int nchunks = (args.KB + KCHUNK / TBK - 1) / (KCHUNK / TBK);  // K chunks of a tile (kEpiLinear)
     const int tiles_n = (int)((args.N + BN - 1) / BN);
-    const int64_t tiles_m = (args.M + TBM - 1) / TBM;
-    const int64_t tiles = tiles_m * tiles_n;
+    const int tiles_m = (int)((args.M + TBM - 1) / TBM);
+    const int tiles = tiles_m * tiles_n;
     // work items: (tile, K range); one K range per tile except for split-K. LSTM epilogues may split
     // the tiles of the last wave into half-width items (the first BN / 2 columns of the tile's W box
     // feed an MMA of N = BN / 2; the px, c and constant boxes are loaded whole)
     const int splits = args.splits;
-    const int64_t full_tiles =
-        (TL::IS_LSTM && args.full_tiles > 0 && args.full_tiles < tiles) ? args.full_tiles : tiles;
-    const int64_t work = full_tiles + 2 * (tiles - full_tiles);  // tile items
-    const int64_t items = work * splits;
+    const int full_tiles = (TL::IS_LSTM && args.full_tiles > 0 && args.full_tiles < tiles) ? (int)args.full_tiles : tiles;
+    const int work = full_tiles + 2 * (tiles - full_tiles);  // tile items
+    const int items = work * splits;
     // origin of tile item w; true for a half-width item
-    auto item_origin = [&](int64_t w, int64_t &m0, int64_t &n0) -> bool {
+    auto item_origin = [&](int w, int64_t &m0, int64_t &n0) -> bool {
         if (w < full_tiles) {
             tile_origin(w, tiles_m, tiles_n, BN, m0, n0);
             return false;
         }
-        const int64_t j = w - full_tiles;
+        const int j = w - full_tiles;
         tile_origin(full_tiles + j / 2, tiles_m, tiles_n, BN, m0, n0);
         n0 += (j & 1) * (BN / 2);
         return true;
     };
     // The k-blocks of an item in two segments: kEpiLstmX's x_t and Wx (segment 0), then A and W (segment 1;
     // an item's own K range for split-K). A stage holds k-blocks of one segment.
-    auto segment = [&](int seg, int64_t item, int &kb, int &end) {
-        kb = seg == 0 || LX ? 0 : (int)(item % splits) * args.kbs;
+    auto segment = [&](int seg, int item, int &kb, int &end) {
+        kb = seg == 0 || LX ? 0 : (item % splits) * args.kbs;
         end = seg == 0 ? args.KB_x : LX ? args.KB : min(args.KB, kb + args.kbs);
     };
     __shared__ int s_abort;
@@ -402,119 +409,123 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     // Persistent: block b takes tiles b, b + grid, ... in grouped order (tile_origin). The k-block
     // and chunk counters run across tiles, so the two accumulator buffers alternate and one tile's
     // epilogue overlaps the next tile's MMAs.
-    if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        // One thread issues every copy and every instruction of its loop is on the critical path of the
-        // operand stream (a few cycles each, one after the other), so the ring position advances
-        // incrementally in 32-bit registers.
-        if (lane == 0) {
-            const uint32_t ring0 = su32(smem);
-            uint32_t dst = ring0, bar = full0;
-            unsigned free_parity = 1;
-            int issued = 0;
-            for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                int64_t m0l, n0l;
-                item_origin(item / splits, m0l, n0l);
-                const int m0 = (int)m0l, n0 = (int)n0l;
+    if (warp < 2 || warp >= 2 + TL::EPI_WARPS) {
+        if constexpr (TL::SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::REGS_ISSUE));
+        if (warp == 0) {
+            // ---------------- TMA producer ----------------
+            // One thread issues every copy and every instruction of its loop is on the critical path of the
+            // operand stream (a few cycles each, one after the other), so the ring position advances
+            // incrementally in 32-bit registers.
+            if (lane == 0) {
+                const uint32_t ring0 = su32(smem);
+                uint32_t dst = ring0, bar = full0;
+                unsigned free_parity = 1;
+                int issued = 0;
+                for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                    int64_t m0l, n0l;
+                    item_origin(item / splits, m0l, n0l);
+                    const int m0 = (int)m0l, n0 = (int)n0l;
 #pragma unroll
-                for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
-                    const CUtensorMap *const ma = seg == 0 ? &mapAX : &mapA, *const mw = seg == 0 ? &mapWX : &mapW;
-                    int kb, end;
-                    segment(seg, item, kb, end);
-                    for (; kb < end; kb += TL::KPS) {
-                        // (not on a slot's first use: an early stage may already be freed again)
-                        if (issued >= STAGES && !mb_wait(bar + 8 * STAGES, free_parity, args.status)) {
-                            s_abort = 1;
-                            break;
-                        }
-                        const int nv = min(TL::KPS, end - kb);   // k-blocks in this stage (the last may be short)
-                        const bool w_sent = issued < w_early;    // W already on its way (expect set with it)
-                        if (issued >= full_early) {              // (else issued whole before the wait)
-                            if (!w_sent) mb_expect(bar, (uint32_t)(nv * TL::SUB_BYTES));
-#pragma unroll
-                            for (int v = 0; v < TL::KPS; ++v) {
-                                if (v >= nv) break;
-                                tma_load_2d(dst + v * A_BYTES, ma, bar, (kb + v) * TBK, m0);
-                                if (!w_sent)
-                                    tma_load_2d(dst + TL::KPS * A_BYTES + v * TL::B_BYTES, mw, bar, (kb + v) * TBK, n0);
-                            }
-                        }
-                        ++issued;
-                        dst += TL::STAGE_BYTES, bar += 8;
-                        if (bar == full0 + 8 * STAGES) dst = ring0, bar = full0, free_parity ^= 1u;
-                    }
-                    if (s_abort) break;
-                }
-            }
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        // Its loop is what a k-block costs when it is longer than the MMAs themselves: four MMAs issue in
-        // about 230 cycles (a floor for N <= 128; 521 at N = 256), a commit takes about 250, and everything
-        // else here adds to that. So the descriptors are 32-bit additions to a running low word (the high
-        // word is constant) and the accumulate flag a constant after the first MMA. Probe of the loop
-        // alone, cycles per 64-wide k-block: 761 with descriptors built per MMA and a 64-bit ring counter;
-        // 535 so (N = 128, one k-block a stage), 381 with two k-blocks a stage, 544 at N = 256.
-        if (lane == 0) {
-            const uint32_t desc0 = smem_desc_lo(su32(smem));
-            uint32_t da = desc0, bar = full0;
-            unsigned parity = 0;
-            unsigned gc = 0;  // chunks accumulated by this block
-            for (int64_t item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
-                const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
-#pragma unroll
-                for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
-                    int kb, end;
-                    segment(seg, item, kb, end);
-                    int kc = 0;  // position in the K chunk (chunks hold whole stages)
-                    uint32_t tmem_d = 0;
-                    for (; kb < end; kb += TL::KPS) {
-                        const bool fresh = kc == 0;
-                        if (fresh) {
-                            // kEpiLstmX: x's k-blocks into the buffer's first accumulator, h's into the second
-                            tmem_d = tmem_base + (gc & 1) * TL::ACC_COLS + (LX && seg == 1 ? BN : 0);
-                            if ((!LX || seg == 0) && gc >= 2 &&
-                                !mb_wait(drained0 + 8 * (gc & 1), ((gc >> 1) - 1) & 1, args.status)) {  // buffer free
+                    for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
+                        const CUtensorMap *const ma = seg == 0 ? &mapAX : &mapA, *const mw = seg == 0 ? &mapWX : &mapW;
+                        int kb, end;
+                        segment(seg, item, kb, end);
+                        for (; kb < end; kb += TL::KPS) {
+                            // (not on a slot's first use: an early stage may already be freed again)
+                            if (issued >= STAGES && !mb_wait(bar + 8 * STAGES, free_parity, args.status)) {
                                 s_abort = 1;
                                 break;
                             }
-                        }
-                        if (!mb_wait(bar, parity, args.status)) {
-                            s_abort = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t db = da + ((TL::KPS * A_BYTES) >> 4);
+                            const int nv = min(TL::KPS, end - kb);   // k-blocks in this stage (the last may be short)
+                            const bool w_sent = issued < w_early;    // W already on its way (expect set with it)
+                            if (issued >= full_early) {              // (else issued whole before the wait)
+                                if (!w_sent) mb_expect(bar, (uint32_t)(nv * TL::SUB_BYTES));
 #pragma unroll
-                        for (int v = 0; v < TL::KPS; ++v) {
-                            if (v > 0 && kb + v >= end) break;
-#pragma unroll
-                            for (int k = 0; k < TBK / 16; ++k) {
-                                // advance 16 fp16 = 32 bytes along K inside the swizzled 128-byte rows
-                                const uint32_t x = da + ((v * A_BYTES + 32 * k) >> 4), w = db + ((v * TL::B_BYTES + 32 * k) >> 4);
-                                if (v == 0 && k == 0)
-                                    mma_f16_lo(tmem_d, x, w, idesc, fresh ? 0u : 1u);
-                                else
-                                    mma_f16_lo(tmem_d, x, w, idesc, 1u);
+                                for (int v = 0; v < TL::KPS; ++v) {
+                                    if (v >= nv) break;
+                                    tma_load_2d(dst + v * A_BYTES, ma, bar, (kb + v) * TBK, m0);
+                                    if (!w_sent)
+                                        tma_load_2d(dst + TL::KPS * A_BYTES + v * TL::B_BYTES, mw, bar, (kb + v) * TBK, n0);
+                                }
                             }
+                            ++issued;
+                            dst += TL::STAGE_BYTES, bar += 8;
+                            if (bar == full0 + 8 * STAGES) dst = ring0, bar = full0, free_parity ^= 1u;
                         }
-                        mma_commit(bar + 8 * STAGES);  // frees the stage when these MMAs have read it
-                        kc += TL::KPS;
-                        const bool last = kb + TL::KPS >= end;
-                        if (LX ? (seg == 1 && last) : (kc == KCHUNK / TBK || last)) {
-                            mma_commit(chunk0 + 8 * (gc & 1));
-                            ++gc;
-                            kc = 0;
+                        if (s_abort) break;
+                    }
+                }
+            }
+        } else if (warp == 1) {
+            // ---------------- MMA issuer ----------------
+            // Its loop is what a k-block costs when it is longer than the MMAs themselves: four MMAs issue in
+            // about 230 cycles (a floor for N <= 128; 521 at N = 256), a commit takes about 250, and everything
+            // else here adds to that. So the descriptors are 32-bit additions to a running low word (the high
+            // word is constant) and the accumulate flag a constant after the first MMA. Probe of the loop
+            // alone, cycles per 64-wide k-block: 761 with descriptors built per MMA and a 64-bit ring counter;
+            // 535 so (N = 128, one k-block a stage), 381 with two k-blocks a stage, 544 at N = 256.
+            if (lane == 0) {
+                const uint32_t desc0 = smem_desc_lo(su32(smem));
+                uint32_t da = desc0, bar = full0;
+                unsigned parity = 0;
+                unsigned gc = 0;  // chunks accumulated by this block
+                for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                    const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
+#pragma unroll
+                    for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
+                        int kb, end;
+                        segment(seg, item, kb, end);
+                        int kc = 0;  // position in the K chunk (chunks hold whole stages)
+                        uint32_t tmem_d = 0;
+                        for (; kb < end; kb += TL::KPS) {
+                            const bool fresh = kc == 0;
+                            if (fresh) {
+                                // kEpiLstmX: x's k-blocks into the buffer's first accumulator, h's into the second
+                                tmem_d = tmem_base + (gc & 1) * TL::ACC_COLS + (LX && seg == 1 ? BN : 0);
+                                if ((!LX || seg == 0) && gc >= 2 &&
+                                    !mb_wait(drained0 + 8 * (gc & 1), ((gc >> 1) - 1) & 1, args.status)) {  // buffer free
+                                    s_abort = 1;
+                                    break;
+                                }
+                            }
+                            if (!mb_wait(bar, parity, args.status)) {
+                                s_abort = 1;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t db = da + ((TL::KPS * A_BYTES) >> 4);
+#pragma unroll
+                            for (int v = 0; v < TL::KPS; ++v) {
+                                if (v > 0 && kb + v >= end) break;
+#pragma unroll
+                                for (int k = 0; k < TBK / 16; ++k) {
+                                    // advance 16 fp16 = 32 bytes along K inside the swizzled 128-byte rows
+                                    const uint32_t x = da + ((v * A_BYTES + 32 * k) >> 4), w = db + ((v * TL::B_BYTES + 32 * k) >> 4);
+                                    if (v == 0 && k == 0)
+                                        mma_f16_lo(tmem_d, x, w, idesc, fresh ? 0u : 1u);
+                                    else
+                                        mma_f16_lo(tmem_d, x, w, idesc, 1u);
+                                }
+                            }
+                            mma_commit(bar + 8 * STAGES);  // frees the stage when these MMAs have read it
+                            kc += TL::KPS;
+                            const bool last = kb + TL::KPS >= end;
+                            if (LX ? (seg == 1 && last) : (kc == KCHUNK / TBK || last)) {
+                                mma_commit(chunk0 + 8 * (gc & 1));
+                                ++gc;
+                                kc = 0;
+                            }
+                            da += TL::STAGE_BYTES >> 4, bar += 8;
+                            if (bar == full0 + 8 * STAGES) da = desc0, bar = full0, parity ^= 1u;
                         }
-                        da += TL::STAGE_BYTES >> 4, bar += 8;
-                        if (bar == full0 + 8 * STAGES) da = desc0, bar = full0, parity ^= 1u;
+                        if (s_abort) break;
                     }
                     if (s_abort) break;
                 }
-                if (s_abort) break;
             }
         }
     } else if constexpr (EPI == kEpiLinear) {
+        if constexpr (TL::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::REGS_EPI));
         // ---------------- epilogue (warps 2..9): recovered product, any K ----------------
         // Each lane owns one output row and one column half of the tile. Every K chunk is drained
         // from tensor memory into int32 running sums in registers; after the last chunk the sums
@@ -525,14 +536,14 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         uint8_t *const stg = smem + STAGES * TL::STAGE_BYTES + (warp - 2) * TL::STG_BYTES;
         ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES + TL::EPI_WARPS * TL::STG_BYTES);
         ColUnit *sunit = reinterpret_cast<ColUnit *>(scol + 2 * BN);
-        const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
+        const int q = hw & 3;                   // tensor-memory lane quarter this warp may read
         const int half = (warp - 2) >> 2;       // column half: [0, BN/2) or [BN/2, BN)
         const int ew = warp - 2;
         const int K = args.K;
         const bool vec = args.Y && (args.ldy % 4 == 0) && ((reinterpret_cast<uintptr_t>(args.Y) & 15) == 0);
         int64_t gc = 0, it = 0;
         bool failed = false;
-        for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
             int64_t m0, n0;
             tile_origin(tile, tiles_m, tiles_n, BN, m0, n0);
             ColConst *cc = scol + (it & 1) * BN;
@@ -601,7 +612,8 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 // outputs then cost a few instructions each (with a 64-bit sum and an IEEE divide apiece the
                 // tile's epilogue outlasts the two K chunks the accumulators can run ahead), and leave through the
                 // warp's staging, 16 columns at a time (stored from registers, a lane its own row: 16384 x 8192 x 8192
-                // 1593 us, so 1527; 9374 x 3033 x 2052, whose rows no 16-byte store fits, 308 us, so 185).
+                // 1593 us, so 1520; 9374 x 3033 x 2052, whose rows no 16-byte store fits, 308 us, so 185; before the
+                // register split above).
                 if (args.Y && cu[c0].unit >= 0 && cu[c0].unit == cu[c0 + 31].unit) {
                     const int zw = cc[c0].zw;
                     const float den = __fmul_rn(Qa, cc[c0].Qw);
@@ -677,6 +689,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         }
         if (lane == 0) bulk_wait();  // (the staging buffers are read until then)
     } else if constexpr (EPI == kEpiRow) {
+        if constexpr (TL::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::REGS_EPI));
         // ---------------- epilogue (warps 2..17): recovered product, one row per lane ----------------
         // Each lane owns one output row; the four warps of a lane quarter take a quarter of its columns
         // each: eq. (1)'s offsets and eq. (3)'s recovery per element. The column constants of the tile are
@@ -685,7 +698,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         uint8_t *const stg = smem + STAGES * TL::STAGE_BYTES + (warp - 2) * TL::STG_BYTES;
         ColConst *scol = reinterpret_cast<ColConst *>(smem + STAGES * TL::STAGE_BYTES + TL::EPI_WARPS * TL::STG_BYTES);
         ColUnit *sunit = reinterpret_cast<ColUnit *>(scol + 2 * BN);
-        const int q = warp & 3;
+        const int q = hw & 3;
         const int part = (warp - 2) >> 2;
         const int ew = warp - 2;
         const int K = args.K;
@@ -694,7 +707,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         // up, the remaining tiles are skipped without waiting.
         int64_t gc = 0;
         bool failed = false;
-        for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
             int64_t m0, n0;
             tile_origin(tile, tiles_m, tiles_n, BN, m0, n0);
             ColConst *cc = scol + (gc & 1) * BN;
@@ -832,12 +845,12 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         // ---------------- epilogue (warps 2..17): split-K partial sums ----------------
         // The item's K range is at most one accumulation chunk, so its fp32 accumulator holds the
         // exact integer sum of centered products; each lane stores its row's 16-column blocks.
-        const int q = warp & 3;
+        const int q = hw & 3;
         const int part = (warp - 2) >> 2;
         int64_t gc = 0;
         bool ok = true;
         const bool vec = args.ldpart % 4 == 0;
-        for (int64_t item = blockIdx.x; item < items && ok; item += gridDim.x, ++gc) {
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++gc) {
             int64_t m0, n0;
             item_origin(item / splits, m0, n0);
             int32_t *dst = args.part + (item % splits) * args.M * args.ldpart;
@@ -872,6 +885,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             if (lane == 0) mb_arrive(drained0 + 8 * buf);
         }
     } else {
+        if constexpr (TL::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::REGS_EPI));
         // ---------------- epilogue: LSTM cell update ----------------
         // Column n of the tile is gate g = (n % 32) / 8 of cell 8 * (n / 32) + n % 8. Each lane owns
         // one batch row; the warps of a lane quarter take slices of CPS cells in turn, reading the
@@ -880,7 +894,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         constexpr int CPS = TL::CPS;
         constexpr int SLICES = BN / (4 * CPS);   // slices per tile
         constexpr int SPG = 8 / CPS;             // slices per 8-cell group
-        const int q = warp & 3;
+        const int q = hw & 3;
         const int eh = (warp - 2) >> 2;
         const int K = args.K;
         const TcLstmOut &E = args.lstm;
@@ -943,7 +957,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         float Qa = 1.0f, Qx = 1.0f;
         // kEpiLstmX: every warp runs every tile (the quarter's barriers count on it); after a wait gave up
         // the remaining tiles are skipped without waiting
-        for (int64_t tile = blockIdx.x; tile < work && (LX || ok); tile += gridDim.x) {
+        for (int tile = blockIdx.x; tile < work && (LX || ok); tile += gridDim.x) {
             int64_t m0, n0;
             const bool half = item_origin(tile, m0, n0);
             const int slices = half ? SLICES / 2 : SLICES;  // half-width items: half the slices
@@ -1123,9 +1137,9 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                         st_vec(E.c + b * (int64_t)H + j0, cst);
                         st_vec(E.h + b * E.h_ld + j0, mst);
                     }
-                    if (s == eh && issuer && gc > 0 && tile + (int64_t)gridDim.x < work &&
+                    if (s == eh && issuer && gc > 0 && tile + (int)gridDim.x < work &&
                         mb_wait(pxempty0 + 8 * (pbuf ^ 1), (unsigned)((gc - 1) / 2) & 1, args.status))
-                        issue_px(tile + (int64_t)gridDim.x, pbuf ^ 1);
+                        issue_px(tile + (int)gridDim.x, pbuf ^ 1);
                     continue;
                 }
                 uint32_t r[4][CPS];
@@ -1201,9 +1215,9 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 }
             }
             // refill the buffer with the tile two ahead once every epilogue warp has released it
-            if (!LX && issuer && tile + 2 * (int64_t)gridDim.x < work &&
+            if (!LX && issuer && tile + 2 * (int)gridDim.x < work &&
                 mb_wait(pxempty0 + 8 * pbuf, (unsigned)(gc / 2) & 1, args.status))
-                issue_px(tile + 2 * (int64_t)gridDim.x, pbuf);
+                issue_px(tile + 2 * (int)gridDim.x, pbuf);
             ++gc;
         }
         if (LX && lane == 0) bulk_wait();
@@ -1397,6 +1411,7 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
         configured = dev;
     }
     const int64_t items = ((a.M + TBM - 1) / TBM) * ((a.N + BN - 1) / BN) * a.splits;  // (tile, K range) pairs
+    if (items > INT32_MAX / 4) return QNN_FAIL(QNN_ERR_INVALID_ARG);
     // persistent: one block per SM (a block holding tensor memory has its SM to itself)
     const int64_t blocks = op.max_blocks > 0 ? std::min(op.max_blocks, sm_count()) : sm_count();
     const unsigned grid = (unsigned)std::min<int64_t>(items, blocks);
