@@ -26,6 +26,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "qnn_device.cuh"
@@ -36,6 +37,7 @@
 namespace qnn {
 namespace {
 
+constexpr int kPairBn = 512;  // the width by which callers name kEpiPair's tiles
 constexpr int TBM = 128, TBK = 64;               // rows of A per tile; fp16 elements per k-block (128 bytes)
 constexpr int A_BYTES = TBM * TBK * 2;            // 16 KB
 constexpr int KCHUNK = 1024;                      // exact fp32 accumulation bound (see above)
@@ -48,7 +50,9 @@ constexpr unsigned long long TC_WAIT_NS = 2000000000ull;
 // those HBM loads delay the tile's TMA stream.)
 // kEpiPartial: split-K, each work item (tile, K range of at most 1024) stores its exact centered
 // integer sums P as int32 into its own slice of a partial-sum buffer; a consumer adds the slices.
-enum Epilogue { kEpiLinear = 0, kEpiLstm = 1, kEpiRow = 2, kEpiPartial = 4, kEpiLstmX = 5 };
+// kEpiPair: kEpiLinear on tiles of 256 x 256 by pairs of blocks (cta_group::2), a block 128 rows of A, half of
+// the tile's rows of W and the outputs of its rows.
+enum Epilogue { kEpiLinear = 0, kEpiLstm = 1, kEpiRow = 2, kEpiPartial = 4, kEpiLstmX = 5, kEpiPair = 6 };
 
 struct ColConst {  // per-output-column constants of kEpiRow, staged in shared memory per tile
     int cs, zw;
@@ -67,21 +71,22 @@ struct ColUnit {  // and the weight unit of each column (-1 past N)
 // tensor-memory lane quarter); eighteen to twenty warps fit the register file at 96 registers a thread.
 template <int BN, int EPI>
 struct Tile {
-    static_assert(EPI == kEpiLinear || BN <= 128, "row and LSTM epilogues take tiles of at most 128 columns");
+    static constexpr bool PAIR = EPI == kEpiPair, LINEAR = EPI == kEpiLinear || PAIR;
+    static_assert(LINEAR || BN <= 128, "row and LSTM epilogues take tiles of at most 128 columns");
     // a 96-column LSTM tile has six 4-cell slices per lane quarter: 24 epilogue warps, one slice each
     // kEpiLstmX: the LSTM step with the input product fused in (a second operand pair and accumulator)
     static constexpr bool IS_LSTM = EPI == kEpiLstm || EPI == kEpiLstmX;
     static constexpr bool LSTM96 = IS_LSTM && BN == 96;
-    static constexpr int EPI_WARPS = EPI == kEpiLinear ? 8 : (LSTM96 ? 24 : 16);
+    static constexpr int EPI_WARPS = LINEAR ? 8 : (LSTM96 ? 24 : 16);
     // LSTM: cells per epilogue slice (a 32-column tile has 8 cells: 2-cell slices keep 4 warps busy)
     static constexpr int CPS = BN == 32 ? 2 : 4;
     // SPLIT: the epilogue warps come first and the two issuing ones after them, in a warpgroup of their own that
     // leaves most of its registers to the epilogue's. (At the registers an even share leaves a thread the
     // epilogues spill, and their reloads go through the same port as the operands: 16384 x 8192 x 8192 1521 us,
     // so 1421; 9374 x 3032 x 2052 142 and 128; LSTMP 5 x 2048p512, B = 1024, 100 frames 20.35 and 19.88 ms.)
-    static constexpr bool SPLIT = EPI == kEpiLinear || EPI == kEpiRow || (IS_LSTM && !LSTM96);
+    static constexpr bool SPLIT = LINEAR || EPI == kEpiRow || (IS_LSTM && !LSTM96);
     static constexpr int THREADS = 32 * ((SPLIT ? 4 : 2) + EPI_WARPS);
-    static constexpr int B_BYTES = BN * TBK * 2;
+    static constexpr int B_BYTES = BN / (PAIR ? 2 : 1) * TBK * 2;
     // a pipeline stage carries KPS consecutive k-blocks (A sub-tiles first, then the W sub-tiles):
     // the operand stream advances by stages at a pace that hardly depends on their size, so short
     // reductions (K <= 1024) take several k-blocks a stage: four for narrow LSTM tiles (two stages in
@@ -93,7 +98,7 @@ struct Tile {
                                                : ((EPI == kEpiPartial || EPI == kEpiRow) ? 2 : 1);
     static constexpr int SUB_BYTES = A_BYTES + B_BYTES;
     static constexpr int STAGE_BYTES = KPS * SUB_BYTES;
-    static constexpr int BASE_STAGES = EPI == kEpiLinear    ? (BN == 256 ? 4 : 6)
+    static constexpr int BASE_STAGES = LINEAR               ? (BN == 256 && !PAIR ? 4 : 6)
                                        : EPI == kEpiPartial ? 6  // one K range per item: keep it all in flight
                                                             : (BN == 128 ? 4 : 6);
     // LSTM: the tile's input products px (4 gates x 128 rows x BN/4 cells) and cell state c (128 x
@@ -109,9 +114,9 @@ struct Tile {
     // [4 gates][32 rows] float4 (1/dx, 1/dh, rt_x, rt_h), then [4 gates][32 rows] float2 (dx, dh)
     static constexpr int OUT_BYTES = EPI == kEpiLstmX ? PX_BOX : 0;
     static constexpr int RC_BYTES = EPI == kEpiLstmX ? 4 * 24 * 32 * 4 : 0;
-    // kEpiRow, kEpiLinear: each epilogue warp's staging of outputs, 32 rows x ROW_COLS fp32 columns
+    // kEpiRow, kEpiLinear, kEpiPair: each epilogue warp's staging of outputs, 32 rows x ROW_COLS fp32 columns
     static constexpr int ROW_COLS = EPI == kEpiRow ? BN / 4 : 16;
-    static constexpr int STG_BYTES = EPI == kEpiRow || EPI == kEpiLinear ? 32 * ROW_COLS * 4 : 0;
+    static constexpr int STG_BYTES = EPI == kEpiRow || LINEAR ? 32 * ROW_COLS * 4 : 0;
     static constexpr int EPI_BYTES = IS_LSTM              ? 2 * LSTM_BUF + OUT_BYTES + RC_BYTES
                                      : EPI == kEpiPartial ? 0
                                                           : 2 * BN * (int)(sizeof(ColConst) + sizeof(ColUnit)) +
@@ -127,11 +132,11 @@ struct Tile {
                            : (2 * ACC_COLS <= 64 ? 64 : (2 * ACC_COLS <= 128 ? 128 : (2 * ACC_COLS <= 256 ? 256 : 512)));
     // warps sit on the four SM sub-partitions by index: 18 warps put 5 on one (5 x 32 x 96 <= 16384),
     // 26 warps put 7 on one (7 x 32 x 72 <= 16384)
-    static constexpr int MAX_REGS = EPI == kEpiLinear ? 168 : (LSTM96 ? 72 : 96);
+    static constexpr int MAX_REGS = LINEAR ? 168 : (LSTM96 ? 72 : 96);
     // SPLIT: per warpgroup, EPI_WARPS / 4 REGS_EPI + REGS_ISSUE <= (EPI_WARPS / 4 + 1) MAX_REGS
     static constexpr int REGS_ISSUE = 32, REGS_EPI = EPI_WARPS == 8 ? 232 : 112;
     static_assert(!SPLIT || EPI_WARPS / 4 * REGS_EPI + REGS_ISSUE <= (EPI_WARPS / 4 + 1) * MAX_REGS, "registers of the block");
-    static constexpr uint32_t IDESC = mma_idesc_f16(TBM, BN);
+    static constexpr uint32_t IDESC = mma_idesc_f16(PAIR ? 2 * TBM : TBM, BN);
     static constexpr uint32_t IDESC_HALF = mma_idesc_f16(TBM, BN / 2 >= 16 ? BN / 2 : 16);  // half-width items
     static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + EPI_BYTES + 256;
 };
@@ -169,7 +174,7 @@ struct TcArgs {
     const int32_t *csW_x;
     const float *bias_x;
     int K_x, KB_x;
-    int y_map;  // kEpiRow, kEpiLinear: mapPX is a map of Y for TMA stores
+    int y_map;  // kEpiRow, kEpiLinear, kEpiPair: mapPX is a map of Y for TMA stores
     // LSTM epilogues: tiles from full_tiles on (the last, partial wave of the persistent grid) run as
     // two half-width items each, so that the blocks of that wave finish together (0: none)
     int64_t full_tiles;
@@ -309,10 +314,13 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     // roles by `warp`: 0 producer, 1 MMA issuer, 2 .. EPI_WARPS + 1 epilogue (tensor-memory lane quarter hw & 3)
     const int hw = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int warp = !TL::SPLIT || hw >= TL::EPI_WARPS + 2 ? hw : hw < TL::EPI_WARPS ? hw + 2 : hw - TL::EPI_WARPS;
-    constexpr bool LX = EPI == kEpiLstmX;
+    constexpr bool LX = EPI == kEpiLstmX, PAIR = TL::PAIR;
+    // blocks working on one item, this block's place among them, the first item and the step to the next
+    constexpr int TEAM = PAIR ? 2 : 1;
+    const int rank = PAIR ? (int)cluster_rank() : 0, first_item = blockIdx.x / TEAM, item_step = gridDim.x / TEAM;
     const int nchunks = (args.KB + KCHUNK / TBK - 1) / (KCHUNK / TBK);  // K chunks of a tile (kEpiLinear)
     const int tiles_n = (int)((args.N + BN - 1) / BN);
-    const int tiles_m = (int)((args.M + TBM - 1) / TBM);
+    const int tiles_m = (int)((args.M + TEAM * TBM - 1) / (TEAM * TBM));
     const int tiles = tiles_m * tiles_n;
     // work items: (tile, K range); one K range per tile except for split-K. LSTM epilogues may split
     // the tiles of the last wave into half-width items (the first BN / 2 columns of the tile's W box
@@ -325,6 +333,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
     auto item_origin = [&](int w, int64_t &m0, int64_t &n0) -> bool {
         if (w < full_tiles) {
             tile_origin(w, tiles_m, tiles_n, BN, m0, n0);
+            if (PAIR) m0 = 2 * m0 + TBM * rank;
             return false;
         }
         const int j = w - full_tiles;
@@ -348,7 +357,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         }
         for (int i = 0; i < 2; ++i) {
             mb_init(chunk0 + 8 * i, 1);      // MMA -> epilogue: chunk accumulated in buffer i
-            mb_init(drained0 + 8 * i, TL::EPI_WARPS);  // epilogue -> MMA: buffer i read out by every epilogue warp
+            mb_init(drained0 + 8 * i, TEAM * TL::EPI_WARPS);  // epilogue -> MMA: buffer i read out by every epilogue warp
             mb_init(pxfull0 + 8 * i, 1);
             mb_init(pxempty0 + 8 * i, LX ? 4 : TL::EPI_WARPS);  // by epilogue warp, or row quarter (LX)
         }
@@ -356,13 +365,21 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {  // allocate the two accumulators
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                     "n"(TL::TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
+                         "n"(TL::TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
+                         "n"(TL::TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();  // the other block's barriers and tensor memory are there too
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
     // Static weights: the producer starts the W tiles of its first stages before the wait below
@@ -379,7 +396,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapAX)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapWX)) : "memory");
         }
-        if (args.w_static && blockIdx.x < items) {
+        if (!PAIR && args.w_static && blockIdx.x < items) {
             int64_t m0, n0;
             item_origin(blockIdx.x / splits, m0, n0);
 #pragma unroll
@@ -421,7 +438,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 uint32_t dst = ring0, bar = full0;
                 unsigned free_parity = 1;
                 int issued = 0;
-                for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                for (int item = first_item; item < items && !s_abort; item += item_step) {
                     int64_t m0l, n0l;
                     item_origin(item / splits, m0l, n0l);
                     const int m0 = (int)m0l, n0 = (int)n0l;
@@ -438,7 +455,13 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                             }
                             const int nv = min(TL::KPS, end - kb);   // k-blocks in this stage (the last may be short)
                             const bool w_sent = issued < w_early;    // W already on its way (expect set with it)
-                            if (issued >= full_early) {              // (else issued whole before the wait)
+                            if constexpr (PAIR) {
+                                // both blocks' loads count on the even one's barrier
+                                if (rank == 0) mb_expect(bar, 2 * TL::SUB_BYTES);
+                                const uint32_t at = cluster_addr(bar, 0);
+                                tma_load_2d_pair(dst, ma, at, kb * TBK, m0);
+                                tma_load_2d_pair(dst + A_BYTES, mw, at, kb * TBK, n0 + BN / 2 * rank);
+                            } else if (issued >= full_early) {       // (else issued whole before the wait)
                                 if (!w_sent) mb_expect(bar, (uint32_t)(nv * TL::SUB_BYTES));
 #pragma unroll
                                 for (int v = 0; v < TL::KPS; ++v) {
@@ -455,6 +478,18 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                         if (s_abort) break;
                     }
                 }
+                // a pair's slots are freed by the even block: none of its arrivals is under way when this one leaves
+                if (PAIR && !s_abort) {
+                    if (issued < STAGES) bar = full0, free_parity = 0;
+                    for (int i = min(issued, STAGES); i > 0; --i) {
+                        if (!mb_wait(bar + 8 * STAGES, free_parity, args.status)) {
+                            s_abort = 1;
+                            break;
+                        }
+                        bar += 8;
+                        if (bar == full0 + 8 * STAGES) bar = full0, free_parity ^= 1u;
+                    }
+                }
             }
         } else if (warp == 1) {
             // ---------------- MMA issuer ----------------
@@ -464,12 +499,12 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             // word is constant) and the accumulate flag a constant after the first MMA. Probe of the loop
             // alone, cycles per 64-wide k-block: 761 with descriptors built per MMA and a 64-bit ring counter;
             // 535 so (N = 128, one k-block a stage), 381 with two k-blocks a stage, 544 at N = 256.
-            if (lane == 0) {
+            if (lane == 0 && rank == 0) {
                 const uint32_t desc0 = smem_desc_lo(su32(smem));
                 uint32_t da = desc0, bar = full0;
                 unsigned parity = 0;
                 unsigned gc = 0;  // chunks accumulated by this block
-                for (int item = blockIdx.x; item < items && !s_abort; item += gridDim.x) {
+                for (int item = first_item; item < items && !s_abort; item += item_step) {
                     const uint32_t idesc = item / splits < full_tiles ? TL::IDESC : TL::IDESC_HALF;
 #pragma unroll
                     for (int seg = LX ? 0 : 1; seg < 2; ++seg) {
@@ -501,17 +536,26 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                                 for (int k = 0; k < TBK / 16; ++k) {
                                     // advance 16 fp16 = 32 bytes along K inside the swizzled 128-byte rows
                                     const uint32_t x = da + ((v * A_BYTES + 32 * k) >> 4), w = db + ((v * TL::B_BYTES + 32 * k) >> 4);
-                                    if (v == 0 && k == 0)
+                                    if constexpr (PAIR)
+                                        mma_f16_lo_pair(tmem_d, x, w, idesc, v == 0 && k == 0 && fresh ? 0u : 1u);
+                                    else if (v == 0 && k == 0)
                                         mma_f16_lo(tmem_d, x, w, idesc, fresh ? 0u : 1u);
                                     else
                                         mma_f16_lo(tmem_d, x, w, idesc, 1u);
                                 }
                             }
-                            mma_commit(bar + 8 * STAGES);  // frees the stage when these MMAs have read it
+                            // frees the stage when these MMAs have read it
+                            if constexpr (PAIR)
+                                mma_commit_pair(bar + 8 * STAGES);
+                            else
+                                mma_commit(bar + 8 * STAGES);
                             kc += TL::KPS;
                             const bool last = kb + TL::KPS >= end;
                             if (LX ? (seg == 1 && last) : (kc == KCHUNK / TBK || last)) {
-                                mma_commit(chunk0 + 8 * (gc & 1));
+                                if constexpr (PAIR)
+                                    mma_commit_pair(chunk0 + 8 * (gc & 1));
+                                else
+                                    mma_commit(chunk0 + 8 * (gc & 1));
                                 ++gc;
                                 kc = 0;
                             }
@@ -524,7 +568,7 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 }
             }
         }
-    } else if constexpr (EPI == kEpiLinear) {
+    } else if constexpr (TL::LINEAR) {
         if constexpr (TL::SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::REGS_EPI));
         // ---------------- epilogue (warps 2..9): recovered product, any K ----------------
         // Each lane owns one output row and one column half of the tile. Every K chunk is drained
@@ -543,9 +587,9 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         const bool vec = args.Y && (args.ldy % 4 == 0) && ((reinterpret_cast<uintptr_t>(args.Y) & 15) == 0);
         int64_t gc = 0, it = 0;
         bool failed = false;
-        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+        for (int tile = first_item; tile < tiles; tile += item_step, ++it) {
             int64_t m0, n0;
-            tile_origin(tile, tiles_m, tiles_n, BN, m0, n0);
+            item_origin(tile, m0, n0);
             ColConst *cc = scol + (it & 1) * BN;
             ColUnit *cu = sunit + (it & 1) * BN;
             for (int c = ew * 32 + lane; c < BN; c += 32 * TL::EPI_WARPS) {
@@ -591,7 +635,12 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mb_arrive(drained0 + 8 * buf);
+                if (lane == 0) {
+                    if constexpr (PAIR)
+                        mb_arrive_cluster(cluster_addr(drained0 + 8 * buf, 0));
+                    else
+                        mb_arrive(drained0 + 8 * buf);
+                }
             }
             const int64_t m = m0 + 32 * q + lane;
             if (failed || m0 + 32 * q >= args.M) continue;
@@ -1232,10 +1281,16 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
         while (gtime() - t0 < 4000000ull) __nanosleep(1000);
     }
     __syncthreads();
+    __syncwarp();
+    if constexpr (PAIR) cluster_sync();  // neither block leaves, or frees its tensor memory, before the other is done
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(TL::TMEM_COLS)
-                     : "memory");
+        if constexpr (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(TL::TMEM_COLS)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(TL::TMEM_COLS)
+                         : "memory");
     }
 }
 
@@ -1391,6 +1446,7 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
                      const CUtensorMap *map_h = nullptr) {
     using TL = Tile<BN, EPI>;
     static int configured = -1;
+    static std::atomic<int> pairs{0};
     int dev = 0;
     QNN_CUDA_TRY(cudaGetDevice(&dev));
     if (configured != dev) {
@@ -1408,13 +1464,26 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
                          fa.maxThreadsPerBlock, fa.numRegs, fa.sharedSizeBytes, TL::SMEM, fa.localSizeBytes, n);
         }
         if (n < 1) return QNN_FAIL(QNN_ERR_CUDA);
+        if (TL::PAIR) {  // pairs of blocks that fit the device at once
+            cudaLaunchConfig_t c = {};
+            c.gridDim = dim3(2 * sm_count()), c.blockDim = dim3(TL::THREADS), c.dynamicSmemBytes = TL::SMEM;
+            cudaLaunchAttribute cl[1];
+            cl[0].id = cudaLaunchAttributeClusterDimension;
+            cl[0].val.clusterDim.x = 2, cl[0].val.clusterDim.y = cl[0].val.clusterDim.z = 1;
+            c.attrs = cl, c.numAttrs = 1;
+            int np = 0;
+            QNN_CUDA_TRY(cudaOccupancyMaxActiveClusters(&np, qgemm_tc_kernel<BN, EPI>, &c));
+            if (np < 1) return QNN_FAIL(QNN_ERR_CUDA);
+            pairs.store(np);
+        }
         configured = dev;
     }
-    const int64_t items = ((a.M + TBM - 1) / TBM) * ((a.N + BN - 1) / BN) * a.splits;  // (tile, K range) pairs
+    constexpr int TEAM = TL::PAIR ? 2 : 1;
+    const int64_t items = ((a.M + TEAM * TBM - 1) / (TEAM * TBM)) * ((a.N + BN - 1) / BN) * a.splits;  // (tile, K range) pairs
     if (items > INT32_MAX / 4) return QNN_FAIL(QNN_ERR_INVALID_ARG);
     // persistent: one block per SM (a block holding tensor memory has its SM to itself)
-    const int64_t blocks = op.max_blocks > 0 ? std::min(op.max_blocks, sm_count()) : sm_count();
-    const unsigned grid = (unsigned)std::min<int64_t>(items, blocks);
+    const int64_t blocks = TL::PAIR ? 2 * pairs.load() : op.max_blocks > 0 ? std::min(op.max_blocks, sm_count()) : sm_count();
+    const unsigned grid = (unsigned)std::min<int64_t>(TEAM * items, blocks);
     // LSTM tiles of 64 or 128 columns: when the last wave is partial and its tiles, halved, fit one
     // wave, they run as two half-width items each (the busiest block then does half a tile less;
     // QNN_TC_HALF=0 keeps whole tiles)
@@ -1432,10 +1501,15 @@ qnn_status launch_tc(const TcOperands &op, const TcArgs &a, const char *name, cu
     cfg.dynamicSmemBytes = TL::SMEM;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    if (TL::PAIR) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2, attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = op.pdl ? 1 : 0;
+    cfg.numAttrs = op.pdl || TL::PAIR ? 1 : 0;
     // the px, c, x, Wx and output maps are read by the LSTM kernels only (the others get A's map, unused)
     QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, qgemm_tc_kernel<BN, EPI>, op.a, op.w, map_px ? *map_px : op.a,
                                     map_c ? *map_c : op.a, map_ax ? *map_ax : op.a, map_wx ? *map_wx : op.w, map_h ? *map_h : op.a, args));
@@ -1461,6 +1535,7 @@ qnn_status dispatch_linear(const TcOperands &op, const TcArgs &a, cudaStream_t s
         case 64: return launch_tc<64, kEpiLinear>(op, r, "qgemm_tc", st, my);
         case 128: return launch_tc<128, kEpiLinear>(op, r, "qgemm_tc", st, my);
         case 256: return launch_tc<256, kEpiLinear>(op, r, "qgemm_tc", st, my);
+        case kPairBn: return launch_tc<256, kEpiPair>(op, r, "qgemm_tc", st, my);
         default: return QNN_ERR_INVALID_ARG;
     }
 }
@@ -1523,8 +1598,14 @@ int tc_pick_bn(int64_t M, int64_t N, int64_t kp) {
     if (kp > KCHUNK) {  // chunked drains: the widest tile whose tiles fill three quarters of the SMs
         if (const char *e = std::getenv("QNN_TC_BN")) {
             const int v = std::atoi(e);
-            if (v == 64 || v == 128 || v == 256) return v;
+            if (v == 64 || v == 128 || v == 256 || v == kPairBn) return v;
         }
+        // the largest products by pairs of blocks: a block's operand traffic in shared memory, 768 cycles a
+        // k-block of 128 x 256, becomes 512. Long reductions only, where a tile's start and end do not count, and
+        // seven rounds of tiles, where the last one does not (16384 x 8192 x 8192: 1419 us by single blocks, 1349 by
+        // pairs; 8192 x 8192 x 5000 485 and 467, x 4096 390 and 386, x 3000 300 and 298; 4096 x 4096 x 4096 130
+        // and 131; 2048 x 8192 x 2048 81 and 84)
+        if (kp >= 4096 && ((M + 255) / 256) * ((N + 255) / 256) >= 512) return kPairBn;
         const int64_t mt = (M + TBM - 1) / TBM;
         for (int bn : {256, 128})
             if (4 * mt * ((N + bn - 1) / bn) >= 3 * (int64_t)sm_count()) return bn;
@@ -1535,10 +1616,10 @@ int tc_pick_bn(int64_t M, int64_t N, int64_t kp) {
 }
 
 qnn_status tc_operands(TcOperands *op, const __half *A16, int64_t M, const __half *W16, int64_t N, int64_t kp, int bn) {
-    if (bn != 32 && bn != 64 && bn != 96 && bn != 128 && bn != 256) return QNN_ERR_INVALID_ARG;
+    if (bn != 32 && bn != 64 && bn != 96 && bn != 128 && bn != 256 && bn != kPairBn) return QNN_ERR_INVALID_ARG;
     if (kp <= 0 || kp % TBK != 0 || M <= 0 || N <= 0) return QNN_ERR_INVALID_ARG;
     QNN_TRY(make_map(&op->a, A16, M, kp, TBM));
-    QNN_TRY(make_map(&op->w, W16, N, kp, bn));
+    QNN_TRY(make_map(&op->w, W16, N, kp, bn == kPairBn ? 128 : bn));
     op->M = M, op->N = N, op->kp = kp, op->bn = bn, op->pdl = false;
     op->row_epilogue = kp <= KCHUNK && (bn == 64 || bn == 128);
     return QNN_OK;

@@ -14,7 +14,7 @@
 namespace qnn {
 
 // The two operands of one product, as TMA tensor maps: A [M][kp] and W [N][kp]. `bn` is the tile
-// width (rows of W per tile: 32, 64, 128 or 256; the LSTM epilogue takes 32, 64 or 128, the row
+// width (rows of W per tile: 32, 64, 128 or 256, or 512 for tiles of 256 x 256 by pairs of blocks; the LSTM epilogue takes 32, 64 or 128, the row
 // epilogue 64 or 128); the maps depend on
 // it. With `pdl` set the product is launched as a programmatic dependent launch: its block setup
 // may overlap the previous kernel of the stream (it waits for that kernel before reading).

@@ -86,7 +86,7 @@ def test_float_output_layer_tiles(qnn, B, T, H, C):
 # The tensor-core product's outputs without raw sums: K <= 1024 stores them by TMA from staging buffers
 # (whole units, ragged rows and columns, rows further apart than N, unaligned rows by plain stores), longer K
 # whole blocks of 32 columns in 32-bit sums; offsets beyond the fp32 and the 32-bit forms take the others.
-@pytest.mark.parametrize("bn", ["64", "128", "256"])
+@pytest.mark.parametrize("bn", ["64", "128", "256", "512"])
 @pytest.mark.parametrize("M,N,K,pad", [(1, 8, 1, 0), (33, 64, 64, 0), (128, 256, 64, 4), (130, 260, 100, 0), (257, 2000, 500, 8),
                                        (200, 136, 1000, 1), (384, 512, 1024, 0), (129, 260, 1025, 0), (257, 320, 3000, 4), (140, 261, 1100, 0),
                                        (260, 515, 2100, 1), (161, 163, 300, 0)])
