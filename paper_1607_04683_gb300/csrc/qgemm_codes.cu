@@ -13,10 +13,10 @@
 // of one row of A are 32 consecutive floats. BN = 64 while those tiles are one wave, else 128.
 //
 // Bound: the shared-memory port (a 128 x 128 k-block loads 16 KB of codes, stores 32 KB and has the MMAs read
-// 32 KB: 640 clk at 128 bytes a clk) and the latencies around it. M = 256, 8192 x 8192: 83 us, 1200 clk a
+// 32 KB: 640 clk at 128 bytes a clk) and the latencies around it. M = 256, 8192 x 8192: 72 us, 1050 clk a
 // k-block; 132 us with eight converting warps and k-blocks one by one (each then waits, converts and loads in
 // turn), 148 us when a test of the matrix's ends stood before every load (nothing stayed in flight). The
-// centering pass and the fp16 product take 46 + 55 us there. M = 256, 2048 x 2048: 28.8 us, so 18.3.
+// centering pass and the fp16 product take 37 + 54 us there. M = 256, 2048 x 2048: 20.6 us, so 17.8.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -32,7 +32,7 @@ namespace {
 
 constexpr int kRowsW = 128, kBK = 64, kKps = 2;  // W rows of a tile, codes of a k-block, k-blocks of a stage
 constexpr int kChunk = 1024 / (kKps * kBK);      // stages of a chunk
-constexpr int kConv = 16, kThreads = 32 * (kConv + 1);
+constexpr int kConv = 16, kThreads = 32 * (kConv + 4);  // (three warps only complete the issuing warpgroup)
 constexpr int kStages = 3;
 constexpr unsigned long long kWaitNs = 2000000000ull;
 
@@ -99,7 +99,9 @@ __device__ __noinline__ uint4 edge_unit(const uint8_t *p, const uint8_t *lo, con
 template <int BN>
 struct CodesTile {
     static constexpr int THREADS = kThreads;
-    static constexpr int MAX_REGS = 96;  // five of the warps share a sub-partition: 5 x 32 x 96 <= 16384
+    // 96 registers a thread at launch; the issuing warpgroup leaves its to the four converting ones, which spill
+    // at 96 (M = 256, 8192 x 8192: 83 us, so 72)
+    static constexpr int MAX_REGS = 96, REGS_CONV = 112, REGS_ISSUE = 32;
     static constexpr int SUB = (kRowsW + BN) * kBK * 2, STAGE = kKps * SUB;  // bytes of a k-block and a stage
     static constexpr size_t SMEM = (size_t)kStages * STAGE + 1024;
 };
@@ -155,8 +157,9 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
                (!*reinterpret_cast<volatile int *>(&s_abort) && mbar_wait_bounded(bar, parity, a.status, kWaitNs));
     };
 
-    if (warp == kConv) {
-        if (lane == 0) {
+    if (warp >= kConv) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CodesTile<BN>::REGS_ISSUE));
+        if (warp == kConv && lane == 0) {
             constexpr uint32_t idesc = mma_idesc_f16(kRowsW, BN);
             const uint32_t desc0 = smem_desc_lo(su32(smem));
             uint32_t d = desc0, bar = full0, tmem_d = tmem_base;
@@ -195,6 +198,7 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
             }
         }
     } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CodesTile<BN>::REGS_CONV));
         // lane (r, c): codes 16 c .. 16 c + 15 of every k-block of row r of W and of A; rows past the end repeat
         // the last one (their sums are dropped)
         const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
