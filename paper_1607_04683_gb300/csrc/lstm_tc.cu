@@ -629,13 +629,21 @@ qnn_status tc_layer_begin(TcLayerRun &s, const float *h0, void *work, const TcFu
     // The fused kernel's operand stream (A re-read for every tile of a block) is bounded by the rate at
     // which a block's TMA ring turns over, so with at least a full wave of tiles the widest tile wins
     // (LSTMP 5x2048p512 B=1024: 128 columns 49.6 us per step against 52.0 for 64); with less than a
-    // wave the tile count that fills the SMs best decides, except in a wavefront, where the other
-    // layers' kernels fill the SMs a narrow grid leaves: there the widest tile always wins (5 x 500
-    // B = 256: 32 blocks of 128 columns 8.9M frames/s, 64 of 64 columns 8.5M, 126 of 32 columns 6.0M).
+    // wave the tile count that fills the SMs best decides. In a wavefront the other layers' kernels fill
+    // the SMs a grid leaves, and a wide tile's columns cost the fewest operand bytes; but a narrow one has
+    // the shorter epilogue in every step's chain, which counts while the tiles of all layers find SMs at
+    // once (30 frames, us, 128 against 64 columns: 2 x 800 B = 256, 200 tiles of 64, 826 : 696; 3 x 1000
+    // B = 128, 189, 899 : 789; 2 x 512p128 B = 64, 64, 728 : 658 and 639 with 32 columns; but 2 x 2048p512
+    // B = 64, 256, 956 : 974; 3 x 1024p256 B = 200, 384, 1064 : 1136).
     int bn_gates = fx ? tc_choose_bn(B, 4 * H8, gate_bn_fused, 3) : tc_choose_bn(B, 4 * H8, gate_bn, 4);
-    if (fx && !std::getenv("QNN_TC_BN") &&
-        (s.wave || ((B + 127) / 128) * ((4 * H8 + 127) / 128) >= sm_count()))
-        bn_gates = 128;
+    if (fx && !std::getenv("QNN_TC_BN")) {
+        const int64_t mt = (B + 127) / 128, sms = sm_count();
+        auto all = [&](int64_t bn) { return m->L * mt * ((4 * H8 + bn - 1) / bn); };  // tiles of a step of every layer
+        if (s.wave)
+            bn_gates = all(32) <= sms ? 32 : 3 * all(64) <= 4 * sms ? 64 : 128;
+        else if (mt * ((4 * H8 + 127) / 128) >= sms)
+            bn_gates = 128;
+    }
     QNN_TRY(tc_operands(&s.gates, s.a16, B, tl.wh16, 4 * H8, kh, bn_gates));
     // the projection after the m_t quantizer: split-K partial sums finished (offsets, recovery, next
     // step's quantization) by one row kernel; or one tcgen05 product with its own epilogue per step

@@ -172,3 +172,19 @@ def test_centered_operands(qnn, M, N, K, pad, off, monkeypatch):
                              qnn.params_tensor(pw), gpu(cs), want_acc=True)
     assert qnn.device_status() == qnn.QNN_OK
     assert np.array_equal(acc.cpu().numpy(), ref["acc"])
+
+
+# Gate tiles of 32, 64 and 128 columns in a wavefront of layers, by the tiles of all layers.
+@pytest.mark.parametrize("L,H,P,B", [(2, 512, 128, 70), (3, 512, 64, 130), (3, 520, 0, 260), (2, 1024, 128, 300)])
+def test_gate_tiles_of_a_wavefront(qnn, L, H, P, B, monkeypatch):
+    from paper_1607_04683_gb300 import inputs
+    monkeypatch.setenv("QNN_LSTM_PATH", "tc")
+    wl = inputs.LstmWorkload("wave", seed=L + H + B, num_layers=L, input_dim=20, hidden=H, proj=P, num_classes=0, batch=B,
+                             frames=3, w_range=0.08, forget_bias=1.0, output_mode=0)
+    params, x = wl.make()
+    model = qnn.LstmModel(qnn.lstm_desc(L, 20, H, P, 0), gpu(params))
+    y = model.forward(gpu(x))
+    assert qnn.device_status() == qnn.QNN_OK
+    b = [0, 63, B // 2, B - 1]
+    ref = oracle.lstm_forward(oracle.desc(L, 20, H, P, 0, oracle.OUT_NONE), params, np.ascontiguousarray(x[b]), want_h_all=True)
+    assert np.array_equal(y.cpu().numpy()[b], ref["h_all"][-1])
