@@ -453,6 +453,15 @@ def run_ours(args, wl, rank, world, local):
         roofline["latency"] = {"us_per_frame": us_frame, "floor_us_per_frame": floor_us,
                                "frac": floor_us / us_frame, "cluster_blocks": cs,
                                "floor_kind": "measured (qnn_measure_exchange_floor)"}
+    elif kname == "lstm_persist":
+        # the whole unprojected stack in one launch: the gate products of every layer and frame
+        flops = 2.0 * wl.batch * wl.frames * wl.num_layers * 4 * wl.hidden * (wl.R + gates_input_width(wl))
+        tpk = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
+        roofline = {"bound": "tensor", "kernel": kname, "achieved": flops / avg_s / 1e12, "peak": tpk, "unit": "TFLOP/s",
+                    "frac": flops / avg_s / 1e12 / tpk, "peak_kind": f"{peak_kind} (fp16/bf16 dense, sustained)",
+                    "traffic": traffic_record(kname, wl.name, ["lstm_persist.cu", "qnn_device.cuh", "tc_ptx.cuh"]),
+                    "alg_flops_per_launch": flops, "us_per_frame": avg_s * 1e6 / wl.frames,
+                    "avg_launch_ms": avg_s * 1e3, "share_of_step": share}
     elif kname == "lstm_gates_tc":
         # one recurrent step of one layer: the tcgen05 gate product (with the input product fused
         # in, the library's default) and the LSTM cell in its epilogue. Fused, the step moves few
@@ -490,7 +499,8 @@ def run_ours(args, wl, rank, world, local):
         "clocks": clk.summary(),
         # how the library ran the layers in the timed steps (the kernels' own durations above come
         # from a replay with the layers in sequence)
-        "layer_schedule": ("wavefront: one stream per layer" if wl.num_layers >= 2 and wl.batch >= 64 and
+        "layer_schedule": ("persistent: every layer in one launch" if "lstm_persist" in prof else
+                           "wavefront: one stream per layer" if wl.num_layers >= 2 and wl.batch >= 64 and
                            os.environ.get("QNN_TC_WAVE") != "0" else "sequential"),
     }
     if world == 1 and not args.no_extras:

@@ -22,12 +22,13 @@
 // Bound: the chain of one frame (operand stream of h_{t-1}, gate arithmetic, two exchanges). A step
 // as launches of a quantizer and a gate kernel per layer takes two launches' latency and streams the
 // weights again; the grid barriers of lstm_recurrent_kernel keep one layer at a time on the GPU. 5 x 500
-// cells, 2000 classes, 100 frames, this kernel alone (whole pass before): B = 16 592 us (5.5 ms), B = 64
-// 1030 us (2.3 ms), B = 128 1231 us (2.6 ms), B = 256 1908 us (3.0 ms). A frame at B = 32 took about 15,000
+// cells, 100 frames, this kernel alone (whole pass before): B = 16 593 us (5.5 ms), B = 64 995 us (2.3 ms);
+// B = 256, 500 frames 7.6 ms (13.4 ms). A frame at B = 32 took about 15,000
 // cycles while one row quarter's warps, all on one scheduler, did all its cells: h's operand stream and
 // products 4,700, gates 5,000, range exchange 2,200, codes and release 2,700. With the cells spread over the
-// four schedulers (SP = 4) B = 16 went from 869 to 717 us; two quarters' over all four (SP = 2), 5 x 300, 40
-// frames, B = 48, from 376 to 350 us, 5 x 512 551 to 529, 1 x 128 231 to 224.
+// four schedulers (SP = 4) a B = 16 pass went from 869 to 717 us; two quarters' over all four (SP = 2), 5 x
+// 300, 40 frames, B = 48, from 376 to 350 us, 5 x 512 551 to 529, 1 x 128 231 to 224 (all before the register
+// split below).
 //
 // Every wait is bounded in time: one that gives up records QNN_ERR_TIMEOUT and raises the abort
 // flag, after which all waits return at once and the launch runs to its end with meaningless outputs.
@@ -828,18 +829,18 @@ qnn_status prepare(qnn_lstm_model *m) {
 }  // namespace
 
 // Where the launch-per-step recurrences keep a stack that qualifies. Stacks gain from layers running side
-// by side in one launch (40 frames, this against the best other path, us: 5 x 500 B = 16 472 : 2257,
-// B = 256 1017 : 1211; 2 x 128 B = 256 374 : 635). A single layer is one chain either way, and two row
-// tiles or long reductions share one block's operand stream there, while the tensor-core recurrence
-// spreads a step over every SM: it keeps single layers from its smallest batch on (1 x 500 B = 64 314 : 375,
-// B = 150 564 : 415; 1 x 1024 B = 64 450 : 462, B = 100 524 : 482). With a few rows of a wide layer the
-// layerwise kernel is as good (1 x 1024 B = 1 383 : 369, B = 5 383 : 391). Posteriors in pinned host memory
-// cross the link during the wavefront's recurrence but only after this one: 5 x 500 B = 256 end to end
-// 14.8 : 14.6 ms.
+// by side in one launch (40 frames, this against the best other path, us: 5 x 500 B = 64 486 : 950, B = 256
+// 912 : 1184; 2 x 128 B = 256 356 : 459). A single layer is one chain either way, and two row tiles or long
+// reductions share one block's operand stream there, while the tensor-core recurrence spreads a step over every
+// SM: it keeps single layers from its smallest batch on (1 x 500 B = 64 292 : 354, B = 128 362 : 361, B = 256 480
+// : 393). With a few rows of a wide layer the layerwise kernel is as good (1 x 1024 B = 1 383 : 369, B = 5 383 :
+// 391). Posteriors in pinned host memory cross the link during the wavefront's recurrence but only after this
+// one, which counts where there are many (5 x 500 B = 256, 500 frames, end to end ms, 2000 classes 13.4 : 14.5,
+// 4000 classes 19.1 : 17.0).
 bool persist_preferred(const qnn_lstm_model *m, int64_t B, bool host_posteriors) {
     const bool tc = tc_recurrence_supported(m) && B >= kTcMinBatch;
     if (m->L == 1) return !tc && (m->H <= 512 || B > 4);
-    return !(host_posteriors && B > kTile && tc && tc_stack_supported(m));
+    return !(host_posteriors && B > kTile && m->C > 2048 && tc && tc_stack_supported(m));
 }
 
 qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, int64_t T, float *y, float *logits,
