@@ -547,7 +547,9 @@ __global__ void __launch_bounds__(256) softmax_rows_reg_kernel(const float *__re
 // buffers (k-major), the next step's operands loaded into registers while this one is multiplied.
 // Column pairs use paired multiply-adds: two per issue slot, so that the fp32 pipe stays busy while the
 // other slots carry the shared-memory loads. Bound: the fp32 pipe (2 M C K operations). 6400 x 2000 x
-// 500 (12.8 GFLOP): 990 us with a 32 x 32 tile whose every multiply-add read shared memory, 294 us here.
+// 500 (12.8 GFLOP): 990 us with a 32 x 32 tile whose every multiply-add read shared memory, 294 us with
+// rows tested and addressed at every load, a warp's threads 16 x 2 and outputs stored one by one, 262 us here
+// (0.65 of the fp32 rate; the tiles of the last of three rounds fill two thirds of the SMs).
 template <int TM, int TN>
 __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__restrict__ X, int64_t M, int K,
                                                            const float *__restrict__ Wt, int C,
@@ -557,7 +559,8 @@ __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__res
     // rows of BM (BC) values, 16 bytes apart from a multiple of 128 bytes for the transposed stores
     constexpr int XS = BM + 4, WS = BC + 4;
     __shared__ __align__(16) float xs[2][BK][XS], ws[2][BK][WS];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    // a warp covers 8 columns' threads x 4 rows': eight lanes read 128 consecutive bytes of ws, one of xs
+    const int tx = (threadIdx.x & 7) + 8 * ((threadIdx.x >> 5) & 1), ty = ((threadIdx.x >> 3) & 3) + 4 * (threadIdx.x >> 6);
     const int64_t m0 = (int64_t)(blockIdx.x / tiles_c) * BM;
     const int c0 = (int)(blockIdx.x % tiles_c) * BC;
     const bool vec = (K & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Wt)) & 15) == 0;
@@ -565,28 +568,31 @@ __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__res
     const int lr = threadIdx.x >> 2, lk = (threadIdx.x & 3) * 4;
     constexpr int XG = (BM + 63) / 64, WG = (BC + 63) / 64;
     float4 xv[XG], wv[WG];
-    auto fetch = [&](const float *base, int64_t row, int64_t rows, int k) {
+    // rows past the end repeat the last one (their outputs are dropped)
+    const float *px[XG], *pw[WG];
+#pragma unroll
+    for (int i = 0; i < XG; ++i) px[i] = X + min(m0 + lr + 64 * i, M - 1) * K + lk;
+#pragma unroll
+    for (int i = 0; i < WG; ++i) pw[i] = Wt + (int64_t)min(c0 + lr + 64 * i, C - 1) * K + lk;
+    auto fetch = [&](const float *p, int k) {
         float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (row < rows) {
-            const float *p = base + row * K + k;
-            if (vec && k < K) {
-                v = *reinterpret_cast<const float4 *>(p);
-            } else {
-                if (k < K) v.x = p[0];
-                if (k + 1 < K) v.y = p[1];
-                if (k + 2 < K) v.z = p[2];
-                if (k + 3 < K) v.w = p[3];
-            }
+        if (vec && k + 4 <= K) {
+            v = __ldg(reinterpret_cast<const float4 *>(p));
+        } else {
+            if (k < K) v.x = p[0];
+            if (k + 1 < K) v.y = p[1];
+            if (k + 2 < K) v.z = p[2];
+            if (k + 3 < K) v.w = p[3];
         }
         return v;
     };
     auto load = [&](int k0) {
 #pragma unroll
         for (int i = 0; i < XG; ++i)
-            if (lr + 64 * i < BM) xv[i] = fetch(X, m0 + lr + 64 * i, M, k0 + lk);
+            if (lr + 64 * i < BM) xv[i] = fetch(px[i] + k0, k0 + lk);
 #pragma unroll
         for (int i = 0; i < WG; ++i)
-            if (lr + 64 * i < BC) wv[i] = fetch(Wt, c0 + lr + 64 * i, C, k0 + lk);
+            if (lr + 64 * i < BC) wv[i] = fetch(pw[i] + k0, k0 + lk);
     };
     auto store = [&](int b) {
 #pragma unroll
@@ -603,6 +609,7 @@ __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__res
             }
     };
     // rows and columns of a thread in groups of G (4, or 2 for 2 x 2): group q at q 16 G + G ty (tx)
+    const bool yvec = (C & 3) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
     constexpr int GM = TM < 4 ? TM : 4, GN = TN < 4 ? TN : 4;
     float2 acc[TM][TN / 2];
 #pragma unroll
@@ -655,9 +662,17 @@ __global__ void __launch_bounds__(256, 2) float_linear_kernel(const float *__res
 #pragma unroll
         for (int j = 0; j < TN; j += GN) {
             const int c = c0 + j / GN * 16 * GN + GN * tx;
+            float o[GN];
 #pragma unroll
             for (int e = 0; e < GN; ++e)
-                if (c + e < C) Y[m * C + c + e] = ((e & 1) ? acc[i][(j + e) / 2].y : acc[i][(j + e) / 2].x) + bias[c + e];
+                o[e] = ((e & 1) ? acc[i][(j + e) / 2].y : acc[i][(j + e) / 2].x) + (c + e < C ? bias[c + e] : 0.0f);
+            if (GN == 4 && yvec && c + 4 <= C) {
+                *reinterpret_cast<float4 *>(Y + m * C + c) = make_float4(o[0], o[1], o[2], o[GN - 1]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < GN; ++e)
+                    if (c + e < C) Y[m * C + c + e] = o[e];
+            }
         }
     }
 }
