@@ -217,16 +217,17 @@ qnn_status launch_qgemm_imma(const uint8_t *A, int64_t lda, const qnn_qparams *p
 }
 
 // Datapath choice, between three kernels that differ in what they do to the operands first:
-//   - the streaming integer MMA kernel, nothing at all: up to 32 rows of A (8192 x 8192: 42 us at M = 32 against
-//     72 for the codes kernel), and up to 127 while its blocks (64 rows of A, 32 of W) are one wave (M = 127, 2048 x
-//     2048: 16.5 against 17.8; 4096 x 4096: 49.8 against 29.0);
+//   - the streaming integer MMA kernel, nothing at all: up to 32 rows of A (2048 x 2048: 8.3 us at M = 32 against
+//     10.3 for the codes kernel), and up to 127 for K below 2048 while its blocks (64 rows of A, 32 of W) are one
+//     wave (33 x 1000 x 1000: 12.4 against 14.4; but 64 x 2048 x 2048: 16.5 against 10.4; 127 x 4096 x 4096: 49.8
+//     against 21.0);
 //   - the codes kernel, converting on the way into shared memory: up to 127 rows beyond that (127 x 8000 x 500:
-//     13.4 against 32.9), and from 128 on while its tiles of 128 x 128 are one wave
-//     (M = 256, 8192 x 8192: 72 against 88 us; 256 x 2048 x 2048: 17.8 against 20.6; at two waves M = 512,
-//     8192 x 8192: 161 against 108; 1536 x 2000 x 500: 31 against 25), its rows lie on 128-byte lines or are short
-//     (1100 x 2000 x 500: 15.6 against 16.5) or, on 16-byte boundaries, its tiles of 128 x 64 are one wave (300 x
-//     3004 x 3008: 23.8 against 30.8; 512 x 4096 x 4000: 46 against 39). Rows without an alignment cost it shuffles
-//     and shifts (1000 x 1000 x 3001: 32.5 against 30.8);
+//     13.4 against 32.9), and from 128 on while its tiles of 128 x 128 are one wave (M = 256, 8192 x 8192: 72 against
+//     88 us; at two waves M = 512: 161 against 108; 1536 x 2000 x 500: 31 against 25), and its rows lie on 128-byte
+//     lines or are short (1100 x 2000 x 500: 15.6 against 16.5), or, on 16-byte boundaries, its tiles of 128 x 64 are
+//     one wave (300 x 3004 x 3008: 23.8 against 30.8; 512 x 4096 x 4000: 46 against 39), or these are so few that two
+//     blocks or more share each (600 x 600 x 3001: 22.6 against 28.8; but 1000 x 1000 x 3001, which do not: 32.5
+//     against 30.8);
 //   - the fp16 tensor-core product after a pass that centers both operands into scratch: the rest.
 // QNN_QGEMM=imma, =codes or =tc forces one (tests compare them).
 qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, int ga, const int32_t *rsA, int64_t M,
@@ -238,10 +239,11 @@ qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, in
     enum { kImma, kCodes, kTc } path = kTc;
     const int64_t sms = sm_count();
     if (M < 128) {  // (neither takes scratch: such a call allocates nothing)
-        path = M <= 32 || (M + 63) / 64 * ((N + 31) / 32) <= sms ? kImma : kCodes;
+        path = M <= 32 || (K < 2048 && (M + 63) / 64 * ((N + 31) / 32) <= sms) ? kImma : kCodes;
     } else if ((M + 127) / 128 * ((N + 127) / 128) <= sms) {
         const uintptr_t at = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | (uintptr_t)lda | (uintptr_t)ldw;
-        if (K <= 512 || at % 128 == 0 || (at % 16 == 0 && (M + 63) / 64 * ((N + 127) / 128) <= sms)) path = kCodes;
+        const int64_t tiles = (M + 63) / 64 * ((N + 127) / 128);  // of 128 x 64
+        if (K <= 512 || at % 128 == 0 || (at % 16 == 0 && tiles <= sms) || 16 * tiles <= 7 * sms) path = kCodes;
     }
     if (force && std::strcmp(force, "imma") == 0) path = kImma;
     if (force && std::strcmp(force, "codes") == 0) path = kCodes;

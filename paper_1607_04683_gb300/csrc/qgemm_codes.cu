@@ -12,6 +12,10 @@
 // Tile: 128 rows of W on the tensor-memory lanes x BN rows of A on the columns, so that a warp's outputs
 // of one row of A are 32 consecutive floats. BN = 64 while those tiles are one wave, else 128.
 //
+// Few tiles share their reductions: a cluster of up to 8 blocks takes a tile, each its part of K, and adds the
+// parts through distributed shared memory (128 x 2048 x 2048 17.8 us by 32 blocks, 10.8 by 128; 256 x 1024 x
+// 8192 51.8 and 19.6; 129 x 64 x 8192 52 and 12.3).
+//
 // Bound: the shared-memory port (a 128 x 128 k-block loads 16 KB of codes, stores 32 KB and has the MMAs read
 // 32 KB: 640 clk at 128 bytes a clk) and the latencies around it. M = 256, 8192 x 8192: 72 us, 1050 clk a
 // k-block; 132 us with eight converting warps and k-blocks one by one (each then waits, converts and loads in
@@ -56,6 +60,7 @@ struct CodeArgs {
     int32_t *acc_out;
     int *status;
     unsigned tiles_m;
+    int splits, per;  // blocks of a cluster, which share a tile's reduction, and the stages of each
 };
 
 struct RowConst {  // constants of one row of A
@@ -106,7 +111,7 @@ struct CodesTile {
     static constexpr size_t SMEM = (size_t)kStages * STAGE + 1024;
 };
 
-template <int BN, bool SHIFT>
+template <int BN, bool SHIFT, bool SPLITK>
 __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTile<BN>::MAX_REGS))
     qgemm_codes_kernel(const CodeArgs a) {
     constexpr int kSub = CodesTile<BN>::SUB, kStage = CodesTile<BN>::STAGE;
@@ -121,7 +126,11 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
                    drained0 = su32(bars + 2 * kStages + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = a.K, KB = (K + kBK - 1) / kBK;
-    const int64_t m0 = (int64_t)(blockIdx.x % a.tiles_m) * BN, n0 = (int64_t)(blockIdx.x / a.tiles_m) * kRowsW;
+    const unsigned tile = SPLITK ? blockIdx.x / a.splits : blockIdx.x;
+    const int64_t m0 = (int64_t)(tile % a.tiles_m) * BN, n0 = (int64_t)(tile / a.tiles_m) * kRowsW;
+    // this block's stages of the reduction: st0 .. st0 + steps - 1 of `all`
+    const int all = (KB + kKps - 1) / kKps, rank = SPLITK ? (int)cluster_rank() : 0;
+    const int st0 = SPLITK ? rank * a.per : 0, steps = SPLITK ? min(a.per, all - st0) : all;
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int i = 0; i < kStages; ++i) {
@@ -164,7 +173,6 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
             const uint32_t desc0 = smem_desc_lo(su32(smem));
             uint32_t d = desc0, bar = full0, tmem_d = tmem_base;
             unsigned parity = 0;
-            const int steps = (KB + kKps - 1) / kKps;
             for (int st = 0; st < steps; ++st) {
                 const int c = st / kChunk;
                 const bool fresh = st % kChunk == 0;
@@ -184,7 +192,7 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
                 for (int v = 0; v < kKps; ++v) {
-                    if (v > 0 && kKps * st + v >= KB) break;
+                    if (v > 0 && kKps * (st0 + st) + v >= KB) break;
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
                         const uint32_t w = d + ((v * kSub + 32 * k) >> 4), x = w + ((kRowsW * kBK * 2) >> 4);
@@ -197,6 +205,8 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
                 if (bar == full0 + 8 * kStages) d = desc0, bar = full0, parity ^= 1u;
             }
         }
+        __syncwarp();
+        if constexpr (SPLITK) cluster_sync(), cluster_sync();  // (the converting warps' two)
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CodesTile<BN>::REGS_CONV));
         // lane (r, c): codes 16 c .. 16 c + 15 of every k-block of row r of W and of A; rows past the end repeat
@@ -222,8 +232,8 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
         auto load = [&](Stage &g, int st) {
 #pragma unroll
             for (int v = 0; v < kKps; ++v) {
-                g.v[v][0] = src[0].load(kKps * st + v);
-                if (both) g.v[v][1] = src[1].load(kKps * st + v);
+                g.v[v][0] = src[0].load(kKps * (st0 + st) + v);
+                if (both) g.v[v][1] = src[1].load(kKps * (st0 + st) + v);
             }
         };
         auto mend = [&](uint4 (&v)[2], int kb) {
@@ -294,19 +304,19 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
         int slot = 0;
         unsigned free_parity = 1;
         bool ok = true, is_free = false;
-        const int steps = (KB + kKps - 1) / kKps;
         // stage st from the registers of its loads (and, with SHIFT, of the next stage's) into its slot
         auto convert = [&](Stage &cur, Stage &next, int st) -> bool {
             if (st >= kStages && !__all_sync(0xffffffffu, is_free || wait(empty0 + 8 * slot, free_parity))) return false;
             // units across an end of their matrix are in the first k-block, the last and (with SHIFT) the one after
-            if (st == 0) mend(cur.v[0], 0);
-            if (st + 2 >= steps) {
-                mend(cur.v[0], kKps * st), mend(cur.v[1], kKps * st + 1);
-                if (SHIFT) mend(next.v[0], kKps * st + 2);
+            const int kb = kKps * (st0 + st);
+            if (kb == 0) mend(cur.v[0], 0);
+            if (st0 + st + 2 >= all) {
+                mend(cur.v[0], kb), mend(cur.v[1], kb + 1);
+                if (SHIFT) mend(next.v[0], kb + 2);
             }
 #pragma unroll
             for (int v = 0; v < kKps; ++v) {
-                const int valid = K - kBK * (kKps * st + v) - 16 * c;  // codes of the chunk that lie inside the row
+                const int valid = K - kBK * (kb + v) - 16 * c;  // codes of the chunk that lie inside the row
                 uint8_t *const d = dst0 + slot * kStage + v * kSub;
                 const uint4(&nx)[2] = v + 1 < kKps ? cur.v[(v + 1) % kKps] : next.v[0];
                 put(d, cur.v[v][0], nx[0], sh[0], valid);
@@ -331,29 +341,22 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
         const int chunks = (steps - 1) / kChunk + 1;
         if (ok && chunks > 1 && (steps - 1) % kChunk < 1) ok = drain(chunks - 2);
         if (ok) ok = drain(chunks - 1);
-        if (!ok) {
-            *reinterpret_cast<volatile int *>(&s_abort) = 1;
-        } else if (n0 + 32 * q + lane < a.N) {
-            const int64_t n = n0 + 32 * q + lane;
+        if (!ok) *reinterpret_cast<volatile int *>(&s_abort) = 1;
+        // Outputs of row n of W (P its sum with row i of the tile's rows of A):
+        // S of eq. (1) = P + ra (128 + zw) + za (K zw + cs) + 128 cs - 128^2 K; while K |a' + za| |w' + zw|
+        // stays below 2^31, wrapping 32-bit arithmetic gives it exactly
+        auto outputs = [&](int64_t n, auto for_each) {
             const qnn_qparams qw = a.pw[n / a.rows_per_block];
             const int zw = qw.z, cs = a.csW[n];
             const float bias = a.bias ? a.bias[n] : 0.0f;
-            // S of eq. (1) = P + ra (128 + zw) + za (K zw + cs) + 128 cs - 128^2 K; while K |a' + za| |w' + zw|
-            // stays below 2^31, wrapping 32-bit arithmetic gives it exactly
             const uint32_t z128 = (uint32_t)(128 + zw), kz = (uint32_t)K * (uint32_t)zw + (uint32_t)cs,
                            s0 = 128u * (uint32_t)cs - 16384u * (uint32_t)K;
             const int a_lim = (int)(INT_MAX / ((long long)K * max(abs(zw), abs(zw + 255))));
-            const int rows = (int)min((int64_t)kCols, a.M - m0 - col0);
-            float *y = a.Y ? a.Y + (m0 + col0) * a.ldy + n : nullptr;
-            int32_t *o = a.acc_out ? a.acc_out + (m0 + col0) * a.N + n : nullptr;
-#pragma unroll
-            for (int j = 0; j < kCols; ++j) {
-                if (j >= rows) break;
-                const RowConst rc = s_row[col0 + j];
-                const int P = run[j];
+            for_each([&](int i, int P) {
+                const RowConst rc = s_row[i];
                 const int raw = (int)((uint32_t)P + 128u * (uint32_t)rc.ra + s0);  // raw code product
-                if (o) o[j * a.N] = raw;
-                if (!y) continue;
+                if (a.acc_out) a.acc_out[(m0 + i) * a.N + n] = raw;
+                if (!a.Y) return;
                 const float den = __fmul_rn(rc.Qa, qw.Q);
                 float v;
                 if (rc.amax <= a_lim && den >= 0x1p-60f && den <= 0x1p60f) {
@@ -362,8 +365,43 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
                 } else {
                     v = recover_product(offset_product(raw, rc.za, zw, rc.ra, cs, K), rc.Qa, qw.Q);
                 }
-                y[j * a.ldy] = a.bias ? __fadd_rn(v, bias) : v;
-            }
+                a.Y[(m0 + i) * a.ldy + n] = a.bias ? __fadd_rn(v, bias) : v;
+            });
+        };
+        const int rows = (int)min((int64_t)BN, a.M - m0);
+        if constexpr (!SPLITK) {
+            const int64_t n = n0 + 32 * q + lane;
+            if (ok && n < a.N)
+                outputs(n, [&](auto put) {
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j) {
+                        if (col0 + j >= rows) break;
+                        put(col0 + j, run[j]);
+                    }
+                });
+        } else {
+            // every block's sums into its own (no longer used) ring, [column][W row]; then each block adds the
+            // cluster's sums of its share of the columns and writes their outputs
+            int *const part = reinterpret_cast<int *>(smem);
+#pragma unroll
+            for (int j = 0; j < kCols; ++j) part[(col0 + j) * kRowsW + 32 * q + lane] = run[j];
+            __syncwarp();
+            cluster_sync();
+            const int share = (BN + a.splits - 1) / a.splits, row = threadIdx.x & (kRowsW - 1);
+            if (ok && n0 + row < a.N)
+                outputs(n0 + row, [&](auto put) {
+                    for (int i = rank * share + (threadIdx.x >> 7); i < min(rows, (rank + 1) * share); i += kConv / 4) {
+                        int P = 0;
+                        for (int b = 0; b < a.splits; ++b) {
+                            int v;
+                            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(su32(part + i * kRowsW + row), b)));
+                            P += v;
+                        }
+                        put(i, P);
+                    }
+                });
+            __syncwarp();
+            cluster_sync();  // no block leaves while another reads its sums
         }
     }
     __syncwarp();
@@ -380,32 +418,45 @@ __global__ void __launch_bounds__((CodesTile<BN>::THREADS)) __maxnreg__((CodesTi
     }
 }
 
-template <int BN, bool SHIFT>
-qnn_status launch_codes(CodeArgs &a, cudaStream_t st) {
+template <int BN, bool SHIFT, bool SPLITK>
+qnn_status launch_codes_as(const CodeArgs &a, int64_t tiles, cudaStream_t st) {
     constexpr size_t smem = CodesTile<BN>::SMEM;
     static int configured = -1;
     int dev = 0;
     QNN_CUDA_TRY(cudaGetDevice(&dev));
     if (configured != dev) {
-        QNN_CUDA_TRY(cudaFuncSetAttribute(qgemm_codes_kernel<BN, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        QNN_CUDA_TRY(cudaFuncSetAttribute(qgemm_codes_kernel<BN, SHIFT, SPLITK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         configured = dev;
     }
-    const int64_t tm = (a.M + BN - 1) / BN, tiles = tm * ((a.N + kRowsW - 1) / kRowsW);
-    if (tiles > INT32_MAX) return QNN_FAIL(QNN_ERR_INVALID_ARG);
-    a.tiles_m = (unsigned)tm;
     ProfScope prof("qgemm_codes", st);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)tiles);
+    cfg.gridDim = dim3((unsigned)(tiles * a.splits));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.splits, attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, qgemm_codes_kernel<BN, SHIFT>, a));
+    cfg.numAttrs = SPLITK ? 2 : 1;
+    QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, qgemm_codes_kernel<BN, SHIFT, SPLITK>, a));
     return QNN_OK;
+}
+
+template <int BN, bool SHIFT>
+qnn_status launch_codes(CodeArgs &a, cudaStream_t st) {
+    const int64_t tm = (a.M + BN - 1) / BN, tiles = tm * ((a.N + kRowsW - 1) / kRowsW);
+    if (tiles > INT32_MAX) return QNN_FAIL(QNN_ERR_INVALID_ARG);
+    a.tiles_m = (unsigned)tm;
+    // a tile's reduction over the blocks of a cluster, up to 8 of at least four stages, while they find SMs
+    // (a cluster's blocks share a part of the chip, so an eighth of the SMs is left out)
+    const int64_t steps = (a.K + kKps * kBK - 1) / (kKps * kBK);
+    a.splits = (int)std::max<int64_t>(1, std::min<int64_t>({8, steps / 4, sm_count() * 7 / 8 / tiles}));
+    a.per = (int)((steps + a.splits - 1) / a.splits);
+    a.splits = (int)((steps + a.per - 1) / a.per);
+    return a.splits > 1 ? launch_codes_as<BN, SHIFT, true>(a, tiles, st) : launch_codes_as<BN, SHIFT, false>(a, tiles, st);
 }
 
 }  // namespace
@@ -416,7 +467,7 @@ qnn_status launch_qgemm_codes(const uint8_t *A, int64_t lda, const qnn_qparams *
                               cudaStream_t st) {
     if (M == 0 || N == 0) return QNN_OK;
     CodeArgs a{A, lda, pa, ga == QNN_PER_ROW, rsA, M, (int)K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out,
-               nullptr, 0};
+               nullptr, 0, 1, 0};
     QNN_TRY(status_word(&a.status));
     const uintptr_t at = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | (uintptr_t)lda | (uintptr_t)ldw;
     const bool wide = ((M + 63) / 64) * ((N + kRowsW - 1) / kRowsW) > (int64_t)sm_count();

@@ -118,7 +118,8 @@ def test_tensor_core_outputs(qnn, M, N, K, pad, bn, shift, monkeypatch):
 @pytest.mark.parametrize("M,N,K", [(1, 1, 40), (5, 6, 7), (63, 127, 15), (64, 128, 16), (65, 129, 17), (100, 260, 63), (129, 2000, 64),
                                    (130, 500, 65), (200, 9000, 127), (128, 20000, 193), (128, 130, 256), (129, 136, 321),
                                    (300, 300, 1000), (128, 64, 1024), (130, 132, 1025), (96, 128, 1088), (70, 200, 1153),
-                                   (128, 14600, 1217), (128, 129, 2048), (128, 128, 2113), (66, 65, 3300), (64, 33, 33025)])
+                                   (128, 14600, 1217), (128, 129, 2048), (128, 128, 2113), (66, 65, 3300), (64, 33, 33025),
+                                   (130, 1500, 1500), (40, 300, 1023), (128, 1100, 1025), (300, 700, 2050)])
 @pytest.mark.parametrize("pad,off,shift", [(None, 0, 0.0), (0, 0, 20.0), (4, 4, 3000.0), (3, 1, 0.0), (6, 15, 0.0)])
 def test_codes_bit_exact(qnn, M, N, K, pad, off, shift, monkeypatch):
     monkeypatch.setenv("QNN_QGEMM", "codes")
