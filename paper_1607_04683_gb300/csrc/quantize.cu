@@ -23,7 +23,9 @@ namespace {
 
 constexpr int kRowWarps = 8;  // warps (rows) per block in the per-row kernels
 
-constexpr int kFlight = 8;    // 16-byte loads in flight per lane in the passes over long rows
+constexpr int kFlight = 8;    // 16-byte loads in flight per lane in the passes over rows of at least kMidRow values;
+constexpr int kMidRow = 512;  // shorter ones take one, and the registers of more rows at once (100000 x 60: range 28 us
+                              // with eight, 21 with one)
 
 // Running range of values and whether one was not finite: v * 0 is NaN then, and so is the sum.
 struct Range {
@@ -38,7 +40,7 @@ struct Range {
 };
 
 // Range of one row held by one warp; returns false if a value is not finite.
-template <bool kVec>
+template <bool kVec, int F>
 __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int cols, float &mn, float &mx) {
     const int lane = threadIdx.x & 31;
     Range r;
@@ -46,13 +48,13 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
     if (kVec) {
         const float4 *x4 = reinterpret_cast<const float4 *>(xr);
         const int n4 = cols >> 2;
-        for (int i = lane; i < n4; i += 32 * kFlight) {
-            float4 v[kFlight];
+        for (int i = lane; i < n4; i += 32 * F) {
+            float4 v[F];
 #pragma unroll
-            for (int u = 0; u < kFlight; ++u)
+            for (int u = 0; u < F; ++u)
                 if (i + 32 * u < n4) v[u] = __ldg(x4 + i + 32 * u);
 #pragma unroll
-            for (int u = 0; u < kFlight; ++u)
+            for (int u = 0; u < F; ++u)
                 if (i + 32 * u < n4) r.add(v[u]);
         }
         done = n4 << 2;
@@ -64,7 +66,7 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
 }
 
 // Codes of one row (eq. 2) and their sum, one warp.
-template <bool kVec>
+template <bool kVec, int F>
 __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int cols, float Q, int z,
                                               uint8_t *__restrict__ cr) {
     const int lane = threadIdx.x & 31;
@@ -73,13 +75,13 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
         const float4 *x4 = reinterpret_cast<const float4 *>(xr);
         uint32_t *c4 = reinterpret_cast<uint32_t *>(cr);
         const int n4 = cols >> 2;
-        for (int i = lane; i < n4; i += 32 * kFlight) {
-            float4 v[kFlight];
+        for (int i = lane; i < n4; i += 32 * F) {
+            float4 v[F];
 #pragma unroll
-            for (int u = 0; u < kFlight; ++u)
+            for (int u = 0; u < F; ++u)
                 if (i + 32 * u < n4) v[u] = __ldg(x4 + i + 32 * u);
 #pragma unroll
-            for (int u = 0; u < kFlight; ++u) {
+            for (int u = 0; u < F; ++u) {
                 if (i + 32 * u >= n4) break;
                 const uint32_t a = quant_code(v[u].x, Q, z), b = quant_code(v[u].y, Q, z), c = quant_code(v[u].z, Q, z),
                                d = quant_code(v[u].w, Q, z);
@@ -102,7 +104,7 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
     return warp_sum(s);
 }
 
-template <bool kVec>
+template <bool kVec, int F>
 __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const float *__restrict__ x, int64_t rows,
                                                                       int cols, int64_t ldx, uint8_t *__restrict__ codes,
                                                                       int64_t ldc, qnn_qparams *__restrict__ params,
@@ -111,14 +113,14 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
     if (row >= rows) return;
     const float *xr = x + row * ldx;
     float mn, mx;
-    bool ok = warp_row_range<kVec>(xr, cols, mn, mx);
+    bool ok = warp_row_range<kVec, F>(xr, cols, mn, mx);
     if (!ok) {
         if ((threadIdx.x & 31) == 0) record_status(status, QNN_ERR_NONFINITE);
         mn = 0.0f;
         mx = 0.0f;
     }
     qnn_qparams p = params_from_range(mn, mx);
-    int s = warp_row_codes<kVec>(xr, cols, p.Q, p.z, codes + row * ldc);
+    int s = warp_row_codes<kVec, F>(xr, cols, p.Q, p.z, codes + row * ldc);
     if ((threadIdx.x & 31) == 0) {
         params[row] = p;
         if (sums) sums[row] = s;
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kRowWarps * 32, rows_reg_blocks(NV))
 // Per-matrix pass 1: block partial ranges; the last block folds them into params[0]. The warps take segments
 // of kSegment values of the rows in turn (whole rows leave a last, nearly empty round).
 constexpr int kSegment = 2048;
-template <bool kVec>
+template <bool kVec, int F>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const float *__restrict__ x, int64_t rows,
                                                                      int cols, int64_t ldx, float *__restrict__ partials,
                                                                      unsigned *__restrict__ counter,
@@ -243,10 +245,10 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     const int segs = (cols - 1) / kSegment + 1;
     const int64_t items = rows * segs;
     for (int64_t i = (int64_t)blockIdx.x * kRowWarps + warp; i < items; i += (int64_t)gridDim.x * kRowWarps) {
-        const int64_t row = i / segs;
+        const int64_t row = segs == 1 ? i : i / segs;
         const int k0 = (int)(i - row * segs) * kSegment;
         float a, b;
-        if (!warp_row_range<kVec>(x + row * ldx + k0, min(kSegment, cols - k0), a, b)) {
+        if (!warp_row_range<kVec, F>(x + row * ldx + k0, min(kSegment, cols - k0), a, b)) {
             if (lane == 0) s_bad = 1;
         } else {
             mn = fminf(mn, a);
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_long_rows_kernel(const 
     grid_dependency_wait();
     const float Q = __ldcg(&params[0].Q);
     const int z = __ldcg(&params[0].z);
-    const int s = k0 < cols ? warp_row_codes<kVec>(x + row * ldx + k0, min(part, cols - k0), Q, z, codes + row * ldc + k0) : 0;
+    const int s = k0 < cols ? warp_row_codes<kVec, kFlight>(x + row * ldx + k0, min(part, cols - k0), Q, z, codes + row * ldc + k0) : 0;
     if (!sums) return;
     if ((threadIdx.x & 31) == 0) s_sum[warp] = s;
     __syncthreads();
@@ -320,18 +322,23 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_long_rows_kernel(const 
     }
 }
 
-template <bool kVec>
+template <bool kVec, int F>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_codes_kernel(const float *__restrict__ x, int64_t rows,
                                                                      int cols, int64_t ldx, uint8_t *__restrict__ codes,
                                                                      int64_t ldc, const qnn_qparams *__restrict__ params,
                                                                      int32_t *__restrict__ sums) {
-    const int64_t row = (int64_t)(gridDim.x - 1 - blockIdx.x) * kRowWarps + (threadIdx.x >> 5);
+    const int64_t groups = (rows + kRowWarps - 1) / kRowWarps;
+    // once a block, of a grid of one wave: in blocks of eight short rows the wait took most of the time (197307 x 57:
+    // 87 us, so 32)
     grid_dependency_wait();
-    if (row >= rows) return;
     const float Q = __ldcg(&params[0].Q);
     const int z = __ldcg(&params[0].z);
-    int s = warp_row_codes<kVec>(x + row * ldx, cols, Q, z, codes + row * ldc);
-    if ((threadIdx.x & 31) == 0 && sums) sums[row] = s;
+    for (int64_t b = blockIdx.x; b < groups; b += gridDim.x) {
+        const int64_t row = (groups - 1 - b) * kRowWarps + (threadIdx.x >> 5);
+        if (row >= rows) continue;
+        const int s = warp_row_codes<kVec, F>(x + row * ldx, cols, Q, z, codes + row * ldc);
+        if (sums && (threadIdx.x & 31) == 0) sums[row] = s;
+    }
 }
 
 inline bool vec_ok(const float *x, int64_t ldx, const uint8_t *codes, int64_t ldc) {
@@ -361,9 +368,9 @@ qnn_status launch_quantize_rows(const float *x, int64_t rows, int64_t cols, int6
             default: quantize_rows_reg_kernel<8><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
         }
     } else if (vec_ok(x, ldx, codes, ldc))
-        quantize_rows_kernel<true><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+        quantize_rows_kernel<true, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
     else
-        quantize_rows_kernel<false><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+        quantize_rows_kernel<false, 1><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
     QNN_CUDA_TRY(cudaGetLastError());
     return QNN_OK;
 }
@@ -379,17 +386,20 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     const bool v = vec_ok(x, ldx, codes, ldc);
     {
     ProfScope prof("quantize_matrix_range", st);
-    if (v)
-        matrix_range_kernel<true><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
+    const bool mid = cols >= kMidRow;
+    if (v && mid)
+        matrix_range_kernel<true, kFlight><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
+    else if (v)
+        matrix_range_kernel<true, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     else
-        matrix_range_kernel<false><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
+        matrix_range_kernel<false, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     QNN_CUDA_TRY(cudaGetLastError());
     }
     ProfScope prof("quantize_matrix_codes", st);
     // programmatic dependent launch: the blocks are set up while the range pass ends (they wait for it)
     cudaLaunchConfig_t cfg = {};
     const bool long_rows = cols >= kLongRow && rows <= INT32_MAX;
-    cfg.gridDim = dim3((unsigned)(long_rows ? rows : want));
+    cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, 8 * (int64_t)sm_count())));
     cfg.blockDim = dim3(kRowWarps * 32);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -401,7 +411,7 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
         QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, v ? matrix_long_rows_kernel<true> : matrix_long_rows_kernel<false>, x, (int)cols, ldx,
                                         codes, ldc, (const qnn_qparams *)params, sums));
     else
-        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, v ? matrix_codes_kernel<true> : matrix_codes_kernel<false>, x, rows, (int)cols,
+        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, !v ? matrix_codes_kernel<false, 1> : cols >= kMidRow ? matrix_codes_kernel<true, kFlight> : matrix_codes_kernel<true, 1>, x, rows, (int)cols,
                                         ldx, codes, ldc, (const qnn_qparams *)params, sums));
     return QNN_OK;
 }
