@@ -128,7 +128,7 @@ qnn_status small_stream_launch(const qnn_lstm_model *m, const SmallStreamArgs &s
 
 // Runs qnn_lstm_forward on the persistent tensor-core stack (lstm_persist.cu) if the model and batch
 // qualify (no projection, one unit per gate matrix, at most 256 sequences, a stack whose blocks fit the
-// SMs); *used tells whether it ran. Arguments as for qnn_lstm_forward_logits (logits nullable).
+// SMs and their accumulators the tensor memory, persist_plan.h); *used tells whether it ran. Arguments as for qnn_lstm_forward_logits (logits nullable).
 qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, int64_t T, float *y, float *logits,
                                 float *h_state, float *c_state, float *h_all, cudaStream_t st, bool *used);
 // Whether that path is the better one where it qualifies (see there).

@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "lstm_model.h"
+#include "persist_plan.h"
 #include "qnn_device.cuh"
 #include "tc_gemm.h"
 #include "tc_ptx.cuh"
@@ -49,7 +50,8 @@
 namespace qnn {
 namespace {
 
-constexpr int kMaxL = 8;               // layers of a launch (tensor maps are kernel arguments)
+using namespace persist;
+
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 32 * (kEpiWarps + 4);  // (two warps only complete the last warpgroup)
 // Registers a thread: 96 at launch (640 threads), of which the producer's warpgroup leaves its share to the
@@ -57,11 +59,7 @@ constexpr int kThreads = 32 * (kEpiWarps + 4);  // (two warps only complete the 
 // misses the little L1 that the weights leave: 5 x 500 cells, B = 16 and 64, 100 frames 714 and 1435 us, B = 256,
 // 500 frames 9.59 ms; so 630, 1352 us and 8.37 ms.
 constexpr int kRegsEpi = 112, kRegsIssue = 32;
-constexpr int kMaxSlots = 4;           // operand ring slots
-constexpr int kSlotBytes = 32 * 1024;  // at most (two k-blocks of 128 rows)
-constexpr int kTile = 128;             // rows (sequences) of a tile
 constexpr unsigned long long kWaitLimit = 2000000000ull;
-constexpr int kSmemMax = 227 * 1024;
 
 __host__ __device__ inline int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
@@ -265,16 +263,10 @@ struct Cfg {
     static constexpr int PAIRS = SP > 1 ? (2 * NC + SL - 1) / SL : MT == 1 ? NC / 2 : NC;  // cell pairs of a thread
     static constexpr bool ODD = SP == 1 && MT == 1 && (NC & 1);  // and one more cell
     static constexpr int GIVEN = SP > 1 ? 2 * NC - (2 * NC + SP - 1) / SP : 0;  // pairs handed over per row quarter
-    static constexpr int TMEM_COLS = 3 * MT * N <= 128 ? 128 : (3 * MT * N <= 256 ? 256 : 512);
+    static constexpr int TMEM_USED = tmem_used(NC, MT), TMEM_COLS = TMEM_USED <= 128 ? 128 : TMEM_USED <= 256 ? 256 : kTmemCols;
+    static_assert(TMEM_USED <= kTmemCols, "the accumulators fit the tensor memory");
     static constexpr int KB_BYTES = N * 128;             // a k-block of weights
 };
-
-// Shared memory beside the ring and the weights: barriers, ranges, (MT = 1) the pairs' code sums, and the sums
-// handed over, [quarter][pair][16 words][32 rows].
-constexpr int misc_bytes(int NC, int MT, int SP) {
-    return 8 * (2 * kMaxSlots + 8) + 16 + 4 * kTile * 4 + (MT == 1 ? 2 * NC * 64 : 0) +
-           (SP > 1 ? (2 * NC - (2 * NC + SP - 1) / SP) * (4 / SP) * 64 * 32 : 0);
-}
 
 template <int NC, int MT, int SP>
 __global__ void __launch_bounds__(kThreads, 1) lstm_persist_kernel(const __grid_constant__ PersistArgs a) {
@@ -720,42 +712,11 @@ __global__ void pair_constants_kernel(const float *__restrict__ bias, const int3
     out[3 * i] = b, out[3 * i + 1] = cx, out[3 * i + 2] = ch;
 }
 
-struct Plan {
-    int NC = 0, MT = 1, SP = 1, G = 0;
-    int rows_box = 0, kps = 0, slots = 0, slot_bytes = 0;
-    size_t smem = 0;
-};
-
-// The smallest cell count per block for which the stack's blocks fit the SMs one each and the widest
-// layer's weights leave room for the operand ring.
-bool make_plan(const qnn_lstm_model *m, int64_t B, Plan *p) {
-    if (m->P != 0 || m->S != 1 || m->L > kMaxL || B < 1 || B > 2 * kTile) return false;
-    const int64_t kh = round_up(m->H, 64);
-    if (kh > 1024) return false;
+bool plan_of(const qnn_lstm_model *m, int64_t B, Plan *p) {
+    if (m->P != 0 || m->S != 1) return false;
     int64_t kx = 0;
     for (int64_t l = 0; l < m->L; ++l) kx = std::max(kx, round_up(m->layers[l].kin, 64));
-    if (kx > 1024) return false;
-    p->MT = B > kTile ? 2 : 1;
-    p->rows_box = (int)std::min<int64_t>(kTile, round_up(B, 8));
-    p->SP = B <= 32 ? 4 : B <= 64 ? 2 : 1;
-    for (int NC : {2, 4, 5, 6}) {
-        const int64_t G = (m->H + 4 * NC - 1) / (4 * NC);
-        if (G * m->L > sm_count()) continue;
-        const int64_t weights = (kx + kh) / 64 * NC * 2048;
-        // (by the widest slots, so that a model's layout does not depend on the batch)
-        const int64_t left = kSmemMax - weights - misc_bytes(NC, p->MT, p->SP);
-        if (kSmemMax - weights - std::max(misc_bytes(NC, 1, 1), misc_bytes(NC, 2, 1)) < 2 * kSlotBytes) continue;
-        // (handed-over sums take up to 24 KB: where two whole slots don't fit beside them, two halves do)
-        p->kps = std::max(1, std::min(8, (left >= 2 * kSlotBytes ? kSlotBytes : kSlotBytes / 2) / (p->rows_box * 128)));
-        p->slot_bytes = p->kps * p->rows_box * 128;
-        const int64_t slots = std::min<int64_t>(kMaxSlots, left / p->slot_bytes);
-        p->NC = NC, p->G = (int)G, p->slots = (int)slots;
-        // an operand box of fewer than 128 rows is multiplied as 128: its last slot's reads stay inside
-        const int64_t used = slots * p->slot_bytes + weights + misc_bytes(NC, p->MT, p->SP);
-        p->smem = (size_t)std::min<int64_t>(kSmemMax, std::max(used, slots * p->slot_bytes + kTile * 128));
-        return (int64_t)p->smem >= slots * p->slot_bytes + kTile * 128;
-    }
-    return false;
+    return make_plan(m->L, m->H, kx, round_up(m->H, 64), B, sm_count(), p);
 }
 
 template <int NC, int MT, int SP>
@@ -847,7 +808,7 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
                                 float *h_state, float *c_state, float *h_all, cudaStream_t st, bool *used) {
     *used = false;
     Plan p;
-    if (!make_plan(m, B, &p) || B * T > INT32_MAX / 2 || T >= (1 << 24)) return QNN_OK;
+    if (!plan_of(m, B, &p) || B * T > INT32_MAX / 2 || T >= (1 << 24)) return QNN_OK;
     QNN_TRY(prepare(m));
     const int64_t L = m->L, I = m->I, H = m->H, C = m->C, R = m->R, rows = B * T;
     const int64_t kh = round_up(H, 64), kx0 = round_up(I, 64);
@@ -953,7 +914,12 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
         ProfScope prof("lstm_persist", st);
         auto run = [&](auto nc) -> qnn_status {
             constexpr int NC = decltype(nc)::value;
-            if (p.MT == 2) return launch<NC, 2, 1>(a, p, L, st);
+            if (p.MT == 2) {
+                if constexpr (tmem_used(NC, 2) <= kTmemCols)
+                    return launch<NC, 2, 1>(a, p, L, st);
+                else
+                    return QNN_FAIL(QNN_ERR_INVALID_ARG);  // (no plan asks for it)
+            }
             return p.SP == 4 ? launch<NC, 1, 4>(a, p, L, st) : p.SP == 2 ? launch<NC, 1, 2>(a, p, L, st) : launch<NC, 1, 1>(a, p, L, st);
         };
         using std::integral_constant;

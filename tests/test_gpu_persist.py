@@ -74,7 +74,11 @@ CASES = [dict(L=1, I=1, H=1, B=1, T=3), dict(L=1, I=8, H=8, B=5, T=3), dict(L=2,
          dict(L=3, H=128, B=32, C=50), dict(L=2, H=300, B=33), dict(L=2, H=301, B=64, C=20), dict(L=5, H=500, B=16, T=6, C=200, w=0.08),
          dict(L=4, H=512, B=65, T=3, w=0.08), dict(L=2, H=128, B=128, C=20), dict(L=2, H=129, B=129), dict(L=3, I=320, H=450, B=200, T=3, w=0.08),
          dict(L=5, H=500, B=256, T=3, C=20, w=0.08), dict(L=1, I=600, H=1000, B=9, T=3, w=0.05), dict(L=8, H=64, B=40, T=5),
-         dict(L=2, H=64, B=9, C=10, mode=2)]
+         dict(L=2, H=64, B=9, C=10, mode=2),
+         # the plan's other forms: 16, 20 and 24 cells a block with one, two and four quarters in use
+         dict(L=4, H=512, B=30, T=2, w=0.08), dict(L=4, H=510, B=50, T=2, w=0.08), dict(L=5, H=498, B=60, T=2, w=0.08),
+         dict(L=5, H=500, B=100, T=2, w=0.08), dict(L=8, H=384, B=20, T=2, C=30, w=0.1), dict(L=8, H=383, B=40, T=2, w=0.1),
+         dict(L=8, H=384, B=100, T=2, w=0.1)]
 
 
 @pytest.mark.parametrize("cfg", CASES)
@@ -96,6 +100,23 @@ def test_stack_bit_exact(qnn, cfg):
     b = forward(qnn, model, wl, x[:, 1:], h=a["h"], c=a["c"], h_all=False)
     assert np.array_equal(b["h"], got["h"]) and np.array_equal(b["c"], got["c"])
     assert np.array_equal(np.concatenate([a["y"], b["y"]], 1), got["y"])
+
+
+# Two row tiles of blocks of 24 cells have no tensor memory: such a stack stays on the layer wavefront.
+@pytest.mark.parametrize("H,B", [(384, 130), (384, 256), (381, 129)])
+def test_stack_without_a_plan(qnn, H, B, monkeypatch):
+    monkeypatch.delenv("QNN_LSTM_PATH")
+    wl = workload(L=8, H=H, B=B, T=2, w=0.1)
+    params, x = wl.make()
+    model = model_of(qnn, wl, params)
+    qnn.profile_read()
+    qnn.profile_enable(True)
+    got = forward(qnn, model, wl, x)
+    qnn.profile_enable(False)
+    assert "lstm_persist" not in qnn.profile_read()
+    b = [0, 63, 127, 128, B - 1]
+    ref = reference(wl, params, np.ascontiguousarray(x[b]))
+    assert np.array_equal(got["h_all"][:, b], ref["h_all"]) and np.array_equal(got["c"][:, b], ref["c"])
 
 
 @pytest.mark.parametrize("B", [9, 150])
