@@ -58,7 +58,10 @@ typedef enum { QNN_OUT_NONE = 0, QNN_OUT_QUANT = 1, QNN_OUT_FLOAT = 2 } qnn_outp
  * eq. (2). Code of v: clamp(round(Q v) - z, 0, 255). Recovery (eq. 3): (code + z) / Q.
  * Readings where the paper is silent: Q is raised by single ulps until the range maximum reaches
  * code 255; codes are clamped to [0, 255]; a unit with vmax == vmin, or with |Q vmin| or
- * |Q vmax| >= 2^22, uses Q = 255 / max(|vmin|, |vmax|) (Q = 1 if all values are 0). That rule
+ * |Q vmax| >= 2^22, uses Q = 255 / max(|vmin|, |vmax|) (Q = 1 if all values are 0). Where that
+ * overflows (a maximum below about 7.5e-37) Q is infinite; the conversions to integers saturate (NaN to
+ * 0) and the difference wraps, so that a unit's codes are all 0, or, if its least value is 0, 255 for
+ * every other value; products recover 0 from it. That rule
  * takes the place of a range error: no call fails on a unit without a usable range (an all-zero
  * initial state, a constant row); only non-finite values are errors (QNN_ERR_NONFINITE). */
 typedef struct {

@@ -67,6 +67,17 @@ enum { ORC_OUT_NONE = 0, ORC_OUT_QUANT = 1, ORC_OUT_FLOAT = 2 };
 /* Quantizer, Sec. 3 "Quantizing" and eq. (2)                                                 */
 /* ------------------------------------------------------------------------------------------ */
 
+/* The nearest int32 of a float, saturating, NaN to 0: only a unit of infinite scale (reading R3 with max|v| below
+ * about 7.5e-37) needs more than the plain cast, which C leaves undefined there. */
+static int32_t round_s32(float v)
+{
+    if (v != v) return 0;
+    v = rintf(v);
+    if (v >= 2147483648.0f) return INT32_MAX;
+    if (v < -2147483648.0f) return INT32_MIN;
+    return (int32_t)v;
+}
+
 static float next_up_positive(float q) /* next fp32 above a positive finite q */
 {
     uint32_t u;
@@ -91,7 +102,7 @@ void orc_params_from_range(float vmin, float vmax, orc_qparams *p)
         float amax = fmaxf(fabsf(vmin), fabsf(vmax));
         Q = (amax > 0.0f) ? S / amax : 1.0f;
         p->Q = Q;
-        p->z = (int32_t)rintf(Q * vmin);
+        p->z = round_s32(Q * vmin);
         return;
     }
     int32_t z = (int32_t)rintf(Q * vmin);
@@ -124,7 +135,7 @@ int orc_range(const float *v, int64_t n, int64_t stride, float *vmin, float *vma
 /* Eq. (2): V' = round(Q V) - round(Q Vmin), clamped to [0, S] (reading R2). */
 uint8_t orc_code(float v, const orc_qparams *p)
 {
-    int32_t c = (int32_t)rintf(p->Q * v) - p->z;
+    int32_t c = (int32_t)((uint32_t)round_s32(p->Q * v) - (uint32_t)p->z);
     if (c < 0) c = 0;
     if (c > 255) c = 255;
     return (uint8_t)c;

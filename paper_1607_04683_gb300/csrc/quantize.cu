@@ -67,7 +67,7 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
 
 // Codes of one row (eq. 2) and their sum, one warp.
 template <bool kVec, int F>
-__device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int cols, float Q, int z,
+__device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int cols, const UnitCoder &unit,
                                               uint8_t *__restrict__ cr) {
     const int lane = threadIdx.x & 31;
     int s = 0;
@@ -83,20 +83,20 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
 #pragma unroll
             for (int u = 0; u < F; ++u) {
                 if (i + 32 * u >= n4) break;
-                const uint32_t a = quant_code(v[u].x, Q, z), b = quant_code(v[u].y, Q, z), c = quant_code(v[u].z, Q, z),
-                               d = quant_code(v[u].w, Q, z);
+                const uint32_t a = unit.code(v[u].x), b = unit.code(v[u].y), c = unit.code(v[u].z),
+                               d = unit.code(v[u].w);
                 s += (int)(a + b + c + d);
                 c4[i + 32 * u] = a | (b << 8) | (c << 16) | (d << 24);
             }
         }
         for (int i = (n4 << 2) + lane; i < cols; i += 32) {
-            uint32_t a = quant_code(__ldg(xr + i), Q, z);
+            uint32_t a = unit.code(__ldg(xr + i));
             s += (int)a;
             cr[i] = (uint8_t)a;
         }
     } else {
         for (int i = lane; i < cols; i += 32) {
-            uint32_t a = quant_code(__ldg(xr + i), Q, z);
+            uint32_t a = unit.code(__ldg(xr + i));
             s += (int)a;
             cr[i] = (uint8_t)a;
         }
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
         mx = 0.0f;
     }
     qnn_qparams p = params_from_range(mn, mx);
-    int s = warp_row_codes<kVec, F>(xr, cols, p.Q, p.z, codes + row * ldc);
+    int s = warp_row_codes<kVec, F>(xr, cols, UnitCoder(p.Q, p.z), codes + row * ldc);
     if ((threadIdx.x & 31) == 0) {
         params[row] = p;
         if (sums) sums[row] = s;
@@ -189,14 +189,15 @@ __global__ void __launch_bounds__(kRowWarps * 32, rows_reg_blocks(NV))
             mx = 0.0f;
         }
         const qnn_qparams p = params_from_range(mn, mx);
+        const UnitCoder unit(p.Q, p.z);
         uint8_t *cr = codes + row * ldc;
         int s = 0;
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
             const int k = 4 * (lane + 32 * i);
             if (k >= cols) continue;
-            const uint32_t a = quant_code(v[i].x, p.Q, p.z), b = quant_code(v[i].y, p.Q, p.z),
-                           c = quant_code(v[i].z, p.Q, p.z), d = quant_code(v[i].w, p.Q, p.z);
+            const uint32_t a = unit.code(v[i].x), b = unit.code(v[i].y),
+                           c = unit.code(v[i].z), d = unit.code(v[i].w);
             if (pack && k + 4 <= cols) {  // 4-byte aligned code rows: one store for four codes
                 s += (int)(a + b + c + d);
                 *reinterpret_cast<uint32_t *>(cr + k) = a | (b << 8) | (c << 16) | (d << 24);
@@ -308,9 +309,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_long_rows_kernel(const 
     const int64_t row = gridDim.x - 1 - blockIdx.x;
     const int warp = threadIdx.x >> 5, part = ((cols + kRowWarps - 1) / kRowWarps + 3) & ~3, k0 = warp * part;
     grid_dependency_wait();
-    const float Q = __ldcg(&params[0].Q);
-    const int z = __ldcg(&params[0].z);
-    const int s = k0 < cols ? warp_row_codes<kVec, kFlight>(x + row * ldx + k0, min(part, cols - k0), Q, z, codes + row * ldc + k0) : 0;
+    const UnitCoder unit(__ldcg(&params[0].Q), __ldcg(&params[0].z));
+    const int s = k0 < cols ? warp_row_codes<kVec, kFlight>(x + row * ldx + k0, min(part, cols - k0), unit, codes + row * ldc + k0) : 0;
     if (!sums) return;
     if ((threadIdx.x & 31) == 0) s_sum[warp] = s;
     __syncthreads();
@@ -331,12 +331,11 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_codes_kernel(const floa
     // once a block, of a grid of one wave: in blocks of eight short rows the wait took most of the time (197307 x 57:
     // 87 us, so 32)
     grid_dependency_wait();
-    const float Q = __ldcg(&params[0].Q);
-    const int z = __ldcg(&params[0].z);
+    const UnitCoder unit(__ldcg(&params[0].Q), __ldcg(&params[0].z));
     for (int64_t b = blockIdx.x; b < groups; b += gridDim.x) {
         const int64_t row = (groups - 1 - b) * kRowWarps + (threadIdx.x >> 5);
         if (row >= rows) continue;
-        const int s = warp_row_codes<kVec, F>(x + row * ldx, cols, Q, z, codes + row * ldc);
+        const int s = warp_row_codes<kVec, F>(x + row * ldx, cols, unit, codes + row * ldc);
         if (sums && (threadIdx.x & 31) == 0) sums[row] = s;
     }
 }

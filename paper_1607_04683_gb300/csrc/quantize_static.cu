@@ -107,15 +107,14 @@ __global__ void __launch_bounds__(kStaticWarps * 32) static_codes_kernel(const f
                                                                         const qnn_qparams *__restrict__ params,
                                                                         int32_t *__restrict__ sums) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float Q = params[0].Q;
-    const int z = params[0].z;
+    const UnitCoder unit(params[0].Q, params[0].z);
     const int64_t r0 = (int64_t)blockIdx.x * kStaticRowsPerBlock + warp * kStaticRowsPerWarp;
     for (int64_t row = r0; row < r0 + kStaticRowsPerWarp && row < rows; ++row) {
         const float *xr = x + row * ldx;
         uint8_t *cr = codes + row * ldc;
         int s = 0;
         for (int k = lane; k < cols; k += 32) {
-            uint32_t c = quant_code(xr[k], Q, z);
+            uint32_t c = unit.code(xr[k]);
             cr[k] = (uint8_t)c;
             s += (int)c;
         }

@@ -21,12 +21,18 @@ def qnn():
     return q
 
 
-def check(qnn, x, ld, off, granularity):
+def check(qnn, x, ld, off, granularity, static=False):
     rows, cols = x.shape
     buf = torch.full((off + rows * ld,), float("nan"), device="cuda")
     v = buf[off:].reshape(rows, ld)[:, :cols]
     v.copy_(torch.from_numpy(x))
-    codes, params, sums = qnn.qnn_quantize(v, granularity)
+    if static:
+        codes, params, sums = (torch.empty(n, dtype=t, device="cuda") for n, t in (((rows, cols), torch.uint8), ((1, 4), torch.int32),
+                                                                                   (rows, torch.int32)))
+        assert qnn.lib().qnn_quantize_matrix_static(v.data_ptr(), rows, cols, ld, codes.data_ptr(), cols, params.data_ptr(),
+                                                    sums.data_ptr(), None, None) == qnn.QNN_OK
+    else:
+        codes, params, sums = qnn.qnn_quantize(v, granularity)
     assert qnn.device_status() == qnn.QNN_OK
     c, p, s = oracle.quantize(x, granularity)
     assert np.array_equal(codes.cpu().numpy(), c)
@@ -67,3 +73,24 @@ def test_non_finite_values_are_reported(qnn, rows, cols, value, granularity):
         assert qnn.device_status() == qnn.QNN_ERR_NONFINITE
     qnn.qnn_quantize(torch.from_numpy(x).cuda(), granularity)
     assert qnn.device_status() == qnn.QNN_OK
+
+
+# Units whose scale 255 / max|v| is infinite, of every sign and with zeros, among ordinary rows and alone: on each
+# kernel's widths.
+@pytest.mark.parametrize("form", ["rows", "matrix", "static"])
+@pytest.mark.parametrize("cols,pad,off", [(1, 0, 0), (60, 0, 0), (500, 0, 0), (1000, 4, 0), (57, 3, 1), (1500, 4, 0), (2100, 0, 0),
+                                          (2101, 0, 0)])
+@pytest.mark.parametrize("tiny", [7e-37, 1e-37, 1e-40, 1e-45])
+def test_units_of_infinite_scale(qnn, form, cols, pad, off, tiny):
+    g = np.random.Generator(np.random.PCG64(cols))
+    t = np.float32(tiny)
+    mixed = np.where(g.integers(0, 2, (3, cols)) == 1, t, -t).astype(np.float32)
+    kinds = [mixed, np.abs(mixed), -np.abs(mixed), mixed * g.integers(0, 2, (3, cols)).astype(np.float32),
+             np.abs(mixed) * g.integers(0, 2, (3, cols)).astype(np.float32), -np.abs(mixed) * g.integers(0, 2, (3, cols)).astype(np.float32)]
+    kinds = [k + np.float32(0) for k in kinds]  # (no negative zeros: the sign of a range's zero is not pinned)
+    if form == "rows":
+        x = np.concatenate([np.concatenate([k, values(1, cols, i)]) for i, k in enumerate(kinds)])
+        check(qnn, x, cols + pad, off, oracle.PER_ROW)
+        return
+    for k in kinds:
+        check(qnn, k, cols + pad, off, oracle.PER_MATRIX, static=form == "static")
