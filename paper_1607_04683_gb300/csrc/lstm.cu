@@ -799,6 +799,27 @@ extern "C" void qnn_lstm_model_destroy(qnn_lstm_model *m) {
     delete m;
 }
 
+namespace qnn {
+
+qnn_status model_alloc(qnn_lstm_model *m, void **p, size_t bytes, bool persist) {
+    const char *limit = std::getenv("QNN_MODEL_MEMORY");
+    for (int i = 0; i < 2; ++i) {
+        const size_t held = m->ws_bytes + m->sws_bytes + m->fws_bytes + m->tcw_bytes + m->pw_bytes + m->pws_bytes;
+        cudaError_t e = cudaErrorMemoryAllocation;
+        if (!limit || held + bytes <= std::strtoull(limit, nullptr, 10)) {
+            e = cudaMalloc(p, bytes);
+            if (e == cudaSuccess) return QNN_OK;
+            cudaGetLastError();
+        }
+        if (e != cudaErrorMemoryAllocation) return QNN_FAIL(QNN_ERR_CUDA);
+        if (persist || (!m->pw && !m->pws)) break;
+        persist_release(m);
+    }
+    return QNN_FAIL(QNN_ERR_NO_MEMORY);
+}
+
+}  // namespace qnn
+
 extern "C" qnn_status qnn_lstm_model_create(const qnn_lstm_desc *d, const float *params, qnn_lstm_model **out) {
     if (!out || !params || !valid_desc(d)) return QNN_ERR_INVALID_ARG;
     *out = nullptr;
@@ -1006,7 +1027,7 @@ qnn_status stack_input(qnn_lstm_model *m, const float *x, int64_t B, int64_t T, 
             m->fws = nullptr;
             m->fws_bytes = 0;
         }
-        QNN_CUDA_TRY(cudaMalloc(&m->fws, need));
+        QNN_TRY(model_alloc(m, &m->fws, need));
         m->fws_bytes = need;
     }
     char *w = reinterpret_cast<char *>(m->fws);
@@ -1053,8 +1074,12 @@ qnn_status forward_impl(qnn_lstm_model *m, const float *x, int64_t B, int64_t T,
     }
     if (choice == PathChoice::kPersist || (choice == PathChoice::kAuto && persist_preferred(m, B, y_map != nullptr))) {
         bool used = false;
-        QNN_TRY(persist_path_forward(m, x, B, T, y, logits, h_state, c_state, h_all, st, &used));
+        const qnn_status s = persist_path_forward(m, x, B, T, y, logits, h_state, c_state, h_all, st, &used);
         if (used) return QNN_OK;
+        // without the memory or the cooperative launch, another path may still take the call: the wavefront needs
+        // no such launch, and keeps only a chunk of the logits where the posteriors go to pinned host memory
+        const bool elsewhere = choice == PathChoice::kAuto && (s == QNN_ERR_NO_MEMORY || s == QNN_ERR_NO_COOP);
+        if (s != QNN_OK && !elsewhere) return s;
         if (choice == PathChoice::kPersist) return QNN_ERR_INVALID_ARG;
     }
     // recurrence: tensor cores for large batches, else the persistent integer-MMA kernel
@@ -1144,7 +1169,7 @@ qnn_status forward_impl(qnn_lstm_model *m, const float *x, int64_t B, int64_t T,
             m->ws = nullptr;
             m->ws_bytes = 0;
         }
-        QNN_CUDA_TRY(cudaMalloc(&m->ws, need));
+        QNN_TRY(model_alloc(m, &m->ws, need));
         m->ws_bytes = need;
     }
     char *ws = reinterpret_cast<char *>(m->ws);
@@ -1347,8 +1372,9 @@ qnn_status forward_impl(qnn_lstm_model *m, const float *x, int64_t B, int64_t T,
             a.ups = (int)m->S, a.cpu = (int)(H / m->S), a.ppu = P > 0 ? (int)(P / m->S) : 1;
             void *args[] = {&a};
             ProfScope prof("lstm_recurrent", st);
-            cudaError_t e = cudaLaunchCooperativeKernel((const void *)lstm_recurrent_kernel, dim3(plan.grid),
-                                                        dim3(kRecThreads), args, plan.smem, st);
+            cudaError_t e = coop_refused() ? cudaErrorCooperativeLaunchTooLarge
+                                           : cudaLaunchCooperativeKernel((const void *)lstm_recurrent_kernel, dim3(plan.grid),
+                                                                         dim3(kRecThreads), args, plan.smem, st);
             if (e == cudaErrorCooperativeLaunchTooLarge) {
                 cudaGetLastError();
                 return QNN_ERR_NO_COOP;

@@ -74,6 +74,7 @@ struct qnn_lstm_model {
     uint32_t epoch = 0;
     // fp16 weight copies of the tensor-core recurrence (made on first use)
     void *tcw = nullptr;
+    size_t tcw_bytes = 0;
     // streams of layers 1 .. L - 1 and events of the layer wavefront (made on first use)
     std::vector<cudaStream_t> wave_st;
     std::vector<cudaEvent_t> wave_ev;
@@ -89,6 +90,7 @@ struct qnn_lstm_model {
     // the persistent tensor-core stack's weights (made on first use), the 8-bit output layer's with them,
     // and its workspace
     void *pw = nullptr;
+    size_t pw_bytes = 0;
     __half *pw_wo16 = nullptr;
     std::vector<qnn::PersistWeights> pw_layers;
     void *pws = nullptr;
@@ -129,6 +131,7 @@ qnn_status small_stream_launch(const qnn_lstm_model *m, const SmallStreamArgs &s
 // Runs qnn_lstm_forward on the persistent tensor-core stack (lstm_persist.cu) if the model and batch
 // qualify (no projection, one unit per gate matrix, at most 256 sequences, a stack whose blocks fit the
 // SMs and their accumulators the tensor memory, persist_plan.h); *used tells whether it ran. Arguments as for qnn_lstm_forward_logits (logits nullable).
+// On QNN_ERR_NO_MEMORY and QNN_ERR_NO_COOP nothing has been written to the caller's buffers.
 qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, int64_t T, float *y, float *logits,
                                 float *h_state, float *c_state, float *h_all, cudaStream_t st, bool *used);
 // Whether that path is the better one where it qualifies (see there).
@@ -142,6 +145,12 @@ qnn_status quantize_rows_f16(const float *src, int64_t ld, int64_t rows, int64_t
 // The float output layer: Y [M][C] = X [M][K] Wt^T + bias in fp32 (lstm.cu).
 qnn_status launch_float_linear(const float *X, int64_t M, int64_t K, const float *Wt, int64_t C, const float *bias,
                                float *Y, cudaStream_t st);
+
+// Device memory for a buffer of the model. Where there is none left, what the persistent stack keeps (its weights'
+// copy and workspace, made again on use) is given back first, unless the buffer is one of them (`persist`).
+// QNN_MODEL_MEMORY bounds the bytes of a model's workspaces and weight copies together (tests).
+qnn_status model_alloc(qnn_lstm_model *m, void **p, size_t bytes, bool persist = false);
+void persist_release(qnn_lstm_model *m);
 
 // Which forward path to take, from the QNN_LSTM_PATH environment variable: "layerwise" (the
 // persistent integer-MMA recurrence), "tc" (the tensor-core recurrence), "persist" (the persistent

@@ -738,7 +738,8 @@ qnn_status launch(const PersistArgs &a, const Plan &p, int64_t L, cudaStream_t s
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, lstm_persist_kernel<NC, MT, SP>, a);
+    const cudaError_t e = coop_refused() ? cudaErrorCooperativeLaunchTooLarge
+                                         : cudaLaunchKernelEx(&cfg, lstm_persist_kernel<NC, MT, SP>, a);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         cudaGetLastError();
         return QNN_ERR_NO_COOP;
@@ -756,7 +757,7 @@ qnn_status prepare(qnn_lstm_model *m) {
     size_t bytes = quant_out ? m->C * kh * 2 : 0;
     for (int64_t l = 0; l < L; ++l) bytes += rows * (round_up(m->layers[l].kin, 64) + kh) * 2 + const_bytes;
     void *buf = nullptr;
-    QNN_CUDA_TRY(cudaMalloc(&buf, bytes));
+    QNN_TRY(model_alloc(m, &buf, bytes, true));
     char *w = reinterpret_cast<char *>(buf);
     qnn_status s = QNN_OK;
     std::vector<PersistWeights> pl((size_t)L);
@@ -783,11 +784,19 @@ qnn_status prepare(qnn_lstm_model *m) {
         cudaFree(buf);
         return s;
     }
-    m->pw = buf, m->pw_wo16 = wo, m->pw_layers = std::move(pl);
+    m->pw = buf, m->pw_bytes = bytes, m->pw_wo16 = wo, m->pw_layers = std::move(pl);
     return QNN_OK;
 }
 
 }  // namespace
+
+void persist_release(qnn_lstm_model *m) {
+    cudaDeviceSynchronize();
+    cudaFree(m->pw);
+    cudaFree(m->pws);
+    m->pw = m->pws = nullptr, m->pw_bytes = m->pws_bytes = 0;
+    m->pw_wo16 = nullptr, m->pw_layers.clear();
+}
 
 // Where the launch-per-step recurrences keep a stack that qualifies. Stacks gain from layers running side
 // by side in one launch (40 frames, this against the best other path, us: 5 x 500 B = 64 486 : 950, B = 256
@@ -846,7 +855,7 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
             QNN_CUDA_TRY(cudaFree(m->pws));
             m->pws = nullptr, m->pws_bytes = 0;
         }
-        QNN_CUDA_TRY(cudaMalloc(&m->pws, need));
+        QNN_TRY(model_alloc(m, &m->pws, need, true));
         m->pws_bytes = need;
     }
     char *const ws = reinterpret_cast<char *>(m->pws);

@@ -1020,7 +1020,7 @@ qnn_status small_path_forward(qnn_lstm_model *m, const float *x, int64_t B, int6
             m->sws = nullptr;
             m->sws_bytes = 0;
         }
-        QNN_CUDA_TRY(cudaMalloc(&m->sws, need));
+        QNN_TRY(model_alloc(m, &m->sws, need));
         QNN_CUDA_TRY(cudaMemset(m->sws, 0, need));  // tags 0 never match an epoch (epochs start at 1)
         m->sws_bytes = need;
     }

@@ -475,7 +475,7 @@ qnn_status tc_prepare(qnn_lstm_model *m) {
     const bool wo16 = m->C > 0 && m->d.output_mode == QNN_OUT_QUANT;
     if (wo16) bytes += (size_t)round_up(m->C * kh * 2, 256);
     void *buf = nullptr;
-    QNN_CUDA_TRY(cudaMalloc(&buf, bytes));
+    QNN_TRY(model_alloc(m, &buf, bytes));
     char *p = reinterpret_cast<char *>(buf);
     m->tc_layers.assign(m->L, TcLayer{});
     for (int64_t l = 0; l < m->L; ++l) {
@@ -543,7 +543,7 @@ qnn_status tc_prepare(qnn_lstm_model *m) {
         cudaFree(buf);
         return QNN_FAIL(QNN_ERR_CUDA);
     }
-    m->tcw = buf;
+    m->tcw = buf, m->tcw_bytes = bytes;
     return QNN_OK;
 }
 

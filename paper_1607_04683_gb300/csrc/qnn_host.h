@@ -4,6 +4,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <cuda_runtime.h>
 
 #include "../../include/qnn.h"
@@ -54,6 +55,12 @@ qnn_status status_word(int **out);
 
 // Streaming multiprocessor count of the current device (cached).
 int sm_count();
+
+// QNN_NO_COOP=1: cooperative launches are refused, as on a partition of a GPU too small for their grids (tests).
+inline bool coop_refused() {
+    const char *e = std::getenv("QNN_NO_COOP");
+    return e && std::strcmp(e, "1") == 0;
+}
 
 // While kernel timing is enabled (qnn_profile_enable), brackets the launches made during its
 // lifetime with CUDA events on `st`, accounted under `name` (a static string).

@@ -214,3 +214,75 @@ def test_replayed_graph(qnn):
         g.replay()
         torch.cuda.synchronize()
         parity.check_posteriors(y.cpu().numpy(), reference(wl, params, xk)["y"])
+
+
+# Where the persistent stack cannot run, automatic dispatch hands the call to the path that took it before.
+def test_refused_cooperative_launch(qnn, monkeypatch):
+    monkeypatch.delenv("QNN_LSTM_PATH")
+    monkeypatch.setenv("QNN_NO_COOP", "1")
+    wl = workload(L=2, H=64, B=70, C=12)
+    params, x = wl.make()
+    model = model_of(qnn, wl, params)
+    qnn.profile_read()
+    qnn.profile_enable(True)
+    got = forward(qnn, model, wl, x)
+    qnn.profile_enable(False)
+    assert "lstm_gates_tc" in qnn.profile_read()
+    check(qnn, wl, got, reference(wl, params, x), params)
+    with pytest.raises(qnn.QnnError) as e:  # the layerwise kernel's launch is cooperative too
+        model.forward(torch.from_numpy(x[:20]).cuda())
+    assert e.value.status == qnn.QNN_ERR_NO_COOP
+    monkeypatch.delenv("QNN_NO_COOP")
+    check(qnn, wl, forward(qnn, model, wl, x), reference(wl, params, x), params)
+
+
+def least_memory(qnn, monkeypatch, run):
+    """The least QNN_MODEL_MEMORY (to 1%) with which run() succeeds."""
+    lo, hi = 0, 1 << 28
+    while hi - lo > hi // 100:
+        mid = (lo + hi) // 2
+        monkeypatch.setenv("QNN_MODEL_MEMORY", str(mid))
+        try:
+            run()
+            hi = mid
+        except qnn.QnnError as e:
+            assert e.status == qnn.QNN_ERR_NO_MEMORY
+            lo = mid
+    monkeypatch.delenv("QNN_MODEL_MEMORY")
+    return hi
+
+
+def test_posteriors_that_fit_only_chunk_by_chunk(qnn, monkeypatch):
+    monkeypatch.setenv("QNN_OUT_CHUNK", "1")
+    wl = workload(L=2, H=64, B=130, T=8, C=2000)
+    params, x = wl.make()
+    xd = torch.from_numpy(x).cuda()
+    y = torch.empty((130, 8, 2000)).pin_memory()
+
+    def run(path):
+        monkeypatch.setenv("QNN_LSTM_PATH", path)
+        model_of(qnn, wl, params).forward(xd, y=y)
+        torch.cuda.synchronize()
+
+    least = {path: least_memory(qnn, monkeypatch, lambda: run(path)) for path in ("tc", "persist")}
+    assert 1.2 * least["tc"] < least["persist"]
+    run("persist")
+    ref = y.clone()
+    monkeypatch.setenv("QNN_MODEL_MEMORY", str((least["tc"] + least["persist"]) // 2))
+    y.fill_(float("nan"))
+    run("auto")
+    assert torch.equal(y, ref)  # (both sum a row's terms in one order)
+
+
+def test_memory_of_the_persistent_stack_is_given_back(qnn, monkeypatch):
+    monkeypatch.delenv("QNN_LSTM_PATH")
+    wl = workload(L=2, H=128, B=300, T=8)
+    params, x = wl.make()
+    xd = torch.from_numpy(x).cuda()
+    ref = model_of(qnn, wl, params).forward(xd)
+    least = least_memory(qnn, monkeypatch, lambda: model_of(qnn, wl, params).forward(xd))
+    model = model_of(qnn, wl, params)
+    monkeypatch.setenv("QNN_MODEL_MEMORY", str(least))
+    small = model.forward(xd[:100])  # the persistent stack
+    assert torch.equal(model.forward(xd), ref)  # the wavefront, whose buffers fit only without it
+    assert torch.equal(model.forward(xd[:100]), small)  # (on whichever has room)
