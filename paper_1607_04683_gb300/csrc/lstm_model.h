@@ -146,6 +146,9 @@ qnn_status quantize_rows_f16(const float *src, int64_t ld, int64_t rows, int64_t
 qnn_status launch_float_linear(const float *X, int64_t M, int64_t K, const float *Wt, int64_t C, const float *bias,
                                float *Y, cudaStream_t st);
 
+// Time-major rows (row t B + b of C values) to sequence-major ones (row b T + t), device or mapped memory (lstm.cu).
+qnn_status launch_rows_to_sequences(const float *src, int64_t B, int64_t T, int64_t C, float *dst, cudaStream_t st);
+
 // Device memory for a buffer of the model. Where there is none left, what the persistent stack keeps (its weights'
 // copy and workspace, made again on use) is given back first, unless the buffer is one of them (`persist`).
 // QNN_MODEL_MEMORY bounds the bytes of a model's workspaces and weight copies together (tests).

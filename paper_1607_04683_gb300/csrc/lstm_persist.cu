@@ -849,6 +849,9 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
     const size_t o_ha = (h_all && !ha_dev) ? acct(4 * L * rows * R) : 0;
     const size_t o_lg = C > 0 ? acct(4 * rows * C) : 0;
     const size_t o_y = (y_dev || y_map || C == 0) ? 0 : acct(4 * rows * ycols);
+    // logits in the caller's row order: written there, or staged for one copy to pageable memory
+    float *const lg_to = !logits || !quant_out ? nullptr : is_device_ptr(logits) ? logits : static_cast<float *>(host_mapped_ptr(logits));
+    const size_t o_ls = (logits && quant_out && !lg_to) ? acct(4 * rows * C) : 0;
     if (need > m->pws_bytes) {
         if (m->pws) {
             QNN_CUDA_TRY(cudaStreamSynchronize(st));
@@ -945,9 +948,10 @@ qnn_status persist_path_forward(qnn_lstm_model *m, const float *x, int64_t B, in
         QNN_TRY(tc_operands(&op, codes + (L - 1) * rows * kh, rows, m->pw_wo16, C, kh, tc_pick_bn(rows, C, kh)));
         QNN_TRY(tc_linear(op, prm + (L - 1) * rows, 1, rs + (L - 1) * rows, R, m->wo.params, C, m->wo.sums, m->bo, lg, C,
                           nullptr, st));
-        if (logits)
-            for (int64_t t = 0; t < T; ++t)
-                QNN_CUDA_TRY(cudaMemcpy2DAsync(logits + t * C, T * C * 4, lg + t * B * C, C * 4, C * 4, B, cudaMemcpyDefault, st));
+        if (logits) {
+            QNN_TRY(launch_rows_to_sequences(lg, B, T, C, lg_to ? lg_to : at(o_ls), st));
+            if (!lg_to) QNN_CUDA_TRY(cudaMemcpyAsync(logits, at(o_ls), 4 * rows * C, cudaMemcpyDeviceToHost, st));
+        }
         QNN_TRY(launch_softmax_rows(lg, rows, C, yd, st, B, T, 0));
     } else if (C > 0) {
         QNN_TRY(launch_float_linear(top, rows, R, m->wo_f, C, m->bo, lg, st));

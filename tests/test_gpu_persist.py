@@ -286,3 +286,24 @@ def test_memory_of_the_persistent_stack_is_given_back(qnn, monkeypatch):
     small = model.forward(xd[:100])  # the persistent stack
     assert torch.equal(model.forward(xd), ref)  # the wavefront, whose buffers fit only without it
     assert torch.equal(model.forward(xd[:100]), small)  # (on whichever has room)
+
+
+# Logits leave in one pass over them, whatever the frames, into any kind of buffer and at any alignment.
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable"])
+@pytest.mark.parametrize("B,T,C,off", [(1, 1, 1, 0), (5, 40, 7, 1), (20, 3, 300, 0), (40, 9, 12, 1), (130, 2, 64, 0)])
+def test_logits_in_sequence_order(qnn, B, T, C, off, where):
+    wl = workload(L=1 if B < 5 else 2, H=24, B=B, T=T, C=C)
+    params, x = wl.make()
+    buf = torch.full((off + B * T * C + 1,), 7.0, device="cuda" if where == "device" else "cpu")
+    buf = buf.pin_memory() if where == "pinned" else buf
+    lg = buf[off:-1].reshape(B, T, C)
+    model = model_of(qnn, wl, params)
+    xd, y = torch.from_numpy(x).cuda(), torch.empty((B, T, C), device="cuda")
+    qnn.profile_read()
+    qnn.profile_enable(True)
+    model.forward(xd, y=y, logits=lg)
+    torch.cuda.synchronize()
+    qnn.profile_enable(False)
+    assert qnn.profile_read()["rows_to_sequences"][0] == 1
+    assert np.array_equal(lg.cpu().numpy(), reference(wl, params, x)["logits"])
+    assert float(buf[-1]) == 7.0 and (off == 0 or float(buf[0]) == 7.0)
