@@ -23,9 +23,12 @@ namespace {
 
 constexpr int kRowWarps = 8;  // warps (rows) per block in the per-row kernels
 
-constexpr int kFlight = 8;    // 16-byte loads in flight per lane in the passes over rows of at least kMidRow values;
+constexpr int kFlight = 8;    // loads (of 16 bytes, or of one value where rows are not aligned) in flight per lane in the
+                              // passes over rows of at least kMidRow values (22002 x 2727: 174 us with one, so 101);
 constexpr int kMidRow = 512;  // shorter ones take one, and the registers of more rows at once (100000 x 60: range 28 us
-                              // with eight, 21 with one)
+                              // with eight, 21 with one); rows that are not aligned from kMidLoose values on (256410 x 234:
+                              // 178 us, so 108; 200000 x 95: 67 either way)
+constexpr int kMidLoose = 128;
 
 // Running range of values and whether one was not finite: v * 0 is NaN then, and so is the sum.
 struct Range {
@@ -59,7 +62,19 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
         }
         done = n4 << 2;
     }
-    for (int i = done + lane; i < cols; i += 32) r.add(__ldg(xr + i));
+    if (kVec || F == 1) {
+        for (int i = done + lane; i < cols; i += 32) r.add(__ldg(xr + i));
+    } else {
+        for (int i = lane; i < cols; i += 32 * F) {
+            float v[F];
+#pragma unroll
+            for (int u = 0; u < F; ++u)
+                if (i + 32 * u < cols) v[u] = __ldg(xr + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < F; ++u)
+                if (i + 32 * u < cols) r.add(v[u]);
+        }
+    }
     mn = warp_min(r.mn);
     mx = warp_max(r.mx);
     return __all_sync(0xffffffffu, r.finite());
@@ -95,10 +110,18 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
             cr[i] = (uint8_t)a;
         }
     } else {
-        for (int i = lane; i < cols; i += 32) {
-            uint32_t a = unit.code(__ldg(xr + i));
-            s += (int)a;
-            cr[i] = (uint8_t)a;
+        for (int i = lane; i < cols; i += 32 * F) {
+            float v[F];
+#pragma unroll
+            for (int u = 0; u < F; ++u)
+                if (i + 32 * u < cols) v[u] = __ldg(xr + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < F; ++u) {
+                if (i + 32 * u >= cols) break;
+                const uint32_t a = unit.code(v[u]);
+                s += (int)a;
+                cr[i + 32 * u] = (uint8_t)a;
+            }
         }
     }
     return warp_sum(s);
@@ -228,7 +251,8 @@ __global__ void __launch_bounds__(kRowWarps * 32, rows_reg_blocks(NV))
 }
 
 // Per-matrix pass 1: block partial ranges; the last block folds them into params[0]. The warps take segments
-// of kSegment values of the rows in turn (whole rows leave a last, nearly empty round).
+// of at most kSegment values of the rows in turn, a row's all of one length (whole rows leave a last, nearly empty
+// round).
 constexpr int kSegment = 2048;
 template <bool kVec, int F>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const float *__restrict__ x, int64_t rows,
@@ -243,17 +267,24 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     __syncthreads();
     float mn = FLT_MAX, mx = -FLT_MAX;
     grid_dependents_launch();
-    const int segs = (cols - 1) / kSegment + 1;
-    const int64_t items = rows * segs;
-    for (int64_t i = (int64_t)blockIdx.x * kRowWarps + warp; i < items; i += (int64_t)gridDim.x * kRowWarps) {
-        const int64_t row = segs == 1 ? i : i / segs;
-        const int k0 = (int)(i - row * segs) * kSegment;
+    const int segs = (cols - 1) / kSegment + 1, seg = ((cols + segs - 1) / segs + 3) & ~3;
+    auto add = [&](const float *xs, int n) {
         float a, b;
-        if (!warp_row_range<kVec, F>(x + row * ldx + k0, min(kSegment, cols - k0), a, b)) {
+        if (!warp_row_range<kVec, F>(xs, n, a, b)) {
             if (lane == 0) s_bad = 1;
         } else {
             mn = fminf(mn, a);
             mx = fmaxf(mx, b);
+        }
+    };
+    const int64_t first = (int64_t)blockIdx.x * kRowWarps + warp, step = (int64_t)gridDim.x * kRowWarps;
+    if (segs == 1) {
+        for (int64_t row = first; row < rows; row += step) add(x + row * ldx, cols);
+    } else {
+        for (int64_t i = first; i < rows * segs; i += step) {
+            const int64_t row = i / segs;
+            const int k0 = (int)(i - row * segs) * seg;
+            add(x + row * ldx + k0, min(seg, cols - k0));
         }
     }
     if (lane == 0) {
@@ -296,8 +327,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     }
 }
 
-// Per-matrix pass 2: codes and row sums with the single unit's parameters. Rows of at least kLongRow values
-// take a block each (contiguous parts of the row by warp), shorter ones a warp. Last rows first: the range
+// Per-matrix pass 2: codes and row sums with the single unit's parameters. Rows of at least kLongRow values,
+// four times as many where they are not aligned (a value a load then: 20000 x 2050 70 us by warps, 127 by blocks; 1000 x
+// 20001 40 by blocks, 72 by warps), take a block each (contiguous parts of the row by warp), shorter ones a warp. Last rows first: the range
 // pass read them last, so about an L2 of them is still there.
 constexpr int kLongRow = 2048;
 template <bool kVec>
@@ -328,8 +360,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_codes_kernel(const floa
                                                                      int64_t ldc, const qnn_qparams *__restrict__ params,
                                                                      int32_t *__restrict__ sums) {
     const int64_t groups = (rows + kRowWarps - 1) / kRowWarps;
-    // once a block, of a grid of one wave: in blocks of eight short rows the wait took most of the time (197307 x 57:
-    // 87 us, so 32)
+    // once a block, of a grid of two waves: in blocks of eight short rows the wait took most of the time (197307 x 57:
+    // 87 us, so 31), and with one wave the last rows' blocks leave warps idle (246038 x 24: 38 us, so 35)
     grid_dependency_wait();
     const UnitCoder unit(__ldcg(&params[0].Q), __ldcg(&params[0].z));
     for (int64_t b = blockIdx.x; b < groups; b += gridDim.x) {
@@ -368,8 +400,10 @@ qnn_status launch_quantize_rows(const float *x, int64_t rows, int64_t cols, int6
         }
     } else if (vec_ok(x, ldx, codes, ldc))
         quantize_rows_kernel<true, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
-    else
+    else if (cols < kMidLoose)
         quantize_rows_kernel<false, 1><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+    else
+        quantize_rows_kernel<false, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
     QNN_CUDA_TRY(cudaGetLastError());
     return QNN_OK;
 }
@@ -383,13 +417,15 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     const int64_t range = (rows * ((cols - 1) / kSegment + 1) + kRowWarps - 1) / kRowWarps;
     const unsigned nb = (unsigned)(range < max_blocks ? range : max_blocks);
     const bool v = vec_ok(x, ldx, codes, ldc);
+    const bool mid = cols >= (v ? kMidRow : kMidLoose);
     {
     ProfScope prof("quantize_matrix_range", st);
-    const bool mid = cols >= kMidRow;
     if (v && mid)
         matrix_range_kernel<true, kFlight><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     else if (v)
         matrix_range_kernel<true, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
+    else if (mid)
+        matrix_range_kernel<false, kFlight><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     else
         matrix_range_kernel<false, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     QNN_CUDA_TRY(cudaGetLastError());
@@ -397,8 +433,8 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     ProfScope prof("quantize_matrix_codes", st);
     // programmatic dependent launch: the blocks are set up while the range pass ends (they wait for it)
     cudaLaunchConfig_t cfg = {};
-    const bool long_rows = cols >= kLongRow && rows <= INT32_MAX;
-    cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, 8 * (int64_t)sm_count())));
+    const bool long_rows = cols >= (v ? kLongRow : 4 * kLongRow) && rows <= INT32_MAX;
+    cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, 16 * (int64_t)sm_count())));
     cfg.blockDim = dim3(kRowWarps * 32);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -410,8 +446,10 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
         QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, v ? matrix_long_rows_kernel<true> : matrix_long_rows_kernel<false>, x, (int)cols, ldx,
                                         codes, ldc, (const qnn_qparams *)params, sums));
     else
-        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, !v ? matrix_codes_kernel<false, 1> : cols >= kMidRow ? matrix_codes_kernel<true, kFlight> : matrix_codes_kernel<true, 1>, x, rows, (int)cols,
-                                        ldx, codes, ldc, (const qnn_qparams *)params, sums));
+        QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg,
+                                        v ? (mid ? matrix_codes_kernel<true, kFlight> : matrix_codes_kernel<true, 1>)
+                                          : (mid ? matrix_codes_kernel<false, kFlight> : matrix_codes_kernel<false, 1>),
+                                        x, rows, (int)cols, ldx, codes, ldc, (const qnn_qparams *)params, sums));
     return QNN_OK;
 }
 

@@ -54,7 +54,8 @@ def test_rows(qnn, rows, cols, pad, off):
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 1), (3, 2047), (8, 2048), (9, 2049), (700, 2052), (130, 4099), (5, 16384), (3000, 40),
-                                       (1, 100001), (513, 2500), (20001, 57), (15000, 511), (10003, 512)])
+                                       (1, 100001), (513, 2500), (20001, 57), (15000, 511), (10003, 512),
+                                       (3, 8191), (4, 8192), (5, 8193), (600, 2727), (2, 4097), (70000, 17)])
 @pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
 def test_matrix(qnn, rows, cols, pad, off):
     g = np.random.Generator(np.random.PCG64(rows * 7 + cols))
