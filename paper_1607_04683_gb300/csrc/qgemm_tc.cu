@@ -44,7 +44,7 @@ constexpr int KCHUNK = 1024;                      // exact fp32 accumulation bou
 constexpr unsigned long long TC_WAIT_NS = 2000000000ull;
 
 // kEpiLinear: recovered product, any K (chunked drains), outputs staged through shared memory.
-// kEpiRow: recovered product for K <= 1024, one output row per lane, two blocks per SM.
+// kEpiRow: recovered product for K <= 1024, one output row per lane.
 // kEpiLstm: the LSTM cell update on gate-interleaved columns, K <= 1024. (Issuing its input-product
 // and cell-state loads before the accumulator wait was measured slower even for single-tile grids:
 // those HBM loads delay the tile's TMA stream.)
@@ -797,14 +797,14 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // The usual tile: every warp takes a quarter of the columns of its 32 rows; when they lie in one
-            // weight unit (and no raw products are wanted) the outputs go through the warp's staging buffer,
-            // swizzled so that neither side conflicts, and out as whole row segments, one TMA store where Y has a
-            // map and a row an instruction where it does not (8000 x 2001 x 500: 99 us, so 77). (Stored
+            // weight unit the outputs go through the warp's staging buffer, swizzled so that neither side conflicts, and
+            // out as whole row segments, one TMA store where Y has a map and a row an instruction where it does not
+            // (8000 x 2001 x 500: 99 us, so 77) and for raw products (16384 x 8192 x 512 with both 1890 us, so 545). (Stored
             // from registers, one 16-byte piece of 32 different rows an instruction, they take most of the
             // epilogue's time: 128000 x 2000 x 500 535 us, so 389; 102400 x 8192 x 512 1884 us, so 1343.)
             constexpr int RC = TL::ROW_COLS;
             const int cq = part * RC;
-            const bool staged = args.Y && !args.acc_out && cu[cq].unit >= 0 && cu[cq].unit == cu[cq + RC - 1].unit;
+            const bool staged = args.Y && cu[cq].unit >= 0 && cu[cq].unit == cu[cq + RC - 1].unit;
             if (staged && !failed) {
                 uint32_t r[RC];
                 if constexpr (RC == 32)
@@ -833,6 +833,21 @@ __global__ void __launch_bounds__((Tile<BN, EPI>::THREADS)) __maxnreg__((Tile<BN
                     row_block_fast<false>(r, cc + cq, rt, za128, den, put);
                 }
                 store_staged<RC>(stg, &mapPX, args.y_map, args.Y, args.ldy, m0 + 32 * q, n0 + cq, args.M);
+                if (args.acc_out) {  // raw code products, by the same buffer and plain stores
+                    if (args.y_map) {
+                        if (lane == 0) bulk_wait_read();
+                        __syncwarp();
+                    }
+                    const int base = 128 * ra - 16384 * K;
+#pragma unroll
+                    for (int i = 0; i < RC / 4; ++i) {
+                        int o[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[e] = f32_integer_to_s32(__uint_as_float(r[4 * i + e])) + base + 128 * cc[cq + 4 * i + e].cs;
+                        put(i, make_float4(__int_as_float(o[0]), __int_as_float(o[1]), __int_as_float(o[2]), __int_as_float(o[3])));
+                    }
+                    store_staged<RC>(stg, nullptr, false, reinterpret_cast<float *>(args.acc_out), args.N, m0 + 32 * q, n0 + cq, args.M);
+                }
             }
 #pragma unroll 1
             for (int j = part * (RC / 16); j < (part + 1) * (RC / 16) && !failed && !staged; ++j) {

@@ -144,6 +144,27 @@ def test_codes_bit_exact(qnn, M, N, K, pad, off, shift, monkeypatch):
     assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
 
 
+# Raw sums beside the tensor-core product's outputs for K <= 1024: tiles of 64 and 128 columns, rows of sums of any
+# alignment (N odd), ragged tiles, columns of several weight units, outputs by TMA and by plain stores.
+@pytest.mark.parametrize("bn", ["64", "128"])
+@pytest.mark.parametrize("M,N,K,nb,pad", [(1, 8, 1, 1, 0), (33, 64, 64, 4, 0), (130, 261, 100, 1, 0), (257, 2000, 500, 4, 8), (200, 135, 1000, 3, 1),
+                                          (384, 513, 1024, 1, 0), (129, 2001, 32, 1, 0)])
+def test_tensor_core_raw_sums(qnn, M, N, K, nb, pad, bn, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "tc")
+    monkeypatch.setenv("QNN_TC_BN", bn)
+    g = np.random.Generator(np.random.PCG64(M + N + K))
+    ca, pa, ra = oracle.quantize(g.uniform(0, 1, (M, K)).astype(np.float32), oracle.PER_ROW)
+    parts = [oracle.quantize(g.uniform(-s, s, (N // nb, K)).astype(np.float32), oracle.PER_MATRIX) for s in np.linspace(0.05, 0.4, nb)]
+    cw, pw, cs = (np.concatenate([p[i] for p in parts]) for i in range(3))
+    ref = oracle.qmatmul(ca, pa, oracle.PER_ROW, cw, pw, n_blocks=nb)
+    out = torch.full((M + 1, N + pad), 7.0, device="cuda")
+    _, acc = qnn.qnn_qmatmul(gpu(ca), qnn.params_tensor(pa), oracle.PER_ROW, gpu(ra), gpu(cw), qnn.params_tensor(pw), gpu(cs),
+                             n_blocks=nb, want_acc=True, out=out[:M, :N])
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"]) and np.array_equal(out[:M, :N].cpu().numpy(), ref["y"])
+    assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
+
+
 # Operands too small to hold one aligned unit take another path than the one the sizes ask for.
 @pytest.mark.parametrize("M,N,K", [(130, 1, 1), (200, 2, 15), (129, 1, 30), (128, 1, 31)])
 @pytest.mark.parametrize("off", [0, 1, 15])
