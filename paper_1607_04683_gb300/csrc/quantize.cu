@@ -26,9 +26,10 @@ constexpr int kRowWarps = 8;  // warps (rows) per block in the per-row kernels
 constexpr int kFlight = 8;    // loads (of 16 bytes, or of one value where rows are not aligned) in flight per lane in the
                               // passes over rows of at least kMidRow values (22002 x 2727: 174 us with one, so 101);
 constexpr int kMidRow = 512;  // shorter ones take one, and the registers of more rows at once (100000 x 60: range 28 us
-                              // with eight, 21 with one); rows that are not aligned from kMidLoose values on (256410 x 234:
-                              // 178 us, so 108; 200000 x 95: 67 either way)
-constexpr int kMidLoose = 128;
+                              // with eight, 21 with one)
+// Rows that are not aligned, a value a load: eight in flight from 128 values on, four from 64 (per matrix, one, four and
+// eight: 200000 x 65 57, 51 and 60 us, x 95 67, 57 and 65; 150000 x 129 60, 63 and 54, 256410 x 234 178, 133 and 108).
+inline int loose_flight(int64_t cols) { return cols >= 128 ? kFlight : cols >= 64 ? 4 : 1; }
 
 // Running range of values and whether one was not finite: v * 0 is NaN then, and so is the sum.
 struct Range {
@@ -327,11 +328,12 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_range_kernel(const floa
     }
 }
 
-// Per-matrix pass 2: codes and row sums with the single unit's parameters. Rows of at least kLongRow values,
-// four times as many where they are not aligned (a value a load then: 20000 x 2050 70 us by warps, 127 by blocks; 1000 x
-// 20001 40 by blocks, 72 by warps), take a block each (contiguous parts of the row by warp), shorter ones a warp. Last rows first: the range
-// pass read them last, so about an L2 of them is still there.
-constexpr int kLongRow = 2048;
+// Per-matrix pass 2: codes and row sums with the single unit's parameters. Rows of at least kLongRow values
+// take a block each (contiguous parts of the row by warp), shorter ones a warp (16384 x 2048: 45 us by warps, 83 by
+// blocks; 10000 x 6200 85 and 91; but 4096 x 8192 49 and 48, 100 x 100000 59 and 27; not aligned, a value a load, 20000 x
+// 2050 70 and 127, 1000 x 20001 72 and 40). Last rows first: the range pass read them last, so about an L2 of them is
+// still there.
+constexpr int kLongRow = 8192;
 template <bool kVec>
 __global__ void __launch_bounds__(kRowWarps * 32) matrix_long_rows_kernel(const float *__restrict__ x, int cols, int64_t ldx,
                                                                          uint8_t *__restrict__ codes, int64_t ldc,
@@ -400,10 +402,11 @@ qnn_status launch_quantize_rows(const float *x, int64_t rows, int64_t cols, int6
         }
     } else if (vec_ok(x, ldx, codes, ldc))
         quantize_rows_kernel<true, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
-    else if (cols < kMidLoose)
-        quantize_rows_kernel<false, 1><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
-    else
-        quantize_rows_kernel<false, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+    else {
+        const int f = loose_flight(cols);
+        const auto kern = f == kFlight ? quantize_rows_kernel<false, kFlight> : f == 4 ? quantize_rows_kernel<false, 4> : quantize_rows_kernel<false, 1>;
+        kern<<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+    }
     QNN_CUDA_TRY(cudaGetLastError());
     return QNN_OK;
 }
@@ -417,23 +420,20 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     const int64_t range = (rows * ((cols - 1) / kSegment + 1) + kRowWarps - 1) / kRowWarps;
     const unsigned nb = (unsigned)(range < max_blocks ? range : max_blocks);
     const bool v = vec_ok(x, ldx, codes, ldc);
-    const bool mid = cols >= (v ? kMidRow : kMidLoose);
+    const int f = !v ? loose_flight(cols) : cols >= kMidRow ? kFlight : 1;
     {
     ProfScope prof("quantize_matrix_range", st);
-    if (v && mid)
-        matrix_range_kernel<true, kFlight><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
-    else if (v)
-        matrix_range_kernel<true, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
-    else if (mid)
-        matrix_range_kernel<false, kFlight><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
-    else
-        matrix_range_kernel<false, 1><<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
+    const auto kern = v ? (f == kFlight ? matrix_range_kernel<true, kFlight> : matrix_range_kernel<true, 1>)
+                        : (f == kFlight ? matrix_range_kernel<false, kFlight>
+                           : f == 4     ? matrix_range_kernel<false, 4>
+                                        : matrix_range_kernel<false, 1>);
+    kern<<<nb, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, partials, counter, params, status);
     QNN_CUDA_TRY(cudaGetLastError());
     }
     ProfScope prof("quantize_matrix_codes", st);
     // programmatic dependent launch: the blocks are set up while the range pass ends (they wait for it)
     cudaLaunchConfig_t cfg = {};
-    const bool long_rows = cols >= (v ? kLongRow : 4 * kLongRow) && rows <= INT32_MAX;
+    const bool long_rows = cols >= kLongRow && rows <= INT32_MAX;
     cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, 16 * (int64_t)sm_count())));
     cfg.blockDim = dim3(kRowWarps * 32);
     cfg.stream = st;
@@ -447,8 +447,10 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
                                         codes, ldc, (const qnn_qparams *)params, sums));
     else
         QNN_CUDA_TRY(cudaLaunchKernelEx(&cfg,
-                                        v ? (mid ? matrix_codes_kernel<true, kFlight> : matrix_codes_kernel<true, 1>)
-                                          : (mid ? matrix_codes_kernel<false, kFlight> : matrix_codes_kernel<false, 1>),
+                                        v ? (f == kFlight ? matrix_codes_kernel<true, kFlight> : matrix_codes_kernel<true, 1>)
+                                          : (f == kFlight ? matrix_codes_kernel<false, kFlight>
+                                             : f == 4     ? matrix_codes_kernel<false, 4>
+                                                          : matrix_codes_kernel<false, 1>),
                                         x, rows, (int)cols, ldx, codes, ldc, (const qnn_qparams *)params, sums));
     return QNN_OK;
 }

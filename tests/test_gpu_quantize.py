@@ -47,7 +47,8 @@ def values(rows, cols, seed):
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 1), (7, 127), (9, 128), (5, 129), (3000, 256), (2500, 260), (20000, 500), (9000, 512),
-                                       (9001, 516), (5000, 1000), (17, 1024), (33, 1028), (4, 4100)])
+                                       (9001, 516), (5000, 1000), (17, 1024), (33, 1028), (4, 4100), (50, 63),
+                                       (50, 64), (50, 97)])
 @pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
 def test_rows(qnn, rows, cols, pad, off):
     check(qnn, values(rows, cols, rows + cols), cols + pad, off, oracle.PER_ROW)
@@ -55,7 +56,7 @@ def test_rows(qnn, rows, cols, pad, off):
 
 @pytest.mark.parametrize("rows,cols", [(1, 1), (3, 2047), (8, 2048), (9, 2049), (700, 2052), (130, 4099), (5, 16384), (3000, 40),
                                        (1, 100001), (513, 2500), (20001, 57), (15000, 511), (10003, 512),
-                                       (3, 8191), (4, 8192), (5, 8193), (600, 2727), (2, 4097), (70000, 17)])
+                                       (3, 8191), (4, 8192), (5, 8193), (600, 2727), (2, 4097), (70000, 17), (90, 63), (90, 65), (4000, 119)])
 @pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
 def test_matrix(qnn, rows, cols, pad, off):
     g = np.random.Generator(np.random.PCG64(rows * 7 + cols))
