@@ -23,6 +23,18 @@ def qnn():
     return q
 
 
+def test_quantizer_after_the_wait(qnn):
+    # the wait's result word is not the quantizer's block counter: units of one block would never be written
+    x = torch.arange(8, dtype=torch.float32, device="cuda").reshape(2, 4)
+    before = qnn.qnn_quantize(x, qnn.PER_MATRIX)
+    qnn.selftest_wait_timeout(1000)
+    assert qnn.device_status() == qnn.QNN_ERR_TIMEOUT
+    codes, params, sums = qnn.qnn_quantize(x, qnn.PER_MATRIX)
+    ref = oracle.quantize(x.cpu().numpy(), oracle.PER_MATRIX)
+    assert np.array_equal(codes.cpu().numpy(), ref[0]) and np.array_equal(sums.cpu().numpy(), ref[2])
+    assert torch.equal(codes, before[0]) and torch.equal(params, before[1])
+
+
 def test_bounded_wait_gives_up_and_reports(qnn):
     t0 = time.perf_counter()
     qnn.selftest_wait_timeout(5_000_000)  # 5 ms
