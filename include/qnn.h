@@ -89,7 +89,8 @@ qnn_status qnn_device_status(void *stream);
  *   code_sums  out, nullable: [rows] int32, sum of each row's codes (used by the offset terms of
  *              eq. 1).
  * Non-finite values: the unit's codes are unspecified and QNN_ERR_NONFINITE is recorded.
- * Per-matrix quantization allocates a small library-owned scratch buffer on first use.
+ * Per-matrix quantization allocates a small library-owned scratch buffer on first use; calls on different
+ * streams have parts of their own.
  */
 qnn_status qnn_quantize(const float *x, int64_t rows, int64_t cols, int64_t ldx, int granularity,
                         uint8_t *codes, int64_t ldc, qnn_qparams *params, int32_t *code_sums, void *stream);
@@ -106,7 +107,9 @@ qnn_status qnn_quantize(const float *x, int64_t rows, int64_t cols, int64_t ldx,
  *         S = sum_k (A[m,k] + za)(W[n,k] + zw) = acc + zw*rsA[m] + za*csW[n] + K*za*zw and
  *         the fp32 operations (float)S, Qa*Qw, divide, add, each rounded once.
  *   acc_out [M x N] int32 out, nullable: acc[m,n] = sum_k A[m,k] W[n,k] (the 32-bit accumulator).
- * 1 <= K <= QNN_K_MAX.
+ * 1 <= K <= QNN_K_MAX. Large products take scratch for centered copies of both operands, 2 (M + N)
+ * (K rounded up to 64) bytes, from a pool of the library's on `stream`, so that calls on different streams
+ * never share it. The pool keeps the largest request so far, or 1 GiB, for later calls.
  */
 qnn_status qnn_qmatmul(const uint8_t *A, int64_t lda, const qnn_qparams *pa, int ga, const int32_t *rsA,
                        int64_t M, int64_t K, const uint8_t *W, int64_t ldw, const qnn_qparams *pw,

@@ -14,8 +14,11 @@ namespace {
 constexpr int kMaxDevices = 64;
 
 struct DeviceState {
-    void *scratch[kScratchCount] = {};
-    size_t scratch_bytes[kScratchCount] = {};
+    cudaMemPool_t pool = nullptr;
+    size_t pool_keeps = 0;
+    char *reduce = nullptr;  // kReduceStreams slots
+    unsigned long long reduce_stream[kReduceStreams] = {};
+    int reduce_streams = 0;
     int *status = nullptr;
     int sms = 0;
 };
@@ -51,24 +54,75 @@ void *host_mapped_ptr(void *p) {
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
 
-qnn_status scratch(ScratchSlot slot, size_t bytes, void **out) {
+qnn_status Scratch::take(size_t bytes, cudaStream_t st) {
     int dev = 0;
     QNN_TRY(current(&dev));
-    std::lock_guard<std::mutex> lk(g_mu);
-    DeviceState &d = g_dev[dev];
-    if (d.scratch_bytes[slot] < bytes) {
-        if (d.scratch[slot]) {
-            QNN_CUDA_TRY(cudaDeviceSynchronize());
-            QNN_CUDA_TRY(cudaFree(d.scratch[slot]));
-            d.scratch[slot] = nullptr;
-            d.scratch_bytes[slot] = 0;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        DeviceState &d = g_dev[dev];
+        if (!d.pool) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            QNN_CUDA_TRY(cudaMemPoolCreate(&d.pool, &props));
         }
-        QNN_CUDA_TRY(cudaMalloc(&d.scratch[slot], bytes));
-        QNN_CUDA_TRY(cudaMemset(d.scratch[slot], 0, bytes));
-        d.scratch_bytes[slot] = bytes;
+        const size_t keeps = bytes > (size_t)1 << 30 ? bytes : (size_t)1 << 30;
+        if (keeps > d.pool_keeps) {
+            unsigned long long v = keeps;
+            QNN_CUDA_TRY(cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &v));
+            d.pool_keeps = keeps;
+        }
+        pool = d.pool;
     }
-    *out = d.scratch[slot];
+    QNN_CUDA_TRY(cudaMallocFromPoolAsync(&p_, bytes, pool, st));
+    pooled_ = true, st_ = st;
     return QNN_OK;
+}
+
+qnn_status Scratch::take_reduce(cudaStream_t st) {
+    int dev = 0;
+    QNN_TRY(current(&dev));
+    const size_t slot = kReduceHeader + (sizeof(float) * 2 * kReduceBlocks * (size_t)sm_count() + 255) / 256 * 256;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    QNN_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+        unsigned long long id = 0;  // (of the process's life: a later stream at the same address has another)
+        QNN_CUDA_TRY(cudaStreamGetId(st, &id));
+        std::lock_guard<std::mutex> lk(g_mu);
+        DeviceState &d = g_dev[dev];
+        int i = 0;
+        while (i < d.reduce_streams && d.reduce_stream[i] != id) ++i;
+        if (i < kReduceStreams) {
+            if (!d.reduce) {
+                void *p = nullptr;
+                QNN_CUDA_TRY(cudaMalloc(&p, slot * kReduceStreams));
+                if (cudaMemset(p, 0, slot * kReduceStreams) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+                    cudaFree(p);
+                    return QNN_FAIL(QNN_ERR_CUDA);
+                }
+                d.reduce = static_cast<char *>(p);
+            }
+            if (i == d.reduce_streams) d.reduce_stream[d.reduce_streams++] = id;
+            p_ = d.reduce + (size_t)i * slot;
+            return QNN_OK;
+        }
+    }
+    QNN_TRY(take(slot, st));
+    QNN_CUDA_TRY(cudaMemsetAsync(p_, 0, sizeof(unsigned), st));
+    return QNN_OK;
+}
+
+Scratch::~Scratch() {
+    if (pooled_ && cudaFreeAsync(p_, st_) != cudaSuccess) cudaGetLastError();
+}
+
+void scratch_trim() {
+    int dev = 0;
+    if (current(&dev) != QNN_OK) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (g_dev[dev].pool) cudaMemPoolTrimTo(g_dev[dev].pool, 0);
 }
 
 qnn_status status_word(int **out) {

@@ -843,8 +843,8 @@ qnn_status model_alloc(qnn_lstm_model *m, void **p, size_t bytes, bool persist) 
             cudaGetLastError();
         }
         if (e != cudaErrorMemoryAllocation) return QNN_FAIL(QNN_ERR_CUDA);
-        if (persist || (!m->pw && !m->pws)) break;
-        persist_release(m);
+        scratch_trim();
+        if (i == 0 && !persist && (m->pw || m->pws)) persist_release(m);
     }
     return QNN_FAIL(QNN_ERR_NO_MEMORY);
 }
@@ -891,8 +891,8 @@ extern "C" qnn_status qnn_lstm_model_create(const qnn_lstm_desc *d, const float 
     cudaStream_t s = nullptr;
     float *partials = nullptr;
     unsigned *counter = nullptr;
-    const int max_blocks = 4 * sm_count();
-    void *red = nullptr;
+    const int max_blocks = kReduceBlocks * sm_count();
+    Scratch red;
     if (cudaMalloc(&m->weights, bytes) != cudaSuccess) {
         delete m;
         return QNN_ERR_NO_MEMORY;
@@ -923,11 +923,8 @@ extern "C" qnn_status qnn_lstm_model_create(const qnn_lstm_desc *d, const float 
     }
     float *pdev = bp.take<float>(n_params);
     if (st == QNN_OK && cudaMemcpy(pdev, params, n_params * 4, cudaMemcpyDefault) != cudaSuccess) st = QNN_ERR_CUDA;
-    if (st == QNN_OK) st = scratch(kScratchReduce, 256 + sizeof(float) * 2 * (size_t)max_blocks, &red);
-    if (st == QNN_OK) {
-        counter = reinterpret_cast<unsigned *>(red);
-        partials = reinterpret_cast<float *>(reinterpret_cast<char *>(red) + 256);
-    }
+    if (st == QNN_OK) st = red.take_reduce(s);
+    if (st == QNN_OK) counter = red.counter(), partials = red.partials();
     const float *q = pdev;
     for (int64_t l = 0; l < L && st == QNN_OK; ++l) {
         LayerDev &ly = m->layers[l];

@@ -182,10 +182,10 @@ extern "C" qnn_status qnn_selftest_wait_timeout(int64_t limit_ns, void *stream) 
     if (limit_ns < 1000 || limit_ns > 1000000000) return QNN_ERR_INVALID_ARG;
     int *status = nullptr, *result = nullptr;
     QNN_TRY(qnn::status_word(&status));
-    void *scratch = nullptr;
-    QNN_TRY(qnn::scratch(qnn::kScratchReduce, 256, &scratch));
-    result = reinterpret_cast<int *>(scratch) + 32;  // (its first word is the per-matrix quantizer's block counter, kept 0)
     cudaStream_t st = qnn::as_stream(stream);
+    qnn::Scratch scratch;
+    QNN_TRY(scratch.take(sizeof(int), st));
+    result = static_cast<int *>(scratch.ptr());
     qnn::wait_timeout_kernel<<<1, 32, 0, st>>>(status, (unsigned long long)limit_ns, result);
     QNN_CUDA_TRY(cudaGetLastError());
     int r = 0;

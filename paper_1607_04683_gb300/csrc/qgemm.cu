@@ -253,10 +253,10 @@ qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, in
     if (path == kCodes)
         return launch_qgemm_codes(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out, st);
     if (path == kTc) {
-        void *ws = nullptr;
-        QNN_TRY(scratch(kScratchTc, tc_scratch_bytes(M, N, K), &ws));
-        return launch_qgemm_tc(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out, ws,
-                               st);
+        Scratch ws;
+        QNN_TRY(ws.take(tc_scratch_bytes(M, N, K), st));
+        return launch_qgemm_tc(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out,
+                               ws.ptr(), st);
     }
     return launch_qgemm_imma(A, lda, pa, ga, rsA, M, K, W, ldw, pw, rows_per_block, csW, N, bias, Y, ldy, acc_out, st);
 }

@@ -46,9 +46,36 @@ bool is_device_ptr(const void *p);
 // write a host output through it send each byte over the host link once, with no staging copy.
 void *host_mapped_ptr(void *p);
 
-// Library-owned, grow-only device scratch of the current device (one slot per purpose).
-enum ScratchSlot { kScratchReduce = 0, kScratchTc = 1, kScratchCount = 2 };
-qnn_status scratch(ScratchSlot slot, size_t bytes, void **out);
+// Device scratch of one call on one stream of the current device, never shared with a call that may run at the
+// same time: calls on other streams, and replays of a captured graph, have their own.
+//   take():        from a pool of the library's on the stream's order, given back to it at the end of the scope. The
+//                  pool keeps the largest request, or 1 GiB; what concurrent calls took beyond is freed at a
+//                  synchronization.
+//   take_reduce(): the per-matrix quantizer's block partials (kReduceBlocks of them an SM at most) behind a counter that
+//                  is 0, and that the kernel leaves 0: a slot of the stream's own, for the first kReduceStreams
+//                  streams, or memory as above with the counter cleared on the stream.
+// In a capture both are allocation nodes of the graph.
+constexpr int kReduceBlocks = 4, kReduceStreams = 64;
+constexpr size_t kReduceHeader = 256;
+class Scratch {
+  public:
+    Scratch() = default;
+    ~Scratch();
+    Scratch(const Scratch &) = delete;
+    Scratch &operator=(const Scratch &) = delete;
+    qnn_status take(size_t bytes, cudaStream_t st);
+    qnn_status take_reduce(cudaStream_t st);
+    void *ptr() const { return p_; }
+    unsigned *counter() const { return static_cast<unsigned *>(p_); }
+    float *partials() const { return reinterpret_cast<float *>(static_cast<char *>(p_) + kReduceHeader); }
+
+  private:
+    void *p_ = nullptr;
+    bool pooled_ = false;
+    cudaStream_t st_ = nullptr;
+};
+// Frees what the pool keeps on the current device and no call holds.
+void scratch_trim();
 
 // The device status word of the current device (allocated and zeroed on first use).
 qnn_status status_word(int **out);

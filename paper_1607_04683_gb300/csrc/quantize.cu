@@ -470,10 +470,8 @@ extern "C" qnn_status qnn_quantize(const float *x, int64_t rows, int64_t cols, i
         return QNN_ERR_INVALID_ARG;
     cudaStream_t st = as_stream(stream);
     if (granularity == QNN_PER_ROW) return launch_quantize_rows(x, rows, cols, ldx, codes, ldc, params, code_sums, st);
-    const int max_blocks = 4 * sm_count();
-    void *ws = nullptr;
-    QNN_TRY(scratch(kScratchReduce, 256 + sizeof(float) * 2 * (size_t)max_blocks, &ws));
-    unsigned *counter = reinterpret_cast<unsigned *>(ws);
-    float *partials = reinterpret_cast<float *>(reinterpret_cast<char *>(ws) + 256);
-    return launch_quantize_matrix(x, rows, cols, ldx, codes, ldc, params, code_sums, partials, counter, max_blocks, st);
+    Scratch ws;
+    QNN_TRY(ws.take_reduce(st));
+    return launch_quantize_matrix(x, rows, cols, ldx, codes, ldc, params, code_sums, ws.partials(), ws.counter(),
+                                  kReduceBlocks * sm_count(), st);
 }
