@@ -2,9 +2,9 @@
 //
 // Two passes over each unit: a range pass (exact fp32 min/max, warp shuffles; non-finite values
 // flagged) and a code pass (eq. 2 with the unit's Q and z, four codes per 32-bit store, row code
-// sums). Per-row units (one frame of one sequence) take one warp per row; rows of up to 1024
-// values stay in the warp's registers between the passes (read once), longer ones are re-read
-// from L1/L2. A per-matrix unit first reduces block partials into a small scratch array; the last
+// sums). Per-row units (one frame of one sequence) take one warp per row; aligned rows of up to 1024
+// values, and any of up to 256, stay in the warp's registers between the passes (read once), longer
+// ones are re-read from L1/L2. A per-matrix unit first reduces block partials into a small scratch array; the last
 // block to finish folds them into the unit's parameters, then a second launch writes codes.
 //
 // Bound: HBM (5 bytes a value for rows, 9 for a matrix beyond L2). Per matrix 8192 x 8192: 117 us with one
@@ -27,7 +27,7 @@ constexpr int kFlight = 8;    // loads (of 16 bytes, or of one value where rows 
                               // passes over rows of at least kMidRow values (22002 x 2727: 174 us with one, so 101);
 constexpr int kMidRow = 512;  // shorter ones take one, and the registers of more rows at once (100000 x 60: range 28 us
                               // with eight, 21 with one)
-// Rows that are not aligned, a value a load: eight in flight from 128 values on, four from 64 (per matrix, one, four and
+// Matrix rows that are not aligned, a value a load: eight in flight from 128 values on, four from 64 (one, four and
 // eight: 200000 x 65 57, 51 and 60 us, x 95 67, 57 and 65; 150000 x 129 60, 63 and 54, 256410 x 234 178, 133 and 108).
 inline int loose_flight(int64_t cols) { return cols >= 128 ? kFlight : cols >= 64 ? 4 : 1; }
 
@@ -128,6 +128,50 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
     return warp_sum(s);
 }
 
+// Per-row units of at most 32 N values, a warp a row, N values a lane in registers: short rows of any alignment, and
+// those of up to 256 values that are not aligned. (200000 x 40 by the passes of the kernel below 46 us, so 32; 100000 x 201
+// 31 and 28; aligned, by the kernel after it with one float4 a lane, x 32 49 us, so 29, x 128 44 and 41.)
+template <int N>
+__global__ void __launch_bounds__(kRowWarps * 32) quantize_short_rows_kernel(const float *__restrict__ x, int64_t rows, int cols,
+                                                                            int64_t ldx, uint8_t *__restrict__ codes, int64_t ldc,
+                                                                            qnn_qparams *__restrict__ params,
+                                                                            int32_t *__restrict__ sums, int *status) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = (int64_t)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+    if (row >= rows) return;
+    const float *xr = x + row * ldx + lane;
+    float v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (lane + 32 * i < cols) v[i] = __ldg(xr + 32 * i);
+    Range r;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (lane + 32 * i < cols) r.add(v[i]);
+    float mn = warp_min(r.mn), mx = warp_max(r.mx);
+    if (!__all_sync(0xffffffffu, r.finite())) {
+        if (lane == 0) record_status(status, QNN_ERR_NONFINITE);
+        mn = 0.0f;
+        mx = 0.0f;
+    }
+    const qnn_qparams p = params_from_range(mn, mx);
+    const UnitCoder unit(p.Q, p.z);
+    uint8_t *cr = codes + row * ldc + lane;
+    int s = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (lane + 32 * i < cols) {
+            const uint32_t a = unit.code(v[i]);
+            s += (int)a;
+            cr[32 * i] = (uint8_t)a;
+        }
+    s = warp_sum(s);
+    if (lane == 0) {
+        params[row] = p;
+        if (sums) sums[row] = s;
+    }
+}
+
 template <bool kVec, int F>
 __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const float *__restrict__ x, int64_t rows,
                                                                       int cols, int64_t ldx, uint8_t *__restrict__ codes,
@@ -151,7 +195,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
     }
 }
 
-// Per-row units of at most 1024 values (16-byte aligned input rows): the warp holds its row in
+// Per-row units of 129 to 1024 values (16-byte aligned input rows): the warp holds its row in
 // registers, NV float4 per lane, so the row is read once and the code pass needs no second read. A warp
 // takes every gridDim kRowWarps-th row, and rows of at most 512 values are loaded while the row before is
 // reduced and coded: the loads of one row alone leave memory idle through its reductions (128000 x 500:
@@ -174,7 +218,7 @@ __device__ __forceinline__ void load_row(float4 (&v)[NV], const float *__restric
 }
 
 // Blocks per SM the registers leave room for.
-constexpr int rows_reg_blocks(int NV) { return NV <= 1 ? 7 : NV <= 2 ? 5 : NV <= 4 ? 4 : 3; }
+constexpr int rows_reg_blocks(int NV) { return NV <= 2 ? 5 : NV <= 4 ? 4 : 3; }
 
 template <int NV>
 __global__ void __launch_bounds__(kRowWarps * 32, rows_reg_blocks(NV))
@@ -390,23 +434,25 @@ qnn_status launch_quantize_rows(const float *x, int64_t rows, int64_t cols, int6
     ProfScope prof("quantize_rows", st);
     const int nv = (int)((cols + 127) / 128);  // float4 per lane for a register-resident row
     const bool x_ok = ((reinterpret_cast<uintptr_t>(x) & 15) == 0) && (ldx % 4 == 0);
-    if (x_ok && nv <= 8) {
+    if (cols <= 128 || (!x_ok && cols <= 256)) {
+        const auto kern = cols <= 32    ? quantize_short_rows_kernel<1>
+                          : cols <= 64  ? quantize_short_rows_kernel<2>
+                          : cols <= 128 ? quantize_short_rows_kernel<4>
+                                        : quantize_short_rows_kernel<8>;
+        kern<<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
+    } else if (x_ok && nv <= 8) {
         const bool pack = ((reinterpret_cast<uintptr_t>(codes) & 3) == 0) && (ldc % 4 == 0);
-        const int r = nv <= 1 ? 1 : nv <= 2 ? 2 : nv <= 4 ? 4 : 8;
+        const int r = nv <= 2 ? 2 : nv <= 4 ? 4 : 8;
         grid.x = std::min<unsigned>(grid.x, (unsigned)(sm_count() * rows_reg_blocks(r)));  // one wave
         switch (r) {
-            case 1: quantize_rows_reg_kernel<1><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
             case 2: quantize_rows_reg_kernel<2><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
             case 4: quantize_rows_reg_kernel<4><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
             default: quantize_rows_reg_kernel<8><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status, pack); break;
         }
     } else if (vec_ok(x, ldx, codes, ldc))
         quantize_rows_kernel<true, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
-    else {
-        const int f = loose_flight(cols);
-        const auto kern = f == kFlight ? quantize_rows_kernel<false, kFlight> : f == 4 ? quantize_rows_kernel<false, 4> : quantize_rows_kernel<false, 1>;
-        kern<<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
-    }
+    else
+        quantize_rows_kernel<false, kFlight><<<grid, kRowWarps * 32, 0, st>>>(x, rows, (int)cols, ldx, codes, ldc, params, sums, status);
     QNN_CUDA_TRY(cudaGetLastError());
     return QNN_OK;
 }

@@ -48,7 +48,7 @@ def values(rows, cols, seed):
 
 @pytest.mark.parametrize("rows,cols", [(1, 1), (7, 127), (9, 128), (5, 129), (3000, 256), (2500, 260), (20000, 500), (9000, 512),
                                        (9001, 516), (5000, 1000), (17, 1024), (33, 1028), (4, 4100), (50, 63),
-                                       (50, 64), (50, 97)])
+                                       (50, 64), (50, 97), (40, 31), (41, 32), (42, 33), (30, 65), (70, 200), (60, 257)])
 @pytest.mark.parametrize("pad,off", [(0, 0), (4, 0), (3, 1)])
 def test_rows(qnn, rows, cols, pad, off):
     check(qnn, values(rows, cols, rows + cols), cols + pad, off, oracle.PER_ROW)
