@@ -591,6 +591,7 @@ struct TcLayerRun {
     bool split_proj = false, fused = false;
     int splits = 0;
     TcLstmInput xin;
+    TcStepMaps maps;
     const __half *x16 = nullptr;
     const qnn_qparams *xprm = nullptr;
     const int32_t *xrs = nullptr;
@@ -600,6 +601,13 @@ struct TcLayerRun {
     int *status = nullptr;
 };
 }  // namespace
+
+// Where the gate kernel of step t writes (and, unfused, its input products).
+static TcLstmOut step_out(const TcLayerRun &s, int64_t t) {
+    const int64_t H = s.m->H;
+    return TcLstmOut{s.fused ? nullptr : s.px + t * 4 * H, s.T * 4 * H, s.cbuf, s.m->P > 0 ? s.mbuf : s.out + t * s.out_t,
+                     s.m->P > 0 ? H : s.out_b, (int)H, (int)s.m->S, (int)(H / s.m->S)};
+}
 
 qnn_status tc_layer_begin(TcLayerRun &s, const float *h0, void *work, const TcFusedInput *fx, bool quantize_input) {
     const qnn_lstm_model *m = s.m;
@@ -669,6 +677,7 @@ qnn_status tc_layer_begin(TcLayerRun &s, const float *h0, void *work, const TcFu
         s.xin.x_pitch = tl.kx, s.xin.kx = tl.kx, s.xin.K_x = (int)fx->kin, s.xin.stride = 1;
         s.xin.wx16 = tl.wx16, s.xin.pw4 = ly.wx.params, s.xin.cs = ly.wx.sums, s.xin.bias = ly.bias;
         s.xin.colc = tl.colc;
+        QNN_TRY(tc_step_maps(&s.maps, s.gates, step_out(s, 0), s.xin));
     }
     QNN_TRY(launch_quantize_rows_f16(h0, R, B, R, kh, s.a16, s.prm, s.rs, s.status, false, s.st));
     return QNN_OK;
@@ -685,10 +694,10 @@ qnn_status tc_layer_step(TcLayerRun &s, int64_t t) {
     // the next layer's input codes of this step (wavefront), written with this step's own codes
     const RowCodes next{s.nx16 ? s.nx16 + t * B * kh : nullptr, s.nx16 ? s.nprm + t * B : nullptr,
                         s.nx16 ? s.nrs + t * B : nullptr};
-    TcLstmOut o{s.fused ? nullptr : s.px + t * 4 * H, T * 4 * H, s.cbuf, P > 0 ? s.mbuf : out_t, P > 0 ? H : s.out_b,
-                (int)H, (int)m->S, (int)(H / m->S)};
+    const TcLstmOut o = step_out(s, t);
     if (s.fused) {
         TcLstmInput xin = s.xin;
+        xin.maps = &s.maps;
         xin.x16 = s.x16 + t * B * tl.kx, xin.pa = s.xprm + t * B, xin.rs = s.xrs + t * B;
         QNN_TRY(tc_lstm_gates_x(s.gates, s.prm, s.rs, R, ly.wh.params, ly.wh.sums, o, xin, st));
     } else {

@@ -1689,6 +1689,14 @@ qnn_status tc_lstm_gates(const TcOperands &op, const qnn_qparams *pa, const int3
     return dispatch_lstm(op, a, st);
 }
 
+qnn_status tc_step_maps(TcStepMaps *maps, const TcOperands &op, const TcLstmOut &out, const TcLstmInput &in) {
+    QNN_TRY(make_map_f32(&maps->c, out.c, op.M, out.H, out.H, op.bn / 4, 32, op.bn));
+    QNN_TRY(make_map_f32(&maps->h, out.h, op.M, out.H, out.h_ld, op.bn / 4, 32, op.bn));
+    maps->h_of = out.h;
+    QNN_TRY(make_map_f32(&maps->col, reinterpret_cast<const float *>(in.colc), 12, out.H, out.H, op.bn / 4, 12));
+    return make_map(&maps->wx, in.wx16, op.N, in.kx, op.bn);
+}
+
 qnn_status tc_lstm_gates_x(const TcOperands &op, const qnn_qparams *pa, const int32_t *rsA, int64_t K,
                            const qnn_qparams *pw4, const int32_t *cs, const TcLstmOut &out, const TcLstmInput &in,
                            cudaStream_t st) {
@@ -1706,12 +1714,14 @@ qnn_status tc_lstm_gates_x(const TcOperands &op, const qnn_qparams *pa, const in
              1, kbh + kbx, nullptr, 0, 1};
     a.pa_x = in.pa, a.x_stride = in.stride, a.rsA_x = in.rs, a.pw_x = in.pw4, a.csW_x = in.cs, a.bias_x = in.bias;
     a.K_x = in.K_x, a.KB_x = kbx;
-    CUtensorMap map_c, map_h, map_ax, map_wx, map_col;
-    QNN_TRY(make_map_f32(&map_c, out.c, op.M, out.H, out.H, op.bn / 4, 32, op.bn));
-    QNN_TRY(make_map_f32(&map_h, out.h, op.M, out.H, out.h_ld, op.bn / 4, 32, op.bn));
-    QNN_TRY(make_map_f32(&map_col, reinterpret_cast<const float *>(in.colc), 12, out.H, out.H, op.bn / 4, 12));
+    if (!in.maps) return QNN_ERR_INVALID_ARG;
+    CUtensorMap map_h, map_ax;
+    const CUtensorMap &map_c = in.maps->c, &map_col = in.maps->col, &map_wx = in.maps->wx;
+    if (in.maps->h_of == out.h)
+        map_h = in.maps->h;
+    else
+        QNN_TRY(make_map_f32(&map_h, out.h, op.M, out.H, out.h_ld, op.bn / 4, 32, op.bn));
     QNN_TRY(make_map(&map_ax, in.x16, op.M, in.kx, TBM, in.x_pitch));
-    QNN_TRY(make_map(&map_wx, in.wx16, op.N, in.kx, op.bn));
     switch (op.bn) {
         case 32: return launch_tc<32, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx, &map_h);
         case 64: return launch_tc<64, kEpiLstmX>(op, a, "lstm_gates_tc", st, &map_col, &map_c, &map_ax, &map_wx, &map_h);

@@ -81,7 +81,17 @@ struct TcLstmInput {
     // of gates i f g o, rows 4-7 the Wx row code sums, rows 8-11 the Wh row code sums (integers below
     // 2^24, exact in fp32); 16-byte aligned, H a multiple of 4
     const void *colc = nullptr;
+    const struct TcStepMaps *maps = nullptr;  // of the steps of one run (tc_step_maps)
 };
+
+// The tensor maps that all steps of a layer's run share: the cell state, the column constants, Wx, and with a
+// projection (out.h the same buffer at every step) the cell outputs. Made once a run: a small layer's steps are
+// bound by the host (8 x 60 cells, 327 sequences, 89 frames: five map calls a step 3266 us, two 3177).
+struct TcStepMaps {
+    CUtensorMap c, col, wx, h;
+    const float *h_of = nullptr;  // the outputs h maps
+};
+qnn_status tc_step_maps(TcStepMaps *maps, const TcOperands &op, const TcLstmOut &out, const TcLstmInput &in);
 
 // One recurrent step's gate product and cell update: A = centered codes of h_{t-1} (one unit per
 // row: pa, rsA), W = the four Wh gate matrices interleaved in 8-cell groups [i f g o] x 8 rows
