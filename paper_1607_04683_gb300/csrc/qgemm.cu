@@ -238,7 +238,7 @@ qnn_status launch_qgemm(const uint8_t *A, int64_t lda, const qnn_qparams *pa, in
     const char *force = std::getenv("QNN_QGEMM");
     enum { kImma, kCodes, kTc } path = kTc;
     const int64_t sms = sm_count();
-    if (M < 128) {  // (neither takes scratch: such a call allocates nothing)
+    if (M < 128) {  // (neither takes scratch)
         path = M <= 32 || (K < 2048 && (M + 63) / 64 * ((N + 31) / 32) <= sms) ? kImma : kCodes;
     } else if ((M + 127) / 128 * ((N + 127) / 128) <= sms) {
         const uintptr_t at = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | (uintptr_t)lda | (uintptr_t)ldw;

@@ -428,7 +428,7 @@ qnn_status launch_codes_as(const CodeArgs &a, int64_t tiles, cudaStream_t st) {
         QNN_CUDA_TRY(cudaFuncSetAttribute(qgemm_codes_kernel<BN, SHIFT, SPLITK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         configured = dev;
     }
-    ProfScope prof("qgemm_codes", st);
+    ProfScope prof(SPLITK ? "qgemm_codes_split" : "qgemm_codes", st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * a.splits));
     cfg.blockDim = dim3(kThreads);
@@ -451,12 +451,16 @@ qnn_status launch_codes(CodeArgs &a, cudaStream_t st) {
     if (tiles > INT32_MAX) return QNN_FAIL(QNN_ERR_INVALID_ARG);
     a.tiles_m = (unsigned)tm;
     // a tile's reduction over the blocks of a cluster, up to 8 of at least four stages, while they find SMs
-    // (a cluster's blocks share a part of the chip, so an eighth of the SMs is left out)
-    const int64_t steps = (a.K + kKps * kBK - 1) / (kKps * kBK);
-    a.splits = (int)std::max<int64_t>(1, std::min<int64_t>({8, steps / 4, sm_count() * 7 / 8 / tiles}));
-    a.per = (int)((steps + a.splits - 1) / a.splits);
-    a.splits = (int)((steps + a.per - 1) / a.per);
-    return a.splits > 1 ? launch_codes_as<BN, SHIFT, true>(a, tiles, st) : launch_codes_as<BN, SHIFT, false>(a, tiles, st);
+    // (a cluster's blocks share a part of the chip, so an eighth of the SMs is left out; tiles of 128 rows of A, taken
+    // when those of 64 are more than a wave, never do)
+    if constexpr (BN == 64) {
+        const int64_t steps = (a.K + kKps * kBK - 1) / (kKps * kBK);
+        a.splits = (int)std::max<int64_t>(1, std::min<int64_t>({8, steps / 4, sm_count() * 7 / 8 / tiles}));
+        a.per = (int)((steps + a.splits - 1) / a.splits);
+        a.splits = (int)((steps + a.per - 1) / a.per);
+        if (a.splits > 1) return launch_codes_as<BN, SHIFT, true>(a, tiles, st);
+    }
+    return launch_codes_as<BN, SHIFT, false>(a, tiles, st);
 }
 
 }  // namespace

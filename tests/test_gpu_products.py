@@ -112,9 +112,10 @@ def test_tensor_core_outputs(qnn, M, N, K, pad, bn, shift, monkeypatch):
     assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
 
 
-# The product from the codes: rows of A around its 64 and 128 columns, rows of W around 128, K around 16
-# codes, the ring's four stages and three k-blocks of loads ahead, chunks of 1024 (drained late, a last chunk
-# of one to three k-blocks), every row shift, raw sums, sums of 32 and of 64 bits.
+# The product from the codes: rows of A around its 64 and 128 columns, rows of W around 128, K around 16 codes,
+# a stage of 128 codes (one and two k-blocks of it), the ring's three stages with two of loads ahead, chunks of
+# eight stages (drained a stage into the next; a last chunk of one stage, or of part of one), every row shift, raw
+# sums, sums of 32 and of 64 bits.
 @pytest.mark.parametrize("M,N,K", [(1, 1, 40), (5, 6, 7), (63, 127, 15), (64, 128, 16), (65, 129, 17), (100, 260, 63), (129, 2000, 64),
                                    (130, 500, 65), (200, 9000, 127), (128, 20000, 193), (128, 130, 256), (129, 136, 321),
                                    (300, 300, 1000), (128, 64, 1024), (130, 132, 1025), (96, 128, 1088), (70, 200, 1153),
@@ -163,6 +164,31 @@ def test_tensor_core_raw_sums(qnn, M, N, K, nb, pad, bn, monkeypatch):
     assert qnn.device_status() == qnn.QNN_OK
     assert np.array_equal(acc.cpu().numpy(), ref["acc"]) and np.array_equal(out[:M, :N].cpu().numpy(), ref["y"])
     assert bool((out[M:] == 7.0).all()) and bool((out[:, N:] == 7.0).all())
+
+
+# One and two tiles share their reductions between the blocks of a cluster: `parts` of them with K, the last one of
+# one stage, of less than a stage or of an odd number of k-blocks, and chunks that end inside a part.
+@pytest.mark.parametrize("M,N", [(33, 128), (64, 250), (70, 100)])
+@pytest.mark.parametrize("K,parts", [(1023, 2), (1024, 2), (1600, 3), (1665, 3), (2049, 4), (2600, 5), (2561, 5), (4096, 8), (4100, 7), (8200, 8), (33025, 8)])
+@pytest.mark.parametrize("pad,off", [(None, 0), (0, 0), (3, 1)])
+def test_codes_shared_reductions(qnn, M, N, K, parts, pad, off, monkeypatch):
+    monkeypatch.setenv("QNN_QGEMM", "codes")
+    steps = -(-K // 128)  # stages; the rule of launch_codes where SMs are plenty
+    splits = max(1, min(8, steps // 4))
+    assert -(-steps // -(-steps // splits)) == parts
+    g = np.random.Generator(np.random.PCG64(M + N + K))
+    ca, pa, ra = oracle.quantize(g.normal(0.1, 1.0, (M, K)).astype(np.float32), oracle.PER_ROW)
+    cw, pw, cs = oracle.quantize(g.normal(0.0, 1.0, (N, K)).astype(np.float32), oracle.PER_MATRIX)
+    ref = oracle.qmatmul(ca, pa, oracle.PER_ROW, cw, pw)
+    ld = (K + 15) // 16 * 16 if pad is None else K + pad
+    qnn.profile_read()
+    qnn.profile_enable(True)
+    Y, acc = qnn.qnn_qmatmul(strided(ca, ld, off), qnn.params_tensor(pa), oracle.PER_ROW, gpu(ra), strided(cw, ld, off),
+                             qnn.params_tensor(pw), gpu(cs), want_acc=True)
+    qnn.profile_enable(False)
+    assert "qgemm_codes_split" in qnn.profile_read()
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(acc.cpu().numpy(), ref["acc"]) and np.array_equal(Y.cpu().numpy(), ref["y"])
 
 
 # Operands too small to hold one aligned unit take another path than the one the sizes ask for.
