@@ -9,11 +9,20 @@
 
 namespace qnn {
 
+struct Held {  // a stream's scratch: grown in its order
+    unsigned long long stream = 0;
+    void *p = nullptr;
+    size_t bytes = 0;
+    int calls = 0;  // being made with it
+};
+
 namespace {
 
 constexpr int kMaxDevices = 64;
 
 struct DeviceState {
+    Held held[kHeldStreams];
+    int held_streams = 0;
     cudaMemPool_t pool = nullptr;
     size_t pool_keeps = 0;
     char *reduce = nullptr;  // kReduceStreams slots
@@ -58,6 +67,10 @@ qnn_status Scratch::take(size_t bytes, cudaStream_t st) {
     int dev = 0;
     QNN_TRY(current(&dev));
     cudaMemPool_t pool = nullptr;
+    unsigned long long id = 0;  // (of the process's life: a later stream at the same address has another)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    QNN_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+    if (cap == cudaStreamCaptureStatusNone) QNN_CUDA_TRY(cudaStreamGetId(st, &id));
     {
         std::lock_guard<std::mutex> lk(g_mu);
         DeviceState &d = g_dev[dev];
@@ -75,6 +88,22 @@ qnn_status Scratch::take(size_t bytes, cudaStream_t st) {
             d.pool_keeps = keeps;
         }
         pool = d.pool;
+        int i = 0;
+        while (i < d.held_streams && d.held[i].stream != id) ++i;
+        // (not while another thread launches with it: two calls' kernels could follow one another in any order)
+        if (cap == cudaStreamCaptureStatusNone && bytes <= kHeldBytes && i < kHeldStreams && d.held[i].calls == 0) {
+            Held &h = d.held[i];
+            if (h.bytes < bytes) {
+                if (h.p) QNN_CUDA_TRY(cudaFreeAsync(h.p, st));  // (what used it is on the stream already)
+                h.p = nullptr, h.bytes = 0;
+                QNN_CUDA_TRY(cudaMallocFromPoolAsync(&h.p, bytes, pool, st));
+                h.bytes = bytes;
+            }
+            if (i == d.held_streams) h.stream = id, ++d.held_streams;
+            ++h.calls;
+            p_ = h.p, held_ = &h;
+            return QNN_OK;
+        }
     }
     QNN_CUDA_TRY(cudaMallocFromPoolAsync(&p_, bytes, pool, st));
     pooled_ = true, st_ = st;
@@ -88,7 +117,7 @@ qnn_status Scratch::take_reduce(cudaStream_t st) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     QNN_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
     if (cap == cudaStreamCaptureStatusNone) {
-        unsigned long long id = 0;  // (of the process's life: a later stream at the same address has another)
+        unsigned long long id = 0;
         QNN_CUDA_TRY(cudaStreamGetId(st, &id));
         std::lock_guard<std::mutex> lk(g_mu);
         DeviceState &d = g_dev[dev];
@@ -115,6 +144,10 @@ qnn_status Scratch::take_reduce(cudaStream_t st) {
 }
 
 Scratch::~Scratch() {
+    if (held_) {
+        std::lock_guard<std::mutex> lk(g_mu);
+        --held_->calls;
+    }
     if (pooled_ && cudaFreeAsync(p_, st_) != cudaSuccess) cudaGetLastError();
 }
 
@@ -122,7 +155,14 @@ void scratch_trim() {
     int dev = 0;
     if (current(&dev) != QNN_OK) return;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (g_dev[dev].pool) cudaMemPoolTrimTo(g_dev[dev].pool, 0);
+    DeviceState &d = g_dev[dev];
+    if (!d.pool || cudaDeviceSynchronize() != cudaSuccess) return;
+    for (Held &h : d.held)
+        if (h.p && h.calls == 0) {
+            cudaFree(h.p);
+            h.p = nullptr, h.bytes = 0;
+        }
+    cudaMemPoolTrimTo(d.pool, 0);
 }
 
 qnn_status status_word(int **out) {

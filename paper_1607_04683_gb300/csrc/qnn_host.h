@@ -48,13 +48,16 @@ void *host_mapped_ptr(void *p);
 
 // Device scratch of one call on one stream of the current device, never shared with a call that may run at the
 // same time: calls on other streams, and replays of a captured graph, have their own.
-//   take():        from a pool of the library's on the stream's order, given back to it at the end of the scope. The
-//                  pool keeps the largest request, or 1 GiB; what concurrent calls took beyond is freed at a
-//                  synchronization.
+//   take():        a buffer held for the stream, of up to kHeldBytes and for the first kHeldStreams streams, or memory
+//                  from a pool of the library's on the stream's order, given back to it at the end of the scope (which
+//                  costs about 1.2 us of the stream's time: 4096 x 2048 x 512 28.0 us a product, so 26.8). The pool keeps
+//                  the largest request, or 1 GiB; what concurrent calls took beyond is freed at a synchronization.
 //   take_reduce(): the per-matrix quantizer's block partials (kReduceBlocks of them an SM at most) behind a counter that
 //                  is 0, and that the kernel leaves 0: a slot of the stream's own, for the first kReduceStreams
 //                  streams, or memory as above with the counter cleared on the stream.
 // In a capture both are allocation nodes of the graph.
+constexpr int kHeldStreams = 4;
+constexpr size_t kHeldBytes = (size_t)256 << 20;
 constexpr int kReduceBlocks = 4, kReduceStreams = 64;
 constexpr size_t kReduceHeader = 256;
 class Scratch {
@@ -72,9 +75,10 @@ class Scratch {
   private:
     void *p_ = nullptr;
     bool pooled_ = false;
+    struct Held *held_ = nullptr;
     cudaStream_t st_ = nullptr;
 };
-// Frees what the pool keeps on the current device and no call holds.
+// Frees what is held and what the pool keeps on the current device, apart from the buffers of calls being made.
 void scratch_trim();
 
 // The device status word of the current device (allocated and zeroed on first use).

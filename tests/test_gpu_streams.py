@@ -91,11 +91,12 @@ def test_more_streams_than_slots(qnn, calls):
     assert all(c.right(o) for c, o in outs)
 
 
-def test_threads(qnn, calls):
-    bad = []
+@pytest.mark.parametrize("shared", [False, True])
+def test_threads(qnn, calls, shared):
+    bad, one = [], torch.cuda.Stream()
 
     def work(i):
-        st = torch.cuda.Stream()
+        st = one if shared else torch.cuda.Stream()
         with torch.cuda.stream(st):
             for k in range(30):
                 c = calls[(i + k) % len(calls)]
