@@ -7,8 +7,8 @@
 // ones are re-read from L1/L2. A per-matrix unit first reduces block partials into a small scratch array; the last
 // block to finish folds them into the unit's parameters, then a second launch writes codes.
 //
-// Bound: HBM (5 bytes a value for rows, 9 for a matrix beyond L2). Per matrix 8192 x 8192: 117 us with one
-// 16-byte load in flight a lane and both passes from HBM; 101 us with eight in flight and the code pass
+// Bound: HBM (5 bytes a value for rows, 9 for a matrix beyond L2). Per matrix 8192 x 8192: 118 us with one
+// 16-byte load in flight a lane and both passes from HBM; 98.5 us with eight in flight and the code pass
 // starting where the range pass ended, in rows that L2 still holds.
 #include <algorithm>
 #include <cfloat>
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
 // registers, NV float4 per lane, so the row is read once and the code pass needs no second read. A warp
 // takes every gridDim kRowWarps-th row, and rows of at most 512 values are loaded while the row before is
 // reduced and coded: the loads of one row alone leave memory idle through its reductions (128000 x 500:
-// 71.9 us, 4.5 TB/s, with a row a warp; 59.4 us, 5.4 TB/s, so).
+// 72.0 us, 4.5 TB/s, with a row a warp; 55.3 us, 5.8 TB/s, so).
 template <int NV>
 __device__ __forceinline__ void load_row(float4 (&v)[NV], const float *__restrict__ xr, int cols) {
     const int lane = threadIdx.x & 31;

@@ -184,8 +184,8 @@ def _p(t):
 
 def _stream(stream):
     """Raw handle of stream, or of the current stream of the current device. A product of one frame is bound
-    by the host: 2048 x 2048 took 19.8 us a call with a Stream object and wrapped pointers made for each
-    call, 12.6 us without."""
+    by the host: 13.5 us of its time a call with a Stream object and wrapped pointers made for each call, 7.5 us
+    without (a result passed in; 14 to 17 us a call with one allocated, 2048 x 2048)."""
     if stream is not None:
         return stream.cuda_stream
     import torch
