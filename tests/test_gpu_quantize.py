@@ -96,3 +96,23 @@ def test_units_of_infinite_scale(qnn, form, cols, pad, off, tiny):
         return
     for k in kinds:
         check(qnn, k, cols + pad, off, oracle.PER_MATRIX, static=form == "static")
+
+
+# Frames and states whose units have an infinite scale: the recurrences recover 0 from any of their codes, on each path.
+@pytest.mark.parametrize("path,B", [("small", 2), ("persist", 9), ("layerwise", 9), ("tc", 66)])
+def test_recurrence_on_units_of_infinite_scale(qnn, path, B, monkeypatch):
+    monkeypatch.setenv("QNN_LSTM_PATH", path)
+    L, I, H, T = 2, 24, 32, 3
+    g = np.random.Generator(np.random.PCG64(B))
+    d = oracle.desc(L, I, H, 0, 0, oracle.OUT_NONE)
+    params = g.uniform(-0.5, 0.5, oracle.lstm_param_count(d)).astype(np.float32)
+    x = g.normal(0, 1, (B, T, I)).astype(np.float32)
+    x[:, 0] *= np.float32(1e-38)  # a frame of every sequence, and every frame of some
+    x[::2] *= np.float32(1e-38)
+    h0, c0 = ((g.normal(0, 1, (L, B, H)) * 1e-39).astype(np.float32) for _ in range(2))
+    ref = oracle.lstm_forward(d, params, x, h0=h0, c0=c0, want_h_all=True)
+    model = qnn.LstmModel(qnn.lstm_desc(L, I, H), torch.from_numpy(params).cuda())
+    hs, cs, ha = torch.from_numpy(h0.copy()).cuda(), torch.from_numpy(c0.copy()).cuda(), torch.empty((L, B, T, H), device="cuda")
+    model.forward(torch.from_numpy(x).cuda(), h_state=hs, c_state=cs, h_all=ha)
+    assert qnn.device_status() == qnn.QNN_OK
+    assert np.array_equal(ha.cpu().numpy(), ref["h_all"]) and np.array_equal(cs.cpu().numpy(), ref["c"])
