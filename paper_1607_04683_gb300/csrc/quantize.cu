@@ -28,7 +28,9 @@ constexpr int kFlight = 8;    // loads (of 16 bytes, or of one value where rows 
 constexpr int kMidRow = 512;  // shorter ones take one, and the registers of more rows at once (100000 x 60: range 28 us
                               // with eight, 21 with one)
 // Matrix rows that are not aligned, a value a load: eight in flight from 128 values on, four from 64 (one, four and
-// eight: 200000 x 65 57, 51 and 60 us, x 95 67, 57 and 65; 150000 x 129 60, 63 and 54, 256410 x 234 178, 133 and 108).
+// eight: 200000 x 65 57, 51 and 60 us, x 95 67, 57 and 65; 150000 x 129 60, 63 and 54, 256410 x 234 178, 133 and 108). The last kLooseRest values or fewer
+// go one by one (100000 x 257 58.2 us with a second round of eight for one value, so 53.9).
+constexpr int kLooseRest = 64;
 inline int loose_flight(int64_t cols) { return cols >= 128 ? kFlight : cols >= 64 ? 4 : 1; }
 
 // Running range of values and whether one was not finite: v * 0 is NaN then, and so is the sum.
@@ -63,11 +65,10 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
         }
         done = n4 << 2;
     }
-    if (kVec || F == 1) {
-        for (int i = done + lane; i < cols; i += 32) r.add(__ldg(xr + i));
-    } else {
-        for (int i = lane; i < cols; i += 32 * F) {
+    if (!kVec && F > 1) {
+        for (; cols - done > kLooseRest; done += 32 * F) {
             float v[F];
+            const int i = done + lane;
 #pragma unroll
             for (int u = 0; u < F; ++u)
                 if (i + 32 * u < cols) v[u] = __ldg(xr + i + 32 * u);
@@ -76,6 +77,7 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
                 if (i + 32 * u < cols) r.add(v[u]);
         }
     }
+    for (int i = done + lane; i < cols; i += 32) r.add(__ldg(xr + i));
     mn = warp_min(r.mn);
     mx = warp_max(r.mx);
     return __all_sync(0xffffffffu, r.finite());
@@ -111,8 +113,10 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
             cr[i] = (uint8_t)a;
         }
     } else {
-        for (int i = lane; i < cols; i += 32 * F) {
+        int done = 0;
+        for (; F > 1 && cols - done > kLooseRest; done += 32 * F) {
             float v[F];
+            const int i = done + lane;
 #pragma unroll
             for (int u = 0; u < F; ++u)
                 if (i + 32 * u < cols) v[u] = __ldg(xr + i + 32 * u);
@@ -123,6 +127,11 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
                 s += (int)a;
                 cr[i + 32 * u] = (uint8_t)a;
             }
+        }
+        for (int i = done + lane; i < cols; i += 32) {
+            const uint32_t a = unit.code(__ldg(xr + i));
+            s += (int)a;
+            cr[i] = (uint8_t)a;
         }
     }
     return warp_sum(s);
@@ -406,8 +415,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) matrix_codes_kernel(const floa
                                                                      int64_t ldc, const qnn_qparams *__restrict__ params,
                                                                      int32_t *__restrict__ sums) {
     const int64_t groups = (rows + kRowWarps - 1) / kRowWarps;
-    // once a block, of a grid of two waves: in blocks of eight short rows the wait took most of the time (197307 x 57:
-    // 87 us, so 31), and with one wave the last rows' blocks leave warps idle (246038 x 24: 38 us, so 35)
+    // once a block, of a grid of one wave: in blocks of eight short rows the wait took most of the time (197307 x 57:
+    // 87 us, so 31). Two waves from 48 blocks an SM on, where one leaves warps idle at its end (67556 x 118 of 121 apart
+    // 36.7 us a call, so 34.5; but 20000 x 300 18.5 and 21.7)
     grid_dependency_wait();
     const UnitCoder unit(__ldcg(&params[0].Q), __ldcg(&params[0].z));
     for (int64_t b = blockIdx.x; b < groups; b += gridDim.x) {
@@ -480,7 +490,7 @@ qnn_status launch_quantize_matrix(const float *x, int64_t rows, int64_t cols, in
     // programmatic dependent launch: the blocks are set up while the range pass ends (they wait for it)
     cudaLaunchConfig_t cfg = {};
     const bool long_rows = cols >= kLongRow && rows <= INT32_MAX;
-    cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, 16 * (int64_t)sm_count())));
+    cfg.gridDim = dim3((unsigned)(long_rows ? rows : std::min<int64_t>(want, (want >= 48 * (int64_t)sm_count() ? 16 : 8) * (int64_t)sm_count())));
     cfg.blockDim = dim3(kRowWarps * 32);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
