@@ -29,7 +29,9 @@ constexpr int kMidRow = 512;  // shorter ones take one, and the registers of mor
                               // with eight, 21 with one)
 // Matrix rows that are not aligned, a value a load: eight in flight from 128 values on, four from 64 (one, four and
 // eight: 200000 x 65 57, 51 and 60 us, x 95 67, 57 and 65; 150000 x 129 60, 63 and 54, 256410 x 234 178, 133 and 108). The last kLooseRest values or fewer
-// go one by one (100000 x 257 58.2 us with a second round of eight for one value, so 53.9).
+// go one by one (100000 x 257 58.2 us with a second round of eight for one value, so 53.9). WHOLE: whole rounds take no
+// tests, for rows of their own (7722 x 7770 109 us with a test a value, so 98; 40000 x 600 31 and 27) but not for matrices
+// (22002 x 2727 103 us with tests, 116 without).
 constexpr int kLooseRest = 64;
 inline int loose_flight(int64_t cols) { return cols >= 128 ? kFlight : cols >= 64 ? 4 : 1; }
 
@@ -46,7 +48,7 @@ struct Range {
 };
 
 // Range of one row held by one warp; returns false if a value is not finite.
-template <bool kVec, int F>
+template <bool kVec, int F, bool WHOLE = false>
 __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int cols, float &mn, float &mx) {
     const int lane = threadIdx.x & 31;
     Range r;
@@ -66,6 +68,13 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
         done = n4 << 2;
     }
     if (!kVec && F > 1) {
+        for (; WHOLE && done + 32 * F <= cols; done += 32 * F) {
+            float v[F];
+#pragma unroll
+            for (int u = 0; u < F; ++u) v[u] = __ldg(xr + done + lane + 32 * u);
+#pragma unroll
+            for (int u = 0; u < F; ++u) r.add(v[u]);
+        }
         for (; cols - done > kLooseRest; done += 32 * F) {
             float v[F];
             const int i = done + lane;
@@ -84,7 +93,7 @@ __device__ __forceinline__ bool warp_row_range(const float *__restrict__ xr, int
 }
 
 // Codes of one row (eq. 2) and their sum, one warp.
-template <bool kVec, int F>
+template <bool kVec, int F, bool WHOLE = false>
 __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int cols, const UnitCoder &unit,
                                               uint8_t *__restrict__ cr) {
     const int lane = threadIdx.x & 31;
@@ -114,6 +123,17 @@ __device__ __forceinline__ int warp_row_codes(const float *__restrict__ xr, int 
         }
     } else {
         int done = 0;
+        for (; WHOLE && F > 1 && done + 32 * F <= cols; done += 32 * F) {
+            float v[F];
+#pragma unroll
+            for (int u = 0; u < F; ++u) v[u] = __ldg(xr + done + lane + 32 * u);
+#pragma unroll
+            for (int u = 0; u < F; ++u) {
+                const uint32_t a = unit.code(v[u]);
+                s += (int)a;
+                cr[done + lane + 32 * u] = (uint8_t)a;
+            }
+        }
         for (; F > 1 && cols - done > kLooseRest; done += 32 * F) {
             float v[F];
             const int i = done + lane;
@@ -190,14 +210,14 @@ __global__ void __launch_bounds__(kRowWarps * 32) quantize_rows_kernel(const flo
     if (row >= rows) return;
     const float *xr = x + row * ldx;
     float mn, mx;
-    bool ok = warp_row_range<kVec, F>(xr, cols, mn, mx);
+    bool ok = warp_row_range<kVec, F, true>(xr, cols, mn, mx);
     if (!ok) {
         if ((threadIdx.x & 31) == 0) record_status(status, QNN_ERR_NONFINITE);
         mn = 0.0f;
         mx = 0.0f;
     }
     qnn_qparams p = params_from_range(mn, mx);
-    int s = warp_row_codes<kVec, F>(xr, cols, UnitCoder(p.Q, p.z), codes + row * ldc);
+    int s = warp_row_codes<kVec, F, true>(xr, cols, UnitCoder(p.Q, p.z), codes + row * ldc);
     if ((threadIdx.x & 31) == 0) {
         params[row] = p;
         if (sums) sums[row] = s;
